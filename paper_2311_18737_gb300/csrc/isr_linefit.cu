@@ -11,72 +11,95 @@
 #include <cstdio>
 
 #include "isr.h"
+#include "isr_ff.cuh"
 #include "isr_kernels.cuh"
 
 namespace {
 
 constexpr int kFitThreads = 256;
 
+// One CTA per gate.  4 bytes per bin bound it; the band's sum runs in float-float on the FP32 pipe
+// (an FP64 conversion and addition per bin bound it before: 34.7 us for 1000 gates x 4608 bins), and
+// the three logarithms and the two quotients run side by side in lanes of one warp, each FP64
+// instruction of which occupies the narrow pipe as long for one lane as for all.  A band whose
+// float-float sum is not finite (an infinity, a NaN, or an FP32 overflow) is summed again in FP64.
 __global__ void __launch_bounds__(kFitThreads) peak_fit_kernel(const float* __restrict__ spectra, int nfft,
                                                                int band_lo, int band_hi, double* __restrict__ freq_bin,
                                                                float* __restrict__ snr)
 {
+    constexpr int W = kFitThreads / 32, U = 8;
     const int r = blockIdx.x;
     const float* P = spectra + (size_t)r * nfft;
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     float best = -INFINITY;
     int best_i = band_lo;
-    double sum = 0.0;
-    for (int i = band_lo + threadIdx.x; i < band_hi; i += kFitThreads) {
-        float v = P[i];
+    isr::ff sum{0.f, 0.f};
+    auto take = [&](int i, float v) {
         if (v > best) {  // strided scan in increasing i keeps the lowest index on ties
             best = v;
             best_i = i;
         }
-        sum += (double)v;
+        isr::ff_acc(sum, v);
+    };
+    int i = band_lo + threadIdx.x;
+    for (; i + (U - 1) * kFitThreads < band_hi; i += U * kFitThreads) {
+        float v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = P[i + u * kFitThreads];
+#pragma unroll
+        for (int u = 0; u < U; ++u) take(i + u * kFitThreads, v[u]);
     }
-    // block reduction: max value, lowest index among equal maxima; double sum
-    __shared__ float s_best[kFitThreads / 32];
-    __shared__ int s_idx[kFitThreads / 32];
-    __shared__ double s_sum[kFitThreads / 32];
-    for (int o = 16; o > 0; o >>= 1) {
-        float ob = __shfl_down_sync(0xffffffffu, best, o);
-        int oi = __shfl_down_sync(0xffffffffu, best_i, o);
-        double os = __shfl_down_sync(0xffffffffu, sum, o);
+    for (; i < band_hi; i += kFitThreads) take(i, P[i]);
+    // block reduction: max value, lowest index among equal maxima; sum
+    __shared__ float s_best[W];
+    __shared__ int s_idx[W];
+    __shared__ isr::ff s_sum[W];
+    auto merge = [&](float ob, int oi) {
         if (ob > best || (ob == best && oi < best_i)) {
             best = ob;
             best_i = oi;
         }
-        sum += os;
+    };
+    for (int o = 16; o > 0; o >>= 1) {
+        const float ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, best_i, o);
+        merge(ob, oi);
     }
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    sum = isr::ff_warp_sum(isr::ff_norm(sum.h, sum.l));
     if (l == 0) {
         s_best[w] = best;
         s_idx[w] = best_i;
         s_sum[w] = sum;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        best = s_best[0];
-        best_i = s_idx[0];
-        sum = s_sum[0];
-        for (int k = 1; k < kFitThreads / 32; ++k) {
-            if (s_best[k] > best || (s_best[k] == best && s_idx[k] < best_i)) {
-                best = s_best[k];
-                best_i = s_idx[k];
-            }
-            sum += s_sum[k];
-        }
-        const double mean = sum / (double)(band_hi - band_lo);
-        const double pm = P[(best_i - 1 + nfft) % nfft], p0 = best, pp = P[(best_i + 1) % nfft];
-        double delta = 0.0;
-        if (pm > 0.0 && p0 > 0.0 && pp > 0.0) {
-            const double ym = log(pm), y0 = log(p0), yp = log(pp);
-            const double d = ym - 2.0 * y0 + yp;
-            if (d < 0.0) delta = 0.5 * (ym - yp) / d;
-            delta = fmin(0.5, fmax(-0.5, delta));
-        }
+    if (w != 0) return;
+    best = s_best[0];
+    best_i = s_idx[0];
+    for (int k = 1; k < W; ++k) merge(s_best[k], s_idx[k]);
+    sum = isr::ff_warp_sum(l < W ? s_sum[l] : isr::ff{0.f, 0.f});
+    double total = isr::ff_to_double(sum);
+    if (!isfinite(sum.h) || !isfinite(sum.l)) {
+        total = 0.0;
+        for (int j = band_lo + l; j < band_hi; j += 32) total += (double)P[j];
+        for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+    }
+    // lanes 0, 1, 2: the bins before, at and after the peak
+    const int at = l == 0 ? (best_i - 1 + nfft) % nfft : l == 2 ? (best_i + 1) % nfft : best_i;
+    const double v = l == 1 ? (double)best : (double)P[at];
+    const bool positive = (__ballot_sync(0xffffffffu, v > 0.0) & 7u) == 7u;
+    const double y = positive ? log(v) : 0.0;
+    const double ym = __shfl_sync(0xffffffffu, y, 0), y0 = __shfl_sync(0xffffffffu, y, 1),
+                 yp = __shfl_sync(0xffffffffu, y, 2);
+    const double d = ym - 2.0 * y0 + yp;
+    // lane 0: the parabola's offset; lane 1: peak over mean, as best / (total / n)
+    const double mean = total / (double)(band_hi - band_lo);
+    const double quot = (l == 0 ? 0.5 * (ym - yp) : (double)best) / (l == 0 ? d : mean);
+    if (l == 0) {
+        double delta = positive && d < 0.0 ? quot : 0.0;
+        if (positive) delta = fmin(0.5, fmax(-0.5, delta));
         freq_bin[r] = (double)best_i + delta;
-        snr[r] = mean > 0.0 ? (float)(p0 / mean) : 0.f;
+    } else if (l == 1) {
+        snr[r] = mean > 0.0 ? (float)quot : 0.f;
     }
 }
 
