@@ -153,6 +153,24 @@ def test_features_match_reference():
     e.close()
 
 
+@pytest.mark.parametrize("L", [16, 37, 511, 513, 5120, 5121, 12000])
+def test_features_band_lengths_and_floors(L):
+    """Bands within and beyond the bins a thread keeps in registers, with bins at, below and far above
+    the 1e-30 floor.  The logarithms carry about 2^-42, so a feature is one FP32 rounding (2^-24
+    relative) of the exact one plus 2^-42 / std; 1.2e-7 |x| + 1e-9 covers both at std >= 0.01."""
+    rng = np.random.default_rng(L)
+    P = rng.gamma(30.0, 2.0, size=(4, L + 3)).astype(np.float32)
+    P[1] *= np.exp(rng.uniform(-60, 60, L + 3)).astype(np.float32)
+    P[2, 1:6] = [0.0, -4.0, 1e-30, 1e-31, 3e38]
+    P[3, 4] = np.nan
+    e = est_mod.Estimator(max_batch=4, precision=isr.ISR_EST_FP32, nfft=L + 3, band_lo=1, band_len=L)
+    x = e.features(torch.from_numpy(P).cuda()).cpu().numpy()
+    e.close()
+    P[3, 4] = 0.0                       # NaN counts as the floor
+    want = ref.features(P, 1, L)
+    assert (np.abs(x - want) <= 1.2e-7 * np.abs(want) + 1e-9).all()
+
+
 @pytest.mark.slow
 def test_training_gains_over_peak_fit():
     """Short training on integrator-made spectra (reduced from the full 200k-spectrum run):
