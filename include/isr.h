@@ -153,16 +153,18 @@ isr_status isr_plan_phase_cycles(isr_plan* plan, uint64_t out[5]);
 isr_status isr_plan_set_wait_limit(isr_plan* plan, uint32_t polls);
 
 /* Radix order (0..9) of the kernel used for binary-phase codes with code_len == nfft, for
- * nfft >= 2048 (smaller sizes have one order): 0..2 are three-pass Stockham orders, 3 is a
- * radix-(nfft/1024) decimation-in-frequency pass followed by one 1024-point transform per
- * warp; 4 and 5 (nfft 16384 only) use paired FP32 instructions (two operations each):
- * 4 the passes [4, 16, 16, 16] with each thread transforming two butterflies at once,
- * 5 the passes [16, 32, 32] of order 1 with two butterflies per thread in the first pass
- * and each radix-32 butterfly split into two paired 16-point halves; 6, 7 and 8 (nfft
- * 16384 only) are orders 0, 1 and 2 with every thread's inter-pass twiddles computed once
- * per CTA into tensor memory (all 512 columns of the SM's TMEM, freed when the CTA ends)
- * instead of being formed from tables and recurrences in every IPP; 9 (nfft 16384 only) is
- * order 3 with its twiddles in tensor memory likewise and unit-stride first-pass columns.
+ * nfft >= 2048 (smaller sizes have one order): 0 (the default, and the kernel of every other code
+ * from nfft 1024 up) is the passes [32, 32, nfft / 1024] with the last exchange and the inter-pass
+ * twiddles in tensor memory (all 512 columns of the SM's TMEM, freed when the CTA ends); 1 and 2
+ * are three-pass Stockham orders, 3 is a radix-(nfft/1024) decimation-in-frequency pass followed
+ * by one 1024-point transform per warp; 4 and 5 (nfft 16384 only) use paired FP32 instructions
+ * (two operations each): 4 the passes [4, 16, 16, 16] with each thread transforming two
+ * butterflies at once, 5 the passes [16, 32, 32] of order 1 with two butterflies per thread in
+ * the first pass and each radix-32 butterfly split into two paired 16-point halves; 6 (nfft 16384
+ * only) is order 0; 7 and 8 (nfft 16384 only) are orders 1 and 2 with every thread's inter-pass
+ * twiddles computed once per CTA into tensor memory instead of being formed from tables and
+ * recurrences in every IPP; 9 (nfft 16384 only) is order 3 with its twiddles in tensor memory
+ * likewise and unit-stride first-pass columns.
  * Every order gives the same spectra up to FP32 rounding; they differ in speed, so a caller (or the
  * binding's autotuner) may time them and keep the fastest.  Default 0. */
 isr_status isr_plan_set_order(isr_plan* plan, int32_t order);

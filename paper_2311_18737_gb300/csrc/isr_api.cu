@@ -32,6 +32,27 @@ isr_status fail(isr_status st, const char* fmt, ...)
     return st;
 }
 void clear_error() { g_err[0] = 0; }
+
+cudaError_t prepare_entry(const KernelEntry& ke, int log2n, int dev, cudaStream_t stream)
+{
+    cudaError_t e = cudaSuccess;
+    auto set = [&](const void* fn, int smem) {
+        if (fn && e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    };
+    set(ke.fn, ke.smem);
+    for (int o = 0; o < kNumOrders; ++o) set(ke.fn_order[o], ke.smem_order[o]);
+    set(ke.fn_xt, ke.smem_xt);
+    if (e != cudaSuccess || !ke.fn_tables) return e;
+    // the tables are the same for every user: filled under the lock, complete before it is released
+    static std::mutex mu;
+    static uint32_t filled[64] = {};   // bit log2n per device
+    std::lock_guard<std::mutex> lock(mu);
+    if (dev >= 0 && dev < 64 && (filled[dev] >> log2n & 1u)) return cudaSuccess;
+    e = cudaLaunchKernel(ke.fn_tables, dim3(32), dim3(128), nullptr, 0, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    if (e == cudaSuccess && dev >= 0 && dev < 64) filled[dev] |= 1u << log2n;
+    return e;
+}
 }  // namespace isr
 
 namespace {
@@ -63,6 +84,7 @@ struct DeviceGuard {
 constexpr unsigned kDefaultWaitLimit = 1u << 22;
 constexpr int kDefaultChunk = 256;
 constexpr int64_t kScratchBudget = int64_t(4) << 30;   // bytes of chunk partials
+constexpr int64_t kSignBytes = int64_t(16) << 20;      // packed chip signs of one launch
 constexpr int64_t kHostStageBytes = int64_t(1) << 30;   // per host-input staging buffer
 constexpr int64_t kHostFirstBytes = int64_t(64) << 20;   // first block of a host-input call
 
@@ -157,6 +179,8 @@ struct isr_plan {
     cudaEvent_t hs_free[2] = {nullptr, nullptr};
     cudaEvent_t hs_t[4] = {nullptr, nullptr, nullptr, nullptr};   // block 0: copy start / end, kernels start / end
     int64_t hs_growth = 0;    // block growth the last multi-block host-input call measured (0: none yet)
+    uint32_t* signs = nullptr;   // packed chip signs of per-IPP binary-phase codes, sign_rows x nfft / 32 words
+    int64_t sign_rows = 0;
     unsigned long long* phase = nullptr;   // debug builds: [5] phase cycles of the fused kernel
 };
 
@@ -209,9 +233,12 @@ isr_status launch_block(isr_plan* p, const uint32_t* echo, const char* tx, int64
     const int64_t RN = (int64_t)R * N;
     const int rg = (R + p->ke.gates - 1) / p->ke.gates;
     const int cb = chip_bytes(p->d.tx_type);
+    const bool full = p->d.code_len == p->d.nfft;
+    const bool pack = p->signs && p->precision == ISR_PREC_FP32 && isr::takes_xt(p->ke, full, p->order);
     int64_t done = 0;
     while (done < n) {
         int64_t n_l = std::min<int64_t>(n - done, (int64_t)p->max_chunks * p->ipp_chunk);
+        if (pack) n_l = std::min(n_l, p->sign_rows);
         // chunks: enough for the FP32 sum length cap, and enough CTAs for two waves
         int64_t c_min = (n_l + p->ipp_chunk - 1) / p->ipp_chunk;
         int64_t c_fill = (2 * (int64_t)p->sm_count + rg - 1) / rg;
@@ -236,23 +263,29 @@ isr_status launch_block(isr_plan* p, const uint32_t* echo, const char* tx, int64
         a.wait_limit = p->wait_limit;
         a.drop_ipp = (p->drop_ipp >= done && p->drop_ipp < done + n_l) ? (int)(p->drop_ipp - done) : -1;
         a.phase_cycles = p->phase;
+        a.chip_bytes = cb;
 
+        if (pack) {
+            const int8_t* rows = static_cast<const int8_t*>(a.tx);
+            int n_rows = (int)n_l;
+            void* args[] = {&rows, &a.tx_stride, &a.code_len, &n_rows, &p->signs};
+            const int64_t blocks = std::min<int64_t>((n_l * (N / 32) + 255) / 256, (int64_t)p->sm_count * 8);
+            CUDA_TRY(cudaLaunchKernel(p->ke.fn_pack, dim3((unsigned)blocks), dim3(256), args, 0, p->stream));
+            a.signs = p->signs;
+        }
         std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
         if (p->prof) {
             ev.first = take_event(p);
             ev.second = take_event(p);
             if (ev.first && ev.second) CUDA_TRY(cudaEventRecord(ev.first, p->stream));
         }
-        void* args[] = {&a};
-        const bool full = p->d.code_len == p->d.nfft;
-        const void* fn = full ? p->ke.fn_order[p->order] : p->ke.fn;
-        int smem = full ? p->ke.smem_order[p->order] : p->ke.smem;
         if (p->precision != ISR_PREC_FP32) {
-            fn = p->ke.fn_tc[p->precision];
-            smem = p->ke.smem_tc;
+            void* args[] = {&a};
+            CUDA_TRY(cudaLaunchKernel(p->ke.fn_tc[p->precision], dim3((unsigned)rg, (unsigned)C),
+                                      dim3((unsigned)p->ke.threads), args, (size_t)p->ke.smem_tc, p->stream));
+        } else {
+            CUDA_TRY(isr::launch_integrate(p->ke, a, full, p->order, rg, (int)C, p->sm_count, p->stream));
         }
-        CUDA_TRY(cudaLaunchKernel(fn, dim3((unsigned)rg, (unsigned)C), dim3((unsigned)p->ke.threads), args,
-                                  (size_t)smem, p->stream));
         if (p->prof && ev.first && ev.second) {
             CUDA_TRY(cudaEventRecord(ev.second, p->stream));
             p->ev_pending.push_back(ev);
@@ -409,11 +442,10 @@ isr_status isr_plan_create(isr_plan** out, const isr_plan_desc* desc)
     if (e != cudaSuccess) return bail(fail(ISR_ERR_CUDA, "device query failed: %s", cudaGetErrorString(e)));
     int smem_optin = 0;
     cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (p->ke.smem > smem_optin)
-        return bail(fail(ISR_ERR_UNSUPPORTED, "kernel needs %d B shared memory, device allows %d", p->ke.smem, smem_optin));
-    e = cudaFuncSetAttribute(p->ke.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, p->ke.smem);
-    for (int o = 0; o < isr::kNumOrders && e == cudaSuccess; ++o)
-        e = cudaFuncSetAttribute(p->ke.fn_order[o], cudaFuncAttributeMaxDynamicSharedMemorySize, p->ke.smem_order[o]);
+    const int smem = std::max(p->ke.smem, p->ke.smem_xt);
+    if (smem > smem_optin)
+        return bail(fail(ISR_ERR_UNSUPPORTED, "kernel needs %d B shared memory, device allows %d", smem, smem_optin));
+    e = isr::prepare_entry(p->ke, lg, dev, p->stream);
     if (e != cudaSuccess) return bail(fail(ISR_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e)));
 
     const int64_t RN = (int64_t)d.n_ranges * d.nfft;
@@ -422,6 +454,11 @@ isr_status isr_plan_create(isr_plan** out, const isr_plan_desc* desc)
     e = cudaMalloc(&p->acc, (size_t)(RN * 8));
     if (e == cudaSuccess) e = cudaMalloc(&p->partial, (size_t)(mc * RN * 4));
     if (e == cudaSuccess) e = cudaMalloc(&p->status, sizeof(int));
+    if (e == cudaSuccess && p->ke.fn_pack && d.tx_stride > 0) {
+        const int64_t row = (int64_t)d.nfft / 32 * 4;
+        p->sign_rows = std::min<int64_t>(mc * p->ipp_chunk, kSignBytes / row);
+        e = cudaMalloc(&p->signs, (size_t)(p->sign_rows * row));
+    }
 #ifdef ISR_DEBUG
     if (e == cudaSuccess) e = cudaMalloc(&p->phase, 5 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemsetAsync(p->phase, 0, 5 * sizeof(unsigned long long), p->stream);
@@ -523,7 +560,7 @@ isr_status isr_plan_query(const isr_plan* p, isr_plan_info* info)
     info->n_ranges = p->d.n_ranges;
     info->ranges_per_cta = p->ke.gates;
     info->threads_per_cta = p->ke.threads;
-    info->smem_bytes = p->ke.smem;
+    info->smem_bytes = p->ke.fn_xt ? p->ke.smem_xt : p->ke.smem;
     info->max_chunks = p->max_chunks;
     info->ipp_chunk = p->ipp_chunk;
     info->sm_count = p->sm_count;
@@ -692,10 +729,10 @@ isr_status isr_integrate_static(const isr_plan_desc* desc, const int16_t* echo, 
     int lg = 0;
     while ((1 << lg) < d.nfft) ++lg;
     isr::KernelEntry ke = isr::kernel_entry(lg, d.tx_type);
-    CUDA_TRY(cudaFuncSetAttribute(ke.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, ke.smem));
     int sm_count = 0;
     CUDA_TRY(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev));
     cudaStream_t stream = static_cast<cudaStream_t>(d.stream);
+    CUDA_TRY(isr::prepare_entry(ke, lg, dev, stream));
 
     // Chunks: FP32 sums of at most kDefaultChunk IPPs (the bound the per-bin tolerance rests
     // on), at most c_cap of them in the scratch at once.  The IPPs run in blocks of at most
@@ -733,9 +770,8 @@ isr_status isr_integrate_static(const isr_plan_desc* desc, const int16_t* echo, 
         a.chunk_len = (int)chunk;
         a.wait_limit = kDefaultWaitLimit;
         a.drop_ipp = -1;
-        void* args[] = {&a};
-        CUDA_TRY(cudaLaunchKernel(ke.fn, dim3((unsigned)rg, (unsigned)C), dim3((unsigned)ke.threads), args,
-                                  (size_t)ke.smem, stream));
+        a.chip_bytes = cb;
+        CUDA_TRY(isr::launch_integrate(ke, a, false, 0, rg, (int)C, sm_count, stream));
         reduce_to_spectra_kernel<<<(unsigned)blocks, threads, 0, stream>>>(scratch, (int)C, RN, out, done > 0);
         CUDA_TRY(cudaGetLastError());
         done += n_l;
@@ -774,6 +810,7 @@ void isr_destroy(isr_plan* p)
     cudaFree(p->acc);
     cudaFree(p->partial);
     cudaFree(p->status);
+    cudaFree(p->signs);
     cudaFree(p->phase);
     cudaFree(p->out_stage);
     cudaGetLastError();

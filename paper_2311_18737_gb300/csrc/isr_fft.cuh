@@ -290,4 +290,30 @@ __device__ __forceinline__ void sdft(float2* v)
     if constexpr (R > 1) sdif22_stage<R, R, 0>(v);
 }
 
+// Group I (elements I, I + Q, I + 2Q, I + 3Q, Q = R / 4) of the first radix-2^2 level of sdft<R>, with
+// real factors on its inputs: the transform's inputs are x0, c1 x1, c2 x2 and c1 r31 x3.  The factors
+// ride on the level's additions (FMAs instead of plain adds), so a sign or the cosine of a twiddle
+// costs nothing here.
+template <int R, int I>
+__device__ __forceinline__ void sdft_first(float2* v, float c1, float c2, float r31)
+{
+    constexpr int Q = R / 4;
+    const float2 x0 = v[I], x1 = v[I + Q], x2 = v[I + 2 * Q], x3 = v[I + 3 * Q];
+    const float2 a0 = make_float2(fmaf(c2, x2.x, x0.x), fmaf(c2, x2.y, x0.y));
+    const float2 d0 = make_float2(fmaf(-c2, x2.x, x0.x), fmaf(-c2, x2.y, x0.y));
+    const float2 a1 = make_float2(fmaf(r31, x3.x, x1.x), fmaf(r31, x3.y, x1.y));
+    const float2 d1 = make_float2(fmaf(-r31, x3.x, x1.x), fmaf(-r31, x3.y, x1.y));
+    v[I] = make_float2(fmaf(c1, a1.x, a0.x), fmaf(c1, a1.y, a0.y));
+    v[I + Q] = tw_mul<2 * I, R>(make_float2(fmaf(-c1, a1.x, a0.x), fmaf(-c1, a1.y, a0.y)));
+    v[I + 2 * Q] = tw_mul<I, R>(make_float2(fmaf(c1, d1.y, d0.x), fmaf(-c1, d1.x, d0.y)));
+    v[I + 3 * Q] = tw_mul<3 * I, R>(make_float2(fmaf(-c1, d1.y, d0.x), fmaf(c1, d1.x, d0.y)));
+}
+
+// The levels of sdft<R> after the first.
+template <int R>
+__device__ __forceinline__ void sdft_rest(float2* v)
+{
+    if constexpr (R > 4) sdif22_stage<R, R / 4, 1>(v);
+}
+
 }  // namespace isr

@@ -164,6 +164,10 @@ struct KArgs {
     // debug builds: [5] = SM cycles of the IPP loop's phases summed over CTAs as seen by thread 0
     // (window wait + barrier, pass 0, middle pass, last pass) and the IPPs counted; NULL = off
     unsigned long long* phase_cycles = nullptr;
+    // isr_xt.cuh only: bytes per chip, and the chip signs of per-IPP binary-phase codes packed by
+    // pack_signs_kernel, [n_ipp][nfft / 32] words (NULL: read the chips)
+    int chip_bytes = 1;
+    const uint32_t* signs = nullptr;
 };
 
 // ---------------------------------------------------------------- async-copy primitives

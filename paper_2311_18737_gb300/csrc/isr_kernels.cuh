@@ -4,6 +4,7 @@
 #include "isr.h"
 #include "isr_kernel.cuh"
 #include "isr_paired.cuh"
+#include "isr_xt.cuh"
 
 namespace isr {
 
@@ -11,35 +12,52 @@ namespace isr {
 isr_status fail(isr_status st, const char* fmt, ...);
 void clear_error();
 
-// radix orders: 0-2 Stockham, 3 warp-local, 4-5 paired FP32, 6-8 orders 0-2 with the inter-pass
-// twiddles in tensor memory, 9 the warp-local schedule with its twiddles in tensor memory
+// radix orders: 0 and 6 the tensor-memory exchange (isr_xt.cuh), 1-2 Stockham, 3 warp-local, 4-5 paired
+// FP32, 7-8 orders 1-2 with the inter-pass twiddles in tensor memory, 9 the warp-local schedule with its
+// twiddles in tensor memory
 constexpr int kNumOrders = 10;
 
 struct KernelEntry {
-    const void* fn;   // __global__ integrate_kernel<LOG2N, TXT>
-    const void* fn_full;  // the same for code_len == nfft (binary-phase codes only; else fn)
-    const void* fn_order[kNumOrders];  // fn_full with radix order 0..8 (1-3: nfft >= 2048; 4-8: 16384)
+    const void* fn;   // nfft < 1024: integrate_kernel<LOG2N, TXT>
+    const void* fn_order[kNumOrders];  // nfft < 1024: [0] the same for code_len == nfft; else the radix
+                                       // orders 1-9 of full-length binary phase but 6 (1-3: nfft >= 2048)
     int smem_order[kNumOrders];        // their shared memory
     const void* fn_tc[9];     // [mode] tensor-core first pass (nfft 16384, binary phase): 1-4 mma.sync,
                               // 5-8 tcgen05; [0] unused
     int smem_tc;
-    int smem;         // dynamic shared memory bytes
+    int smem;         // of fn (bytes)
     int gates;        // range gates per CTA (G)
     int threads;      // threads per CTA
+    // nfft >= 1024: the kernel with its last exchange in tensor memory (isr_xt.cuh), persistent, launched
+    // by launch_integrate; pack forms its sign words of per-IPP binary-phase codes
+    const void* fn_xt = nullptr;
+    const void* fn_pack = nullptr;
+    const void* fn_tables = nullptr;   // fills the twiddle tables of the current device
+    int smem_xt = 0;
 };
 
 template <int L>
 KernelEntry entry_for(int txt)
 {
     using S = Sched<L>;
-    const void* f = txt == TX_CI16 ? (const void*)integrate_kernel<L, TX_CI16>
-                  : txt == TX_C32  ? (const void*)integrate_kernel<L, TX_C32>
-                                   : (const void*)integrate_kernel<L, TX_PM1>;
-    const void* ff = txt == TX_PM1 ? (const void*)integrate_kernel<L, TX_PM1, true> : f;
-    KernelEntry e{f, ff, {ff, ff, ff, ff, ff, ff, ff, ff, ff, ff},
-                  {S::SMEM, S::SMEM, S::SMEM, S::SMEM, S::SMEM, S::SMEM, S::SMEM, S::SMEM, S::SMEM, S::SMEM},
-                  {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr},
-                  0, S::SMEM, S::G, kThreads};
+    KernelEntry e{};
+    e.gates = S::G;
+    e.threads = kThreads;
+    if constexpr (L < 10) {
+        e.fn = txt == TX_CI16 ? (const void*)integrate_kernel<L, TX_CI16>
+             : txt == TX_C32  ? (const void*)integrate_kernel<L, TX_C32>
+                              : (const void*)integrate_kernel<L, TX_PM1>;
+        e.fn_order[0] = txt == TX_PM1 ? (const void*)integrate_kernel<L, TX_PM1, true> : e.fn;
+        e.smem = e.smem_order[0] = S::SMEM;
+    }
+    if constexpr (L >= 10) {
+        e.fn_xt = txt == TX_CI16 ? (const void*)integrate_kernel_xt<L, TX_CI16, XtPlanSrc>
+                : txt == TX_C32  ? (const void*)integrate_kernel_xt<L, TX_C32, XtPlanSrc>
+                                 : (const void*)integrate_kernel_xt<L, TX_PM1, XtPlanSrc>;
+        e.fn_pack = txt == TX_PM1 ? (const void*)pack_signs_kernel<SchedX<L>::T> : nullptr;
+        e.fn_tables = (const void*)xt_tables_kernel<L>;
+        e.smem_xt = SchedX<L>::SMEM;
+    }
     if constexpr (L >= 11) {
         if (txt == TX_PM1) {
             e.fn_order[1] = (const void*)integrate_kernel<L, TX_PM1, true, 1>;
@@ -56,8 +74,6 @@ KernelEntry entry_for(int txt)
             e.smem_order[4] = SchedP::SMEM;
             e.fn_order[5] = (const void*)integrate_kernel_q<true>;
             e.smem_order[5] = SchedQ::SMEM;
-            e.fn_order[6] = (const void*)integrate_kernel_tm<14, TX_PM1, true, 0>;
-            e.smem_order[6] = Sched<14, 0, true>::SMEM;
             e.fn_order[7] = (const void*)integrate_kernel_tm<14, TX_PM1, true, 1>;
             e.smem_order[7] = Sched<14, 1, true>::SMEM;
             e.fn_order[8] = (const void*)integrate_kernel_tm<14, TX_PM1, true, 2>;
@@ -90,6 +106,28 @@ inline KernelEntry kernel_entry(int log2n, int txt)
     if (log2n <= 12) return entry_mid(log2n, txt);
     if (log2n == 13) return entry_8192(txt);
     return entry_16384(txt);
+}
+
+// Ready the entry's kernels on the current device `dev` (once per plan): opt them into their shared
+// memory and fill the twiddle tables if that has not happened on this device (synchronises `stream` then).
+cudaError_t prepare_entry(const KernelEntry& ke, int log2n, int dev, cudaStream_t stream);
+
+// whether launch_integrate takes the tensor-memory kernel
+inline bool takes_xt(const KernelEntry& ke, bool full, int order) { return ke.fn_xt && (!full || order == 0 || order == 6); }
+
+// One launch over rg gate groups x n_chunks IPP chunks of `a` with radix order `order`.
+inline cudaError_t launch_integrate(const KernelEntry& ke, KArgs a, bool full, int order, int rg, int n_chunks,
+                                    int sm_count, cudaStream_t stream)
+{
+    if (takes_xt(ke, full, order)) {
+        XtPlanSrc src{a, rg, rg * n_chunks};
+        void* args[] = {&src};
+        const int grid = src.n_units < sm_count ? src.n_units : sm_count;   // persistent: one CTA per SM
+        return cudaLaunchKernel(ke.fn_xt, dim3((unsigned)grid), dim3(kThreads), args, (size_t)ke.smem_xt, stream);
+    }
+    void* args[] = {&a};
+    return cudaLaunchKernel(full ? ke.fn_order[order] : ke.fn, dim3((unsigned)rg, (unsigned)n_chunks),
+                            dim3((unsigned)ke.threads), args, (size_t)(full ? ke.smem_order[order] : ke.smem), stream);
 }
 
 }  // namespace isr
