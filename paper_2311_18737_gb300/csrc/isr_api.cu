@@ -239,11 +239,8 @@ isr_status launch_block(isr_plan* p, const uint32_t* echo, const char* tx, int64
     while (done < n) {
         int64_t n_l = std::min<int64_t>(n - done, (int64_t)p->max_chunks * p->ipp_chunk);
         if (pack) n_l = std::min(n_l, p->sign_rows);
-        // chunks: enough for the FP32 sum length cap, and enough CTAs for two waves
-        int64_t c_min = (n_l + p->ipp_chunk - 1) / p->ipp_chunk;
-        int64_t c_fill = (2 * (int64_t)p->sm_count + rg - 1) / rg;
-        int64_t C = std::max(c_min, std::min(c_fill, n_l));
-        C = std::min<int64_t>(C, p->max_chunks);
+        // at least enough chunks for the FP32 sum length cap
+        int64_t C = isr::pick_chunks(n_l, rg, p->sm_count, (n_l + p->ipp_chunk - 1) / p->ipp_chunk, p->max_chunks, RN);
         int64_t chunk = (n_l + C - 1) / C;
         C = (n_l + chunk - 1) / chunk;
 
@@ -737,12 +734,10 @@ isr_status isr_integrate_static(const isr_plan_desc* desc, const int16_t* echo, 
     // Chunks: FP32 sums of at most kDefaultChunk IPPs (the bound the per-bin tolerance rests
     // on), at most c_cap of them in the scratch at once.  The IPPs run in blocks of at most
     // c_cap * kDefaultChunk: one fused launch and one reduction per block, the reduction of
-    // every block after the first adding into `out`.  Within a block, two waves of CTAs when
-    // the IPP count allows.
+    // every block after the first adding into `out`.
     const int rg = (d.n_ranges + ke.gates - 1) / ke.gates;
     const int64_t c_cap = std::min<int64_t>(65535, ISR_STATIC_SCRATCH_FLOATS / RN);
     const int64_t block_cap = c_cap * kDefaultChunk;
-    const int64_t c_fill = (2 * (int64_t)sm_count + rg - 1) / rg;
 
     CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int), stream));
     const int cb = chip_bytes(d.tx_type);
@@ -751,7 +746,7 @@ isr_status isr_integrate_static(const isr_plan_desc* desc, const int16_t* echo, 
     for (int64_t done = 0; done < n_ipp;) {
         const int64_t n_l = std::min<int64_t>(n_ipp - done, block_cap);
         const int64_t c_min = (n_l + kDefaultChunk - 1) / kDefaultChunk;
-        int64_t C = std::min(c_cap, std::max(c_min, std::min<int64_t>(c_fill, n_l)));
+        int64_t C = isr::pick_chunks(n_l, rg, sm_count, c_min, c_cap, RN);
         const int64_t chunk = (n_l + C - 1) / C;
         C = (n_l + chunk - 1) / chunk;
 

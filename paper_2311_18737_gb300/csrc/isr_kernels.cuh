@@ -1,6 +1,8 @@
 // isr_kernels.cuh -- kernel registry shared by the instantiation units and the host API.
 #pragma once
 
+#include <algorithm>
+
 #include "isr.h"
 #include "isr_kernel.cuh"
 #include "isr_paired.cuh"
@@ -114,6 +116,33 @@ cudaError_t prepare_entry(const KernelEntry& ke, int log2n, int dev, cudaStream_
 
 // whether launch_integrate takes the tensor-memory kernel
 inline bool takes_xt(const KernelEntry& ke, bool full, int order) { return ke.fn_xt && (!full || order == 0 || order == 6); }
+
+// IPP chunks of a launch over n IPPs and rg gate groups on sm_count SMs, c_min .. c_max of them.  One CTA
+// per SM works through rg x C units of ceil(n / C) IPPs each; a unit costs its IPPs (about 4.3 us each
+// for any nfft) and a third of one more for its start and its partial sums, and every chunk's partials
+// (bins floats) are written and read once.  The C with the least sum is taken: about two waves, the
+// rule before, left up to a third of the SMs idle in the last one (777 gates x 333 IPPs at nfft 2048:
+// four chunks made 392 units, three rounds of 84 IPPs; three make two of 111).
+inline int64_t pick_chunks(int64_t n, int64_t rg, int64_t sm_count, int64_t c_min, int64_t c_max, int64_t bins)
+{
+    constexpr double kUnitIpps = 0.33, kChunkIppsPerBin = 8.0 / (6.5e6 * 4.3);   // 8 bytes at 6.5 MB per us
+    c_max = std::min(c_max, n);
+    c_min = std::min(c_min, c_max);
+    // beyond four units per SM a finer split has nothing left to balance
+    const int64_t c_top = std::min(c_max, std::max(c_min + 2, (4 * sm_count + rg - 1) / rg));
+    int64_t best = c_min;
+    double best_cost = 0;
+    for (int64_t c = c_min; c <= c_top; ++c) {
+        const int64_t chunk = (n + c - 1) / c, real = (n + chunk - 1) / chunk;
+        const int64_t rounds = (rg * real + sm_count - 1) / sm_count;
+        const double cost = (double)rounds * ((double)chunk + kUnitIpps) + (double)real * (double)bins * kChunkIppsPerBin;
+        if (c == c_min || cost < best_cost) {
+            best = c;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
 
 // One launch over rg gate groups x n_chunks IPP chunks of `a` with radix order `order`.
 inline cudaError_t launch_integrate(const KernelEntry& ke, KArgs a, bool full, int order, int rg, int n_chunks,
