@@ -2,9 +2,11 @@
 //
 // A plan holds the persistent FP64 accumulators, the IPP-chunk scratch and the launch
 // shape.  isr_integrate splits the requested IPPs into chunks (each summed in FP32 by
-// one CTA per gate group), launches the fused kernel once per block of chunks and adds
-// the chunk partials into the FP64 accumulators with a reduction kernel.  Host inputs
-// are streamed through two device staging buffers on a copy stream.
+// one CTA per gate group) and launches the fused kernel once per block of chunks; the
+// chunk partials stay in the scratch until the read-back sums them straight into the
+// caller's spectra, or until the scratch is full and a reduction adds them to the FP64
+// accumulators.  Host inputs are streamed through two device staging buffers on a copy
+// stream.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -16,6 +18,7 @@
 #include <vector>
 
 #include "isr.h"
+#include "isr_ff.cuh"
 #include "isr_kernels.cuh"
 
 namespace {
@@ -100,7 +103,44 @@ bool is_device_ptr(const void* p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// sum of chunk partials into the FP64 accumulators: acc[i] += sum_c part[c][i]
+// Host copies of the plans' status words: slots of one pinned page, taken and given back by plans of any
+// thread and device.  A pinned allocation per plan would cost 0.2 ms at each creation; the page is made
+// by the first plan and stays, and a plan that finds no slot free allocates its own word.
+struct StatusPool {
+    static constexpr int kSlots = 1024;
+    std::mutex mu;
+    int* page = nullptr;
+    std::vector<int> free_slots;
+    cudaError_t take(int** out)
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        if (!page) {
+            const cudaError_t e = cudaHostAlloc(&page, kSlots * sizeof(int), cudaHostAllocPortable);
+            if (e != cudaSuccess) {
+                page = nullptr;
+                return e;
+            }
+            for (int i = kSlots; i-- > 0;) free_slots.push_back(i);
+        }
+        if (free_slots.empty()) return cudaHostAlloc(out, sizeof(int), cudaHostAllocPortable);
+        *out = page + free_slots.back();
+        free_slots.pop_back();
+        return cudaSuccess;
+    }
+    void give(int* w)
+    {
+        if (!w) return;
+        std::lock_guard<std::mutex> lock(mu);
+        if (page && w >= page && w < page + kSlots) free_slots.push_back((int)(w - page));
+        else cudaFreeHost(w);
+    }
+};
+StatusPool& status_pool()
+{
+    static StatusPool* pool = new StatusPool();   // never destroyed: plans may outlive static destructors
+    return *pool;
+}
+
 // s + x with the rounding error carried in c (Kahan compensated summation, FP32)
 __device__ __forceinline__ void kahan_add(float& s, float& c, float x)
 {
@@ -110,37 +150,112 @@ __device__ __forceinline__ void kahan_add(float& s, float& c, float x)
     s = t;
 }
 
-// acc[i] += sum_c part[c][i]: the chunk partials are summed in FP32 with compensation (error
-// ~2 ulp whatever the chunk count) and added once per bin into the FP64 accumulator, so the
-// kernel streams at memory speed instead of waiting on FP64 conversions and additions
+// chunk partials of four bins summed in FP32 with compensation (error ~2 ulp whatever the chunk count),
+// eight chunks' loads in flight at a time
+__device__ __forceinline__ void sum_partials(const float* __restrict__ part, int n_chunks, int64_t n, float (&s)[4],
+                                             float (&cp)[4])
+{
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k] = cp[k] = 0.f;
+    constexpr int U = 8;
+    int c = 0;
+    for (; c + U <= n_chunks; c += U) {
+        float4 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = __ldcs(reinterpret_cast<const float4*>(part + (int64_t)(c + u) * n));
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            kahan_add(s[0], cp[0], v[u].x);
+            kahan_add(s[1], cp[1], v[u].y);
+            kahan_add(s[2], cp[2], v[u].z);
+            kahan_add(s[3], cp[3], v[u].w);
+        }
+    }
+    for (; c < n_chunks; ++c) {
+        const float4 v = __ldcs(reinterpret_cast<const float4*>(part + (int64_t)c * n));
+        kahan_add(s[0], cp[0], v.x);
+        kahan_add(s[1], cp[1], v.y);
+        kahan_add(s[2], cp[2], v.z);
+        kahan_add(s[3], cp[3], v.w);
+    }
+}
+
+// float -> double on the integer pipe (exact): a conversion instruction holds the FP64 pipe, which
+// bounds the reduction, as long as an addition
+__device__ __forceinline__ double widen(float f)
+{
+    const uint32_t b = __float_as_uint(f), e = b & 0x7f800000u;
+    if (e == 0x7f800000u || (e == 0u && (b << 1) != 0u)) return (double)f;   // infinity, NaN, subnormal
+    const uint32_t hi = (b & 0x80000000u) | ((b << 1) != 0u ? ((b & 0x7fffffffu) >> 3) + 0x38000000u : 0u);
+    return __hiloint2double((int)hi, (int)(b << 29));
+}
+
+// acc[i] (+)= sum_c part[c][i], the sum added once per bin into the FP64 accumulator
+template <bool ADD>
 __global__ void reduce_partials_kernel(const float* __restrict__ part, int n_chunks, int64_t n,
                                        double* __restrict__ acc)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4;
     for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i < n; i += stride) {
-        float s[4] = {0.f, 0.f, 0.f, 0.f}, cp[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int c = 0; c < n_chunks; ++c) {
-            const float4 v = __ldcs(reinterpret_cast<const float4*>(part + (int64_t)c * n + i));
-            kahan_add(s[0], cp[0], v.x);
-            kahan_add(s[1], cp[1], v.y);
-            kahan_add(s[2], cp[2], v.z);
-            kahan_add(s[3], cp[3], v.w);
-        }
         double2* a = reinterpret_cast<double2*>(acc + i);
-        double2 a0 = a[0], a1 = a[1];
-        a0.x += (double)s[0] - (double)cp[0];
-        a0.y += (double)s[1] - (double)cp[1];
-        a1.x += (double)s[2] - (double)cp[2];
-        a1.y += (double)s[3] - (double)cp[3];
-        a[0] = a0;
-        a[1] = a1;
+        double2 a0 = make_double2(0.0, 0.0), a1 = a0;
+        if constexpr (ADD) {
+            a0 = a[0];
+            a1 = a[1];
+        }
+        float s[4], cp[4];
+        sum_partials(part + i, n_chunks, n, s, cp);
+        double d[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) d[k] = widen(s[k]) - widen(cp[k]);
+        if constexpr (ADD) {
+            d[0] += a0.x;
+            d[1] += a0.y;
+            d[2] += a1.x;
+            d[3] += a1.y;
+        }
+        a[0] = make_double2(d[0], d[1]);
+        a[1] = make_double2(d[2], d[3]);
     }
 }
 
-__global__ void convert_kernel(const double* __restrict__ acc, int64_t n, double scale, float* __restrict__ out)
+// out[i] = (float)((acc[i] + sum_c part[c][i]) * scale), and the status word to host memory: the whole
+// read-back in one pass over the partials that no reduction has taken yet.  Without accumulated sums
+// (ACC false) it stays on the FP32 pipe: the product with scale = sc.h + sc.l as a float pair, one
+// rounding.  V4: out is 16-byte aligned.
+template <bool ACC, bool V4>
+__global__ void spectra_kernel(const float* __restrict__ part, int n_chunks, int64_t n, const double* __restrict__ acc,
+                               double scale, isr::ff sc, float* __restrict__ out, const int* __restrict__ status,
+                               int* __restrict__ host_status)
 {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = (float)(acc[i] * scale);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *host_status = *status;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4;
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i < n; i += stride) {
+        float s[4], cp[4], o[4];
+        sum_partials(part + i, n_chunks, n, s, cp);
+        if constexpr (ACC) {
+            const double2 a0 = *reinterpret_cast<const double2*>(acc + i), a1 = *reinterpret_cast<const double2*>(acc + i + 2);
+            const double d[4] = {a0.x, a0.y, a1.x, a1.y};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                double v = d[k];
+                if (n_chunks > 0) v += widen(s[k]) - widen(cp[k]);
+                o[k] = (float)(v * scale);
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float p = __fmul_rn(s[k], sc.h), e = fmaf(s[k], sc.h, -p);
+                o[k] = p + fmaf(s[k], sc.l, fmaf(-cp[k], sc.h, e));
+            }
+        }
+        if constexpr (V4) {
+            *reinterpret_cast<float4*>(out + i) = make_float4(o[0], o[1], o[2], o[3]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) out[i + k] = o[k];
+        }
+    }
 }
 
 }  // namespace
@@ -155,8 +270,18 @@ struct isr_plan {
     double* acc = nullptr;       // [R][N]
     float* partial = nullptr;    // [max_chunks][R][N]
     int max_chunks = 0;
+    // The first `pending` chunks of `partial` are part of the integration but not yet of acc: a launch
+    // appends its chunks, and they are reduced into acc when the scratch is full, or by the read-back
+    // without going through acc.  acc_zero: nothing has been reduced into acc since it was zeroed.
+    // captured: a launch went into a stream capture, whose replays this bookkeeping cannot see; from
+    // then on every launch reduces its own chunks at once (what was pending before stays so), and acc
+    // is always read and zeroed.
+    int pending = 0;
+    bool acc_zero = true;
+    bool captured = false;
     int ipp_chunk = 0;
     int* status = nullptr;       // device word, bit 0 = timed-out wait
+    int* host_status = nullptr;  // its copy in pinned host memory
     float* out_stage = nullptr;  // [R][N] for host readback
     int64_t n_ipp_total = 0;
     int64_t launches = 0;
@@ -225,7 +350,32 @@ isr_status check_geometry(const isr_plan_desc& d, int64_t start, int64_t step)
     return ISR_OK;
 }
 
-// Launch the fused kernel and the reduction for n rows of device-resident input.
+// CTAs of a kernel with four bins per thread: all bins once, at most eight CTAs per SM
+unsigned bin_blocks(const isr_plan* p, int64_t bins, int threads)
+{
+    return (unsigned)std::min<int64_t>((bins / 4 + threads - 1) / threads, (int64_t)p->sm_count * 8);
+}
+// threads per CTA of such a kernel: small spectra are spread over all SMs
+int bin_threads(const isr_plan* p, int64_t bins) { return bins / 4 < (int64_t)p->sm_count * 256 ? 64 : 256; }
+
+// Reduce the pending chunk partials into the accumulators.
+isr_status flush_partials(isr_plan* p)
+{
+    if (p->pending == 0) return ISR_OK;
+    const int64_t RN = (int64_t)p->d.n_ranges * p->d.nfft;
+    const int threads = bin_threads(p, RN);
+    const unsigned blocks = bin_blocks(p, RN, threads);
+    if (p->acc_zero && !p->captured)
+        reduce_partials_kernel<false><<<blocks, threads, 0, p->stream>>>(p->partial, p->pending, RN, p->acc);
+    else
+        reduce_partials_kernel<true><<<blocks, threads, 0, p->stream>>>(p->partial, p->pending, RN, p->acc);
+    CUDA_TRY(cudaGetLastError());
+    p->pending = 0;
+    p->acc_zero = false;
+    return ISR_OK;
+}
+
+// Launch the fused kernel for n rows of device-resident input; its chunk partials are left pending.
 isr_status launch_block(isr_plan* p, const uint32_t* echo, const char* tx, int64_t n, int64_t start, int64_t step)
 {
     const int R = p->d.n_ranges;
@@ -235,12 +385,25 @@ isr_status launch_block(isr_plan* p, const uint32_t* echo, const char* tx, int64
     const int cb = chip_bytes(p->d.tx_type);
     const bool full = p->d.code_len == p->d.nfft;
     const bool pack = p->signs && p->precision == ISR_PREC_FP32 && isr::takes_xt(p->ke, full, p->order);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CUDA_TRY(cudaStreamIsCapturing(p->stream, &cap));
+    if (cap != cudaStreamCaptureStatusNone) p->captured = true;
     int64_t done = 0;
     while (done < n) {
         int64_t n_l = std::min<int64_t>(n - done, (int64_t)p->max_chunks * p->ipp_chunk);
         if (pack) n_l = std::min(n_l, p->sign_rows);
-        // at least enough chunks for the FP32 sum length cap
-        int64_t C = isr::pick_chunks(n_l, rg, p->sm_count, (n_l + p->ipp_chunk - 1) / p->ipp_chunk, p->max_chunks, RN);
+        // at least enough chunks for the FP32 sum length cap, behind those that are pending (never all)
+        int64_t c_min = (n_l + p->ipp_chunk - 1) / p->ipp_chunk;
+        if (p->pending + c_min > p->max_chunks) {
+            if (cap == cudaStreamCaptureStatusNone) {
+                const isr_status st = flush_partials(p);
+                if (st != ISR_OK) return st;
+            } else {   // a replay must not reduce what is pending now once more
+                c_min = p->max_chunks - p->pending;
+                n_l = std::min(n_l, c_min * p->ipp_chunk);
+            }
+        }
+        int64_t C = isr::pick_chunks(n_l, rg, p->sm_count, c_min, p->max_chunks - p->pending, RN);
         int64_t chunk = (n_l + C - 1) / C;
         C = (n_l + chunk - 1) / chunk;
 
@@ -249,7 +412,7 @@ isr_status launch_block(isr_plan* p, const uint32_t* echo, const char* tx, int64
         a.echo_stride = p->d.echo_stride;
         a.tx = tx + (size_t)(done * p->d.tx_stride) * cb;
         a.tx_stride = p->d.tx_stride;
-        a.partial = p->partial;
+        a.partial = p->partial + (int64_t)p->pending * RN;
         a.status = p->status;
         a.n_ranges = R;
         a.range_start = (int)start;
@@ -288,10 +451,18 @@ isr_status launch_block(isr_plan* p, const uint32_t* echo, const char* tx, int64
             p->ev_pending.push_back(ev);
         }
         p->launches += 1;
-        int threads = 256;
-        int64_t blocks = std::min<int64_t>((RN / 4 + threads - 1) / threads, (int64_t)p->sm_count * 8);
-        reduce_partials_kernel<<<(unsigned)blocks, threads, 0, p->stream>>>(p->partial, (int)C, RN, p->acc);
-        CUDA_TRY(cudaGetLastError());
+        if (p->captured) {
+            const int threads = bin_threads(p, RN);
+            reduce_partials_kernel<true><<<bin_blocks(p, RN, threads), threads, 0, p->stream>>>(a.partial, (int)C, RN, p->acc);
+            CUDA_TRY(cudaGetLastError());
+            p->acc_zero = false;
+        } else {
+            p->pending += (int)C;
+            if (p->pending == p->max_chunks) {
+                const isr_status st = flush_partials(p);
+                if (st != ISR_OK) return st;
+            }
+        }
         done += n_l;
     }
     return ISR_OK;
@@ -449,13 +620,16 @@ isr_status isr_plan_create(isr_plan** out, const isr_plan_desc* desc)
     int64_t mc = d.max_chunks > 0 ? d.max_chunks : std::min<int64_t>(64, std::max<int64_t>(1, kScratchBudget / (RN * 4)));
     p->max_chunks = (int)mc;
     e = cudaMalloc(&p->acc, (size_t)(RN * 8));
-    if (e == cudaSuccess) e = cudaMalloc(&p->partial, (size_t)(mc * RN * 4));
-    if (e == cudaSuccess) e = cudaMalloc(&p->status, sizeof(int));
-    if (e == cudaSuccess && p->ke.fn_pack && d.tx_stride > 0) {
-        const int64_t row = (int64_t)d.nfft / 32 * 4;
-        p->sign_rows = std::min<int64_t>(mc * p->ipp_chunk, kSignBytes / row);
-        e = cudaMalloc(&p->signs, (size_t)(p->sign_rows * row));
+    // chunk partials, packed signs and the status word in one allocation
+    const int64_t part_bytes = mc * RN * 4, sign_row = (int64_t)d.nfft / 32 * 4;
+    p->sign_rows = p->ke.fn_pack && d.tx_stride > 0 ? std::min<int64_t>(mc * p->ipp_chunk, kSignBytes / sign_row) : 0;
+    const int64_t sign_bytes = (p->sign_rows * sign_row + 15) / 16 * 16;
+    if (e == cudaSuccess) e = cudaMalloc(&p->partial, (size_t)(part_bytes + sign_bytes + 16));
+    if (e == cudaSuccess) {
+        p->signs = p->sign_rows ? reinterpret_cast<uint32_t*>(p->partial + part_bytes / 4) : nullptr;
+        p->status = reinterpret_cast<int*>(p->partial + (part_bytes + sign_bytes) / 4);
     }
+    if (e == cudaSuccess) e = status_pool().take(&p->host_status);
 #ifdef ISR_DEBUG
     if (e == cudaSuccess) e = cudaMalloc(&p->phase, 5 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemsetAsync(p->phase, 0, 5 * sizeof(unsigned long long), p->stream);
@@ -525,19 +699,26 @@ isr_status isr_spectra(isr_plan* p, float* out, int32_t flags, int64_t* n_ipp_ou
             if (!p->out_stage) CUDA_TRY(cudaMalloc(&p->out_stage, (size_t)(RN * 4)));
             dst = p->out_stage;
         }
-        int threads = 256;
-        int64_t blocks = std::min<int64_t>((RN + threads - 1) / threads, (int64_t)p->sm_count * 8);
-        convert_kernel<<<(unsigned)blocks, threads, 0, p->stream>>>(p->acc, RN, scale, dst);
+        const int threads = bin_threads(p, RN);
+        const unsigned blocks = bin_blocks(p, RN, threads);
+        const isr::ff sc{(float)scale, (float)(scale - (double)(float)scale)};
+        const bool v4 = reinterpret_cast<uintptr_t>(dst) % 16 == 0, from_acc = !p->acc_zero || p->captured;
+        auto* k = from_acc ? (v4 ? spectra_kernel<true, true> : spectra_kernel<true, false>)
+                           : (v4 ? spectra_kernel<false, true> : spectra_kernel<false, false>);
+        k<<<blocks, threads, 0, p->stream>>>(p->partial, p->pending, RN, p->acc, scale, sc, dst, p->status, p->host_status);
         CUDA_TRY(cudaGetLastError());
         if (!dev_out) CUDA_TRY(cudaMemcpyAsync(out, dst, (size_t)(RN * 4), cudaMemcpyDeviceToHost, p->stream));
+    } else {
+        CUDA_TRY(cudaMemcpyAsync(p->host_status, p->status, sizeof(int), cudaMemcpyDeviceToHost, p->stream));
     }
-    int status = 0;
-    CUDA_TRY(cudaMemcpyAsync(&status, p->status, sizeof(int), cudaMemcpyDeviceToHost, p->stream));
     CUDA_TRY(cudaStreamSynchronize(p->stream));
+    const int status = *p->host_status;
     harvest_events(p);
     if (n_ipp_out) *n_ipp_out = p->n_ipp_total;
     if (flags & ISR_RESET_AFTER) {
-        CUDA_TRY(cudaMemsetAsync(p->acc, 0, (size_t)(RN * 8), p->stream));
+        p->pending = 0;
+        if (!p->acc_zero || p->captured) CUDA_TRY(cudaMemsetAsync(p->acc, 0, (size_t)(RN * 8), p->stream));
+        p->acc_zero = true;
         p->n_ipp_total = 0;
     }
     if (status) {
@@ -804,8 +985,7 @@ void isr_destroy(isr_plan* p)
         if (e) cudaEventDestroy(e);
     cudaFree(p->acc);
     cudaFree(p->partial);
-    cudaFree(p->status);
-    cudaFree(p->signs);
+    status_pool().give(p->host_status);
     cudaFree(p->phase);
     cudaFree(p->out_stage);
     cudaGetLastError();

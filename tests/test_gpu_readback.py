@@ -1,0 +1,80 @@
+"""The read-back that sums chunk partials straight into the spectra, in every state the partials can be
+in: none, some pending, scratch full and reduced, a read between calls, resets, a stream capture among
+the calls, and an output that is not 16-byte aligned.  Bins against the FP64 oracle at RTOL."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from gpu_helpers import assert_parity
+from paper_2311_18737_gb300 import isr
+
+pytestmark = pytest.mark.gpu
+
+NFFT, R, STEP = 1024, 5, 3
+
+
+def _echo(seed, P):
+    rng = np.random.default_rng(seed)
+    stride = ((R - 1) * STEP + NFFT + 3) // 4 * 4
+    return (np.clip(np.rint(rng.standard_normal((P, stride, 2)) * 1000), -32768, 32767).astype(np.int16),
+            np.where(rng.random(NFFT) < 0.5, -1, 1).astype(np.int8))
+
+
+def _ref(echo, tx):
+    return oracle.integrate(echo, tx, nfft=NFFT, n_ranges=R, range_start=0, range_step=STEP)
+
+
+def _plan(echo, stream, **kw):
+    return isr.Plan(nfft=NFFT, n_ranges=R, echo_stride=echo.shape[1], range_step=STEP, device=0, stream=stream, **kw)
+
+
+@pytest.mark.parametrize("max_chunks,ipp_chunk", [(0, 0), (1, 4), (2, 3), (3, 2)])
+def test_reads_between_calls_and_resets(max_chunks, ipp_chunk):
+    echo, tx = _echo(1, 23)
+    e, t = torch.from_numpy(echo).cuda(), torch.from_numpy(tx).cuda()
+    with _plan(echo, torch.cuda.current_stream(), max_chunks=max_chunks, ipp_chunk=ipp_chunk) as plan:
+        out, n = plan.spectra()
+        assert n == 0 and not out.any()
+        done = 0
+        for k in (4, 1, 7):
+            plan.integrate(e[done:], t, k)
+            done += k
+            for _ in range(2):          # reading leaves the integration as it was
+                out, n = plan.spectra(flags=isr.ISR_MEAN)
+                assert n == done
+                assert_parity(out.numpy().astype(np.float64), _ref(echo[:done], tx) / done, what=f"after {done}")
+        plan.spectra(out, isr.ISR_RESET_AFTER)
+        assert not plan.spectra()[0].any()
+        plan.integrate(e[done:], t, 11)
+        isr.isr_spectra(plan.handle, None, isr.ISR_RESET_AFTER)
+        plan.integrate(e[:6], t, 6)
+        buf = torch.zeros(R * NFFT + 1, device="cuda")          # an output that is only 4-byte aligned
+        plan.spectra(buf[1:])
+        assert buf[0] == 0
+        assert_parity(buf[1:].reshape(R, NFFT).cpu().numpy().astype(np.float64), _ref(echo[:6], tx), what="unaligned")
+
+
+def test_captured_integration_replayed_between_calls():
+    """A captured isr_integrate adds to the integration at every replay, whatever was pending before it."""
+    echo, tx = _echo(2, 12)
+    e, t = torch.from_numpy(echo).cuda(), torch.from_numpy(tx).cuda()
+    side = torch.cuda.Stream()
+    with _plan(echo, side) as plan:
+        side.wait_stream(torch.cuda.current_stream())
+        plan.integrate(e, t, 4)                                   # pending when the capture starts
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side):
+            plan.integrate(e[4:], t, 5)
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(side):
+            graph.replay()
+            graph.replay()
+        plan.integrate(e[9:], t, 3)
+        out, _ = plan.spectra(flags=isr.ISR_RESET_AFTER)
+        ref = _ref(echo[:4], tx) + 2 * _ref(echo[4:9], tx) + _ref(echo[9:], tx)
+        assert_parity(out.numpy().astype(np.float64), ref, what="two replays")
+        with torch.cuda.stream(side):
+            graph.replay()
+        out, _ = plan.spectra()
+        assert_parity(out.numpy().astype(np.float64), _ref(echo[4:9], tx), what="a replay after the reset")
