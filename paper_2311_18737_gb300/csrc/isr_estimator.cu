@@ -1604,69 +1604,531 @@ __global__ void __launch_bounds__(256) head_chunk_kernel(const T* __restrict__ h
     }
 }
 
-// With pos and pres (inference) it also gives the prediction: position = softmax-weighted mean
-// over the 7 bins around the first arg-max of z (+ band_lo), presence = sigmoid(q).
-__global__ void __launch_bounds__(64) head_mlp_kernel(const float* __restrict__ theta, int L, int nx,
-                                                      const float* __restrict__ pmax, const int* __restrict__ pidx,
-                                                      const float* __restrict__ psum, const float* __restrict__ z,
-                                                      const float* __restrict__ zmax, const int* __restrict__ zidx,
-                                                      int lo, int* __restrict__ amax, float* __restrict__ pooled,
-                                                      float* __restrict__ u, float* __restrict__ q,
-                                                      float* __restrict__ pos, float* __restrict__ pres)
+// Head of one row from its chunk statistics, in HM_THREADS threads: max / first
+// arg-max / mean per channel and the presence MLP; with PREDICT also the prediction: position =
+// softmax-weighted mean over the 7 bins around the first arg-max of z (+ band_lo), presence =
+// sigmoid(q).  Latency bound (a few KB per row): warp w takes the chunks w, w + 8, ... with a lane per
+// channel, the first warp the chunks' largest logits with a lane per chunk, and eight threads share
+// each hidden unit.
+constexpr int HM_THREADS = 256;
+struct HeadScratch {
+    float mx[HM_THREADS / 32][CH], sum[HM_THREADS / 32][CH];
+    float pool[2 * CH], u[CH];
+};
+struct HeadArgs {
+    const float* theta;
+    int L, nx, lo;
+    const float *pmax, *psum, *z, *zmax;
+    const int *pidx, *zidx;
+    int* amax;
+    float *pooled, *u, *q, *pos, *pres;
+};
+
+template <bool PREDICT>
+__global__ void __launch_bounds__(HM_THREADS) head_mlp_kernel(const HeadArgs a)
 {
-    const int b = blockIdx.x;
-    __shared__ float pool_s[2 * CH];
-    __shared__ float u_s[CH];
-    if (pos && threadIdx.x == CH) {
-        float mx = -INFINITY;
-        int mi = 0;
-        for (int xc = 0; xc < nx; ++xc)   // chunks in position order: ties keep the first
-            if (zmax[(size_t)b * nx + xc] > mx) {
-                mx = zmax[(size_t)b * nx + xc];
-                mi = zidx[(size_t)b * nx + xc];
-            }
-        const float* zb = z + (size_t)b * L;
-        const int a = max(0, mi - WIN), e = min(L, mi + WIN + 1);
-        double sw = 0, swi = 0;
-        for (int i = a; i < e; ++i) {
-            const double wgt = exp((double)zb[i] - (double)mx);
-            sw += wgt;
-            swi += wgt * i;
-        }
-        pos[b] = (float)(lo + swi / sw);
-    }
-    if (threadIdx.x < CH) {
-        const int c = threadIdx.x;
+    __shared__ HeadScratch sc;
+    __shared__ int mi_s[HM_THREADS / 32][CH];
+    const int b = blockIdx.x, tid = threadIdx.x;
+    constexpr int NW = HM_THREADS / 32;
+    const int lane = tid & 31, warp = tid >> 5, nx = a.nx, L = a.L;
+    const float* theta = a.theta;
+    // hidden unit j's weights for inputs 8 part .. 8 part + 7, on their way meanwhile
+    const int j = tid >> 3, part = tid & 7;
+    float wa[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) wa[e] = theta[OFF_WA + j * 2 * CH + 8 * part + e];
+    {
         float mx = -INFINITY, sum = 0.f;
         int mi = 0;
-        for (int xc = 0; xc < nx; ++xc) {   // chunks in position order: ties keep the first
-            const size_t o = ((size_t)b * nx + xc) * CH + c;
-            if (pmax[o] > mx) {
-                mx = pmax[o];
-                mi = pidx[o];
+        for (int xc = warp; xc < nx; xc += NW) {   // ascending: ties keep the first
+            const size_t o = ((size_t)b * nx + xc) * CH + lane;
+            const float v = a.pmax[o];
+            if (v > mx) {
+                mx = v;
+                if constexpr (!PREDICT) mi = a.pidx[o];   // only the backward pass asks where
             }
-            sum += psum[o];
+            sum += a.psum[o];
         }
-        pool_s[c] = mx;
-        pool_s[CH + c] = sum / L;
-        amax[b * CH + c] = mi;
+        sc.mx[warp][lane] = mx;
+        sc.sum[warp][lane] = sum;
+        if constexpr (!PREDICT) mi_s[warp][lane] = mi;
+    }
+    if (PREDICT && warp == 0) {
+        float mx = -INFINITY;
+        int mi = 0x7fffffff;
+        for (int xc = lane; xc < nx; xc += 32) {
+            const float v = a.zmax[(size_t)b * nx + xc];
+            if (v > mx) {
+                mx = v;
+                mi = a.zidx[(size_t)b * nx + xc];
+            }
+        }
+        for (int o = 16; o; o >>= 1) {
+            const float om = __shfl_xor_sync(0xffffffffu, mx, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, mi, o);
+            if (om > mx || (om == mx && oi < mi)) {
+                mx = om;
+                mi = oi;
+            }
+        }
+        if (mi == 0x7fffffff) mi = 0;   // no logit above -infinity
+        const int i = mi - WIN + lane;
+        double wgt = 0.0;
+        if (lane <= 2 * WIN && i >= 0 && i < L) wgt = exp((double)a.z[(size_t)b * L + i] - (double)mx);
+        double sw = 0, swi = 0;
+        for (int k = 0; k <= 2 * WIN; ++k) {   // ascending positions
+            const double wk = __shfl_sync(0xffffffffu, wgt, k);
+            const int ik = mi - WIN + k;
+            if (ik < 0 || ik >= L) continue;
+            sw += wk;
+            swi += wk * ik;
+        }
+        if (lane == 0) a.pos[b] = (float)(a.lo + swi / sw);
     }
     __syncthreads();
-    if (threadIdx.x < CH) {
-        const int j = threadIdx.x;
-        float s = theta[OFF_BA + j];
-        for (int e = 0; e < 2 * CH; ++e) s = fmaf(theta[OFF_WA + j * 2 * CH + e], pool_s[e], s);
-        u_s[j] = fmaxf(s, 0.f);
-        u[b * CH + j] = u_s[j];
+    if (tid < CH) {
+        float mx = sc.mx[0][tid], sum = sc.sum[0][tid];
+        int mi = PREDICT ? 0 : mi_s[0][tid];
+        for (int w = 1; w < NW; ++w) {
+            const float om = sc.mx[w][tid];
+            const int oi = PREDICT ? 0 : mi_s[w][tid];
+            if (om > mx || (om == mx && om > -INFINITY && oi < mi)) {
+                mx = om;
+                mi = oi;
+            }
+            sum += sc.sum[w][tid];
+        }
+        sc.pool[tid] = mx;
+        sc.pool[CH + tid] = sum / L;
+        if constexpr (!PREDICT) a.amax[b * CH + tid] = mi;
     }
-    if (threadIdx.x < 2 * CH) pooled[b * 2 * CH + threadIdx.x] = pool_s[threadIdx.x];
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float s = theta[OFF_BB];
-        for (int j = 0; j < CH; ++j) s = fmaf(theta[OFF_WB + j], u_s[j], s);
-        q[b] = s;
-        if (pres) pres[b] = 1.f / (1.f + expf(-s));
+    {
+        float s = 0.f;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) s = fmaf(wa[e], sc.pool[8 * part + e], s);
+        for (int o = 4; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (part == 0) {
+            s += theta[OFF_BA + j];
+            sc.u[j] = fmaxf(s, 0.f);
+            if constexpr (!PREDICT) a.u[b * CH + j] = sc.u[j];
+        }
     }
+    if constexpr (!PREDICT) {
+        if (tid < 2 * CH) a.pooled[b * 2 * CH + tid] = sc.pool[tid];
+    }
+    __syncthreads();
+    if (warp == 0) {
+        float s = theta[OFF_WB + lane] * sc.u[lane];
+        for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) {
+            s += theta[OFF_BB];
+            if constexpr (!PREDICT) a.q[b] = s;
+            else a.pres[b] = 1.f / (1.f + expf(-s));
+        }
+    }
+}
+
+// ---------------------------------------------------------------- fused inference
+// The whole network up to the head's chunk statistics in one kernel (BF16 storage, tcgen05): a tile's
+// activations never leave the SM.  Launched per batch: conv1, three convolutions and the head took
+// 16 + 3 x 33 + 14 us for 128 rows x 4608 positions, bound by staging channel-major rows into the
+// operand layout and writing them back; here the epilogue of a layer writes the next layer's operand.
+//
+// A tile is FI_W = 512 positions of one row, of which FI_P = 488 come out of the fourth layer (four
+// 9-tap layers use up 8 positions each, the first computes 512 of the 520 the second could read).  It
+// goes to the tensor cores as 128 rows of four positions each:
+//   D[r][32 p' + co] = sum_{t, ci} X[4 r + t][ci] W[co][ci][t - p],   p' = 3 - p,  t = 0 .. 11,
+// M = 128, N = 128 (four positions x 32 channels), K = 12 taps x 32 channels, 24 MMAs of 64 cycles where
+// four M = 128, N = 32 tiles are 72 of 46: a quarter of the products are with zeros, but an N = 32 MMA is
+// bound by reading its A operand.  The operand B of tap t is the 128 rows starting at tap t of the
+// weights laid out [8-channel group][3 zero taps, 9 taps][32 co][8 ci] (the next group's zeros follow), so
+// the Toeplitz matrix costs little more room than the weights.  Positions of equal index mod 4 form the planes of A
+// ([8-channel group][index mod 4][index / 4][8 ci]), so tap t is plane t mod 4 started t / 4 rows later.
+// Each output accumulates the same products in the same order as in conv_tc05_kernel (the added ones
+// are zeros), so the activations are equal bit by bit; a zero times an infinity would not be, so a tile
+// that holds one issues the products of each p' alone, without the zero taps.
+//
+// A CTA (one per SM) holds the three layers' weights and FI_SLOTS tiles, each worked on by eight warps
+// with 128 TMEM columns of its own: while one tile's MMAs run, the others are in their first layer or
+// epilogues.  The activations are overwritten in place once a layer's MMAs have completed.
+// Measured, 128 rows x 4608 positions: 58 us a call with the head's 9, where the separate kernels took
+// 139; two tiles per CTA 68 us, a turn for issuing one tile's MMAs after the other's 60 us, the row's head
+// in its last tile's warps (one atomic per tile) 70 us.  The tensor pipe is active on about 45 % of cycles:
+// the tiles run through their phases nearly together, three rounds of them per call.
+constexpr int FI_W = 512, FI_P = FI_W - 24;      // positions of a tile, positions it finishes
+constexpr int FI_SLOTS = 3, FI_ST = 256;         // tiles in flight per CTA, threads per tile
+constexpr int FI_COLS = FI_SLOTS > 2 ? 512 : 256; // TMEM columns (a power of two)
+constexpr int FI_ROWS = FI_W / 4 + 2;            // rows of a plane (taps reach two rows beyond)
+constexpr int FI_PLANE = FI_ROWS * 16;           // bytes; 8 banks past a multiple of 32, so planes interleave
+constexpr int FI_BUF = 16 * FI_PLANE;
+constexpr int FI_WCG = (KT + 3) * CH * 16;       // bytes between 8-channel groups: 3 zero taps and 9 taps
+constexpr int FI_WLAYER = 4 * FI_WCG;
+constexpr int FI_WBYTES = 3 * FI_WLAYER + 3 * CH * 16;   // the last group's taps are followed by zeros too
+constexpr int FI_XW = FI_W + KT - 1;
+static_assert((FI_PLANE / 4) % 32 == 8 && FI_PLANE % 16 == 0, "plane pitch");
+struct FiSlot {
+    uint64_t mbar;
+    float zm[8];
+    int zi[8];
+    float mx[8][CH], sum[8][CH];
+    alignas(16) float x[FI_XW];
+};
+struct FiShared {
+    float w1[CH][12];    // W1[co][0..8], b1[co]
+    float bias[3][CH];
+    float w5[CH];
+    uint32_t tslot;
+    FiSlot slot[FI_SLOTS];
+};
+constexpr int FI_OFF_BUF = (FI_WBYTES + 127) / 128 * 128;
+constexpr int FI_OFF_SH = FI_OFF_BUF + FI_SLOTS * FI_BUF;
+constexpr int FI_SMEM = FI_OFF_SH + (int)sizeof(FiShared);
+static_assert(FI_SMEM <= 232448 && FI_OFF_BUF % 128 == 0 && FI_OFF_SH % 16 == 0, "shared memory");
+
+// relu of two values as stored: rounded to BF16, then max with 0 (NaN becomes 0, as fmaxf gives)
+__device__ __forceinline__ uint32_t fi_relu2(float a, float b)
+{
+    const __nv_bfloat162 h = __hmax2(__floats2bfloat162_rn(a, b), __floats2bfloat162_rn(0.f, 0.f));
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+__device__ __forceinline__ uint32_t fi_max2(uint32_t a, uint32_t b)
+{
+    const __nv_bfloat162 h = __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+// whether either half of a word of non-negative BF16 values is an infinity
+__device__ __forceinline__ bool fi_inf2(uint32_t m) { return (m & 0x7fffu) == 0x7f80u || (m >> 16 & 0x7fffu) == 0x7f80u; }
+__device__ __forceinline__ float fi_half(uint32_t w, int half) { return __uint_as_float(half ? (w & 0xffff0000u) : (w << 16)); }
+
+// sum of v[c] over the warp's lanes for 32 channels c: lane c receives channel c's (31 exchanges)
+__device__ __forceinline__ float fi_scatter_sum(float (&v)[CH], int lane)
+{
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int k = 0; k < o; ++k) {
+            const float keep = up ? v[k + o] : v[k], give = up ? v[k] : v[k + o];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    return v[0];
+}
+// the same for the maximum of BF16 pairs: m[k] = channels 2 k, 2 k + 1
+__device__ __forceinline__ float fi_scatter_max(uint32_t (&m)[CH / 2], int lane)
+{
+#pragma unroll
+    for (int o = 8; o; o >>= 1) {
+        const bool up = (lane & (2 * o)) != 0;
+#pragma unroll
+        for (int k = 0; k < o; ++k) {
+            const uint32_t keep = up ? m[k + o] : m[k], give = up ? m[k] : m[k + o];
+            m[k] = fi_max2(keep, __shfl_xor_sync(0xffffffffu, give, 2 * o));
+        }
+    }
+    m[0] = fi_max2(m[0], __shfl_xor_sync(0xffffffffu, m[0], 1));
+    return fi_half(m[0], lane & 1);
+}
+
+__global__ void __launch_bounds__(FI_SLOTS * FI_ST, 1) infer_kernel(const float* __restrict__ x, const __nv_bfloat16* __restrict__ w1,
+                                                                    const __nv_bfloat16* __restrict__ wt,
+                                                                    int n_rows, float* __restrict__ z, float* __restrict__ pmax,
+                                                                    float* __restrict__ psum, float* __restrict__ zmax,
+                                                                    int* __restrict__ zidx, const float* __restrict__ theta,
+                                                                    int L, int nx)
+{
+    extern __shared__ __align__(128) unsigned char fi_smem[];
+    FiShared& sh = *reinterpret_cast<FiShared*>(fi_smem + FI_OFF_SH);
+    const int tid = threadIdx.x, slot = tid / FI_ST, st = tid - slot * FI_ST;
+    const int lane = tid & 31, w = __shfl_sync(0xffffffffu, st >> 5, 0);   // warp of the slot
+    FiSlot& sl = sh.slot[slot];
+    unsigned char* buf = fi_smem + FI_OFF_BUF + slot * FI_BUF;
+    const uint32_t mbar = isr::smem_u32(&sl.mbar);
+
+    if (st == 0) isr::mbar_init(mbar, 1);
+    isr::fence_barrier_init();
+    if (tid < 32) isr::tmem_alloc(isr::smem_u32(&sh.tslot), FI_COLS);
+    // weights of layers 2-4: rows [co][tap][ci] to [ci / 8][tap + 3][co][8 ci], zeros around the taps
+    {
+        constexpr int NT = FI_SLOTS * FI_ST, PER = (FI_WBYTES / 16 + NT - 1) / NT;
+        uint4 v[PER];   // all loads first
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int e = tid + i * NT, co = e % CH, tp = e / CH % (KT + 3), gr = e / (CH * (KT + 3)), l = gr / 4, cg = gr % 4;
+            v[i] = make_uint4(0u, 0u, 0u, 0u);
+            if (tp >= 3 && e < FI_WBYTES / 16)
+                v[i] = __ldg(reinterpret_cast<const uint4*>(wt + ((size_t)(l * CH + co) * KT + (tp - 3)) * CH + cg * 8));
+        }
+#pragma unroll
+        for (int i = 0; i < PER; ++i)
+            if (tid + i * NT < FI_WBYTES / 16) *reinterpret_cast<uint4*>(fi_smem + (tid + i * NT) * 16) = v[i];
+    }
+    for (int e = tid; e < CH * 12; e += FI_SLOTS * FI_ST) {
+        const int co = e / 12, k = e - co * 12;
+        sh.w1[co][k] = k < KT ? ld<__nv_bfloat16>(w1, (size_t)k * CH + co) : (k == KT ? theta[OFF_B1 + co] : 0.f);
+    }
+    for (int e = tid; e < 3 * CH; e += FI_SLOTS * FI_ST) sh.bias[e / CH][e % CH] = theta[b_off(2 + e / CH) + e % CH];
+    if (tid < CH) sh.w5[tid] = theta[OFF_W5 + tid];
+    for (int e = tid; e < FI_SLOTS * FI_BUF / 16; e += FI_SLOTS * FI_ST)   // the last two rows are read, never written
+        *reinterpret_cast<uint4*>(fi_smem + FI_OFF_BUF + e * 16) = make_uint4(0u, 0u, 0u, 0u);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    isr::tmem_fence_before_sync();
+    __syncthreads();
+    isr::tmem_fence_after_sync();
+    const uint32_t tacc = sh.tslot + 128u * slot;   // this tile's accumulator
+    const float b5 = theta[OFF_B5];
+
+    auto slot_or = [&](bool pred) -> bool {
+        uint32_t any;
+        asm volatile(
+            "{\n\t.reg .pred p, q;\n\t"
+            "setp.ne.u32 p, %1, 0;\n\t"
+            "bar.red.or.pred q, %2, %3, p;\n\t"
+            "selp.u32 %0, 1, 0, q;\n\t}"
+            : "=r"(any)
+            : "r"((uint32_t)pred), "r"(1 + slot), "n"(FI_ST)
+            : "memory");
+        return any != 0;
+    };
+    // one thread: the MMAs of layer l (0 .. 2) on this slot's buffer
+    auto issue = [&](int l, bool inf) {
+        constexpr uint32_t idesc32 = isr::tc05_idesc<true>();
+        constexpr uint32_t idesc = (idesc32 & ~(0x3fu << 17)) | ((128u >> 3) << 17);   // N = 128
+        const uint64_t ad = isr::tc05_desc(isr::smem_u32(buf), 4 * FI_PLANE, 128);
+        const uint64_t bd = isr::tc05_desc(isr::smem_u32(fi_smem) + l * FI_WLAYER, FI_WCG, 128);
+        if (!inf) {
+#pragma unroll
+            for (int t = 0; t < KT + 3; ++t)
+#pragma unroll
+                for (int ks = 0; ks < 2; ++ks)
+                    isr::tc05_mma(tacc, ad + (uint32_t)(((2 * ks * 4 + (t & 3)) * FI_PLANE + (t >> 2) * 16) >> 4),
+                                  bd + (uint32_t)((2 * ks * FI_WCG + t * CH * 16) >> 4), idesc, (t | ks) != 0);
+        } else {
+#pragma unroll 1
+            for (int p = 0; p < 4; ++p)
+#pragma unroll 1
+                for (int tap = 0; tap < KT; ++tap)
+#pragma unroll 1
+                    for (int ks = 0; ks < 2; ++ks) {
+                        const int t = tap + p;
+                        isr::tc05_mma(tacc + 32u * (3 - p), ad + (uint32_t)(((2 * ks * 4 + (t & 3)) * FI_PLANE + (t >> 2) * 16) >> 4),
+                                      bd + (uint32_t)((2 * ks * FI_WCG + (tap + 3) * CH * 16) >> 4), idesc32, (tap | ks) != 0);
+                    }
+        }
+        isr::tc05_commit(mbar);
+    };
+
+    const int n_tiles = n_rows * nx, step = gridDim.x * FI_SLOTS;
+    // x of a tile: positions i0 - 16 .. , rounded to BF16 as the network reads it
+    constexpr int XPER = (FI_XW + FI_ST - 1) / FI_ST;
+    float xr[XPER];
+    auto load_x = [&](int tile) {
+        const int b = tile / nx, i0 = (tile - b * nx) * FI_P;
+#pragma unroll
+        for (int k = 0; k < XPER; ++k) {
+            const int j = st + k * FI_ST, pos = i0 - 16 + j;
+            xr[k] = (j < FI_XW && pos >= 0 && pos < L) ? __ldg(x + (size_t)b * L + pos) : 0.f;
+        }
+    };
+    uint32_t phase = 0;
+    int tile = slot * gridDim.x + blockIdx.x;   // what is left after full rounds goes to different SMs
+    if (tile < n_tiles) load_x(tile);
+    for (; tile < n_tiles; tile += step) {
+        const int b = tile / nx, xc = tile - b * nx, i0 = xc * FI_P;
+#pragma unroll
+        for (int k = 0; k < XPER; ++k) {
+            const int j = st + k * FI_ST;
+            if (j < FI_XW) sl.x[j] = __bfloat162float(__float2bfloat16_rn(xr[k]));
+        }
+        slot_or(false);
+        if (tile + step < n_tiles) load_x(tile + step);
+        // ---- layer 1: positions i0 - 12 + 4 r .. + 3 of row r = st % 128, half of the channels
+        bool inf = false;
+        {
+            const int r = st & (FI_W / 4 - 1), half = st / (FI_W / 4);
+            float xv[KT + 3];
+#pragma unroll
+            for (int k = 0; k < KT + 3; k += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(&sl.x[4 * r + k]);
+                xv[k] = v.x, xv[k + 1] = v.y, xv[k + 2] = v.z, xv[k + 3] = v.w;
+            }
+            uint32_t in[4], top = 0u;
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                const int pos = i0 - 12 + 4 * r + p;
+                in[p] = pos >= 0 && pos < L ? ~0u : 0u;
+            }
+#pragma unroll 1
+            for (int cg = 2 * half; cg < 2 * half + 2; ++cg) {
+                uint32_t q[4][4];   // [position][channel pair]
+#pragma unroll
+                for (int c2 = 0; c2 < 4; ++c2) {
+                    float a[2][4];
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        const float* wr = sh.w1[8 * cg + 2 * c2 + c];
+                        const float4 wa = *reinterpret_cast<const float4*>(wr), wb = *reinterpret_cast<const float4*>(wr + 4);
+                        const float2 wc = *reinterpret_cast<const float2*>(wr + 8);
+                        const float wk[KT] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w, wc.x};
+#pragma unroll
+                        for (int p = 0; p < 4; ++p) a[c][p] = wc.y;
+#pragma unroll
+                        for (int k = 0; k < KT; ++k)
+#pragma unroll
+                            for (int p = 0; p < 4; ++p) a[c][p] = fmaf(wk[k], xv[p + k], a[c][p]);
+                    }
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) {
+                        q[p][c2] = fi_relu2(a[0][p], a[1][p]) & in[p];
+                        top = fi_max2(top, q[p][c2]);
+                    }
+                }
+#pragma unroll
+                for (int p = 0; p < 4; ++p)
+                    *reinterpret_cast<uint4*>(buf + (cg * 4 + p) * FI_PLANE + r * 16) = make_uint4(q[p][0], q[p][1], q[p][2], q[p][3]);
+            }
+            inf = fi_inf2(top);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        inf = slot_or(inf);
+        if (st == 0) issue(0, inf);
+        // ---- layers 2-4: row 32 (w % 4) + lane of the accumulator, positions 4 row + 3 - p' of the two
+        // p' = 2 (w / 4), 2 (w / 4) + 1
+        const int row = 32 * (w & 3) + lane, pp = 2 * (w >> 2);
+        // relu(accumulator + bias) of layer l for p' = pp + h, as stored: word k = channels 2 k, 2 k + 1
+        auto outputs = [&](int l, int h, uint32_t (&q)[CH / 2]) {
+            uint32_t r[32];
+            isr::tmem_ld32(isr::tmem_warp_lane_base(tacc) + 32u * (pp + h), r);
+            isr::tmem_wait_ld32(r);
+#pragma unroll
+            for (int c4 = 0; c4 < CH / 4; ++c4) {
+                const float4 bv = *reinterpret_cast<const float4*>(&sh.bias[l][4 * c4]);
+                q[2 * c4] = fi_relu2(__uint_as_float(r[4 * c4]) + bv.x, __uint_as_float(r[4 * c4 + 1]) + bv.y);
+                q[2 * c4 + 1] = fi_relu2(__uint_as_float(r[4 * c4 + 2]) + bv.z, __uint_as_float(r[4 * c4 + 3]) + bv.w);
+            }
+        };
+#pragma unroll 1
+        for (int l = 0; l < 2; ++l) {
+            const bool done = isr::mbar_wait(mbar, phase, 1u << 26);
+            phase ^= 1u;
+            isr::tmem_fence_after_sync();
+            uint32_t top = 0u;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint32_t q[CH / 2];
+                outputs(l, h, q);
+                const int p = 3 - pp - h, pos = i0 - 8 + 4 * l + 4 * row + p;
+                const uint32_t in = done && pos >= 0 && pos < L ? ~0u : 0u;
+                unsigned char* d = buf + p * FI_PLANE + row * 16;
+#pragma unroll
+                for (int k = 0; k < CH / 2; ++k) {
+                    q[k] &= in;
+                    top = fi_max2(top, q[k]);
+                }
+#pragma unroll
+                for (int cg = 0; cg < 4; ++cg)
+                    *reinterpret_cast<uint4*>(d + cg * 4 * FI_PLANE) = make_uint4(q[4 * cg], q[4 * cg + 1], q[4 * cg + 2], q[4 * cg + 3]);
+            }
+            inf = fi_inf2(top);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            isr::tmem_fence_before_sync();
+            inf = slot_or(inf);
+            isr::tmem_fence_after_sync();
+            if (st == 0) issue(l + 1, inf);
+        }
+        // ---- layer 4 stays in registers: h4 as stored (BF16), its logit, and what the head keeps of it
+        float zm = -INFINITY;
+        int zi = 0x7fffffff;
+        uint32_t h4[2][CH / 2];
+        const bool done = isr::mbar_wait(mbar, phase, 1u << 26);
+        phase ^= 1u;
+        isr::tmem_fence_after_sync();
+#pragma unroll
+        for (int h = 1; h >= 0; --h) {   // ascending positions
+            outputs(2, h, h4[h]);
+            const int pos = i0 + 4 * row + 3 - pp - h;
+            const bool ok = done && pos < i0 + FI_P && pos < L;
+            // in the order of head_chunk_kernel
+            float s = b5;
+#pragma unroll
+            for (int c4 = 0; c4 < CH / 4; ++c4) {
+                const float4 w5 = *reinterpret_cast<const float4*>(&sh.w5[4 * c4]);
+                const uint32_t p0 = h4[h][2 * c4], p1 = h4[h][2 * c4 + 1];
+                float part = (L & 7) == 0 ? 0.f : s;
+                part = fmaf(w5.x, fi_half(p0, 0), part);
+                part = fmaf(w5.y, fi_half(p0, 1), part);
+                part = fmaf(w5.z, fi_half(p1, 0), part);
+                part = fmaf(w5.w, fi_half(p1, 1), part);
+                s = (L & 7) == 0 ? s + part : part;
+            }
+            if (ok) {
+                z[(size_t)b * L + pos] = s;
+                if (s > zm) {
+                    zm = s;
+                    zi = pos;
+                }
+            }
+            // other positions count as 0 in the head's sums and, as every activation is >= 0 and every
+            // tile has a position of its own, in its maxima
+#pragma unroll
+            for (int k = 0; k < CH / 2; ++k) h4[h][k] = ok ? h4[h][k] : 0u;
+        }
+        isr::tmem_fence_before_sync();
+        // ---- chunk statistics of the head
+        {
+            float m = zm;
+            int mi = zi;
+            for (int o = 16; o; o >>= 1) {
+                const float om = __shfl_xor_sync(0xffffffffu, m, o);
+                const int oi = __shfl_xor_sync(0xffffffffu, mi, o);
+                if (om > m || (om == m && oi < mi)) {
+                    m = om;
+                    mi = oi;
+                }
+            }
+            float t[CH];
+#pragma unroll
+            for (int c = 0; c < CH; ++c) t[c] = fi_half(h4[0][c / 2], c & 1) + fi_half(h4[1][c / 2], c & 1);
+            sl.sum[w][lane] = fi_scatter_sum(t, lane);
+#pragma unroll
+            for (int k = 0; k < CH / 2; ++k) h4[0][k] = fi_max2(h4[0][k], h4[1][k]);
+            sl.mx[w][lane] = fi_scatter_max(h4[0], lane);
+            if (lane == 0) {
+                sl.zm[w] = m;
+                sl.zi[w] = mi;
+            }
+        }
+        slot_or(false);
+        isr::tmem_fence_after_sync();
+        if (w == 0) {
+            float m = sl.mx[0][lane], a = sl.sum[0][lane];
+#pragma unroll
+            for (int k = 1; k < 8; ++k) {
+                m = fmaxf(m, sl.mx[k][lane]);
+                a += sl.sum[k][lane];
+            }
+            const size_t o = ((size_t)b * nx + xc) * CH + lane;
+            pmax[o] = m;
+            psum[o] = a;
+            if (lane == 0) {
+                float best = sl.zm[0];
+                int at = sl.zi[0];
+                for (int k = 1; k < 8; ++k)
+                    if (sl.zm[k] > best || (sl.zm[k] == best && sl.zi[k] < at)) {
+                        best = sl.zm[k];
+                        at = sl.zi[k];
+                    }
+                zmax[(size_t)b * nx + xc] = best;
+                zidx[(size_t)b * nx + xc] = at;
+            }
+        }
+    }
+    isr::tmem_fence_before_sync();
+    __syncthreads();
+    isr::tmem_fence_after_sync();
+    if (tid < 32) isr::tmem_dealloc(sh.tslot, FI_COLS);
 }
 
 __device__ __forceinline__ float block_sum(float v, float* red)
@@ -1994,6 +2456,7 @@ isr_status set_smem_attrs()
     EST_TRY(cudaFuncSetAttribute(conv_kernel<float, T, float, T, CH, false>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, big));
     if constexpr (kTensorConv<T>) {
+        EST_TRY(cudaFuncSetAttribute(infer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FI_SMEM));
         EST_TRY(cudaFuncSetAttribute(conv_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)tc_smem_bytes(true)));
         EST_TRY(cudaFuncSetAttribute(conv_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2015,6 +2478,11 @@ isr_status set_smem_attrs()
     return ISR_OK;
 }
 
+HeadArgs head_args(const isr_est* e, int nx, float* pos, float* pres)
+{
+    return HeadArgs{e->theta, e->L, nx, e->lo, e->pmax, e->psum, e->z, e->zmax, e->pidx, e->zidx, e->amax, e->pooled, e->u, e->q, pos, pres};
+}
+
 // pos / pres: the prediction outputs (inference), or NULL
 template <class T>
 isr_status forward_t(isr_est* e, const float* x, int n, float* pos = nullptr, float* pres = nullptr)
@@ -2024,12 +2492,23 @@ isr_status forward_t(isr_est* e, const float* x, int n, float* pos = nullptr, fl
     T* act[5];
     for (int i = 0; i < 5; ++i) act[i] = static_cast<T*>(e->act[i]);
     const size_t nx = (size_t)n * L;
-    cast_kernel<T><<<(unsigned)std::min<size_t>((nx + 255) / 256, 4096), 256, 0, s>>>(x, nx, act[0]);
     if (e->weights_stale) {   // working weights follow the master copy only after it changed
         relayout_kernel<T><<<(CH * KT + 3 * CH * CH * KT + 255) / 256, 256, 0, s>>>(
             e->theta, static_cast<T*>(e->wf), static_cast<T*>(e->wb), static_cast<T*>(e->tf), static_cast<T*>(e->tb));
         e->weights_stale = false;
     }
+    if constexpr (kTensorConv<T>) {
+        if (pos && e->conv05) {
+            const int nxi = (L + FI_P - 1) / FI_P, tiles = n * nxi;
+            infer_kernel<<<std::min(e->sms, tiles), FI_SLOTS * FI_ST, FI_SMEM, s>>>(
+                x, static_cast<const T*>(e->wf), static_cast<const T*>(e->tf), n, e->z, e->pmax, e->psum, e->zmax,
+                e->zidx, e->theta, L, nxi);
+            head_mlp_kernel<true><<<n, HM_THREADS, 0, s>>>(head_args(e, nxi, pos, pres));
+            EST_TRY(cudaGetLastError());
+            return ISR_OK;
+        }
+    }
+    cast_kernel<T><<<(unsigned)std::min<size_t>((nx + 255) / 256, 4096), 256, 0, s>>>(x, nx, act[0]);
     const T* wf = static_cast<const T*>(e->wf);
     dim3 grid((L + CT - 1) / CT, n);
     // a training pass (no prediction outputs) of the tcgen05 engine leaves the ReLU masks of h1..h3
@@ -2057,8 +2536,8 @@ isr_status forward_t(isr_est* e, const float* x, int n, float* pos = nullptr, fl
     const int nxh = (L + HD_CT - 1) / HD_CT;
     head_chunk_kernel<T><<<dim3(nxh, n), 256, 0, s>>>(act[4], e->theta, L, nxh, e->z, e->pmax, e->pidx, e->psum,
                                                       e->zmax, e->zidx);
-    head_mlp_kernel<<<n, 64, 0, s>>>(e->theta, L, nxh, e->pmax, e->pidx, e->psum, e->z, e->zmax, e->zidx, e->lo,
-                                     e->amax, e->pooled, e->u, e->q, pos, pres);
+    if (pos) head_mlp_kernel<true><<<n, HM_THREADS, 0, s>>>(head_args(e, nxh, pos, pres));
+    else head_mlp_kernel<false><<<n, HM_THREADS, 0, s>>>(head_args(e, nxh, nullptr, nullptr));
     EST_TRY(cudaGetLastError());
     return ISR_OK;
 }
@@ -2190,7 +2669,8 @@ isr_status isr_est_create(isr_est** out, int32_t nfft, int32_t band_lo, int32_t 
     A((void**)&e->q, 4 * B);
     A((void**)&e->loss, 4);
     A((void**)&e->amax, 4 * B * CH);
-    const size_t nxh = (L + HD_CT - 1) / HD_CT;
+    const size_t nxh = (L + FI_P - 1) / FI_P;   // head chunks of the fused inference (training has no more)
+    static_assert(FI_P <= HD_CT, "head partials");
     A((void**)&e->pmax, 4 * B * nxh * CH);
     A((void**)&e->pidx, 4 * B * nxh * CH);
     A((void**)&e->psum, 4 * B * nxh * CH);
