@@ -238,18 +238,36 @@ __global__ void __launch_bounds__(256) conv_kernel(const TIN* __restrict__ in, c
                                                    int L, TOUT* __restrict__ out)
 {
     constexpr int XW = CT + KT - 1;
-    extern __shared__ float conv_smem[];
+    extern __shared__ __align__(16) float conv_smem[];
     float* xs = conv_smem;                 // [CIN][XW]
     float* ws = conv_smem + CIN * XW;      // [CIN][KT][CH]
     const int b = blockIdx.y;
     const int i0 = blockIdx.x * CT;
     const TIN* inb = in + (size_t)b * CIN * L;
-    for (int e = threadIdx.x; e < CIN * XW; e += 256) {
-        int ci = e / XW, j = e % XW;
-        int pos = i0 + j - HALF;
-        xs[e] = (pos >= 0 && pos < L) ? ld<TIN>(inb, (size_t)ci * L + pos) : 0.f;
+    // staging, every load of the thread in flight before its first store (with a few at a time the
+    // 54 KB took half of the kernel)
+    constexpr int XPER = (CIN * XW + 255) / 256, WPER = CIN * KT * CH / 4 / 256;
+    static_assert(CIN * KT * CH == WPER * 4 * 256, "whole 16-byte pieces per thread");
+    float xq[XPER];
+#pragma unroll
+    for (int u = 0; u < XPER; ++u) {
+        const int e = threadIdx.x + u * 256, ci = e / XW, pos = i0 + e % XW - HALF;
+        xq[u] = (e < CIN * XW && pos >= 0 && pos < L) ? ld<TIN>(inb, (size_t)ci * L + pos) : 0.f;
     }
-    for (int e = threadIdx.x; e < CIN * KT * CH; e += 256) ws[e] = ld<TW>(w, e);
+    if constexpr (std::is_same<TW, float>::value) {
+        float4 wq[WPER];
+#pragma unroll
+        for (int u = 0; u < WPER; ++u) wq[u] = reinterpret_cast<const float4*>(w)[threadIdx.x + u * 256];
+#pragma unroll
+        for (int u = 0; u < WPER; ++u) reinterpret_cast<float4*>(ws)[threadIdx.x + u * 256] = wq[u];
+    } else {
+        for (int e = threadIdx.x; e < CIN * KT * CH; e += 256) ws[e] = ld<TW>(w, e);
+    }
+#pragma unroll
+    for (int u = 0; u < XPER; ++u) {
+        const int e = threadIdx.x + u * 256;
+        if (e < CIN * XW) xs[e] = xq[u];
+    }
     __syncthreads();
     const int co = threadIdx.x & 31;
     const int p0 = (threadIdx.x >> 5) * 16;
@@ -258,9 +276,10 @@ __global__ void __launch_bounds__(256) conv_kernel(const TIN* __restrict__ in, c
 #pragma unroll
     for (int p = 0; p < 16; ++p) acc[p] = bv;
     for (int ci = 0; ci < CIN; ++ci) {
-        float xv[16 + KT - 1];
+        float xv[16 + KT - 1];   // the same for all lanes: six 16-byte loads (XW and p0 are multiples of 4)
 #pragma unroll
-        for (int j = 0; j < 16 + KT - 1; ++j) xv[j] = xs[ci * XW + p0 + j];
+        for (int j = 0; j < 16 + KT - 1; j += 4)
+            *reinterpret_cast<float4*>(xv + j) = *reinterpret_cast<const float4*>(xs + ci * XW + p0 + j);
 #pragma unroll
         for (int k = 0; k < KT; ++k) {
             const float wv = ws[(ci * KT + k) * CH + co];
@@ -1187,66 +1206,82 @@ __global__ void __launch_bounds__(W5_BLOCK, 1) wgrad_tc05_kernel(const __nv_bflo
 }
 
 // dW[co][ci][k] += sum_i da[b][co][i] h[b][ci][i + k - 4];  db[co] += sum_i da[b][co][i]
-// CTA: one row b, positions [i0, i0 + WG_SPAN); lane = co, warp = group of CIN/8 input channels
-constexpr int WG_SPAN = 1152;
+// CTA: one row b, positions [i0, i0 + span); lane = co, warp = four input channels.  Bound by shared
+// loads and FMAs: the activations are the same for all lanes, so they come 16 bytes at a time (16 loads
+// per 144 FMAs instead of 52).  The span shrinks until the launch has about four CTAs per SM: with one of
+// 1152 positions per row, 37 rows of 1101 left three quarters of the SMs idle (121 -> 32 us).  The sums
+// go out through shared memory so that the atomics of a warp fall on runs of 18 addresses instead of 32
+// sectors.
+constexpr int WG_MAX_SPAN = 1152;
 
-template <class TH, int CIN>
-__global__ void __launch_bounds__(256) wgrad_kernel(const TH* __restrict__ h, const float* __restrict__ da, int L,
+inline int wgrad_span(int L, int n, int sms)
+{
+    int span = WG_MAX_SPAN;
+    while (span > CT && (int64_t)n * ((L + span - 1) / span) < 4 * (int64_t)sms) span -= CT;
+    return span;
+}
+
+template <class TH>
+__global__ void __launch_bounds__(256) wgrad_kernel(const TH* __restrict__ h, const float* __restrict__ da, int L, int span,
                                                     float* __restrict__ dW, float* __restrict__ db)
 {
-    constexpr int CPW = CIN >= 8 ? CIN / 8 : 1;       // input channels per warp
-    constexpr int WARPS_USED = CIN >= 8 ? 8 : CIN;
-    __shared__ float das[CT][CH + 1];
-    __shared__ float hs[CIN][CT + KT - 1];
+    constexpr int CPW = CH / 8, HW = CT + KT - 1, RUN = CPW / 2 * KT;
+    static_assert(HW % 4 == 0 && WG_MAX_SPAN % CT == 0, "aligned window rows, whole tiles");
+    __shared__ __align__(16) float sm[CT * (CH + 1) + CH * HW];
+    static_assert(8 * CH * RUN <= CT * (CH + 1) + CH * HW, "output staging");
+    float* das = sm;                    // [CT][CH + 1]
+    float* hs = sm + CT * (CH + 1);     // [CH][HW]
+    static_assert(CT * (CH + 1) % 4 == 0, "16-byte rows");
     const int b = blockIdx.y;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool active = warp < WARPS_USED;
     float acc[CPW][KT];
 #pragma unroll
     for (int c = 0; c < CPW; ++c)
 #pragma unroll
         for (int k = 0; k < KT; ++k) acc[c][k] = 0.f;
     float dbacc = 0.f;
-    const int span_end = min(L, (int)(blockIdx.x + 1) * WG_SPAN);
-    for (int i0 = blockIdx.x * WG_SPAN; i0 < span_end; i0 += CT) {
+    const int span_end = min(L, (int)(blockIdx.x + 1) * span);
+    for (int i0 = blockIdx.x * span; i0 < span_end; i0 += CT) {
         __syncthreads();
         for (int e = threadIdx.x; e < CT * CH; e += 256) {
-            int co = e / CT, j = e % CT;
-            int pos = i0 + j;
-            das[j][co] = pos < span_end ? da[((size_t)b * CH + co) * L + pos] : 0.f;
+            const int co = e / CT, j = e % CT, pos = i0 + j;
+            das[j * (CH + 1) + co] = pos < span_end ? da[((size_t)b * CH + co) * L + pos] : 0.f;
         }
-        for (int e = threadIdx.x; e < CIN * (CT + KT - 1); e += 256) {
-            int ci = e / (CT + KT - 1), j = e % (CT + KT - 1);
-            int pos = i0 + j - HALF;
-            hs[ci][j] = (pos >= 0 && pos < L) ? ld<TH>(h, ((size_t)b * CIN + ci) * L + pos) : 0.f;
+        for (int e = threadIdx.x; e < CH * HW; e += 256) {
+            const int ci = e / HW, j = e % HW, pos = i0 + j - HALF;
+            hs[e] = (pos >= 0 && pos < L) ? ld<TH>(h, ((size_t)b * CH + ci) * L + pos) : 0.f;
         }
         __syncthreads();
-        if (active) {
-            for (int j = 0; j < CT; j += 4) {
-                float d[4];
+        for (int j = 0; j < CT; j += 4) {
+            float d[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) d[q] = das[j + q][lane];
-                if (warp == 0) dbacc += d[0] + d[1] + d[2] + d[3];
+            for (int q = 0; q < 4; ++q) d[q] = das[(j + q) * (CH + 1) + lane];
+            if (warp == 0) dbacc += d[0] + d[1] + d[2] + d[3];
 #pragma unroll
-                for (int c = 0; c < CPW; ++c) {
-                    const float* hr = hs[warp * CPW + c] + j;
-                    float hv[4 + KT - 1];
+            for (int c = 0; c < CPW; ++c) {
+                const float* hr = hs + (warp * CPW + c) * HW + j;
+                float hv[4 + KT - 1];
 #pragma unroll
-                    for (int q = 0; q < 4 + KT - 1; ++q) hv[q] = hr[q];
+                for (int q = 0; q < 4 + KT - 1; q += 4)
+                    *reinterpret_cast<float4*>(hv + q) = *reinterpret_cast<const float4*>(hr + q);
 #pragma unroll
-                    for (int k = 0; k < KT; ++k)
+                for (int k = 0; k < KT; ++k)
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) acc[c][k] = fmaf(d[q], hv[q + k], acc[c][k]);
-                }
+                    for (int q = 0; q < 4; ++q) acc[c][k] = fmaf(d[q], hv[q + k], acc[c][k]);
             }
         }
     }
-    if (active) {
+    if (warp == 0) atomicAdd(&db[lane], dbacc);
+    float* st = sm + warp * CH * RUN;   // [co][two channels x 9 taps]
 #pragma unroll
-        for (int c = 0; c < CPW; ++c)
+    for (int half = 0; half < 2; ++half) {
+        if (half == 0) __syncthreads();
+        else __syncwarp();
 #pragma unroll
-            for (int k = 0; k < KT; ++k) atomicAdd(&dW[((size_t)lane * CIN + warp * CPW + c) * KT + k], acc[c][k]);
-        if (warp == 0) atomicAdd(&db[lane], dbacc);
+        for (int r = 0; r < RUN; ++r) st[lane * RUN + r] = acc[half * (CPW / 2) + r / KT][r % KT];
+        __syncwarp();
+        for (int e = lane; e < CH * RUN; e += 32)
+            atomicAdd(&dW[(size_t)(e / RUN) * CH * KT + (warp * CPW + half * (CPW / 2)) * KT + e % RUN], st[e]);
     }
 }
 
@@ -2558,8 +2593,8 @@ isr_status backward_t(isr_est* e, int n, const float* fpos, const float* pres)
     const T* wbk = static_cast<const T*>(e->wb);
     float* da = e->da0;
     float* dn = e->da1;
-    dim3 gw((L + WG_SPAN - 1) / WG_SPAN, n);
     dim3 gc((L + CT - 1) / CT, n);
+    const int fspan = wgrad_span(L, n, std::max(1, e->sms));
     const int span = TC_CT * wgrad_span_chunks(L, n, std::max(1, e->wgrad_slots));
     for (int l = 4; l >= 1; --l) {
         if (l == 1) {
@@ -2578,7 +2613,8 @@ isr_status backward_t(isr_est* e, int n, const float* fpos, const float* pres)
                         act[l - 1], da, L, span, e->grad + w_off(l), e->grad + b_off(l));
                 }
             } else
-                wgrad_kernel<T, CH><<<gw, 256, 0, s>>>(act[l - 1], da, L, e->grad + w_off(l), e->grad + b_off(l));
+                wgrad_kernel<T><<<dim3((L + fspan - 1) / fspan, n), 256, 0, s>>>(act[l - 1], da, L, fspan, e->grad + w_off(l),
+                                                                                 e->grad + b_off(l));
             // gradient into the layer below, masked by its ReLU: da_{l-1} = (W_l^T * da_l) (h_{l-1} > 0)
             if constexpr (kTensorConv<T>) {
                 const T* w = static_cast<const T*>(e->tb) + (size_t)(l - 2) * CH * CH * KT;

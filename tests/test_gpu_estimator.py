@@ -171,6 +171,54 @@ def test_features_band_lengths_and_floors(L):
     assert (np.abs(x - want) <= 1.2e-7 * np.abs(want) + 1e-9).all()
 
 
+@pytest.mark.parametrize("B,L", [(1, 16), (2, 129), (5, 1153)])
+def test_fp32_gradients_over_spans_and_rows(B, L):
+    """FP32 storage where the weight gradient splits its rows differently: one short tile, and one position
+    into a second tile or span; the bound of the other FP32 gradient test (2e-4 of each block's largest
+    gradient)."""
+    rng = np.random.default_rng(B + L)
+    theta = (ref.init_params(3) + 0.05 * rng.standard_normal(ref.N_PARAMS)).astype(np.float32)
+    x = rng.standard_normal((B, L)).astype(np.float32)
+    f = rng.uniform(3, L - 3, B).astype(np.float32)
+    y = np.resize(np.array([1, 0, 1, 1], dtype=np.float32), B)
+    e = est_mod.Estimator(max_batch=B, precision=isr.ISR_EST_FP32, nfft=L, band_lo=0, band_len=L)
+    e.set_params(theta)
+    loss, g = e.grad(*[torch.from_numpy(a).cuda() for a in (x, f, y)])
+    e.close()
+    rl, rg = ref.loss_and_grad(theta.astype(np.float64), x, f, y)
+    assert abs(loss - rl) <= 1e-5 * abs(rl)
+    gd, rd = ref.unpack(g.astype(np.float64)), ref.unpack(rg)
+    gmax = np.abs(rg).max()
+    for name, _ in ref.SHAPES:
+        scale = max(np.abs(rd[name]).max(), 1e-3 * gmax)
+        err = np.abs(gd[name] - rd[name]).max() / scale
+        assert err <= 2e-4, f"{name}: max error {err:.2e} of the block's largest gradient"
+
+
+def test_fp32_batch_gradient_is_the_mean_over_its_rows():
+    """300 rows at once (spans of 128 positions, several waves) against the same rows one at a time (one
+    span per tile): the forward pass and its masks are the same per row, so the batch gradient is the
+    mean of the rows' up to FP32 summation, 300 x 130 terms in any order: 1e-4 of each block's largest."""
+    B, L = 300, 130
+    rng = np.random.default_rng(B + L)
+    theta = (ref.init_params(3) + 0.05 * rng.standard_normal(ref.N_PARAMS)).astype(np.float32)
+    arrays = [torch.from_numpy(a).cuda() for a in (rng.standard_normal((B, L)).astype(np.float32),
+                                                   rng.uniform(3, L - 3, B).astype(np.float32),
+                                                   np.resize(np.array([1, 0, 1, 1], dtype=np.float32), B))]
+    e = est_mod.Estimator(max_batch=B, precision=isr.ISR_EST_FP32, nfft=L, band_lo=0, band_len=L)
+    e.set_params(theta)
+    _, g = e.grad(*arrays)
+    rows = np.zeros(ref.N_PARAMS)
+    for r in range(B):
+        rows += e.grad(*[a[r:r + 1].contiguous() for a in arrays])[1].astype(np.float64)
+    e.close()
+    gd, rd = ref.unpack(g.astype(np.float64)), ref.unpack(rows / B)
+    gmax = np.abs(rows / B).max()
+    for name, _ in ref.SHAPES:
+        scale = max(np.abs(rd[name]).max(), 1e-3 * gmax)
+        assert np.abs(gd[name] - rd[name]).max() <= 1e-4 * scale, name
+
+
 @pytest.mark.slow
 def test_training_gains_over_peak_fit():
     """Short training on integrator-made spectra (reduced from the full 200k-spectrum run):
