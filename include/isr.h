@@ -313,14 +313,16 @@ isr_status isr_est_predict(isr_est* est, const float* x, int32_t n, float* line_
 void isr_est_destroy(isr_est* est);
 
 /*
- * Batched integration of many windows of uneven shape in one persistent launch.  Radars
+ * Batched integration of many windows of uneven shape as one run.  Radars
  * integrate several windows at once, e.g. the up- and down-shifted plasma-line channels
  * (the line appears at +-f_r, Sec. 2.1) with different range extents and resolutions.
  * Each window is an independent integration (Eqs. 7-8) with its own echo, code and
  * geometry; isr_batch_run writes, for every window, the sum over its n_ipp IPPs as float
- * [n_ranges][nfft] into its `out`.  All (gate group, IPP chunk) units of all windows
- * form one queue, longest first, served by one CTA per SM.  Buffers are device memory and
- * stay bound to the batch: refill them between runs.  Limits: nfft in {2048, 4096, 8192,
+ * [n_ranges][nfft] into its `out`.  The (gate group, IPP chunk) units of the default radix
+ * order are dealt to one persistent CTA per SM and transform length, longest first to the CTA
+ * with the least work, one launch per length on streams that fork from and join the batch's;
+ * units of orders 1 to 3 form one queue served by one CTA per SM.  Buffers are device memory
+ * and stay bound to the batch: refill them between runs.  Limits: nfft in {2048, 4096, 8192,
  * 16384}; binary-phase codes (ISR_TX_PM1) only.
  */
 typedef struct {

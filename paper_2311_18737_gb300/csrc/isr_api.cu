@@ -45,6 +45,7 @@ cudaError_t prepare_entry(const KernelEntry& ke, int log2n, int dev, cudaStream_
     set(ke.fn, ke.smem);
     for (int o = 0; o < kNumOrders; ++o) set(ke.fn_order[o], ke.smem_order[o]);
     set(ke.fn_xt, ke.smem_xt);
+    set(ke.fn_xt_batch, ke.smem_xt);
     if (e != cudaSuccess || !ke.fn_tables) return e;
     // the tables are the same for every user: filled under the lock, complete before it is released
     static std::mutex mu;

@@ -1,18 +1,22 @@
-// isr_batch.cu -- many integration windows of uneven shape in one persistent launch.
+// isr_batch.cu -- many integration windows of uneven shape as one run.
 //
 // A radar usually integrates several windows at once: up- and down-shifted plasma-line
 // channels (the line sits at +-f_r, Sec. 2.1 of the paper), different range extents and
-// spectral resolutions.  Here every window's (gate group, IPP chunk) work units form one
-// queue, ordered longest first; one CTA per SM pulls units from the queue with an atomic
-// counter and runs the fused decode -> FFT -> |X|^2 unit of the matching transform length.
-// The launch and the chunk reduction can be captured once in a CUDA graph and replayed.
-// The Stockham radix order of each transform length can be picked by timing the
-// candidates on the windows themselves (autotuning).
+// spectral resolutions.  Every window is cut into (gate group, IPP chunk) work units.  The
+// units of the default radix order are dealt to one persistent CTA per SM and transform
+// length, longest first to the CTA with the least work (their cost is known: it goes by IPPs), and
+// run in the fused kernel with its exchange in tensor memory, one launch per transform
+// length on streams of their own, so that an SM that is done with one length starts the next
+// (32 windows with 10-100 IPPs: 22.7 ms from one queue of every shape in one kernel, 18.5 ms so).
+// Units of the other radix orders form one queue, longest first, from which one CTA per SM
+// pulls with an atomic counter.  The launches and the chunk reduction can be captured once in
+// a CUDA graph and replayed.  The radix order of each transform length can be picked by
+// timing the candidates on the windows themselves (autotuning).
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <new>
-#include <numeric>
+#include <queue>
 #include <vector>
 
 #include "isr.h"
@@ -26,17 +30,9 @@ constexpr int kMinLog2 = 11, kMaxLog2 = 14;
 constexpr int kChunk = 256;
 constexpr unsigned kWaitLimit = 1u << 22;
 
-struct BatchWin {
-    isr::KArgs a;
-    int log2n;
-    int order;
-    int n_gx;   // gate groups
-    int n_cy;   // IPP chunks
-};
-
-struct BatchUnit {
-    int win, gx, cy, pad;
-};
+using isr::BatchUnit;
+using isr::BatchWin;
+using isr::XtBatchSrc;
 
 template <int L, int O>
 constexpr int smem_of() { return isr::Sched<L, O>::SMEM; }
@@ -44,8 +40,7 @@ constexpr int smem_of() { return isr::Sched<L, O>::SMEM; }
 constexpr int max_smem()
 {
     int m = 0;
-    int v[] = {smem_of<11, 0>(), smem_of<11, 1>(), smem_of<11, 2>(), smem_of<12, 0>(), smem_of<12, 1>(),
-               smem_of<12, 2>(), smem_of<13, 0>(), smem_of<13, 1>(), smem_of<13, 2>(), smem_of<14, 0>(),
+    int v[] = {smem_of<11, 1>(), smem_of<11, 2>(), smem_of<12, 1>(), smem_of<12, 2>(), smem_of<13, 1>(), smem_of<13, 2>(),
                smem_of<14, 1>(), smem_of<14, 2>(), isr::SchedWL<11>::SMEM, isr::SchedWL<12>::SMEM,
                isr::SchedWL<13>::SMEM, isr::SchedWL<14>::SMEM};
     for (int x : v) m = x > m ? x : m;
@@ -71,7 +66,7 @@ __device__ __noinline__ bool run_unit(const BatchWin& w, const BatchUnit& u, uns
     }
 }
 
-// Persistent: one CTA per SM pulls work units until the queue is empty.
+// Persistent, radix orders 1 to 3: one CTA per SM pulls work units until the queue is empty.
 __global__ void __launch_bounds__(isr::kThreads, 1) batch_kernel(const BatchWin* __restrict__ wins,
                                                                  const BatchUnit* __restrict__ units, int n_units,
                                                                  int* __restrict__ counter)
@@ -108,19 +103,15 @@ __global__ void __launch_bounds__(isr::kThreads, 1) batch_kernel(const BatchWin*
         const bool setup = key != prev_key;
         bool ok = true;
         switch (key) {
-        case 11 * 4 + 0: ok = run_unit<11, 0>(w, u, smem, s_phase, setup); break;
         case 11 * 4 + 1: ok = run_unit<11, 1>(w, u, smem, s_phase, setup); break;
         case 11 * 4 + 2: ok = run_unit<11, 2>(w, u, smem, s_phase, setup); break;
         case 11 * 4 + 3: ok = run_unit<11, 3>(w, u, smem, s_phase, setup); break;
-        case 12 * 4 + 0: ok = run_unit<12, 0>(w, u, smem, s_phase, setup); break;
         case 12 * 4 + 1: ok = run_unit<12, 1>(w, u, smem, s_phase, setup); break;
         case 12 * 4 + 2: ok = run_unit<12, 2>(w, u, smem, s_phase, setup); break;
         case 12 * 4 + 3: ok = run_unit<12, 3>(w, u, smem, s_phase, setup); break;
-        case 13 * 4 + 0: ok = run_unit<13, 0>(w, u, smem, s_phase, setup); break;
         case 13 * 4 + 1: ok = run_unit<13, 1>(w, u, smem, s_phase, setup); break;
         case 13 * 4 + 2: ok = run_unit<13, 2>(w, u, smem, s_phase, setup); break;
         case 13 * 4 + 3: ok = run_unit<13, 3>(w, u, smem, s_phase, setup); break;
-        case 14 * 4 + 0: ok = run_unit<14, 0>(w, u, smem, s_phase, setup); break;
         case 14 * 4 + 1: ok = run_unit<14, 1>(w, u, smem, s_phase, setup); break;
         case 14 * 4 + 2: ok = run_unit<14, 2>(w, u, smem, s_phase, setup); break;
         case 14 * 4 + 3: ok = run_unit<14, 3>(w, u, smem, s_phase, setup); break;
@@ -148,7 +139,7 @@ struct RedSeg {
 };
 
 // out[i] = sum_c part[c][i], FP32 with Kahan compensation (error ~2 ulp for any chunk count);
-// one window per blockIdx.y
+// one window per blockIdx.y.  A window of one chunk needs none: its units write into out.
 __global__ void batch_reduce_kernel(const RedSeg* __restrict__ segs)
 {
     const RedSeg s = segs[blockIdx.y];
@@ -190,9 +181,19 @@ struct isr_batch {
     cudaStream_t cap_stream = nullptr;
     std::vector<isr_window> w;
     std::vector<BatchWin> hw;
+    // units in launch order: transform lengths 2048 .. 16384 of order 0, dealt to CTAs (first[L] holds the
+    // bounds of each CTA's), then the queue of the other orders
     std::vector<BatchUnit> hu;
+    std::vector<int> first[4];
+    int n_queue = 0;
+    isr::KernelEntry ke[4];
+    cudaStream_t side[4] = {nullptr, nullptr, nullptr, nullptr};
+    cudaEvent_t fork = nullptr, join[4] = {nullptr, nullptr, nullptr, nullptr};
+    int n_segs = 0;
+    int64_t n_units = 0;
     BatchWin* d_wins = nullptr;
     BatchUnit* d_units = nullptr;
+    int* d_first = nullptr;   // [4][sm_count + 1]
     RedSeg* d_segs = nullptr;
     float* partial = nullptr;
     int* counter = nullptr;
@@ -207,43 +208,94 @@ struct isr_batch {
 
 namespace {
 
-// unit list of the chosen windows (all if only < 0), longest work first
-void build_units(isr_batch* b, int only_log2n, std::vector<BatchUnit>& out)
+// Units of the chosen windows (all if only < 0), longest work first; with limit > 0 the first `limit` of them.
+void build_units(isr_batch* b, int only_log2n, size_t limit)
 {
-    out.clear();
+    std::vector<BatchUnit> all;
     for (int i = 0; i < (int)b->hw.size(); ++i) {
         const BatchWin& w = b->hw[i];
         if (only_log2n >= 0 && w.log2n != only_log2n) continue;
         for (int c = 0; c < w.n_cy; ++c)
-            for (int g = 0; g < w.n_gx; ++g) out.push_back(BatchUnit{i, g, c, 0});
+            for (int g = 0; g < w.n_gx; ++g) all.push_back(BatchUnit{i, g, c, 0});
     }
+    // 16384 points per CTA per IPP for every shape; a unit's start and end cost about a third of an IPP
     auto cost = [&](const BatchUnit& u) {
         const BatchWin& w = b->hw[u.win];
         const int p0 = u.cy * w.a.chunk_len;
-        const int n = std::min(p0 + w.a.chunk_len, w.a.n_ipp) - p0;
-        return (double)n * w.log2n;   // 16384 points per CTA per IPP for every shape
+        return (std::min(p0 + w.a.chunk_len, w.a.n_ipp) - p0 + 0.33) * w.log2n;
     };
-    std::stable_sort(out.begin(), out.end(), [&](const BatchUnit& x, const BatchUnit& y) { return cost(x) > cost(y); });
+    std::stable_sort(all.begin(), all.end(), [&](const BatchUnit& x, const BatchUnit& y) { return cost(x) > cost(y); });
+    if (limit > 0) all.resize(std::min(all.size(), limit));
+
+    b->hu.clear();
+    for (int l = 0; l < 4; ++l) {
+        // the next unit goes to the CTA with the least work so far
+        std::vector<std::vector<BatchUnit>> mine(b->sm_count);
+        using Load = std::pair<double, int>;
+        std::priority_queue<Load, std::vector<Load>, std::greater<Load>> load;
+        for (int c = 0; c < b->sm_count; ++c) load.push(Load(0.0, c));
+        for (const BatchUnit& u : all) {
+            if (b->hw[u.win].log2n != kMinLog2 + l || b->hw[u.win].order != 0) continue;
+            Load t = load.top();
+            load.pop();
+            mine[t.second].push_back(u);
+            load.push(Load(t.first + cost(u), t.second));
+        }
+        b->first[l].assign(b->sm_count + 1, 0);
+        for (int c = 0; c < b->sm_count; ++c) {
+            b->first[l][c] = (int)b->hu.size();
+            b->hu.insert(b->hu.end(), mine[c].begin(), mine[c].end());
+        }
+        b->first[l][b->sm_count] = (int)b->hu.size();
+    }
+    const size_t dealt = b->hu.size();
+    for (const BatchUnit& u : all)
+        if (b->hw[u.win].order != 0) b->hu.push_back(u);
+    b->n_queue = (int)(b->hu.size() - dealt);
 }
 
-isr_status upload(isr_batch* b, const std::vector<BatchUnit>& units, cudaStream_t s)
+isr_status upload(isr_batch* b, cudaStream_t s)
 {
     B_TRY(cudaMemcpyAsync(b->d_wins, b->hw.data(), sizeof(BatchWin) * b->hw.size(), cudaMemcpyHostToDevice, s));
-    B_TRY(cudaMemcpyAsync(b->d_units, units.data(), sizeof(BatchUnit) * units.size(), cudaMemcpyHostToDevice, s));
+    B_TRY(cudaMemcpyAsync(b->d_units, b->hu.data(), sizeof(BatchUnit) * b->hu.size(), cudaMemcpyHostToDevice, s));
+    for (int l = 0; l < 4; ++l)
+        B_TRY(cudaMemcpyAsync(b->d_first + l * (b->sm_count + 1), b->first[l].data(), sizeof(int) * (b->sm_count + 1),
+                              cudaMemcpyHostToDevice, s));
     return ISR_OK;
 }
 
-isr_status enqueue(isr_batch* b, int n_units, bool reduce, cudaStream_t s)
+isr_status enqueue(isr_batch* b, bool reduce, cudaStream_t s)
 {
-    B_TRY(cudaMemsetAsync(b->counter, 0, sizeof(int), s));
-    batch_kernel<<<b->sm_count, isr::kThreads, kBatchSmem, s>>>(b->d_wins, b->d_units, n_units, b->counter);
-    B_TRY(cudaGetLastError());
-    if (reduce) {
+    const int n_dealt = (int)b->hu.size() - b->n_queue;
+    // longest lists first, each on a stream of its own between fork and join
+    int by_work[4] = {0, 1, 2, 3};
+    auto units_of = [&](int l) { return b->first[l][b->sm_count] - b->first[l][0]; };
+    std::sort(by_work, by_work + 4, [&](int x, int y) { return units_of(x) > units_of(y); });
+    B_TRY(cudaEventRecord(b->fork, s));
+    bool used[4] = {false, false, false, false};
+    for (int l : by_work) {
+        if (units_of(l) == 0) continue;
+        used[l] = true;
+        B_TRY(cudaStreamWaitEvent(b->side[l], b->fork, 0));
+        XtBatchSrc src{b->d_wins, b->d_units, b->d_first + l * (b->sm_count + 1), kWaitLimit, b->status};
+        void* args[] = {&src};
+        B_TRY(cudaLaunchKernel(b->ke[l].fn_xt_batch, dim3((unsigned)std::min(b->sm_count, units_of(l))), dim3(isr::kThreads),
+                               args, (size_t)b->ke[l].smem_xt, b->side[l]));
+        B_TRY(cudaEventRecord(b->join[l], b->side[l]));
+    }
+    if (b->n_queue > 0) {
+        B_TRY(cudaMemsetAsync(b->counter, 0, sizeof(int), s));
+        batch_kernel<<<b->sm_count, isr::kThreads, kBatchSmem, s>>>(b->d_wins, b->d_units + n_dealt, b->n_queue, b->counter);
+        B_TRY(cudaGetLastError());
+    }
+    for (int l = 0; l < 4; ++l)
+        if (used[l]) B_TRY(cudaStreamWaitEvent(s, b->join[l], 0));
+    if (reduce && b->n_segs > 0) {
         // memory-bound: about four waves of 256-thread CTAs over all windows (8 per SM resident),
         // at most one CTA per 256 elements of the largest window
-        const int64_t want = (4 * 8 * (int64_t)b->sm_count + (int64_t)b->w.size() - 1) / (int64_t)b->w.size();
+        const int64_t want = (4 * 8 * (int64_t)b->sm_count + b->n_segs - 1) / b->n_segs;
         const int64_t gx = std::max<int64_t>(1, std::min<int64_t>(want, (b->max_bins + 255) / 256));
-        batch_reduce_kernel<<<dim3((unsigned)gx, (unsigned)b->w.size()), 256, 0, s>>>(b->d_segs);
+        batch_reduce_kernel<<<dim3((unsigned)gx, (unsigned)b->n_segs), 256, 0, s>>>(b->d_segs);
         B_TRY(cudaGetLastError());
     }
     return ISR_OK;
@@ -254,7 +306,6 @@ isr_status autotune(isr_batch* b)
     cudaEvent_t e0, e1;
     B_TRY(cudaEventCreate(&e0));
     B_TRY(cudaEventCreate(&e1));
-    std::vector<BatchUnit> units;
     for (int L = kMinLog2; L <= kMaxLog2; ++L) {
         bool used = false;
         for (auto& w : b->hw) used |= w.log2n == L;
@@ -267,15 +318,14 @@ isr_status autotune(isr_batch* b)
         for (int o = 0; o < isr::kOrders; ++o) {
             for (auto& w : b->hw)
                 if (w.log2n == L) w.order = o;
-            build_units(b, L, units);
             // a probe of a few waves is enough to rank the orders
-            units.resize(std::min<size_t>(units.size(), (size_t)b->sm_count * 3));
-            isr_status st = upload(b, units, b->cap_stream);
+            build_units(b, L, (size_t)b->sm_count * 3);
+            isr_status st = upload(b, b->cap_stream);
             if (st != ISR_OK) return st;
-            st = enqueue(b, (int)units.size(), false, b->cap_stream);   // warm-up
+            st = enqueue(b, false, b->cap_stream);   // warm-up
             if (st != ISR_OK) return st;
             B_TRY(cudaEventRecord(e0, b->cap_stream));
-            st = enqueue(b, (int)units.size(), false, b->cap_stream);
+            st = enqueue(b, false, b->cap_stream);
             if (st != ISR_OK) return st;
             B_TRY(cudaEventRecord(e1, b->cap_stream));
             B_TRY(cudaEventSynchronize(e1));
@@ -344,8 +394,20 @@ isr_status isr_batch_create(isr_batch** out, const isr_window* windows, int32_t 
         return bail(fail(ISR_ERR_CUDA, "device query failed"));
     cudaError_t e = cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBatchSmem);
     if (e != cudaSuccess) return bail(fail(ISR_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e)));
-    if (cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking) != cudaSuccess)
+    if (cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) != cudaSuccess)
         return bail(fail(ISR_ERR_CUDA, "stream creation failed"));
+    for (int l = 0; l < 4; ++l) {
+        bool used = false;
+        for (int i = 0; i < n_windows; ++i) used |= windows[i].nfft == 1 << (kMinLog2 + l);
+        if (!used) continue;
+        b->ke[l] = isr::kernel_entry(kMinLog2 + l, isr::TX_PM1);
+        if (cudaStreamCreateWithFlags(&b->side[l], cudaStreamNonBlocking) != cudaSuccess ||
+            cudaEventCreateWithFlags(&b->join[l], cudaEventDisableTiming) != cudaSuccess)
+            return bail(fail(ISR_ERR_CUDA, "stream creation failed"));
+        e = isr::prepare_entry(b->ke[l], kMinLog2 + l, dev, b->cap_stream);
+        if (e != cudaSuccess) return bail(fail(ISR_ERR_CUDA, "kernel preparation: %s", cudaGetErrorString(e)));
+    }
 
     // chunking and scratch layout
     int64_t part_floats = 0;
@@ -373,13 +435,14 @@ isr_status isr_batch_create(isr_batch** out, const isr_window* windows, int32_t 
         bw.a.chunk_len = chunk;
         bw.a.wait_limit = kWaitLimit;
         bw.a.drop_ipp = -1;
+        bw.a.chip_bytes = 1;
         part_off[i] = part_floats;
-        part_floats += (int64_t)bw.n_cy * w.n_ranges * w.nfft;
+        if (bw.n_cy > 1) part_floats += (int64_t)bw.n_cy * w.n_ranges * w.nfft;
         b->hw.push_back(bw);
         b->transforms += (int64_t)w.n_ranges * w.n_ipp;
         b->max_bins = std::max<int64_t>(b->max_bins, (int64_t)w.n_ranges * w.nfft);
     }
-    e = cudaMalloc(&b->partial, sizeof(float) * part_floats);
+    e = cudaMalloc(&b->partial, sizeof(float) * std::max<int64_t>(part_floats, 1));
     if (e == cudaSuccess) e = cudaMalloc(&b->counter, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&b->status, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_wins, sizeof(BatchWin) * n_windows);
@@ -387,31 +450,36 @@ isr_status isr_batch_create(isr_batch** out, const isr_window* windows, int32_t 
     int64_t max_units = 0;
     for (auto& bw : b->hw) max_units += (int64_t)bw.n_gx * bw.n_cy;
     if (e == cudaSuccess) e = cudaMalloc(&b->d_units, sizeof(BatchUnit) * max_units);
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_first, sizeof(int) * 4 * (b->sm_count + 1));
     if (e != cudaSuccess)
         return bail(fail(e == cudaErrorMemoryAllocation ? ISR_ERR_NO_MEMORY : ISR_ERR_CUDA, "allocation failed: %s",
                          cudaGetErrorString(e)));
-    std::vector<RedSeg> segs(n_windows);
+    std::vector<RedSeg> segs;
     for (int i = 0; i < n_windows; ++i) {
-        b->hw[i].a.partial = b->partial + part_off[i];
+        const bool direct = b->hw[i].n_cy == 1;
+        b->hw[i].a.partial = direct ? windows[i].out : b->partial + part_off[i];
         b->hw[i].a.status = b->status;
-        segs[i] = RedSeg{b->partial + part_off[i], windows[i].out, (int64_t)windows[i].n_ranges * windows[i].nfft,
-                         b->hw[i].n_cy};
+        if (!direct)
+            segs.push_back(RedSeg{b->partial + part_off[i], windows[i].out, (int64_t)windows[i].n_ranges * windows[i].nfft,
+                                  b->hw[i].n_cy});
     }
-    e = cudaMemcpy(b->d_segs, segs.data(), sizeof(RedSeg) * n_windows, cudaMemcpyHostToDevice);
+    b->n_segs = (int)segs.size();
+    e = segs.empty() ? cudaSuccess : cudaMemcpy(b->d_segs, segs.data(), sizeof(RedSeg) * segs.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(b->status, 0, sizeof(int));
     if (e != cudaSuccess) return bail(fail(ISR_ERR_CUDA, "upload failed: %s", cudaGetErrorString(e)));
 
     isr_status st = ISR_OK;
     if (flags & ISR_BATCH_AUTOTUNE) st = autotune(b);
     if (st != ISR_OK) return bail(st);
-    build_units(b, -1, b->hu);
-    st = upload(b, b->hu, b->cap_stream);
+    build_units(b, -1, 0);
+    b->n_units = (int64_t)b->hu.size();
+    st = upload(b, b->cap_stream);
     if (st == ISR_OK && cudaStreamSynchronize(b->cap_stream) != cudaSuccess) st = fail(ISR_ERR_CUDA, "upload failed");
     if (st != ISR_OK) return bail(st);
     if (flags & ISR_BATCH_GRAPH) {
         e = cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return bail(fail(ISR_ERR_CUDA, "begin capture: %s", cudaGetErrorString(e)));
-        st = enqueue(b, (int)b->hu.size(), true, b->cap_stream);
+        st = enqueue(b, true, b->cap_stream);
         e = cudaStreamEndCapture(b->cap_stream, &b->graph);
         if (st != ISR_OK) return bail(st);
         if (e != cudaSuccess) return bail(fail(ISR_ERR_CUDA, "end capture: %s", cudaGetErrorString(e)));
@@ -435,7 +503,7 @@ isr_status isr_batch_run(isr_batch* b)
         cudaError_t e = cudaGraphLaunch(b->exec, b->user_stream);
         if (e != cudaSuccess) st = fail(ISR_ERR_CUDA, "graph launch: %s", cudaGetErrorString(e));
     } else {
-        st = enqueue(b, (int)b->hu.size(), true, b->user_stream);
+        st = enqueue(b, true, b->user_stream);
     }
     if (prev >= 0) cudaSetDevice(prev);
     return st;
@@ -464,7 +532,7 @@ isr_status isr_batch_query(const isr_batch* b, isr_batch_info* info)
     if (!b || !info) return fail(ISR_ERR_INVALID_ARG, "NULL argument");
     info->n_windows = (int32_t)b->w.size();
     info->graph = b->exec != nullptr;
-    info->n_units = (int64_t)b->hu.size();
+    info->n_units = b->n_units;
     info->transforms = b->transforms;
     for (int i = 0; i < 4; ++i) {
         info->order[i] = b->order[i];
@@ -484,11 +552,17 @@ void isr_batch_destroy(isr_batch* b)
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->graph) cudaGraphDestroy(b->graph);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
+    for (int l = 0; l < 4; ++l) {
+        if (b->side[l]) cudaStreamDestroy(b->side[l]);
+        if (b->join[l]) cudaEventDestroy(b->join[l]);
+    }
+    if (b->fork) cudaEventDestroy(b->fork);
     cudaFree(b->partial);
     cudaFree(b->counter);
     cudaFree(b->status);
     cudaFree(b->d_wins);
     cudaFree(b->d_units);
+    cudaFree(b->d_first);
     cudaFree(b->d_segs);
     cudaGetLastError();
     if (prev >= 0) cudaSetDevice(prev);

@@ -33,6 +33,7 @@ struct KernelEntry {
     // nfft >= 1024: the kernel with its last exchange in tensor memory (isr_xt.cuh), persistent, launched
     // by launch_integrate; pack forms its sign words of per-IPP binary-phase codes
     const void* fn_xt = nullptr;
+    const void* fn_xt_batch = nullptr;   // the same kernel over the units of a batch (binary phase, nfft >= 2048)
     const void* fn_pack = nullptr;
     const void* fn_tables = nullptr;   // fills the twiddle tables of the current device
     int smem_xt = 0;
@@ -57,6 +58,8 @@ KernelEntry entry_for(int txt)
                 : txt == TX_C32  ? (const void*)integrate_kernel_xt<L, TX_C32, XtPlanSrc>
                                  : (const void*)integrate_kernel_xt<L, TX_PM1, XtPlanSrc>;
         e.fn_pack = txt == TX_PM1 ? (const void*)pack_signs_kernel<SchedX<L>::T> : nullptr;
+        if constexpr (L >= 11)
+            if (txt == TX_PM1) e.fn_xt_batch = (const void*)integrate_kernel_xt<L, TX_PM1, XtBatchSrc>;
         e.fn_tables = (const void*)xt_tables_kernel<L>;
         e.smem_xt = SchedX<L>::SMEM;
     }

@@ -248,6 +248,7 @@ struct XtUnit {
     int n;                   // IPPs
     int un;                  // index of the unit in its launch
     uint32_t it0;            // IPPs of this gate before the unit
+    int wipe;                // the stage behind the code may hold samples of another unit
     int drop;                // test hook: the IPP that is never staged, -1 = none
     int ok;                  // debug builds: the window lies in its row
 };
@@ -287,10 +288,40 @@ struct XtPlanSrc {
     {
         xt_fill<LOG2N>(x, a, un % rg, un / rg, g, t);
     }
-    __device__ __forceinline__ bool short_codes(int nfft) const { return a.code_len < nfft; }
     __device__ __forceinline__ unsigned wait_limit() const { return a.wait_limit; }
     __device__ __forceinline__ int* status() const { return a.status; }
     __device__ __forceinline__ unsigned long long* phase_cycles() const { return a.phase_cycles; }
+};
+
+// Work of a batch: CTA b takes units [first[b], first[b + 1]) of windows of one nfft.
+struct BatchWin {
+    KArgs a;
+    int log2n;
+    int order;
+    int n_gx;   // gate groups
+    int n_cy;   // IPP chunks
+};
+struct BatchUnit {
+    int win, gx, cy, pad;
+};
+struct XtBatchSrc {
+    const BatchWin* wins;
+    const BatchUnit* units;
+    const int* starts;
+    unsigned limit;
+    int* stat;
+    __device__ __forceinline__ int first() const { return __ldg(starts + blockIdx.x); }
+    __device__ __forceinline__ int next(int un) const { return un + 1; }
+    __device__ __forceinline__ bool valid(int un) const { return un < __ldg(starts + blockIdx.x + 1); }
+    template <int LOG2N>
+    __device__ __forceinline__ void fill(XtUnit& x, int un, int g, int t) const
+    {
+        const BatchUnit u = units[un];
+        xt_fill<LOG2N>(x, wins[u.win].a, u.gx, u.cy, g, t);
+    }
+    __device__ __forceinline__ unsigned wait_limit() const { return limit; }
+    __device__ __forceinline__ int* status() const { return stat; }
+    __device__ __forceinline__ unsigned long long* phase_cycles() const { return nullptr; }
 };
 
 // ---------------------------------------------------------------- the kernel
@@ -314,17 +345,12 @@ __global__ void __launch_bounds__(kThreads, 1) integrate_kernel_xt(const __grid_
         if (x.ok && i != x.drop) bulk_load(smem_u32(stage), x.src + i * x.stride, x.bytes, bar);
     };
 
-    if (work.short_codes(N)) {
-        // the windows of codes shorter than nfft never fill the stage: what they leave stays zero
-        for (int i = tid; i < S::STAGE_WORDS * G; i += kThreads)
-            reinterpret_cast<uint32_t*>(smem + S::OFF_STAGE)[i] = 0u;
-        fence_proxy_async();
-        __syncthreads();
-    }
     auto begin = [&](XtUnit& x, int un, uint32_t it0) {   // thread 0 of the gate: unit un, its first window
         work.template fill<LOG2N>(x, un, g, t);
         x.un = un;
         x.it0 = it0;
+        // words behind a short code are cleared once, and again after a unit with a longer one
+        x.wipe = x.code_len < N && (it0 == 0 || units[&x == units].code_len > x.code_len);
         issue(x, 0);
     };
     const bool any = work.valid(work.first());
@@ -445,13 +471,20 @@ __global__ void __launch_bounds__(kThreads, 1) integrate_kernel_xt(const __grid_
 #endif
             float2 v[32];
             {
-                // ---- pass 0: decode, 32-point DFT.  A copy of a window shorter than nfft is rounded up
-                // to 16 bytes: its thread clears what that left behind the last chip (at most 6 words)
+                // ---- pass 0: decode, 32-point DFT.  The samples behind a code shorter than nfft read as
+                // zeros: a unit's first IPP clears them all if need be, and as copies are rounded to 16
+                // bytes, every IPP what that left behind the last chip (at most 6 words).  A thread
+                // clears the words that it alone reads.
                 uint32_t* win = stage + x->off + t;
                 const int L = x->code_len;
                 if (L != N) {
                     const int d = (t - L) & (T - 1);
-                    if (d < 6 && L + d < N) {
+                    if (x->wipe && it == x->it0) {
+                        for (int pos = L + d; pos < N; pos += T) win[pos - t] = 0u;
+                        // the words that a unit with a larger offset reads beyond these
+                        if (t < 4 && N + t >= x->off + L) stage[N + t] = 0u;
+                        fence_proxy_async();
+                    } else if (d < 6 && L + d < N) {
                         win[L + d - t] = 0u;
                         fence_proxy_async();
                     }

@@ -83,3 +83,41 @@ def test_reused_per_window_plans_match_fresh_plans(bufs, reference):
                 assert_parity(o.cpu().numpy().astype(np.float64), r, rtol=RTOL, what=f"reused plan, window {i}")
     finally:
         pw.close()
+
+
+def test_mixed_code_lengths_and_gate_counts_in_one_launch():
+    """Windows of one transform length with short and full codes in turn (a CTA takes units of several,
+    and what a longer window left in its stage must not enter a shorter one), more CTAs than units for
+    some lengths, several chunks (a reduction) for others, and per-IPP codes."""
+    rng = np.random.default_rng(17)
+    dev = torch.device("cuda:0")
+    shapes = [(2048, 2048, 200, 3, 0), (2048, 1025, 700, 2, 0), (2048, 2041, 900, 2, 1), (2048, 2048, 1500, 2, 0),
+              (4096, 4095, 3, 5, 0), (4096, 2049, 650, 2, 0), (4096, 4096, 700, 2, 1), (8192, 8190, 2, 600, 0),
+              (16384, 9000, 160, 2, 0), (16384, 16384, 170, 2, 0), (16384, 16383, 180, 2, 0), (16384, 8193, 200, 2, 1)]
+    keep, ws = [], []
+    for nfft, L, R, P, per in shapes:
+        stride = (2 + (R - 1) * 3 + L + 3) // 4 * 4
+        echo = np.clip(np.rint(rng.standard_normal((P, stride, 2)) * 1000), -32768, 32767).astype(np.int16)
+        code = np.where(rng.random((P, L) if per else (L,)) < 0.5, -1, 1).astype(np.int8)
+        e, c = torch.from_numpy(echo).to(dev), torch.from_numpy(code).to(dev)
+        o = torch.empty((R, nfft), device=dev)
+        keep.append((echo, code, e, c, o))
+        x = isr.IsrWindow()
+        x.echo, x.tx_code, x.out = e.data_ptr(), c.data_ptr(), o.data_ptr()
+        x.echo_stride, x.tx_stride, x.nfft, x.code_len = stride, L if per else 0, nfft, L
+        x.n_ranges, x.range_start, x.range_step, x.n_ipp, x.order, x.reserved = R, 2, 3, P, -1, 0
+        ws.append(x)
+    torch.cuda.synchronize()
+    h = isr.isr_batch_create(ws, 0, 0, torch.cuda.current_stream())
+    for _ in range(2):
+        isr.isr_batch_run(h)
+        isr.isr_batch_wait(h)
+    for (nfft, L, R, P, per), (echo, code, _, _, o) in zip(shapes, keep):
+        sel = sorted({0, 1, R // 2, R - 1})
+        ref = oracle.integrate(echo, code, nfft=nfft, n_ranges=R, range_start=2, range_step=3, code_len=L,
+                               per_ipp_tx=bool(per), sel=sel)
+        got = o.cpu().numpy().astype(np.float64)[sel]
+        # few IPPs: a bin far below the mean shares the mean's rounding
+        tol = RTOL * np.maximum(ref, 0.01 * ref.mean(axis=1, keepdims=True))
+        assert (np.abs(got - ref) <= tol).all(), (nfft, L, R, P, per)
+    isr.isr_batch_destroy(h)
