@@ -1765,11 +1765,12 @@ __global__ void __launch_bounds__(HM_THREADS) head_mlp_kernel(const HeadArgs a)
     }
 }
 
-// ---------------------------------------------------------------- fused inference
-// The whole network up to the head's chunk statistics in one kernel (BF16 storage, tcgen05): a tile's
-// activations never leave the SM.  Launched per batch: conv1, three convolutions and the head took
-// 16 + 3 x 33 + 14 us for 128 rows x 4608 positions, bound by staging channel-major rows into the
-// operand layout and writing them back; here the epilogue of a layer writes the next layer's operand.
+// ---------------------------------------------------------------- fused forward pass (BF16, tcgen05)
+// The whole network up to the head's chunk statistics in one kernel: a tile's activations never leave the
+// SM (in training they are written out for the backward pass, but not read again).  Launched per layer,
+// conv1, three convolutions and the head took 16 + 3 x 33 + 14 us for 128 rows x 4608 positions, bound by
+// staging channel-major rows into the operand layout; here the epilogue of a layer writes the next
+// layer's operand.
 //
 // A tile is FI_W = 512 positions of one row, of which FI_P = 488 come out of the fourth layer (four
 // 9-tap layers use up 8 positions each, the first computes 512 of the 520 the second could read).  It
@@ -1779,50 +1780,36 @@ __global__ void __launch_bounds__(HM_THREADS) head_mlp_kernel(const HeadArgs a)
 // four M = 128, N = 32 tiles are 72 of 46: a quarter of the products are with zeros, but an N = 32 MMA is
 // bound by reading its A operand.  The operand B of tap t is the 128 rows starting at tap t of the
 // weights laid out [8-channel group][3 zero taps, 9 taps][32 co][8 ci] (the next group's zeros follow), so
-// the Toeplitz matrix costs little more room than the weights.  Positions of equal index mod 4 form the planes of A
-// ([8-channel group][index mod 4][index / 4][8 ci]), so tap t is plane t mod 4 started t / 4 rows later.
-// Each output accumulates the same products in the same order as in conv_tc05_kernel (the added ones
-// are zeros), so the activations are equal bit by bit; a zero times an infinity would not be, so a tile
-// that holds one issues the products of each p' alone, without the zero taps.
+// the Toeplitz matrix costs little more room than the weights.  Positions of equal index mod 4 form the
+// planes of A ([8-channel group][index mod 4][index / 4][8 ci]), so tap t is plane t mod 4 started t / 4
+// rows later.  Each output accumulates the same products in the same order as one 9-tap convolution
+// (the added ones are zeros); a zero times an infinity would not be one, so a tile that holds an infinity
+// or a NaN issues the products of each p' alone, without the zero taps.
 //
-// A CTA (one per SM) holds the three layers' weights and FI_SLOTS tiles, each worked on by eight warps
-// with 128 TMEM columns of its own: while one tile's MMAs run, the others are in their first layer or
+// A CTA (one per SM) holds the three layers' weights and SLOTS tiles, each worked on by eight warps with
+// 128 TMEM columns of its own: while one tile's MMAs run, the others are in their first layer or
 // epilogues.  The activations are overwritten in place once a layer's MMAs have completed.
-// Measured, 128 rows x 4608 positions: 58 us a call with the head's 9, where the separate kernels took
-// 139; two tiles per CTA 68 us, a turn for issuing one tile's MMAs after the other's 60 us, the row's head
-// in its last tile's warps (one atomic per tile) 70 us.  The tensor pipe is active on about 45 % of cycles:
-// the tiles run through their phases nearly together, three rounds of them per call.
+// Measured, 128 rows x 4608 positions: inference 59 us with the head's 9 (separate kernels 139), training
+// 76 us (separate 136).  Two tiles in inference 68 us, a turn for issuing one tile's MMAs after the
+// other's 60 us, the row's head in its last tile's warps (one atomic per tile) 70 us.  The tensor pipe is
+// active on about 45 % of cycles: the tiles run through their phases nearly together.  Thread
+// (warp w, lane) of a tile: row r = 32 (w mod 4) + lane, its four positions, channels 16 (w / 4) .. + 15.
 constexpr int FI_W = 512, FI_P = FI_W - 24;      // positions of a tile, positions it finishes
-constexpr int FI_SLOTS = 3, FI_ST = 256;         // tiles in flight per CTA, threads per tile
-constexpr int FI_COLS = FI_SLOTS > 2 ? 512 : 256; // TMEM columns (a power of two)
+constexpr int FI_ST = 256;                       // threads per tile
 constexpr int FI_ROWS = FI_W / 4 + 2;            // rows of a plane (taps reach two rows beyond)
 constexpr int FI_PLANE = FI_ROWS * 16;           // bytes; 8 banks past a multiple of 32, so planes interleave
-constexpr int FI_BUF = 16 * FI_PLANE;
+constexpr int FI_BUF = 16 * FI_PLANE;            // one part (32 channels) of a tile
 constexpr int FI_WCG = (KT + 3) * CH * 16;       // bytes between 8-channel groups: 3 zero taps and 9 taps
 constexpr int FI_WLAYER = 4 * FI_WCG;
 constexpr int FI_WBYTES = 3 * FI_WLAYER + 3 * CH * 16;   // the last group's taps are followed by zeros too
-constexpr int FI_XW = FI_W + KT - 1;
-static_assert((FI_PLANE / 4) % 32 == 8 && FI_PLANE % 16 == 0, "plane pitch");
-struct FiSlot {
-    uint64_t mbar;
-    float zm[8];
-    int zi[8];
-    float mx[8][CH], sum[8][CH];
-    alignas(16) float x[FI_XW];
-};
-struct FiShared {
-    float w1[CH][12];    // W1[co][0..8], b1[co]
-    float bias[3][CH];
-    float w5[CH];
-    uint32_t tslot;
-    FiSlot slot[FI_SLOTS];
-};
 constexpr int FI_OFF_BUF = (FI_WBYTES + 127) / 128 * 128;
-constexpr int FI_OFF_SH = FI_OFF_BUF + FI_SLOTS * FI_BUF;
-constexpr int FI_SMEM = FI_OFF_SH + (int)sizeof(FiShared);
-static_assert(FI_SMEM <= 232448 && FI_OFF_BUF % 128 == 0 && FI_OFF_SH % 16 == 0, "shared memory");
+constexpr int FI_XW = FI_W + KT - 1;
+constexpr int HC = CH / 2;                       // channels of a thread
+static_assert((FI_PLANE / 4) % 32 == 8 && FI_PLANE % 16 == 0, "plane pitch");
 
-// relu of two values as stored: rounded to BF16, then max with 0 (NaN becomes 0, as fmaxf gives)
+__host__ __device__ constexpr int fi_cols(int slots) { return slots > 2 ? 512 : 128 * slots; }   // a power of two
+
+// two values as stored (BF16), and relu of them: max with 0 after rounding (NaN becomes 0, as fmaxf gives)
 __device__ __forceinline__ uint32_t fi_relu2(float a, float b)
 {
     const __nv_bfloat162 h = __hmax2(__floats2bfloat162_rn(a, b), __floats2bfloat162_rn(0.f, 0.f));
@@ -1833,129 +1820,235 @@ __device__ __forceinline__ uint32_t fi_max2(uint32_t a, uint32_t b)
     const __nv_bfloat162 h = __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
     return *reinterpret_cast<const uint32_t*>(&h);
 }
-// whether either half of a word of non-negative BF16 values is an infinity
-__device__ __forceinline__ bool fi_inf2(uint32_t m) { return (m & 0x7fffu) == 0x7f80u || (m >> 16 & 0x7fffu) == 0x7f80u; }
+// whether a word that is the maximum of magnitude bit patterns has an infinity or NaN in either half
+__device__ __forceinline__ bool fi_inf2(uint32_t m) { return (m & 0x7fffu) >= 0x7f80u || (m >> 16 & 0x7fffu) >= 0x7f80u; }
 __device__ __forceinline__ float fi_half(uint32_t w, int half) { return __uint_as_float(half ? (w & 0xffff0000u) : (w << 16)); }
 
-// sum of v[c] over the warp's lanes for 32 channels c: lane c receives channel c's (31 exchanges)
-__device__ __forceinline__ float fi_scatter_sum(float (&v)[CH], int lane)
+// v[c] (16 channels) combined over the warp's lanes: lanes 2 c, 2 c + 1 receive channel c's
+template <class T, class OP>
+__device__ __forceinline__ T fi_scatter(T (&v)[HC], int lane, OP op)
 {
 #pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int k = 0; k < o; ++k) {
-            const float keep = up ? v[k + o] : v[k], give = up ? v[k] : v[k + o];
-            v[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-        }
-    }
-    return v[0];
-}
-// the same for the maximum of BF16 pairs: m[k] = channels 2 k, 2 k + 1
-__device__ __forceinline__ float fi_scatter_max(uint32_t (&m)[CH / 2], int lane)
-{
-#pragma unroll
-    for (int o = 8; o; o >>= 1) {
+    for (int o = HC / 2; o; o >>= 1) {
         const bool up = (lane & (2 * o)) != 0;
 #pragma unroll
         for (int k = 0; k < o; ++k) {
-            const uint32_t keep = up ? m[k + o] : m[k], give = up ? m[k] : m[k + o];
-            m[k] = fi_max2(keep, __shfl_xor_sync(0xffffffffu, give, 2 * o));
+            const T keep = up ? v[k + o] : v[k], give = up ? v[k] : v[k + o];
+            v[k] = op(keep, __shfl_xor_sync(0xffffffffu, give, 2 * o));
         }
     }
-    m[0] = fi_max2(m[0], __shfl_xor_sync(0xffffffffu, m[0], 1));
-    return fi_half(m[0], lane & 1);
+    return op(v[0], __shfl_xor_sync(0xffffffffu, v[0], 1));
 }
 
-__global__ void __launch_bounds__(FI_SLOTS * FI_ST, 1) infer_kernel(const float* __restrict__ x, const __nv_bfloat16* __restrict__ w1,
-                                                                    const __nv_bfloat16* __restrict__ wt,
-                                                                    int n_rows, float* __restrict__ z, float* __restrict__ pmax,
-                                                                    float* __restrict__ psum, float* __restrict__ zmax,
-                                                                    int* __restrict__ zidx, const float* __restrict__ theta,
-                                                                    int L, int nx)
+// the barrier of a slot's 256 threads, with a vote
+__device__ __forceinline__ bool fi_slot_or(int slot, bool pred)
 {
-    extern __shared__ __align__(128) unsigned char fi_smem[];
-    FiShared& sh = *reinterpret_cast<FiShared*>(fi_smem + FI_OFF_SH);
+    uint32_t any;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "bar.red.or.pred q, %2, %3, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(any)
+        : "r"((uint32_t)pred), "r"(1 + slot), "n"(FI_ST)
+        : "memory");
+    return any != 0;
+}
+
+// weights of three layers, rows [co][tap][ci], to [layer][ci / 8][3 zero taps, 9 taps][co][8 ci]
+template <int NT>
+__device__ __forceinline__ void fi_stage_weights(unsigned char* dst, const __nv_bfloat16* __restrict__ wt, int tid)
+{
+    constexpr int PER = (FI_WBYTES / 16 + NT - 1) / NT;
+    uint4 v[PER];   // all loads first
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int e = tid + i * NT, co = e % CH, tp = e / CH % (KT + 3), gr = e / (CH * (KT + 3)), l = gr / 4, cg = gr % 4;
+        v[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (tp >= 3 && e < FI_WBYTES / 16)
+            v[i] = __ldg(reinterpret_cast<const uint4*>(wt + ((size_t)(l * CH + co) * KT + (tp - 3)) * CH + cg * 8));
+    }
+#pragma unroll
+    for (int i = 0; i < PER; ++i)
+        if (tid + i * NT < FI_WBYTES / 16) *reinterpret_cast<uint4*>(dst + (tid + i * NT) * 16) = v[i];
+}
+
+// one thread: the MMAs of a layer on a tile of PARTS operand parts (hi and lo of a split operand), into the
+// 128 TMEM columns at d, committed to mbar
+template <int PARTS>
+__device__ __forceinline__ void fi_issue(uint32_t d, uint32_t mbar, const unsigned char* buf, const unsigned char* w, bool inf)
+{
+    constexpr uint32_t idesc32 = isr::tc05_idesc<true>();                                  // M 128, N 32
+    constexpr uint32_t idesc = (idesc32 & ~(0x3fu << 17)) | ((128u >> 3) << 17);           // N 128
+    const uint64_t ad = isr::tc05_desc(isr::smem_u32(buf), 4 * FI_PLANE, 128);
+    const uint64_t bd = isr::tc05_desc(isr::smem_u32(w), FI_WCG, 128);
+    // descriptors step in 16-byte units of the start field (addresses stay below 0x40000)
+    auto a_at = [&](int part, int t, int ks) {
+        return ad + (uint32_t)((part * FI_BUF + (2 * ks * 4 + (t & 3)) * FI_PLANE + (t >> 2) * 16) >> 4);
+    };
+    auto b_at = [&](int tap, int ks) { return bd + (uint32_t)((2 * ks * FI_WCG + tap * CH * 16) >> 4); };
+    if (!inf) {
+#pragma unroll 1
+        for (int part = 0; part < PARTS; ++part)
+#pragma unroll
+            for (int t = 0; t < KT + 3; ++t)
+#pragma unroll
+                for (int ks = 0; ks < 2; ++ks)
+                    isr::tc05_mma(d, a_at(part, t, ks), b_at(t, ks), idesc, (part | t | ks) != 0);
+    } else {
+#pragma unroll 1
+        for (int p = 0; p < 4; ++p)
+#pragma unroll 1
+            for (int part = 0; part < PARTS; ++part)
+#pragma unroll 1
+                for (int tap = 0; tap < KT; ++tap)
+#pragma unroll 1
+                    for (int ks = 0; ks < 2; ++ks)
+                        isr::tc05_mma(d + 32u * (3 - p), a_at(part, tap + p, ks), b_at(tap + 3, ks), idesc32, (part | tap | ks) != 0);
+    }
+    isr::tc05_commit(mbar);
+}
+
+// Eight channels (group g of this thread's two) of its four positions: registers stay few that way.
+constexpr int GC = CH / 4;
+using FiQuad = uint32_t[4][GC / 2];   // [position][channel pair], as stored
+
+__device__ __forceinline__ void fi_read(uint32_t tacc, int half, int g, float (&v)[4][GC])
+{
+    const uint32_t t = isr::tmem_warp_lane_base(tacc) + (uint32_t)(HC * half + GC * g);
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=f"(v[p][0]), "=f"(v[p][1]), "=f"(v[p][2]), "=f"(v[p][3]), "=f"(v[p][4]), "=f"(v[p][5]),
+                       "=f"(v[p][6]), "=f"(v[p][7])
+                     : "r"(t + 32u * (3 - p)));
+#pragma unroll
+    for (int p = 0; p < 4; ++p)   // the registers pass through the wait, so that no use moves ahead of it
+        asm volatile("tcgen05.wait::ld.sync.aligned;"
+                     : "+f"(v[p][0]), "+f"(v[p][1]), "+f"(v[p][2]), "+f"(v[p][3]), "+f"(v[p][4]), "+f"(v[p][5]),
+                       "+f"(v[p][6]), "+f"(v[p][7]));
+}
+
+// to the planes of row r
+__device__ __forceinline__ void fi_to_planes(unsigned char* buf, int r, int half, int g, const FiQuad& q)
+{
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+        *reinterpret_cast<uint4*>(buf + ((2 * half + g) * 4 + p) * FI_PLANE + r * 16) = make_uint4(q[p][0], q[p][1], q[p][2], q[p][3]);
+}
+
+// Training forward: the stored activations of four positions pos .. (a multiple of 4, the first `count`
+// exist) of row b
+__device__ __forceinline__ void fi_to_rows(__nv_bfloat16* __restrict__ h, int b, int L, int pos, int count, int half, int g,
+                                           const FiQuad& q)
+{
+    unsigned short* o = reinterpret_cast<unsigned short*>(h) + ((size_t)b * CH + HC * half + GC * g) * L + pos;
+    if ((L & 3) == 0) {   // whole groups of four, 8-byte aligned
+#pragma unroll
+        for (int c = 0; c < GC; ++c) {
+            const uint32_t sel = c & 1 ? 0x7632u : 0x5410u;
+            *reinterpret_cast<uint2*>(o + (size_t)c * L) =
+                make_uint2(__byte_perm(q[0][c / 2], q[1][c / 2], sel), __byte_perm(q[2][c / 2], q[3][c / 2], sel));
+        }
+    } else {
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+            if (p < count)
+#pragma unroll
+                for (int c = 0; c < GC; ++c) o[(size_t)c * L + p] = (unsigned short)(q[p][c / 2] >> (16 * (c & 1)));
+    }
+}
+// and their ReLU masks (bit co of word (b, i): h[b][co][i] > 0): eight channels of each position into m,
+// then this thread's sixteen to memory
+__device__ __forceinline__ void fi_mask(uint32_t (&m)[4], int g, const FiQuad& q)
+{
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int k = 0; k < GC / 2; ++k) {
+            const uint32_t t = __vsetgts2(q[p][k], 0u);   // 1 per half above zero
+            m[p] |= ((t | t >> 15) & 3u) << (GC * g + 2 * k);
+        }
+}
+__device__ __forceinline__ void fi_mask_to_rows(uint32_t* __restrict__ bits, int b, int L, int pos, int count, int half,
+                                                const uint32_t (&m)[4])
+{
+    unsigned short* o = reinterpret_cast<unsigned short*>(bits + (size_t)b * L + pos) + half;
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+        if (p < count) o[2 * p] = (unsigned short)m[p];
+}
+
+struct FiFwdSlot {
+    uint64_t mbar;
+    float zm[4];
+    int zi[4];
+    float mx[4][CH], sum[4][CH];
+    int mi[4][CH];
+    alignas(16) float z[FI_W];       // logits of the lower channels
+    alignas(16) float x[FI_XW];
+};
+template <int SLOTS>
+struct FiFwdShared {
+    float w1[CH][12];    // W1[co][0..8], b1[co]
+    float bias[3][CH];
+    float w5[CH];
+    uint32_t tslot;
+    FiFwdSlot slot[SLOTS];
+};
+// tiles in flight per CTA: 80 registers a thread for three in inference; the stores of training need more
+template <bool TRAIN> __host__ __device__ constexpr int fi_slots() { return TRAIN ? 2 : 3; }
+template <bool TRAIN> __host__ __device__ constexpr int fi_smem()
+{
+    return FI_OFF_BUF + fi_slots<TRAIN>() * FI_BUF + (int)sizeof(FiFwdShared<fi_slots<TRAIN>()>);
+}
+static_assert(fi_smem<false>() <= 232448 && fi_smem<true>() <= 232448, "shared memory");
+struct FiFwdArgs {
+    const float* x;
+    const __nv_bfloat16 *w1, *wt;
+    const float* theta;
+    int L, n_rows, nx;
+    float *z, *pmax, *psum, *zmax;
+    int *pidx, *zidx;
+    __nv_bfloat16* h[4];       // training: h1 .. h4
+    uint32_t* bits[3];         // training: ReLU masks of h1 .. h3
+};
+
+template <bool TRAIN>
+__global__ void __launch_bounds__(fi_slots<TRAIN>() * FI_ST, 1) forward_kernel(const __grid_constant__ FiFwdArgs a)
+{
+    constexpr int SLOTS = fi_slots<TRAIN>(), NT = SLOTS * FI_ST;
+    extern __shared__ __align__(128) unsigned char fi_smem_raw[];
+    unsigned char* smem = fi_smem_raw;
+    auto& sh = *reinterpret_cast<FiFwdShared<SLOTS>*>(smem + FI_OFF_BUF + SLOTS * FI_BUF);
     const int tid = threadIdx.x, slot = tid / FI_ST, st = tid - slot * FI_ST;
     const int lane = tid & 31, w = __shfl_sync(0xffffffffu, st >> 5, 0);   // warp of the slot
-    FiSlot& sl = sh.slot[slot];
-    unsigned char* buf = fi_smem + FI_OFF_BUF + slot * FI_BUF;
+    const int half = w >> 2, r = 32 * (w & 3) + lane;
+    FiFwdSlot& sl = sh.slot[slot];
+    unsigned char* buf = smem + FI_OFF_BUF + slot * FI_BUF;
     const uint32_t mbar = isr::smem_u32(&sl.mbar);
+    const int L = a.L, nx = a.nx;
 
     if (st == 0) isr::mbar_init(mbar, 1);
     isr::fence_barrier_init();
-    if (tid < 32) isr::tmem_alloc(isr::smem_u32(&sh.tslot), FI_COLS);
-    // weights of layers 2-4: rows [co][tap][ci] to [ci / 8][tap + 3][co][8 ci], zeros around the taps
-    {
-        constexpr int NT = FI_SLOTS * FI_ST, PER = (FI_WBYTES / 16 + NT - 1) / NT;
-        uint4 v[PER];   // all loads first
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const int e = tid + i * NT, co = e % CH, tp = e / CH % (KT + 3), gr = e / (CH * (KT + 3)), l = gr / 4, cg = gr % 4;
-            v[i] = make_uint4(0u, 0u, 0u, 0u);
-            if (tp >= 3 && e < FI_WBYTES / 16)
-                v[i] = __ldg(reinterpret_cast<const uint4*>(wt + ((size_t)(l * CH + co) * KT + (tp - 3)) * CH + cg * 8));
-        }
-#pragma unroll
-        for (int i = 0; i < PER; ++i)
-            if (tid + i * NT < FI_WBYTES / 16) *reinterpret_cast<uint4*>(fi_smem + (tid + i * NT) * 16) = v[i];
-    }
-    for (int e = tid; e < CH * 12; e += FI_SLOTS * FI_ST) {
+    if (tid < 32) isr::tmem_alloc(isr::smem_u32(&sh.tslot), fi_cols(SLOTS));
+    fi_stage_weights<NT>(smem, a.wt, tid);
+    for (int e = tid; e < CH * 12; e += NT) {
         const int co = e / 12, k = e - co * 12;
-        sh.w1[co][k] = k < KT ? ld<__nv_bfloat16>(w1, (size_t)k * CH + co) : (k == KT ? theta[OFF_B1 + co] : 0.f);
+        sh.w1[co][k] = k < KT ? ld<__nv_bfloat16>(a.w1, (size_t)k * CH + co) : (k == KT ? a.theta[OFF_B1 + co] : 0.f);
     }
-    for (int e = tid; e < 3 * CH; e += FI_SLOTS * FI_ST) sh.bias[e / CH][e % CH] = theta[b_off(2 + e / CH) + e % CH];
-    if (tid < CH) sh.w5[tid] = theta[OFF_W5 + tid];
-    for (int e = tid; e < FI_SLOTS * FI_BUF / 16; e += FI_SLOTS * FI_ST)   // the last two rows are read, never written
-        *reinterpret_cast<uint4*>(fi_smem + FI_OFF_BUF + e * 16) = make_uint4(0u, 0u, 0u, 0u);
+    for (int e = tid; e < 3 * CH; e += NT) sh.bias[e / CH][e % CH] = a.theta[b_off(2 + e / CH) + e % CH];
+    if (tid < CH) sh.w5[tid] = a.theta[OFF_W5 + tid];
+    for (int e = tid; e < SLOTS * FI_BUF / 16; e += NT)   // the last two rows are read, never written
+        *reinterpret_cast<uint4*>(smem + FI_OFF_BUF + e * 16) = make_uint4(0u, 0u, 0u, 0u);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     isr::tmem_fence_before_sync();
     __syncthreads();
     isr::tmem_fence_after_sync();
     const uint32_t tacc = sh.tslot + 128u * slot;   // this tile's accumulator
-    const float b5 = theta[OFF_B5];
+    const float b5 = a.theta[OFF_B5];
 
-    auto slot_or = [&](bool pred) -> bool {
-        uint32_t any;
-        asm volatile(
-            "{\n\t.reg .pred p, q;\n\t"
-            "setp.ne.u32 p, %1, 0;\n\t"
-            "bar.red.or.pred q, %2, %3, p;\n\t"
-            "selp.u32 %0, 1, 0, q;\n\t}"
-            : "=r"(any)
-            : "r"((uint32_t)pred), "r"(1 + slot), "n"(FI_ST)
-            : "memory");
-        return any != 0;
-    };
-    // one thread: the MMAs of layer l (0 .. 2) on this slot's buffer
-    auto issue = [&](int l, bool inf) {
-        constexpr uint32_t idesc32 = isr::tc05_idesc<true>();
-        constexpr uint32_t idesc = (idesc32 & ~(0x3fu << 17)) | ((128u >> 3) << 17);   // N = 128
-        const uint64_t ad = isr::tc05_desc(isr::smem_u32(buf), 4 * FI_PLANE, 128);
-        const uint64_t bd = isr::tc05_desc(isr::smem_u32(fi_smem) + l * FI_WLAYER, FI_WCG, 128);
-        if (!inf) {
-#pragma unroll
-            for (int t = 0; t < KT + 3; ++t)
-#pragma unroll
-                for (int ks = 0; ks < 2; ++ks)
-                    isr::tc05_mma(tacc, ad + (uint32_t)(((2 * ks * 4 + (t & 3)) * FI_PLANE + (t >> 2) * 16) >> 4),
-                                  bd + (uint32_t)((2 * ks * FI_WCG + t * CH * 16) >> 4), idesc, (t | ks) != 0);
-        } else {
-#pragma unroll 1
-            for (int p = 0; p < 4; ++p)
-#pragma unroll 1
-                for (int tap = 0; tap < KT; ++tap)
-#pragma unroll 1
-                    for (int ks = 0; ks < 2; ++ks) {
-                        const int t = tap + p;
-                        isr::tc05_mma(tacc + 32u * (3 - p), ad + (uint32_t)(((2 * ks * 4 + (t & 3)) * FI_PLANE + (t >> 2) * 16) >> 4),
-                                      bd + (uint32_t)((2 * ks * FI_WCG + (tap + 3) * CH * 16) >> 4), idesc32, (tap | ks) != 0);
-                    }
-        }
-        isr::tc05_commit(mbar);
-    };
-
-    const int n_tiles = n_rows * nx, step = gridDim.x * FI_SLOTS;
+    const int n_tiles = a.n_rows * nx, step = gridDim.x * SLOTS;
     // x of a tile: positions i0 - 16 .. , rounded to BF16 as the network reads it
     constexpr int XPER = (FI_XW + FI_ST - 1) / FI_ST;
     float xr[XPER];
@@ -1964,157 +2057,238 @@ __global__ void __launch_bounds__(FI_SLOTS * FI_ST, 1) infer_kernel(const float*
 #pragma unroll
         for (int k = 0; k < XPER; ++k) {
             const int j = st + k * FI_ST, pos = i0 - 16 + j;
-            xr[k] = (j < FI_XW && pos >= 0 && pos < L) ? __ldg(x + (size_t)b * L + pos) : 0.f;
+            xr[k] = (j < FI_XW && pos >= 0 && pos < L) ? __ldg(a.x + (size_t)b * L + pos) : 0.f;
         }
     };
     uint32_t phase = 0;
     int tile = slot * gridDim.x + blockIdx.x;   // what is left after full rounds goes to different SMs
     if (tile < n_tiles) load_x(tile);
     for (; tile < n_tiles; tile += step) {
-        const int b = tile / nx, xc = tile - b * nx, i0 = xc * FI_P;
+        const int b = tile / nx, xc = tile - b * nx, i0 = xc * FI_P, end = min(i0 + FI_P, L);
 #pragma unroll
         for (int k = 0; k < XPER; ++k) {
             const int j = st + k * FI_ST;
             if (j < FI_XW) sl.x[j] = __bfloat162float(__float2bfloat16_rn(xr[k]));
         }
-        slot_or(false);
+        fi_slot_or(slot, false);
         if (tile + step < n_tiles) load_x(tile + step);
-        // ---- layer 1: positions i0 - 12 + 4 r .. + 3 of row r = st % 128, half of the channels
+        // a tile writes out the positions it owns, i0 .. end - 1, of every layer (whole groups of four but
+        // at the end of a row)
+        auto owned = [&](int pos) { return pos >= i0 && pos < end ? min(4, end - pos) : 0; };
+        // zero outside the row
+        auto inside = [&](int pos) { return pos >= 0 && pos < L ? ~0u : 0u; };
+        // ---- layer 1: positions i0 - 12 + 4 r .. + 3
         bool inf = false;
         {
-            const int r = st & (FI_W / 4 - 1), half = st / (FI_W / 4);
             float xv[KT + 3];
 #pragma unroll
             for (int k = 0; k < KT + 3; k += 4) {
                 const float4 v = *reinterpret_cast<const float4*>(&sl.x[4 * r + k]);
                 xv[k] = v.x, xv[k + 1] = v.y, xv[k + 2] = v.z, xv[k + 3] = v.w;
             }
-            uint32_t in[4], top = 0u;
-#pragma unroll
-            for (int p = 0; p < 4; ++p) {
-                const int pos = i0 - 12 + 4 * r + p;
-                in[p] = pos >= 0 && pos < L ? ~0u : 0u;
-            }
+            const int pos = i0 - 12 + 4 * r;
+            uint32_t top = 0u, mask[4] = {0u, 0u, 0u, 0u};
 #pragma unroll 1
-            for (int cg = 2 * half; cg < 2 * half + 2; ++cg) {
-                uint32_t q[4][4];   // [position][channel pair]
+            for (int g = 0; g < 2; ++g) {
+                FiQuad q;
 #pragma unroll
-                for (int c2 = 0; c2 < 4; ++c2) {
-                    float a[2][4];
+                for (int c2 = 0; c2 < GC / 2; ++c2) {
+                    float s[2][4];
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
-                        const float* wr = sh.w1[8 * cg + 2 * c2 + c];
+                        const float* wr = sh.w1[HC * half + GC * g + 2 * c2 + c];
                         const float4 wa = *reinterpret_cast<const float4*>(wr), wb = *reinterpret_cast<const float4*>(wr + 4);
                         const float2 wc = *reinterpret_cast<const float2*>(wr + 8);
                         const float wk[KT] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w, wc.x};
 #pragma unroll
-                        for (int p = 0; p < 4; ++p) a[c][p] = wc.y;
+                        for (int p = 0; p < 4; ++p) s[c][p] = wc.y;
 #pragma unroll
                         for (int k = 0; k < KT; ++k)
 #pragma unroll
-                            for (int p = 0; p < 4; ++p) a[c][p] = fmaf(wk[k], xv[p + k], a[c][p]);
+                            for (int p = 0; p < 4; ++p) s[c][p] = fmaf(wk[k], xv[p + k], s[c][p]);
                     }
 #pragma unroll
                     for (int p = 0; p < 4; ++p) {
-                        q[p][c2] = fi_relu2(a[0][p], a[1][p]) & in[p];
+                        q[p][c2] = fi_relu2(s[0][p], s[1][p]) & inside(pos + p);
                         top = fi_max2(top, q[p][c2]);
                     }
                 }
-#pragma unroll
-                for (int p = 0; p < 4; ++p)
-                    *reinterpret_cast<uint4*>(buf + (cg * 4 + p) * FI_PLANE + r * 16) = make_uint4(q[p][0], q[p][1], q[p][2], q[p][3]);
+                fi_to_planes(buf, r, half, g, q);
+                if constexpr (TRAIN) {
+                    if (const int n = owned(pos)) fi_to_rows(a.h[0], b, L, pos, n, half, g, q);
+                    fi_mask(mask, g, q);
+                }
             }
+            if constexpr (TRAIN) fi_mask_to_rows(a.bits[0], b, L, pos, owned(pos), half, mask);
             inf = fi_inf2(top);
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        inf = slot_or(inf);
-        if (st == 0) issue(0, inf);
-        // ---- layers 2-4: row 32 (w % 4) + lane of the accumulator, positions 4 row + 3 - p' of the two
-        // p' = 2 (w / 4), 2 (w / 4) + 1
-        const int row = 32 * (w & 3) + lane, pp = 2 * (w >> 2);
-        // relu(accumulator + bias) of layer l for p' = pp + h, as stored: word k = channels 2 k, 2 k + 1
-        auto outputs = [&](int l, int h, uint32_t (&q)[CH / 2]) {
-            uint32_t r[32];
-            isr::tmem_ld32(isr::tmem_warp_lane_base(tacc) + 32u * (pp + h), r);
-            isr::tmem_wait_ld32(r);
+        inf = fi_slot_or(slot, inf);
+        if (st == 0) fi_issue<1>(tacc, mbar, buf, smem, inf);
+        // relu(accumulator + bias) of layer l + 2, as stored
+        auto outputs = [&](int l, int g, FiQuad& q) {
+            float v[4][GC];
+            fi_read(tacc, half, g, v);
 #pragma unroll
-            for (int c4 = 0; c4 < CH / 4; ++c4) {
-                const float4 bv = *reinterpret_cast<const float4*>(&sh.bias[l][4 * c4]);
-                q[2 * c4] = fi_relu2(__uint_as_float(r[4 * c4]) + bv.x, __uint_as_float(r[4 * c4 + 1]) + bv.y);
-                q[2 * c4 + 1] = fi_relu2(__uint_as_float(r[4 * c4 + 2]) + bv.z, __uint_as_float(r[4 * c4 + 3]) + bv.w);
+            for (int c4 = 0; c4 < GC / 4; ++c4) {
+                const float4 bv = *reinterpret_cast<const float4*>(&sh.bias[l][HC * half + GC * g + 4 * c4]);
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    q[p][2 * c4] = fi_relu2(v[p][4 * c4] + bv.x, v[p][4 * c4 + 1] + bv.y);
+                    q[p][2 * c4 + 1] = fi_relu2(v[p][4 * c4 + 2] + bv.z, v[p][4 * c4 + 3] + bv.w);
+                }
             }
         };
+        // ---- layers 2 and 3
 #pragma unroll 1
         for (int l = 0; l < 2; ++l) {
             const bool done = isr::mbar_wait(mbar, phase, 1u << 26);
             phase ^= 1u;
             isr::tmem_fence_after_sync();
+            const int pos = i0 - 8 + 4 * l + 4 * r;
+            FiQuad q[2];
             uint32_t top = 0u;
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                uint32_t q[CH / 2];
-                outputs(l, h, q);
-                const int p = 3 - pp - h, pos = i0 - 8 + 4 * l + 4 * row + p;
-                const uint32_t in = done && pos >= 0 && pos < L ? ~0u : 0u;
-                unsigned char* d = buf + p * FI_PLANE + row * 16;
+            for (int g = 0; g < 2; ++g) {
+                outputs(l, g, q[g]);
 #pragma unroll
-                for (int k = 0; k < CH / 2; ++k) {
-                    q[k] &= in;
-                    top = fi_max2(top, q[k]);
+                for (int p = 0; p < 4; ++p) {
+                    const uint32_t in = done ? inside(pos + p) : 0u;
+#pragma unroll
+                    for (int k = 0; k < GC / 2; ++k) {
+                        q[g][p][k] &= in;
+                        top = fi_max2(top, q[g][p][k]);
+                    }
                 }
-#pragma unroll
-                for (int cg = 0; cg < 4; ++cg)
-                    *reinterpret_cast<uint4*>(d + cg * 4 * FI_PLANE) = make_uint4(q[4 * cg], q[4 * cg + 1], q[4 * cg + 2], q[4 * cg + 3]);
+                fi_to_planes(buf, r, half, g, q[g]);
             }
-            inf = fi_inf2(top);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             isr::tmem_fence_before_sync();
-            inf = slot_or(inf);
+            inf = fi_slot_or(slot, fi_inf2(top));
             isr::tmem_fence_after_sync();
-            if (st == 0) issue(l + 1, inf);
+            if (st == 0) fi_issue<1>(tacc, mbar, buf, smem + (l + 1) * FI_WLAYER, inf);
+            if constexpr (TRAIN) {   // beside the next layer's MMAs
+                if (const int n = owned(pos)) {
+                    uint32_t mask[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+                    for (int g = 0; g < 2; ++g) {
+                        fi_to_rows(a.h[l + 1], b, L, pos, n, half, g, q[g]);
+                        fi_mask(mask, g, q[g]);
+                    }
+                    fi_mask_to_rows(a.bits[l + 1], b, L, pos, n, half, mask);
+                }
+            }
         }
-        // ---- layer 4 stays in registers: h4 as stored (BF16), its logit, and what the head keeps of it
-        float zm = -INFINITY;
-        int zi = 0x7fffffff;
-        uint32_t h4[2][CH / 2];
+        // ---- layer 4 stays in registers: the logits (lower channels first, the order of head_chunk_kernel)
+        // and the head's statistics
         const bool done = isr::mbar_wait(mbar, phase, 1u << 26);
         phase ^= 1u;
         isr::tmem_fence_after_sync();
+        const int pos = i0 + 4 * r, n_own = done ? owned(pos) : 0;
+        auto logits = [&](int g, const FiQuad& q, float (&s)[4]) {
 #pragma unroll
-        for (int h = 1; h >= 0; --h) {   // ascending positions
-            outputs(2, h, h4[h]);
-            const int pos = i0 + 4 * row + 3 - pp - h;
-            const bool ok = done && pos < i0 + FI_P && pos < L;
-            // in the order of head_chunk_kernel
-            float s = b5;
+            for (int c4 = 0; c4 < GC / 4; ++c4) {
+                const float4 w5 = *reinterpret_cast<const float4*>(&sh.w5[HC * half + GC * g + 4 * c4]);
 #pragma unroll
-            for (int c4 = 0; c4 < CH / 4; ++c4) {
-                const float4 w5 = *reinterpret_cast<const float4*>(&sh.w5[4 * c4]);
-                const uint32_t p0 = h4[h][2 * c4], p1 = h4[h][2 * c4 + 1];
-                float part = (L & 7) == 0 ? 0.f : s;
-                part = fmaf(w5.x, fi_half(p0, 0), part);
-                part = fmaf(w5.y, fi_half(p0, 1), part);
-                part = fmaf(w5.z, fi_half(p1, 0), part);
-                part = fmaf(w5.w, fi_half(p1, 1), part);
-                s = (L & 7) == 0 ? s + part : part;
-            }
-            if (ok) {
-                z[(size_t)b * L + pos] = s;
-                if (s > zm) {
-                    zm = s;
-                    zi = pos;
+                for (int p = 0; p < 4; ++p) {
+                    const uint32_t p0 = q[p][2 * c4], p1 = q[p][2 * c4 + 1];
+                    float part = (L & 7) == 0 ? 0.f : s[p];
+                    part = fmaf(w5.x, fi_half(p0, 0), part);
+                    part = fmaf(w5.y, fi_half(p0, 1), part);
+                    part = fmaf(w5.z, fi_half(p1, 0), part);
+                    part = fmaf(w5.w, fi_half(p1, 1), part);
+                    s[p] = (L & 7) == 0 ? s[p] + part : part;
                 }
             }
-            // other positions count as 0 in the head's sums and, as every activation is >= 0 and every
-            // tile has a position of its own, in its maxima
+        };
+        float t[HC];                                   // sums over this thread's positions
+        uint32_t key[TRAIN ? HC : HC / 2];             // their maxima (training: with the position)
+        FiQuad q[2];
+        float s[4] = {b5, b5, b5, b5};
 #pragma unroll
-            for (int k = 0; k < CH / 2; ++k) h4[h][k] = ok ? h4[h][k] : 0u;
+        for (int g = 0; g < 2; ++g) {
+            outputs(2, g, q[g]);
+            if constexpr (TRAIN) {
+                if (n_own) fi_to_rows(a.h[3], b, L, pos, n_own, half, g, q[g]);
+            }
+            if (half == 0) logits(g, q[g], s);
+            // other positions count as 0 in the sums and, as every activation is >= 0 and every tile has a
+            // position of its own, in the maxima
+            FiQuad o;
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+#pragma unroll
+                for (int k = 0; k < GC / 2; ++k) o[p][k] = p < n_own ? q[g][p][k] : 0u;
+#pragma unroll
+            for (int c = 0; c < GC; ++c)
+                t[GC * g + c] = (fi_half(o[0][c / 2], c & 1) + fi_half(o[1][c / 2], c & 1)) +
+                                (fi_half(o[2][c / 2], c & 1) + fi_half(o[3][c / 2], c & 1));
+            if constexpr (TRAIN) {
+                // largest value, first position: the value's bits above the position counted down; a
+                // position that is not owned has the key 0, below any other's
+#pragma unroll
+                for (int c = 0; c < GC; ++c) {
+                    key[GC * g + c] = 0u;
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) {
+                        const uint32_t bits = c & 1 ? o[p][c / 2] & 0xffff0000u : o[p][c / 2] << 16;
+                        key[GC * g + c] = max(key[GC * g + c], p < n_own ? bits | (uint32_t)(FI_W - 1 - 4 * r - p) : 0u);
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < GC / 2; ++k)   // channel pairs
+                    key[GC / 2 * g + k] = fi_max2(fi_max2(o[0][k], o[1][k]), fi_max2(o[2][k], o[3][k]));
+            }
         }
         isr::tmem_fence_before_sync();
-        // ---- chunk statistics of the head
+        if (half == 0) *reinterpret_cast<float4*>(&sl.z[4 * r]) = make_float4(s[0], s[1], s[2], s[3]);
         {
-            float m = zm;
-            int mi = zi;
+            const float cs = fi_scatter(t, lane, [](float u, float v) { return u + v; });
+            if ((lane & 1) == 0) sl.sum[w & 3][HC * half + (lane >> 1)] = cs;
+            if constexpr (TRAIN) {
+                const uint32_t ck = fi_scatter(key, lane, [](uint32_t u, uint32_t v) { return max(u, v); });
+                if ((lane & 1) == 0) {
+                    const int c = HC * half + (lane >> 1);
+                    sl.mx[w & 3][c] = __uint_as_float(ck & 0xffff0000u);
+                    sl.mi[w & 3][c] = i0 + FI_W - 1 - (int)(ck & 0xffffu);
+                }
+            } else {
+#pragma unroll
+                for (int o = HC / 4; o; o >>= 1) {
+                    const bool up = (lane & (4 * o)) != 0;
+#pragma unroll
+                    for (int k = 0; k < o; ++k) {
+                        const uint32_t keep = up ? key[k + o] : key[k], give = up ? key[k] : key[k + o];
+                        key[k] = fi_max2(keep, __shfl_xor_sync(0xffffffffu, give, 4 * o));
+                    }
+                }
+                key[0] = fi_max2(key[0], __shfl_xor_sync(0xffffffffu, key[0], 2));
+                key[0] = fi_max2(key[0], __shfl_xor_sync(0xffffffffu, key[0], 1));
+                if ((lane & 2) == 0) sl.mx[w & 3][HC * half + 2 * (lane >> 2) + (lane & 1)] = fi_half(key[0], lane & 1);
+            }
+        }
+        fi_slot_or(slot, false);
+        isr::tmem_fence_after_sync();
+        if (half == 1) {
+            const float4 s0 = *reinterpret_cast<const float4*>(&sl.z[4 * r]);
+            s[0] = s0.x, s[1] = s0.y, s[2] = s0.z, s[3] = s0.w;
+            logits(0, q[0], s);
+            logits(1, q[1], s);
+            float m = -INFINITY;
+            int mi = 0x7fffffff;
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+                if (p < n_own && s[p] > m) {
+                    m = s[p];
+                    mi = pos + p;
+                }
+            float* zo = a.z + (size_t)b * L + pos;
+            if ((L & 3) == 0) {
+                if (n_own) *reinterpret_cast<float4*>(zo) = make_float4(s[0], s[1], s[2], s[3]);
+            } else {
+                for (int p = 0; p < n_own; ++p) zo[p] = s[p];
+            }
             for (int o = 16; o; o >>= 1) {
                 const float om = __shfl_xor_sync(0xffffffffu, m, o);
                 const int oi = __shfl_xor_sync(0xffffffffu, mi, o);
@@ -2123,47 +2297,46 @@ __global__ void __launch_bounds__(FI_SLOTS * FI_ST, 1) infer_kernel(const float*
                     mi = oi;
                 }
             }
-            float t[CH];
-#pragma unroll
-            for (int c = 0; c < CH; ++c) t[c] = fi_half(h4[0][c / 2], c & 1) + fi_half(h4[1][c / 2], c & 1);
-            sl.sum[w][lane] = fi_scatter_sum(t, lane);
-#pragma unroll
-            for (int k = 0; k < CH / 2; ++k) h4[0][k] = fi_max2(h4[0][k], h4[1][k]);
-            sl.mx[w][lane] = fi_scatter_max(h4[0], lane);
             if (lane == 0) {
-                sl.zm[w] = m;
-                sl.zi[w] = mi;
+                sl.zm[w & 3] = m;
+                sl.zi[w & 3] = mi;
             }
-        }
-        slot_or(false);
-        isr::tmem_fence_after_sync();
-        if (w == 0) {
-            float m = sl.mx[0][lane], a = sl.sum[0][lane];
+        } else if (w == 0) {
+            float m = sl.mx[0][lane], s = sl.sum[0][lane];
+            int mi = TRAIN ? sl.mi[0][lane] : 0;
 #pragma unroll
-            for (int k = 1; k < 8; ++k) {
-                m = fmaxf(m, sl.mx[k][lane]);
-                a += sl.sum[k][lane];
+            for (int k = 1; k < 4; ++k) {   // ascending positions: ties keep the first
+                const float om = sl.mx[k][lane];
+                if (om > m) {
+                    m = om;
+                    if constexpr (TRAIN) mi = sl.mi[k][lane];
+                }
+                s += sl.sum[k][lane];
             }
             const size_t o = ((size_t)b * nx + xc) * CH + lane;
-            pmax[o] = m;
-            psum[o] = a;
-            if (lane == 0) {
+            a.pmax[o] = m;
+            a.psum[o] = s;
+            if constexpr (TRAIN) a.pidx[o] = mi;
+        }
+        if constexpr (!TRAIN) {   // only the prediction asks for the largest logit
+            fi_slot_or(slot, false);
+            if (st == 0) {
                 float best = sl.zm[0];
                 int at = sl.zi[0];
-                for (int k = 1; k < 8; ++k)
-                    if (sl.zm[k] > best || (sl.zm[k] == best && sl.zi[k] < at)) {
+                for (int k = 1; k < 4; ++k)   // ascending positions
+                    if (sl.zm[k] > best) {
                         best = sl.zm[k];
                         at = sl.zi[k];
                     }
-                zmax[(size_t)b * nx + xc] = best;
-                zidx[(size_t)b * nx + xc] = at;
+                a.zmax[(size_t)b * nx + xc] = best;
+                a.zidx[(size_t)b * nx + xc] = at;
             }
         }
     }
     isr::tmem_fence_before_sync();
     __syncthreads();
     isr::tmem_fence_after_sync();
-    if (tid < 32) isr::tmem_dealloc(sh.tslot, FI_COLS);
+    if (tid < 32) isr::tmem_dealloc(sh.tslot, fi_cols(SLOTS));
 }
 
 __device__ __forceinline__ float block_sum(float v, float* red)
@@ -2491,7 +2664,8 @@ isr_status set_smem_attrs()
     EST_TRY(cudaFuncSetAttribute(conv_kernel<float, T, float, T, CH, false>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, big));
     if constexpr (kTensorConv<T>) {
-        EST_TRY(cudaFuncSetAttribute(infer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FI_SMEM));
+        EST_TRY(cudaFuncSetAttribute(forward_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fi_smem<false>()));
+        EST_TRY(cudaFuncSetAttribute(forward_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, fi_smem<true>()));
         EST_TRY(cudaFuncSetAttribute(conv_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)tc_smem_bytes(true)));
         EST_TRY(cudaFuncSetAttribute(conv_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2533,12 +2707,33 @@ isr_status forward_t(isr_est* e, const float* x, int n, float* pos = nullptr, fl
         e->weights_stale = false;
     }
     if constexpr (kTensorConv<T>) {
-        if (pos && e->conv05) {
+        if (e->conv05) {
             const int nxi = (L + FI_P - 1) / FI_P, tiles = n * nxi;
-            infer_kernel<<<std::min(e->sms, tiles), FI_SLOTS * FI_ST, FI_SMEM, s>>>(
-                x, static_cast<const T*>(e->wf), static_cast<const T*>(e->tf), n, e->z, e->pmax, e->psum, e->zmax,
-                e->zidx, e->theta, L, nxi);
-            head_mlp_kernel<true><<<n, HM_THREADS, 0, s>>>(head_args(e, nxi, pos, pres));
+            FiFwdArgs a{};
+            a.x = x;
+            a.w1 = static_cast<const T*>(e->wf);
+            a.wt = static_cast<const T*>(e->tf);
+            a.theta = e->theta;
+            a.L = L;
+            a.n_rows = n;
+            a.nx = nxi;
+            a.z = e->z;
+            a.pmax = e->pmax;
+            a.psum = e->psum;
+            a.zmax = e->zmax;
+            a.pidx = e->pidx;
+            a.zidx = e->zidx;
+            if (pos) {
+                forward_kernel<false><<<std::min(e->sms, tiles), fi_slots<false>() * FI_ST, fi_smem<false>(), s>>>(a);
+                head_mlp_kernel<true><<<n, HM_THREADS, 0, s>>>(head_args(e, nxi, pos, pres));
+            } else {
+                // the weight gradient of the first layer reads x as stored
+                cast_kernel<T><<<(unsigned)std::min<size_t>((nx + 255) / 256, 4096), 256, 0, s>>>(x, nx, act[0]);
+                for (int l = 0; l < 4; ++l) a.h[l] = act[l + 1];
+                for (int l = 0; l < 3; ++l) a.bits[l] = e->hbits + (size_t)l * e->max_batch * L;
+                forward_kernel<true><<<std::min(e->sms, tiles), fi_slots<true>() * FI_ST, fi_smem<true>(), s>>>(a);
+                head_mlp_kernel<false><<<n, HM_THREADS, 0, s>>>(head_args(e, nxi, nullptr, nullptr));
+            }
             EST_TRY(cudaGetLastError());
             return ISR_OK;
         }
