@@ -53,15 +53,6 @@ template <> __device__ __forceinline__ float ld<__nv_bfloat16>(const __nv_bfloat
 template <class T> __device__ __forceinline__ T cvt(float v);
 template <> __device__ __forceinline__ float cvt<float>(float v) { return v; }
 template <> __device__ __forceinline__ __nv_bfloat16 cvt<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
-// whether v, once stored as T, reads back above zero (the test of the backward pass's ReLU mask);
-// for BF16 the sign and magnitude bits of the stored pattern: positive and not zero
-template <class T> __device__ __forceinline__ bool positive_as_stored(float v);
-template <> __device__ __forceinline__ bool positive_as_stored<float>(float v) { return v > 0.f; }
-template <> __device__ __forceinline__ bool positive_as_stored<__nv_bfloat16>(float v)
-{
-    return (int16_t)__bfloat16_as_ushort(__float2bfloat16_rn(v)) > 0;
-}
-
 // ---------------------------------------------------------------- features
 // x[i] = (ln max(P[lo+i], 1e-30) - mean) / (std + 1e-6) over the band; one CTA per gate.
 // Bytes bound it (4 in, 4 out per bin), so the logarithm and both moments run in float-float on the
@@ -529,37 +520,18 @@ __global__ void __launch_bounds__(CF_THREADS) conv_tc_kernel(const void* __restr
     }
 }
 
-// ---------------------------------------------------------------- tcgen05 convolution
-// Layers 2-4 with BF16 storage on the fifth-generation tensor cores: the same GEMM as
-// conv_tc_kernel with positions as M,
-//   D[i][co] = sum_{k, ci} X[i + k - 4][ci] W[co][ci][k]     (M = 128 positions per tile, N = 32, K = 288),
-// issued by one thread as tcgen05.mma (kind::f16, BF16 operands from shared memory, FP32
-// accumulator in tensor memory).  The input tile is staged position-major in four "planes" of
-// eight channels, [rows][8 ch] with 16-byte rows, so every 8 x 16-byte core matrix of the
-// K-major no-swizzle layout is eight consecutive rows of one plane (SBO = 128 B between 8-row
-// groups, LBO = plane stride between the two 8-channel halves of a K = 16 step), and the A
-// operand of tap k is the same tile started k rows later: descriptor start + 16 k bytes.  The
-// weights are 36 planes [tap][8-channel group] of [32 co][8 ci].  A tile is TPC M tiles of 128
-// positions (128 TPC threads; 18 MMAs per M tile, 36 in the backward-data pass, which multiplies
-// the hi and lo parts of its FP32 input) and 32 TPC TMEM columns; warp w reads M tile w / 4 at its
-// lane quarter and writes the epilogue (bias + ReLU to BF16, or the FP32 gradient masked by the
-// layer below) straight from registers, one coalesced 32-position store per channel.  Every
-// thread issues all of its staging loads before its first shared store.
-// TPC = M tiles of 128 positions per tile (1, 2 or 4): 128 TPC threads, four warps per M tile
+// ---------------------------------------------------------------- tcgen05 operand staging
+// Activations as operand planes of the tcgen05 weight gradient: a tile of 128 TPC positions (halo
+// included) position-major in four planes of eight channels, [rows][8 ch] with 16-byte rows, so every
+// 8 x 16-byte core matrix of the no-swizzle layout is eight consecutive rows of one plane, and tap k is
+// the same tile started k rows later.
 template <int TPC> struct C5 {
-    static constexpr int CT = 128 * TPC;                   // positions per CTA
-    static constexpr int THREADS = 128 * TPC;
+    static constexpr int CT = 128 * TPC;                   // positions per tile
     static constexpr int XW = CT + KT - 1;                 // staged rows (halo included)
     static constexpr int PLANE = XW * 16 + 16;             // bytes per channel plane (+16: planes 4 banks apart)
     static constexpr int PART = 4 * PLANE;                 // one staged part (32 channels)
-    static constexpr int COLS = TPC <= 1 ? 32 : 32 * TPC;  // TMEM columns: one N = 32 tile per M tile
-    // the persistent convolution: two staging buffers of 1 (forward) or 2 (hi, lo) parts, the
-    // weight planes, two mbarriers and the TMEM address slot
-    static constexpr size_t smem(bool fwd) { return (size_t)2 * (fwd ? 1 : 2) * PART + KT * 4 * 512 + 32; }
     static_assert(PLANE % 16 == 0 && (PLANE / 4) % 32 == 4, "planes 16-byte aligned, four banks apart");
 };
-constexpr int C5_WBYTES = KT * 4 * 512;                    // weight planes
-constexpr int C5_TPC = 2;                                  // the launched shape
 
 // 16-bit index of (row j, channel c) in a staged part of plane size PLANE bytes
 template <int PLANE>
@@ -569,14 +541,13 @@ __device__ __forceinline__ int c5_idx(int j, int c) { return (c >> 3) * (PLANE /
 // planes, in two phases so that a pipelined caller keeps the global loads in flight while it does
 // other work: c5_act_load issues every global load of the thread into registers, c5_act_store
 // writes them to the planes.  When L is not a multiple of 8 the 16-byte loads do not apply:
-// c5_act_load does nothing and c5_act_store stages word by word.  Called by THREADS threads.
-// NT = the calling threads (C5<TPC>::THREADS unless a caller stages with more).
-template <int TPC, int NT = C5<TPC>::THREADS> struct C5Act {
+// c5_act_load does nothing and c5_act_store stages word by word.  Called by NT threads.
+template <int TPC, int NT> struct C5Act {
     static constexpr int NITEM = CH * (C5<TPC>::XW / 8 + 1);   // (channel, 8-position block) pieces
     static constexpr int PER = (NITEM + NT - 1) / NT;
 };
 
-template <int TPC, int NT = C5<TPC>::THREADS>
+template <int TPC, int NT>
 __device__ __forceinline__ void c5_act_load(const unsigned short* __restrict__ rows, int L, int i0,
                                             uint4 (&q)[C5Act<TPC, NT>::PER])
 {
@@ -592,7 +563,7 @@ __device__ __forceinline__ void c5_act_load(const unsigned short* __restrict__ r
     }
 }
 
-template <int TPC, int NT = C5<TPC>::THREADS>
+template <int TPC, int NT>
 __device__ __forceinline__ void c5_act_store(const unsigned short* __restrict__ rows, int L, int i0,
                                              const uint4 (&q)[C5Act<TPC, NT>::PER], unsigned short* xs)
 {
@@ -633,255 +604,6 @@ __device__ __forceinline__ void c5_act_store(const unsigned short* __restrict__ 
             *reinterpret_cast<uint32_t*>(xs + c5_idx<P>(j, 2 * cp)) = v0 | (v1 << 16);
         }
     }
-}
-
-template <int TPC>
-__device__ __forceinline__ void c5_stage_act(const unsigned short* __restrict__ rows, int L, int i0, unsigned short* xs)
-{
-    uint4 q[C5Act<TPC>::PER];
-    c5_act_load<TPC>(rows, L, i0, q);
-    c5_act_store<TPC>(rows, L, i0, q, xs);
-}
-
-// The same from FP32 rows, split into BF16 hi (part xh) and lo (part xl), in the same two phases.
-template <int TPC> struct C5Split {
-    static constexpr int NITEM = CH * (C5<TPC>::XW / 4);        // (channel, 4-position block) pieces
-    static constexpr int PER = (NITEM + C5<TPC>::THREADS - 1) / C5<TPC>::THREADS;
-};
-
-template <int TPC>
-__device__ __forceinline__ void c5_split_load(const float* __restrict__ rows, int L, int i0,
-                                              float4 (&q)[C5Split<TPC>::PER])
-{
-    constexpr int NITEM = C5Split<TPC>::NITEM, PER = C5Split<TPC>::PER, THREADS = C5<TPC>::THREADS;
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-        const int e = threadIdx.x + u * THREADS;
-        const int c = e & (CH - 1), v = e / CH;
-        const int pos0 = i0 - HALF + 4 * v;
-        const float* src = rows + (size_t)c * L;
-        q[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (e < NITEM) {
-            if ((L & 3) == 0 && pos0 >= 0 && pos0 + 4 <= L) {
-                q[u] = *reinterpret_cast<const float4*>(src + pos0);
-            } else {
-                q[u].x = (pos0 >= 0 && pos0 < L) ? src[pos0] : 0.f;
-                q[u].y = (pos0 + 1 >= 0 && pos0 + 1 < L) ? src[pos0 + 1] : 0.f;
-                q[u].z = (pos0 + 2 >= 0 && pos0 + 2 < L) ? src[pos0 + 2] : 0.f;
-                q[u].w = (pos0 + 3 >= 0 && pos0 + 3 < L) ? src[pos0 + 3] : 0.f;
-            }
-        }
-    }
-}
-
-template <int TPC>
-__device__ __forceinline__ void c5_split_store(const float4 (&q)[C5Split<TPC>::PER], unsigned short* xh,
-                                               unsigned short* xl)
-{
-    constexpr int NITEM = C5Split<TPC>::NITEM, PER = C5Split<TPC>::PER, THREADS = C5<TPC>::THREADS;
-    constexpr int P = C5<TPC>::PLANE;
-    static_assert(NITEM % 32 == 0 && THREADS % 32 == 0, "whole warps per item round (the shuffles)");
-    static_assert((C5<TPC>::PART / 4) % 32 == 16, "the hi and lo parts 16 banks apart");
-    // lane = channel c; lanes c, c ^ 1 swap parts: the even lane gets the hi words of both
-    // channels and the odd lane the lo words, and each writes one 32-bit word (channels c & ~1,
-    // c | 1) per position, so every store fills rows j of both parts, 32 distinct banks
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-        const int e = threadIdx.x + u * THREADS;
-        if (e >= NITEM) break;
-        const int c = e & (CH - 1), v = e / CH, odd = c & 1;
-        uint32_t hi0, lo0, hi1, lo1;
-        isr::split2<true>(q[u].x, q[u].y, hi0, lo0);
-        isr::split2<true>(q[u].z, q[u].w, hi1, lo1);
-        const uint32_t r0 = __shfl_xor_sync(0xffffffffu, odd ? hi0 : lo0, 1);
-        const uint32_t r1 = __shfl_xor_sync(0xffffffffu, odd ? hi1 : lo1, 1);
-        const uint32_t m0 = odd ? lo0 : hi0, m1 = odd ? lo1 : hi1;
-        const uint32_t e0 = odd ? r0 : m0, o0 = odd ? m0 : r0;   // even / odd channel, positions 0-1
-        const uint32_t e1 = odd ? r1 : m1, o1 = odd ? m1 : r1;   // positions 2-3
-        const uint32_t w[4] = {__byte_perm(e0, o0, 0x5410), __byte_perm(e0, o0, 0x7632),
-                               __byte_perm(e1, o1, 0x5410), __byte_perm(e1, o1, 0x7632)};
-        unsigned short* x = odd ? xl : xh;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) *reinterpret_cast<uint32_t*>(x + c5_idx<P>(4 * v + k, c & ~1)) = w[k];
-    }
-}
-
-// FWD: in = BF16 activations [B][32][L], out = BF16 relu(conv + bias); with BITS (a training pass)
-//   also the ReLU mask, bits[b * L + i] bit co = (stored output [b][co][i] > 0).
-// !FWD: in = FP32 gradient [B][32][L], out = FP32 conv masked by the layer below's ReLU, read as
-//   those bits (one word per position, loaded before the epilogue waits for the tile's MMAs), no bias.
-// wt: GEMM rows [out channel][tap][in channel] (BF16), as for conv_tc_kernel.
-// Persistent: CTA c takes tiles c, c + gridDim.x, ... of the n_rows x ceil(L / CT) tiles (row-major)
-// with a two-deep pipeline over two staging buffers, two TMEM accumulators and two mbarriers.  In
-// the iteration of tile t: the global loads of tile t + gridDim.x are issued into registers, the
-// epilogue of tile t runs (its MMAs were issued one iteration earlier), the registers are written
-// to the other staging buffer (whose MMAs completed before the previous epilogue), and after one
-// barrier thread 0 issues that tile's MMAs into the other accumulator.  The weights are staged
-// once per CTA.  A wait that runs out of polls ends the CTA's loop (the vote at the barrier makes
-// that uniform) and the tiles left are not written.
-constexpr int C5_CTAS_PER_SM = 2;
-static_assert(C5_CTAS_PER_SM * 2 * C5<C5_TPC>::COLS <= 512, "TMEM columns of the resident CTAs");
-template <bool FWD, bool BITS = !FWD>
-__global__ void __launch_bounds__(C5<C5_TPC>::THREADS, C5_CTAS_PER_SM) conv_tc05_kernel(const void* __restrict__ in,
-                                                                         const __nv_bfloat16* __restrict__ wt,
-                                                                         const float* __restrict__ bias,
-                                                                         uint32_t* __restrict__ bits, int L,
-                                                                         int n_rows, void* __restrict__ out)
-{
-    using G = C5<C5_TPC>;
-    constexpr int NX = FWD ? 1 : 2;
-    constexpr int C5_CT = G::CT, CF_THREADS = G::THREADS, C5_PART = G::PART, C5_PLANE = G::PLANE, C5_COLS = G::COLS;
-    static_assert(C5_PLANE % 16 == 0 && C5_PART % 16 == 0, "descriptor steps are whole 16-byte units");
-    extern __shared__ __align__(128) unsigned char c5_smem[];
-    unsigned char* xs = c5_smem;                                  // [2 buffers][NX parts of 4 planes]
-    unsigned char* ws = c5_smem + 2 * NX * C5_PART;               // 36 weight planes
-    uint64_t* mbar = reinterpret_cast<uint64_t*>(ws + C5_WBYTES); // [2]
-    uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 2);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tiles_per_row = (L + C5_CT - 1) / C5_CT, n_tiles = n_rows * tiles_per_row;
-    if ((int)blockIdx.x >= n_tiles) return;   // uniform per CTA, before any barrier or allocation
-
-    if (tid == 0) {
-        isr::mbar_init(isr::smem_u32(&mbar[0]), 1);
-        isr::mbar_init(isr::smem_u32(&mbar[1]), 1);
-    }
-    if (warp == 0) isr::tmem_alloc(isr::smem_u32(tslot), 2 * C5_COLS);
-    // weights: 16-byte piece (co, tap, 8-channel group g) of row co to plane (tap, g), row co
-    {
-        const uint4* w4 = reinterpret_cast<const uint4*>(wt);
-        constexpr int WPER = (CH * KT * 4 + CF_THREADS - 1) / CF_THREADS;
-        uint4 wq[WPER];
-#pragma unroll
-        for (int u = 0; u < WPER; ++u) {
-            const int e = tid + u * CF_THREADS;
-            if (e < CH * KT * 4) wq[u] = w4[e];
-        }
-#pragma unroll
-        for (int u = 0; u < WPER; ++u) {
-            const int e = tid + u * CF_THREADS;
-            if (e >= CH * KT * 4) break;
-            const int co = e / (KT * 4), r = e - co * (KT * 4);  // r = tap * 4 + g
-            *reinterpret_cast<uint4*>(ws + (r * CH + co) * 16) = wq[u];
-        }
-    }
-
-    // staging of tile t: global loads into registers, then shared stores into buffer `buf`
-    uint4 qa[FWD ? C5Act<C5_TPC>::PER : 1];
-    float4 qs[FWD ? 1 : C5Split<C5_TPC>::PER];
-    auto load = [&](int t) {
-        const int b = t / tiles_per_row, i0 = (t - b * tiles_per_row) * C5_CT;
-        if constexpr (FWD)
-            c5_act_load<C5_TPC>(static_cast<const unsigned short*>(in) + (size_t)b * CH * L, L, i0, qa);
-        else
-            c5_split_load<C5_TPC>(static_cast<const float*>(in) + (size_t)b * CH * L, L, i0, qs);
-    };
-    auto store = [&](int t, int buf) {
-        const int b = t / tiles_per_row, i0 = (t - b * tiles_per_row) * C5_CT;
-        unsigned char* x = xs + buf * NX * C5_PART;
-        if constexpr (FWD)
-            c5_act_store<C5_TPC>(static_cast<const unsigned short*>(in) + (size_t)b * CH * L, L, i0, qa,
-                                 reinterpret_cast<unsigned short*>(x));
-        else
-            c5_split_store<C5_TPC>(qs, reinterpret_cast<unsigned short*>(x), reinterpret_cast<unsigned short*>(x + C5_PART));
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tile, for the tensor cores
-    };
-    // thread 0: the MMAs of the tile in buffer `buf` into accumulator `buf`, committed to mbar[buf]
-    auto issue = [&](uint32_t tbase, int buf) {
-        constexpr uint32_t idesc = isr::tc05_idesc<true>();      // BF16, FP32 accumulate, M 128, N 32
-        // descriptors built once and stepped in 16-byte units of the start field (addresses stay
-        // below 0x40000 B, so the 14-bit field never carries): tap k starts the A tile k rows
-        // (16 B each) later and B at weight plane 4 k; K-step ks moves A by two channel planes
-        // and B by two weight planes (512 B each)
-        const uint64_t bd0 = isr::tc05_desc(isr::smem_u32(ws), 512, 128);
-        const uint32_t xb = isr::smem_u32(xs) + buf * NX * C5_PART;
-#pragma unroll 1
-        for (int m = 0; m < C5_CT / 128; ++m) {
-            const uint32_t d = tbase + (uint32_t)(buf * C5_COLS) + 32u * m;
-            uint32_t acc = 0;
-#pragma unroll 1
-            for (int part = 0; part < NX; ++part) {
-                // rows 128 m + tap of the tile, channels 16 ks .. (planes 2 ks, 2 ks + 1)
-                const uint64_t ad0 = isr::tc05_desc(xb + part * C5_PART + 128 * m * 16, C5_PLANE, 128);
-#pragma unroll
-                for (int tap = 0; tap < KT; ++tap)
-#pragma unroll
-                    for (int ks = 0; ks < 2; ++ks) {
-                        isr::tc05_mma(d, ad0 + (uint32_t)(tap + ks * (2 * C5_PLANE / 16)),
-                                      bd0 + (uint32_t)((tap * 4 + 2 * ks) * (512 / 16)), idesc, acc);
-                        acc = 1;
-                    }
-            }
-        }
-        isr::tc05_commit(isr::smem_u32(&mbar[buf]));
-    };
-
-    int t = blockIdx.x;
-    load(t);
-    store(t, 0);
-    isr::fence_barrier_init();
-    isr::tmem_fence_before_sync();
-    __syncthreads();
-    isr::tmem_fence_after_sync();
-    const uint32_t tbase = *tslot;
-    if (tid == 0) issue(tbase, 0);
-
-    // epilogue: warp w, tile m = w / 4, lane quarter w % 4 -> position i
-    const int m = warp >> 2;
-    for (int k = 0;; ++k) {
-        const int buf = k & 1, tn = t + (int)gridDim.x;
-        const bool more = tn < n_tiles;
-        if (more) load(tn);
-        uint32_t mbits = 0;   // backward: the ReLU mask of this thread's position, in flight during the wait
-        if constexpr (!FWD) {
-            const int b = t / tiles_per_row, i = (t - b * tiles_per_row) * C5_CT + 128 * m + 32 * (warp & 3) + lane;
-            if (i < L) mbits = bits[(size_t)b * L + i];
-        }
-        const bool done = isr::mbar_wait(isr::smem_u32(&mbar[buf]), (uint32_t)(k >> 1) & 1u, 1u << 26);
-        isr::tmem_fence_after_sync();
-        {
-            const int b = t / tiles_per_row, i0 = (t - b * tiles_per_row) * C5_CT;
-            const int i = i0 + 128 * m + 32 * (warp & 3) + lane;
-            uint32_t r[32];
-            isr::tmem_ld32(isr::tmem_warp_lane_base(tbase) + (uint32_t)(buf * C5_COLS) + 32u * m, r);
-            isr::tmem_wait_ld32(r);
-            if (done && i < L) {
-                const size_t row = (size_t)b * CH * L + i;
-                uint32_t fbits = 0;
-#pragma unroll
-                for (int co = 0; co < CH; ++co) {
-                    const float v = __uint_as_float(r[co]);
-                    if constexpr (FWD) {
-                        const __nv_bfloat16 hv = __float2bfloat16_rn(fmaxf(v + __ldg(bias + co), 0.f));
-                        static_cast<__nv_bfloat16*>(out)[row + (size_t)co * L] = hv;
-                        if constexpr (BITS) fbits |= (uint32_t)((int16_t)__bfloat16_as_ushort(hv) > 0) << co;
-                    } else {
-                        static_cast<float*>(out)[row + (size_t)co * L] = (mbits >> co) & 1u ? v : 0.f;
-                    }
-                }
-                if constexpr (FWD && BITS) bits[(size_t)b * L + i] = fbits;
-            }
-        }
-        // the other staging buffer and accumulator were last used by tile t - gridDim.x, whose
-        // MMAs completed (waited on in the previous iteration) and whose epilogue is done
-        if (more) store(tn, buf ^ 1);
-        isr::tmem_fence_before_sync();
-        const bool ok = __syncthreads_and(done) != 0;
-        isr::tmem_fence_after_sync();
-        if (!more || !ok) break;
-        if (tid == 0) issue(tbase, buf ^ 1);
-        t = tn;
-    }
-    isr::tmem_fence_before_sync();
-    __syncthreads();
-    isr::tmem_fence_after_sync();
-    if (warp == 0) isr::tmem_dealloc(tbase, 2 * C5_COLS);
-}
-
-// Persistent CTAs of conv_tc05_kernel: one per tile, up to `slots` (the resident count on all SMs).
-inline int conv_tc05_grid(int L, int n_rows, int slots)
-{
-    const int tiles = n_rows * ((L + C5<C5_TPC>::CT - 1) / C5<C5_TPC>::CT);
-    return std::max(1, std::min(tiles, slots));
 }
 
 __device__ __forceinline__ void ldsm_x4_trans(uint32_t (&r)[4], uint32_t addr)
@@ -1391,25 +1113,9 @@ template <> __device__ __forceinline__ void store_pair<__nv_bfloat16>(__nv_bfloa
 {
     *reinterpret_cast<__nv_bfloat162*>(o) = __floats2bfloat162_rn(a, b);
 }
-// the same, returning in bits 0 / 1 whether a / b read back above zero as stored
-template <class T> __device__ __forceinline__ uint32_t store_pair_signs(T* o, float a, float b);
-template <> __device__ __forceinline__ uint32_t store_pair_signs<float>(float* o, float a, float b)
-{
-    store_pair<float>(o, a, b);
-    return (uint32_t)(a > 0.f) | ((uint32_t)(b > 0.f) << 1);
-}
-template <> __device__ __forceinline__ uint32_t store_pair_signs<__nv_bfloat16>(__nv_bfloat16* o, float a, float b)
-{
-    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    *reinterpret_cast<__nv_bfloat162*>(o) = h;
-    const uint32_t w = *reinterpret_cast<const uint32_t*>(&h);
-    return (uint32_t)((int16_t)(w & 0xffffu) > 0) | ((uint32_t)((int32_t)w > 0x0000ffff) << 1);
-}
-
-template <class T, bool BITS>
+template <class T>
 __global__ void __launch_bounds__(256) conv1_kernel(const T* __restrict__ x, const T* __restrict__ w1,
-                                                    const float* __restrict__ b1, int L, T* __restrict__ out,
-                                                    uint32_t* __restrict__ bits)
+                                                    const float* __restrict__ b1, int L, T* __restrict__ out)
 {
     __shared__ float xs[L1_CT + KT - 1];
     __shared__ __align__(16) float ws[CH][12];   // W1[co][0..8], b1[co], 0, 0
@@ -1430,7 +1136,6 @@ __global__ void __launch_bounds__(256) conv1_kernel(const T* __restrict__ x, con
 #pragma unroll
     for (int j = 0; j < KT + 1; ++j) xv[j] = xs[p + j];
     const bool pair = i + 1 < L && (L & 1) == 0;   // even row offsets: aligned pair stores
-    uint32_t m0 = 0, m1 = 0;                        // ReLU mask bits of positions i, i + 1 (BITS)
 #pragma unroll 4
     for (int co = 0; co < CH; ++co) {
         const float4 wa = *reinterpret_cast<const float4*>(&ws[co][0]);
@@ -1447,25 +1152,11 @@ __global__ void __launch_bounds__(256) conv1_kernel(const T* __restrict__ x, con
         s1 = fmaxf(s1, 0.f);
         T* o = out + ((size_t)b * CH + co) * L + i;
         if (pair) {
-            if constexpr (BITS) {
-                const uint32_t sg = store_pair_signs<T>(o, s0, s1);
-                m0 |= (sg & 1u) << co;
-                m1 |= (sg >> 1) << co;
-            } else {
-                store_pair<T>(o, s0, s1);
-            }
+            store_pair<T>(o, s0, s1);
         } else {
-            if constexpr (BITS) {
-                m0 |= (uint32_t)positive_as_stored<T>(s0) << co;
-                m1 |= (uint32_t)positive_as_stored<T>(s1) << co;
-            }
             o[0] = cvt<T>(s0);
             if (i + 1 < L) o[1] = cvt<T>(s1);
         }
-    }
-    if constexpr (BITS) {
-        bits[(size_t)b * L + i] = m0;
-        if (i + 1 < L) bits[(size_t)b * L + i + 1] = m1;
     }
 }
 
@@ -2588,6 +2279,220 @@ __global__ void __launch_bounds__(256, 2) head_bwd_chunk_kernel(const T* __restr
     }
 }
 
+// ---------------------------------------------------------------- fused backward pass (BF16, tcgen05)
+// The gradient of the loss from the head down through the three 32-channel layers in one kernel, with the
+// tiles, operand layout and slots of forward_kernel: dL/dz and the masked gradient of h4 as
+// head_bwd_chunk_kernel forms them, then per layer the convolution with the flipped transposed weights
+// on the FP32 gradient split into BF16 hi + lo (48 MMAs), masked by the layer below's ReLU bits.  Every
+// masked gradient is written once, in FP32, for the weight gradients, and none is read back: launched
+// per layer these passes took 39 + 3 x 55 us for 128 rows x 4608 positions, bound by 75 MB in and out per
+// layer and the staging between; together they take 126 us, for 323 MB of which 302 MB are the four
+// gradients written (42 us at 7.6 TB/s): two tiles a SM leave the MMAs and the element passes of one
+// exposed when the other waits too, and shared memory has no room for a third.  Gradient sums of w5 and
+// b5 stay in registers over a CTA's tiles.
+constexpr int FB_SLOTS = 2;
+struct FiBwdSlot {
+    uint64_t mbar;
+    float mean[CH], peak[CH], scal[HB_SCAL];   // per channel: pooling gradients of the row
+    int at[CH];                                 // position of the channel's maximum
+};
+struct FiBwdShared {
+    float w5[CH];
+    uint32_t tslot;
+    FiBwdSlot slot[FB_SLOTS];
+};
+constexpr int FB_OFF_SH = FI_OFF_BUF + FB_SLOTS * 2 * FI_BUF;
+constexpr int FB_SMEM = FB_OFF_SH + (int)sizeof(FiBwdShared);
+static_assert(FB_SMEM <= 232448 && FB_OFF_SH % 16 == 0, "shared memory");
+struct FiBwdArgs {
+    const __nv_bfloat16 *h4, *wt;
+    const float *theta, *z, *scal, *dpool;
+    const int* amax;
+    const uint32_t* bits[3];   // masks of h3, h2, h1
+    float* da[4];              // masked gradients of h4 .. h1
+    float* grad;
+    int L, n_rows, nx;
+};
+
+__global__ void __launch_bounds__(FB_SLOTS * FI_ST, 1) backward_kernel(const __grid_constant__ FiBwdArgs a)
+{
+    constexpr int NT = FB_SLOTS * FI_ST;
+    extern __shared__ __align__(128) unsigned char fb_smem[];
+    auto& sh = *reinterpret_cast<FiBwdShared*>(fb_smem + FB_OFF_SH);
+    const int tid = threadIdx.x, slot = tid / FI_ST, st = tid - slot * FI_ST;
+    const int lane = tid & 31, w = __shfl_sync(0xffffffffu, st >> 5, 0);
+    const int half = w >> 2, r = 32 * (w & 3) + lane;
+    FiBwdSlot& sl = sh.slot[slot];
+    unsigned char* buf = fb_smem + FI_OFF_BUF + slot * 2 * FI_BUF;   // hi part, lo part
+    const uint32_t mbar = isr::smem_u32(&sl.mbar);
+    const int L = a.L, nx = a.nx;
+    const bool vec = (L & 3) == 0;   // groups of four positions are whole and aligned
+
+    if (st == 0) isr::mbar_init(mbar, 1);
+    isr::fence_barrier_init();
+    if (tid < 32) isr::tmem_alloc(isr::smem_u32(&sh.tslot), fi_cols(FB_SLOTS));
+    fi_stage_weights<NT>(fb_smem, a.wt, tid);
+    if (tid < CH) sh.w5[tid] = a.theta[OFF_W5 + tid];
+    for (int e = tid; e < FB_SLOTS * 2 * FI_BUF / 16; e += NT)   // the last two rows are read, never written
+        *reinterpret_cast<uint4*>(fb_smem + FI_OFF_BUF + e * 16) = make_uint4(0u, 0u, 0u, 0u);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    isr::tmem_fence_before_sync();
+    __syncthreads();
+    isr::tmem_fence_after_sync();
+    const uint32_t tacc = sh.tslot + 128u * slot;
+
+    // v[p][c]: FP32 gradients of eight channels (group g) at four positions -> memory (the first `count`
+    // positions) ...
+    auto to_rows = [&](float* __restrict__ da, int b, int pos, int count, int g, const float (&v)[4][GC]) {
+        float* o = da + ((size_t)b * CH + HC * half + GC * g) * L + pos;
+        if (vec) {
+            if (count)
+#pragma unroll
+                for (int c = 0; c < GC; ++c)
+                    *reinterpret_cast<float4*>(o + (size_t)c * L) = make_float4(v[0][c], v[1][c], v[2][c], v[3][c]);
+        } else {
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+                if (p < count)
+#pragma unroll
+                    for (int c = 0; c < GC; ++c) o[(size_t)c * L + p] = v[p][c];
+        }
+    };
+    // ... and, split into BF16 hi + lo, to the operand planes; the magnitudes' largest bits into top
+    auto to_planes = [&](int g, const float (&v)[4][GC], uint32_t& top) {
+        FiQuad hi, lo;
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+            for (int k = 0; k < GC / 2; ++k) {
+                isr::split2<true>(v[p][2 * k], v[p][2 * k + 1], hi[p][k], lo[p][k]);
+                top = __vmaxu2(top, hi[p][k] & 0x7fff7fffu);
+            }
+        fi_to_planes(buf, r, half, g, hi);
+        fi_to_planes(buf + FI_BUF, r, half, g, lo);
+    };
+
+    const int n_tiles = a.n_rows * nx, step = gridDim.x * FB_SLOTS;
+    float dw5[HC], db5 = 0.f;
+#pragma unroll
+    for (int c = 0; c < HC; ++c) dw5[c] = 0.f;
+    uint32_t phase = 0;
+    for (int tile = slot * gridDim.x + blockIdx.x; tile < n_tiles; tile += step) {
+        const int b = tile / nx, xc = tile - b * nx, i0 = xc * FI_P, end = min(i0 + FI_P, L);
+        auto owned = [&](int pos) { return pos >= i0 && pos < end ? min(4, end - pos) : 0; };
+        auto inside = [&](int pos) { return pos >= 0 && pos < L; };
+        if (st < CH) {
+            sl.peak[st] = a.dpool[(size_t)b * 2 * CH + st];
+            sl.mean[st] = a.dpool[(size_t)b * 2 * CH + CH + st] / L;
+            sl.at[st] = a.amax[b * CH + st];
+        } else if (st < CH + HB_SCAL) {
+            sl.scal[st - CH] = a.scal[(size_t)b * HB_SCAL + st - CH];
+        }
+        fi_slot_or(slot, false);
+        // ---- gradient of h4 at positions i0 - 12 + 4 r .. + 3
+        uint32_t top = 0u;
+        {
+            const int pos = i0 - 12 + 4 * r, n_own = owned(pos);
+            const float lse = sl.scal[0], inv_st = sl.scal[1], ys = sl.scal[2], f = sl.scal[3];
+            float dz[4];
+            const float* zb = a.z + (size_t)b * L;
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                const int i = pos + p;
+                const float d = (i - f) / SIGMA_T;
+                dz[p] = inside(i) && ys != 0.f ? ys * (__expf(zb[i] - lse) - __expf(-0.5f * d * d) * inv_st) : 0.f;
+                if (half == 0 && p < n_own) db5 += dz[p];
+            }
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                const __nv_bfloat16* hb = a.h4 + ((size_t)b * CH + HC * half + GC * g) * L + pos;
+                uint2 hq[GC];   // four positions of a channel
+#pragma unroll
+                for (int c = 0; c < GC; ++c) {
+                    hq[c] = make_uint2(0u, 0u);
+                    if (vec) {
+                        if (inside(pos)) hq[c] = *reinterpret_cast<const uint2*>(hb + (size_t)c * L);
+                    } else {
+                        const unsigned short* hs = reinterpret_cast<const unsigned short*>(hb) + (size_t)c * L;
+                        uint32_t h[4];
+#pragma unroll
+                        for (int p = 0; p < 4; ++p) h[p] = inside(pos + p) ? hs[p] : 0u;
+                        hq[c] = make_uint2(h[0] | h[1] << 16, h[2] | h[3] << 16);
+                    }
+                }
+                float v[4][GC];
+#pragma unroll
+                for (int c = 0; c < GC; ++c) {
+                    const int ch = HC * half + GC * g + c;
+                    const float w5 = sh.w5[ch], mean = sl.mean[ch], peak = sl.peak[ch];
+                    const int at = sl.at[ch];
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) {
+                        const float h = fi_half(p < 2 ? hq[c].x : hq[c].y, p & 1);
+                        if (p < n_own) dw5[GC * g + c] = fmaf(dz[p], h, dw5[GC * g + c]);
+                        float d = fmaf(w5, dz[p], mean);
+                        if (pos + p == at) d += peak;
+                        v[p][c] = h > 0.f ? d : 0.f;
+                    }
+                }
+                to_rows(a.da[0], b, pos, n_own, g, v);
+                to_planes(g, v, top);
+            }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        bool inf = fi_slot_or(slot, fi_inf2(top));
+        if (st == 0) fi_issue<2>(tacc, mbar, buf, fb_smem + 2 * FI_WLAYER, inf);
+        // ---- layers 4, 3, 2: gradients of h3, h2, h1
+#pragma unroll 1
+        for (int l = 0; l < 3; ++l) {
+            const int pos = i0 - 8 + 4 * l + 4 * r, n_own = owned(pos);
+            uint32_t m[4] = {0u, 0u, 0u, 0u};   // ReLU masks, on their way during the MMAs
+            const uint32_t* mb = a.bits[l] + (size_t)b * L + pos;
+            if (vec) {
+                if (inside(pos)) {
+                    const uint4 q = *reinterpret_cast<const uint4*>(mb);
+                    m[0] = q.x, m[1] = q.y, m[2] = q.z, m[3] = q.w;
+                }
+            } else {
+#pragma unroll
+                for (int p = 0; p < 4; ++p)
+                    if (inside(pos + p)) m[p] = mb[p];
+            }
+            const bool done = isr::mbar_wait(mbar, phase, 1u << 26);
+            phase ^= 1u;
+            isr::tmem_fence_after_sync();
+            top = 0u;
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                float v[4][GC];
+                fi_read(tacc, half, g, v);
+#pragma unroll
+                for (int p = 0; p < 4; ++p)
+#pragma unroll
+                    for (int c = 0; c < GC; ++c)
+                        v[p][c] = done && (m[p] >> (HC * half + GC * g + c) & 1u) ? v[p][c] : 0.f;
+                to_rows(a.da[l + 1], b, pos, n_own, g, v);
+                if (l < 2) to_planes(g, v, top);
+            }
+            isr::tmem_fence_before_sync();
+            if (l < 2) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            inf = fi_slot_or(slot, fi_inf2(top));
+            isr::tmem_fence_after_sync();
+            if (l < 2 && st == 0) fi_issue<2>(tacc, mbar, buf, fb_smem + (1 - l) * FI_WLAYER, inf);
+        }
+    }
+    const float d5 = fi_scatter(dw5, lane, [](float u, float v) { return u + v; });
+    if ((lane & 1) == 0) atomicAdd(&a.grad[OFF_W5 + HC * half + (lane >> 1)], d5);
+    if (half == 0) {
+        for (int o = 16; o; o >>= 1) db5 += __shfl_xor_sync(0xffffffffu, db5, o);
+        if (lane == 0) atomicAdd(&a.grad[OFF_B5], db5);
+    }
+    isr::tmem_fence_before_sync();
+    __syncthreads();
+    isr::tmem_fence_after_sync();
+    if (tid < 32) isr::tmem_dealloc(sh.tslot, fi_cols(FB_SLOTS));
+}
+
 __global__ void adam_kernel(float* __restrict__ theta, const float* __restrict__ g, float* __restrict__ m,
                             float* __restrict__ v, int n, float lr, float b1, float b2, float eps, float c1, float c2)
 {
@@ -2623,9 +2528,8 @@ struct isr_est {
     int wgrad_slots = 0;                      // resident tensor-core weight-gradient CTAs (all SMs)
     bool conv05 = false;                      // BF16 convolutions on tcgen05 (else mma.sync)
     int sms = 0;                              // multiprocessors of the device
-    int c5_slots[2] = {1, 1};                 // persistent tcgen05 convolution CTAs, backward / forward
     int* pidx = nullptr;
-    float *da0 = nullptr, *da1 = nullptr; // gradient ping-pong [B][32][L]
+    float* da[4] = {};                    // masked gradients [B][32][L]: of h4 .. h1 (tcgen05 engine), else two in turn
     // tcgen05 engine: ReLU masks of h1..h3 as written by a training forward pass, [3][B][L] words,
     // bit co of word (b, i) set when h_l[b][co][i] > 0 as stored
     uint32_t* hbits = nullptr;
@@ -2659,11 +2563,13 @@ struct Dev {
 template <class T>
 isr_status set_smem_attrs()
 {
-    const int big = (int)conv_smem_bytes(CH);
-    EST_TRY(cudaFuncSetAttribute(conv_kernel<T, T, T, T, CH, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-    EST_TRY(cudaFuncSetAttribute(conv_kernel<float, T, float, T, CH, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-    if constexpr (kTensorConv<T>) {
+    [[maybe_unused]] const int big = (int)conv_smem_bytes(CH);
+    if constexpr (!kTensorConv<T>) {
+        EST_TRY(cudaFuncSetAttribute(conv_kernel<T, T, T, T, CH, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+        EST_TRY(cudaFuncSetAttribute(conv_kernel<float, T, float, T, CH, false>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+    } else {
+        EST_TRY(cudaFuncSetAttribute(backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FB_SMEM));
         EST_TRY(cudaFuncSetAttribute(forward_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fi_smem<false>()));
         EST_TRY(cudaFuncSetAttribute(forward_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, fi_smem<true>()));
         EST_TRY(cudaFuncSetAttribute(conv_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2674,15 +2580,6 @@ isr_status set_smem_attrs()
                                      (int)wgrad_tc_smem_bytes()));
         EST_TRY(cudaFuncSetAttribute(wgrad_tc05_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)W5_SMEM_LAUNCH));
-        for (auto k : {conv_tc05_kernel<true, false>, conv_tc05_kernel<true, true>}) {
-            EST_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C5<C5_TPC>::smem(true)));
-            EST_TRY(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                         (int)cudaSharedmemCarveoutMaxShared));
-        }
-        EST_TRY(cudaFuncSetAttribute(conv_tc05_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)C5<C5_TPC>::smem(false)));
-        EST_TRY(cudaFuncSetAttribute(conv_tc05_kernel<false>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     (int)cudaSharedmemCarveoutMaxShared));
     }
     return ISR_OK;
 }
@@ -2741,27 +2638,15 @@ isr_status forward_t(isr_est* e, const float* x, int n, float* pos = nullptr, fl
     cast_kernel<T><<<(unsigned)std::min<size_t>((nx + 255) / 256, 4096), 256, 0, s>>>(x, nx, act[0]);
     const T* wf = static_cast<const T*>(e->wf);
     dim3 grid((L + CT - 1) / CT, n);
-    // a training pass (no prediction outputs) of the tcgen05 engine leaves the ReLU masks of h1..h3
-    // as bits for the backward-data convolutions
-    auto hbits = [&](int l) -> uint32_t* {
-        return (pos == nullptr && e->hbits && l <= 3) ? e->hbits + (size_t)(l - 1) * e->max_batch * L : nullptr;
-    };
-    (hbits(1) ? conv1_kernel<T, true> : conv1_kernel<T, false>)<<<dim3((L + L1_CT - 1) / L1_CT, n), 256, 0, s>>>(
-        act[0], wf, e->theta + OFF_B1, L, act[1], hbits(1));
+    conv1_kernel<T><<<dim3((L + L1_CT - 1) / L1_CT, n), 256, 0, s>>>(act[0], wf, e->theta + OFF_B1, L, act[1]);
     for (int l = 2; l <= 4; ++l) {
-        if constexpr (kTensorConv<T>) {
-            const T* w = static_cast<const T*>(e->tf) + (size_t)(l - 2) * CH * CH * KT;
-            if (e->conv05)
-                (hbits(l) ? conv_tc05_kernel<true, true> : conv_tc05_kernel<true, false>)<<<
-                    conv_tc05_grid(L, n, e->c5_slots[1]), C5<C5_TPC>::THREADS, C5<C5_TPC>::smem(true), s>>>(
-                    act[l - 1], w, e->theta + b_off(l), hbits(l), L, n, act[l]);
-            else
-                conv_tc_kernel<true><<<dim3((L + CF_CT - 1) / CF_CT, n), CF_THREADS, tc_smem_bytes(true), s>>>(
-                    act[l - 1], w, e->theta + b_off(l), nullptr, L, act[l]);
-        } else {
+        if constexpr (kTensorConv<T>)
+            conv_tc_kernel<true><<<dim3((L + CF_CT - 1) / CF_CT, n), CF_THREADS, tc_smem_bytes(true), s>>>(
+                act[l - 1], static_cast<const T*>(e->tf) + (size_t)(l - 2) * CH * CH * KT, e->theta + b_off(l), nullptr, L,
+                act[l]);
+        else
             conv_kernel<T, T, T, T, CH, true><<<grid, 256, conv_smem_bytes(CH), s>>>(
                 act[l - 1], wf + CH * KT + (size_t)(l - 2) * CH * CH * KT, e->theta + b_off(l), nullptr, L, act[l]);
-        }
     }
     const int nxh = (L + HD_CT - 1) / HD_CT;
     head_chunk_kernel<T><<<dim3(nxh, n), 256, 0, s>>>(act[4], e->theta, L, nxh, e->z, e->pmax, e->pidx, e->psum,
@@ -2783,11 +2668,39 @@ isr_status backward_t(isr_est* e, int n, const float* fpos, const float* pres)
     EST_TRY(cudaMemsetAsync(e->loss, 0, sizeof(float), s));
     head_bwd_row_kernel<<<n, 256, 0, s>>>(e->theta, L, n, e->z, e->pooled, e->u, e->q, fpos, pres, e->hscal,
                                           e->dpool, e->grad, e->loss);
+    if constexpr (kTensorConv<T>) {
+        if (e->conv05) {
+            const int nxi = (L + FI_P - 1) / FI_P;
+            FiBwdArgs a{};
+            a.h4 = act[4];
+            a.wt = static_cast<const T*>(e->tb);
+            a.theta = e->theta;
+            a.z = e->z;
+            a.scal = e->hscal;
+            a.dpool = e->dpool;
+            a.amax = e->amax;
+            for (int i = 0; i < 3; ++i) a.bits[i] = e->hbits + (size_t)(2 - i) * e->max_batch * L;
+            for (int i = 0; i < 4; ++i) a.da[i] = e->da[i];
+            a.grad = e->grad;
+            a.L = L;
+            a.n_rows = n;
+            a.nx = nxi;
+            backward_kernel<<<std::min(e->sms, n * nxi), FB_SLOTS * FI_ST, FB_SMEM, s>>>(a);
+            const int chunks = n * ((L + W5_CHUNK - 1) / W5_CHUNK), spans = n * ((L + W1_SPAN - 1) / W1_SPAN);
+            for (int l = 4; l >= 2; --l)
+                wgrad_tc05_kernel<<<std::min(chunks, e->sms), W5_BLOCK, W5_SMEM_LAUNCH, s>>>(
+                    act[l - 1], e->da[4 - l], L, n, e->grad + w_off(l), e->grad + b_off(l));
+            wgrad1_kernel<T><<<std::min(spans, 2 * std::max(1, e->sms)), 256, 0, s>>>(act[0], e->da[3], L, n,
+                                                                                     e->grad + OFF_W1, e->grad + OFF_B1);
+            EST_TRY(cudaGetLastError());
+            return ISR_OK;
+        }
+    }
     head_bwd_chunk_kernel<T><<<dim3((L + HD_CT - 1) / HD_CT, n), 256, 0, s>>>(act[4], e->theta, L, e->z, e->amax,
-                                                                              e->hscal, e->dpool, e->da0, e->grad);
+                                                                              e->hscal, e->dpool, e->da[0], e->grad);
     const T* wbk = static_cast<const T*>(e->wb);
-    float* da = e->da0;
-    float* dn = e->da1;
+    float* da = e->da[0];
+    float* dn = e->da[1];
     dim3 gc((L + CT - 1) / CT, n);
     const int fspan = wgrad_span(L, n, std::max(1, e->sms));
     const int span = TC_CT * wgrad_span_chunks(L, n, std::max(1, e->wgrad_slots));
@@ -2797,30 +2710,17 @@ isr_status backward_t(isr_est* e, int n, const float* fpos, const float* pres)
             wgrad1_kernel<T><<<std::min(spans, 2 * std::max(1, e->sms)), 256, 0, s>>>(act[0], da, L, n,
                                                                                      e->grad + OFF_W1, e->grad + OFF_B1);
         } else {
-            if constexpr (kTensorConv<T>) {
-                if (e->conv05) {
-                    const int chunks = n * ((L + W5_CHUNK - 1) / W5_CHUNK);
-                    wgrad_tc05_kernel<<<std::min(chunks, e->sms), W5_BLOCK, W5_SMEM_LAUNCH, s>>>(
-                        reinterpret_cast<const __nv_bfloat16*>(act[l - 1]), da, L, n, e->grad + w_off(l),
-                        e->grad + b_off(l));
-                } else {
-                    wgrad_tc_kernel<<<dim3((L + span - 1) / span, n), 256, wgrad_tc_smem_bytes(), s>>>(
-                        act[l - 1], da, L, span, e->grad + w_off(l), e->grad + b_off(l));
-                }
-            } else
+            if constexpr (kTensorConv<T>)
+                wgrad_tc_kernel<<<dim3((L + span - 1) / span, n), 256, wgrad_tc_smem_bytes(), s>>>(
+                    act[l - 1], da, L, span, e->grad + w_off(l), e->grad + b_off(l));
+            else
                 wgrad_kernel<T><<<dim3((L + fspan - 1) / fspan, n), 256, 0, s>>>(act[l - 1], da, L, fspan, e->grad + w_off(l),
                                                                                  e->grad + b_off(l));
             // gradient into the layer below, masked by its ReLU: da_{l-1} = (W_l^T * da_l) (h_{l-1} > 0)
-            if constexpr (kTensorConv<T>) {
-                const T* w = static_cast<const T*>(e->tb) + (size_t)(l - 2) * CH * CH * KT;
-                if (e->conv05)
-                    conv_tc05_kernel<false><<<conv_tc05_grid(L, n, e->c5_slots[0]), C5<C5_TPC>::THREADS,
-                                              C5<C5_TPC>::smem(false), s>>>(
-                        da, w, nullptr, e->hbits + (size_t)(l - 2) * e->max_batch * L, L, n, dn);
-                else
-                    conv_tc_kernel<false><<<dim3((L + CF_CT - 1) / CF_CT, n), CF_THREADS, tc_smem_bytes(false), s>>>(
-                        da, w, nullptr, act[l - 1], L, dn);
-            } else
+            if constexpr (kTensorConv<T>)
+                conv_tc_kernel<false><<<dim3((L + CF_CT - 1) / CF_CT, n), CF_THREADS, tc_smem_bytes(false), s>>>(
+                    da, static_cast<const T*>(e->tb) + (size_t)(l - 2) * CH * CH * KT, nullptr, act[l - 1], L, dn);
+            else
                 conv_kernel<float, T, float, T, CH, false><<<gc, 256, conv_smem_bytes(CH), s>>>(
                     da, wbk + (size_t)(l - 2) * CH * CH * KT, nullptr, act[l - 1], L, dn);
             std::swap(da, dn);
@@ -2909,8 +2809,7 @@ isr_status isr_est_create(isr_est** out, int32_t nfft, int32_t band_lo, int32_t 
     A((void**)&e->dpool, 4 * B * 2 * CH);
     A((void**)&e->zmax, 4 * B * nxh);
     A((void**)&e->zidx, 4 * B * nxh);
-    A((void**)&e->da0, 4 * B * CH * L);
-    A((void**)&e->da1, 4 * B * CH * L);
+    for (int i = 0; i < (e->conv05 ? 4 : 2); ++i) A((void**)&e->da[i], 4 * B * CH * L);
     if (e->conv05) A((void**)&e->hbits, 4 * 3 * B * L);
     if (r == cudaSuccess) r = cudaMemset(e->theta, 0, 4 * NPARAM);
     if (r == cudaSuccess) r = cudaMemset(e->m, 0, 4 * NPARAM);
@@ -2928,9 +2827,6 @@ isr_status isr_est_create(isr_est** out, int32_t nfft, int32_t band_lo, int32_t 
             int occ = 0;
             r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, wgrad_tc_kernel, 256, wgrad_tc_smem_bytes());
             e->wgrad_slots = std::max(1, occ) * e->sms;
-            // two CTAs per SM, the shape the kernel is built for (__launch_bounds__ minimum): 128
-            // registers x 256 threads, at most 86 KB of shared memory and 128 TMEM columns each
-            e->c5_slots[0] = e->c5_slots[1] = C5_CTAS_PER_SM * e->sms;
         }
     }
     if (r != cudaSuccess) {
@@ -3033,7 +2929,7 @@ void isr_est_destroy(isr_est* e)
     Dev guard(e->dev);
     cudaStreamSynchronize(e->stream);
     void* ptrs[] = {e->theta, e->m, e->v, e->grad, e->wf, e->wb, e->tf, e->tb, e->act[0], e->act[1], e->act[2], e->act[3],
-                    e->act[4], e->z, e->pooled, e->u, e->q, e->loss, e->amax, e->da0, e->da1,
+                    e->act[4], e->z, e->pooled, e->u, e->q, e->loss, e->amax, e->da[0], e->da[1], e->da[2], e->da[3],
                     e->pmax, e->pidx, e->psum, e->hscal, e->dpool, e->zmax, e->zidx, e->hbits};
     for (void* p : ptrs) cudaFree(p);
     cudaGetLastError();

@@ -255,3 +255,22 @@ def test_bf16_gradients_many_rows_several_chunks_per_cta(precision):
         err = np.abs(gd[name] - rd[name]).max() / scale
         assert err <= 1e-3, f"{name}: max error {err:.2e} of the block's largest gradient"
     e.close()
+
+
+@pytest.mark.parametrize("B,L", [(1, 16), (3, 487), (2, 488), (2, 489), (3, 976), (2, 977), (320, 1000)])
+def test_bf16_fused_gradients_at_tile_edges(B, L):
+    """Forward and backward passes of the tcgen05 engine work in tiles of 488 positions, two to
+    a CTA: one short, one full and one position more, rows that are not whole groups of four
+    positions, and more tiles than CTAs take at a time.  The bound of the other exact-input
+    gradient tests."""
+    e, theta, x, f, y, (xd, fd, yd) = _dyadic_case(B=B, L=L, seed=11)
+    loss, g = e.grad(xd, fd, yd)
+    rl, rg = ref.loss_and_grad(theta.astype(np.float64), x, f, y, store=ref.round_bf16)
+    assert abs(loss - rl) <= 1e-4 * abs(rl)
+    gd, rd = ref.unpack(g.astype(np.float64)), ref.unpack(rg)
+    gmax = np.abs(rg).max()
+    for name, _ in ref.SHAPES:
+        scale = max(np.abs(rd[name]).max(), 1e-3 * gmax)
+        err = np.abs(gd[name] - rd[name]).max() / scale
+        assert err <= 1e-3, f"{name}: max error {err:.2e} of the block's largest gradient"
+    e.close()
