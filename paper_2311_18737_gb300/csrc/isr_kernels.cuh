@@ -125,25 +125,30 @@ inline bool takes_xt(const KernelEntry& ke, bool full, int order) { return ke.fn
 // for any nfft) and a third of one more for its start and its partial sums, and every chunk's partials
 // (bins floats) are written and read once.  The C with the least sum is taken: about two waves, the
 // rule before, left up to a third of the SMs idle in the last one (777 gates x 333 IPPs at nfft 2048:
-// four chunks made 392 units, three rounds of 84 IPPs; three make two of 111).
+// four chunks made 392 units, three rounds of 84 IPPs; three make two of 111).  Weighed are the few
+// least counts, which many gate groups want, and the most chunks that fit in each of the next 16 numbers
+// of rounds; with no more than four units per SM to choose from, 500 gates x 200 IPPs at nfft 4096 had no
+// split better than one chunk on 125 of the SMs (843 us; six chunks, five rounds of 34 IPPs: 726 us).
 inline int64_t pick_chunks(int64_t n, int64_t rg, int64_t sm_count, int64_t c_min, int64_t c_max, int64_t bins)
 {
     constexpr double kUnitIpps = 0.33, kChunkIppsPerBin = 8.0 / (6.5e6 * 4.3);   // 8 bytes at 6.5 MB per us
     c_max = std::min(c_max, n);
     c_min = std::min(c_min, c_max);
-    // beyond four units per SM a finer split has nothing left to balance
-    const int64_t c_top = std::min(c_max, std::max(c_min + 2, (4 * sm_count + rg - 1) / rg));
     int64_t best = c_min;
-    double best_cost = 0;
-    for (int64_t c = c_min; c <= c_top; ++c) {
+    double best_cost = -1;
+    auto weigh = [&](int64_t c) {
+        c = std::max(c_min, std::min(c, c_max));
         const int64_t chunk = (n + c - 1) / c, real = (n + chunk - 1) / chunk;
         const int64_t rounds = (rg * real + sm_count - 1) / sm_count;
         const double cost = (double)rounds * ((double)chunk + kUnitIpps) + (double)real * (double)bins * kChunkIppsPerBin;
-        if (c == c_min || cost < best_cost) {
+        if (best_cost < 0 || cost < best_cost) {
             best = c;
             best_cost = cost;
         }
-    }
+    };
+    for (int64_t c = c_min; c < c_min + 4; ++c) weigh(c);
+    const int64_t rounds_min = (rg * c_min + sm_count - 1) / sm_count;
+    for (int64_t k = rounds_min; k < rounds_min + 16; ++k) weigh(k * sm_count / rg);
     return best;
 }
 
