@@ -540,26 +540,29 @@ __device__ __forceinline__ int c5_idx(int j, int c) { return (c >> 3) * (PLANE /
 // Staging of one row's 32 channels, positions i0 - 4 + j for j < XW (zero outside [0, L)), into
 // planes, in two phases so that a pipelined caller keeps the global loads in flight while it does
 // other work: c5_act_load issues every global load of the thread into registers, c5_act_store
-// writes them to the planes.  When L is not a multiple of 8 the 16-byte loads do not apply:
-// c5_act_load does nothing and c5_act_store stages word by word.  Called by NT threads.
+// writes them to the planes.  A warp takes pieces of eight positions, four neighbouring ones (lane >> 3)
+// of eight channels (lane & 7): 64 bytes of a row at a time, since a load costs the L1 a cycle for every
+// line that its lanes touch (one channel per lane: 32 lines).  When L is not a multiple of 8 the 16-byte
+// loads do not apply: c5_act_load does nothing and c5_act_store stages word by word.  Called by NT threads.
 template <int TPC, int NT> struct C5Act {
-    static constexpr int NITEM = CH * (C5<TPC>::XW / 8 + 1);   // (channel, 8-position block) pieces
-    static constexpr int PER = (NITEM + NT - 1) / NT;
+    static constexpr int NV = C5<TPC>::XW / 8 + 1;             // pieces of a row
+    static constexpr int ROUNDS = CH / 8 * ((NV + 3) / 4);     // warp rounds: channel group fastest
+    static constexpr int PER = (ROUNDS + NT / 32 - 1) / (NT / 32);
 };
 
 template <int TPC, int NT>
 __device__ __forceinline__ void c5_act_load(const unsigned short* __restrict__ rows, int L, int i0,
                                             uint4 (&q)[C5Act<TPC, NT>::PER])
 {
-    constexpr int NITEM = C5Act<TPC, NT>::NITEM, PER = C5Act<TPC, NT>::PER, THREADS = NT;
     if ((L & 7) != 0) return;
 #pragma unroll
-    for (int u = 0; u < PER; ++u) {
-        const int e = threadIdx.x + u * THREADS;
-        const int c = e & (CH - 1), v = e / CH;
+    for (int u = 0; u < C5Act<TPC, NT>::PER; ++u) {
+        const int e = (threadIdx.x >> 5) + u * (NT / 32), lane = threadIdx.x & 31;
+        const int c = 8 * (e & 3) + (lane & 7), v = 4 * (e >> 2) + (lane >> 3);
         const int pos0 = i0 - 8 + 8 * v;   // a multiple of 8 (i0 is): the piece lies inside [0, L) or outside
         q[u] = make_uint4(0u, 0u, 0u, 0u);
-        if (e < NITEM && pos0 >= 0 && pos0 + 8 <= L) q[u] = *reinterpret_cast<const uint4*>(rows + (size_t)c * L + pos0);
+        if (v < C5Act<TPC, NT>::NV && pos0 >= 0 && pos0 + 8 <= L)
+            q[u] = *reinterpret_cast<const uint4*>(rows + (size_t)c * L + pos0);
     }
 }
 
@@ -569,18 +572,17 @@ __device__ __forceinline__ void c5_act_store(const unsigned short* __restrict__ 
 {
     using G = C5<TPC>;
     constexpr int XW = G::XW, THREADS = NT, P = G::PLANE;
-    constexpr int NITEM = C5Act<TPC, NT>::NITEM, PER = C5Act<TPC, NT>::PER;
-    static_assert(NITEM % 32 == 0 && THREADS % 32 == 0, "whole warps per item round (the shuffles)");
+    static_assert(CH == 32, "four channel groups");
     if ((L & 7) == 0) {
-        // lane = channel c; lanes c, c ^ 1 swap halves of their 8 positions, so that the even lane
-        // holds positions 0-3 and the odd lane positions 4-7 of both channels and writes one 32-bit
-        // word (channels c & ~1, c | 1) per position: per store the even lanes fill rows j (16
-        // banks over the four planes) and the odd lanes rows j + 4 (the other 16)
+        // lanes c, c ^ 1 swap halves of their 8 positions, so that the even lane holds positions 0-3 and
+        // the odd lane positions 4-7 of both channels and writes one 32-bit word (channels c & ~1, c | 1)
+        // per position.  Pieces v are 32 banks apart, so lanes of piece v start with position v & 3: the
+        // four pieces, two halves and four channel pairs of a store fill 32 banks.
 #pragma unroll
-        for (int u = 0; u < PER; ++u) {
-            const int e = threadIdx.x + u * THREADS;
-            if (e >= NITEM) break;
-            const int c = e & (CH - 1), v = e / CH, odd = c & 1;
+        for (int u = 0; u < C5Act<TPC, NT>::PER; ++u) {
+            const int e = (threadIdx.x >> 5) + u * (NT / 32), lane = threadIdx.x & 31;
+            if (e >= C5Act<TPC, NT>::ROUNDS) break;
+            const int c = 8 * (e & 3) + (lane & 7), v = 4 * (e >> 2) + (lane >> 3), odd = c & 1, rot = v & 3;
             const uint32_t r0 = __shfl_xor_sync(0xffffffffu, odd ? q[u].x : q[u].z, 1);
             const uint32_t r1 = __shfl_xor_sync(0xffffffffu, odd ? q[u].y : q[u].w, 1);
             const uint32_t m0 = odd ? q[u].z : q[u].x, m1 = odd ? q[u].w : q[u].y;
@@ -588,10 +590,15 @@ __device__ __forceinline__ void c5_act_store(const unsigned short* __restrict__ 
             const uint32_t e1 = odd ? r1 : m1, o1 = odd ? m1 : r1;   // positions 2-3
             const uint32_t w[4] = {__byte_perm(e0, o0, 0x5410), __byte_perm(e0, o0, 0x7632),
                                    __byte_perm(e1, o1, 0x5410), __byte_perm(e1, o1, 0x7632)};
+            uint32_t x[4], y[4];   // y[k] = w[(k + rot) & 3]
+#pragma unroll
+            for (int k = 0; k < 4; ++k) x[k] = rot & 1 ? w[(k + 1) & 3] : w[k];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) y[k] = rot & 2 ? x[(k + 2) & 3] : x[k];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const int j = 8 * v - HALF + 4 * odd + k;
-                if (j >= 0 && j < XW) *reinterpret_cast<uint32_t*>(xs + c5_idx<P>(j, c & ~1)) = w[k];
+                const int j = 8 * v - HALF + 4 * odd + ((k + rot) & 3);
+                if (j >= 0 && j < XW) *reinterpret_cast<uint32_t*>(xs + c5_idx<P>(j, c & ~1)) = y[k];
             }
         }
     } else {
@@ -730,15 +737,24 @@ __global__ void __launch_bounds__(256, 4) wgrad_tc_kernel(const __nv_bfloat16* _
 // MN-major operand whose 8-row M-groups are 16 bytes apart, so M-group k reads channels 8 g + i at
 // position p + k, i.e. tap k (groups 9-15 are padding); B = the gradient's BF16 hi parts (rows
 // 0-31) and lo parts (rows 32-63; their sum keeps ~16 bits of the FP32 gradient), K-major 8 x 8
-// blocks staged from the channel-major rows; N = 64, M = 128, TMEM columns 64 g, 256 in all.  In
+// blocks staged from the channel-major rows; N = 64, M = 128, TMEM columns 64 g, 256 a set.  In
 // the no-swizzle layouts of both majors the descriptor's leading-byte offset steps along K and its
 // stride-byte offset along M or N.  Four 128 x 64 x 16 MMAs per K-step (64 per chunk) read 6 KB of
 // shared memory each: 384 KB per chunk, where 32-column MMAs per tap needed 144 MMAs and 720 KB,
 // which the tensor pipe could not stream while the CTA staged the next chunk.  Chunks of 256
 // positions are double-buffered; 16 warps stage (and run the epilogue), one more issues the MMAs;
-// the n_rows x ceil(L / 256) chunks, row after row, are split into gridDim.x contiguous ranges of
-// equal length (+-1), so a CTA's range may cross from one row into the next: the sum over
-// positions and rows does not care.  One CTA per SM.
+// the CTAs are dealt to the three layers in turn and a layer's n_rows x ceil(L / 256) chunks, row after
+// row, split into contiguous ranges of equal length (+-1) over its CTAs, so a CTA's range may cross
+// from one row into the next: the sum over positions and rows does not care.  One CTA per SM.
+// The accumulators drop low bits at every MMA, an error that grows with the MMAs behind a sum, so a sum
+// is taken over to shared memory after as many chunks as a launch of one layer on all SMs would give it,
+// while the next ones go to the other of two sets of accumulators.
+// At 128 rows x 4608 positions the three layers take 132 us in this one launch (46 chunks a CTA); a
+// launch per layer over all SMs, with one channel per lane in the loads, took 3 x 51.  The MMAs alone
+// would take about 115 us (75 cycles each: A's core matrices start off the 128-byte lines), the staging
+// alone 104, the loads alone 71; without drains it is 126.  Loads one chunk further ahead (+4 us:
+// registers) and M = 64 with tap 8 as a fifth product, for no padding rows (+19 us: as many cycles per
+// MMA), gave nothing.
 // one arrival (release semantics at CTA scope) on the barrier's current phase
 __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 {
@@ -748,15 +764,25 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 constexpr int W5_CHUNK = 256;                    // positions per chunk (16 K-steps)
 constexpr int W5_THREADS = 512;                  // staging (and epilogue) threads
 constexpr int W5_BLOCK = W5_THREADS + 32;        // + one warp that issues the MMAs
-constexpr int W5_ASBO = W5_CHUNK / 8 * 128;      // bytes per 8-row group of A (all its 8-position blocks)
-constexpr int W5_ABUF = 8 * W5_ASBO;             // one A buffer: 8 real row groups (hi 0-3, lo 4-7)
+constexpr int W5_ASBO = W5_CHUNK / 8 * 128;      // bytes per 8-row group of the gradient (all its blocks)
+constexpr int W5_ABUF = 8 * W5_ASBO;             // one gradient buffer: 8 row groups (hi 0-3, lo 4-7)
+constexpr int W5_LAYERS = 3;                     // layers 2-4, one launch
+struct W5Args {
+    const __nv_bfloat16* h[W5_LAYERS];
+    const float* da[W5_LAYERS];
+    float *dW[W5_LAYERS], *db[W5_LAYERS];
+    int L, n_rows, drain;   // chunks between drains of the accumulators
+};
 using W5X = C5<2>;                               // activation tile: 256 + 8 rows, 4 planes
 static_assert(W5X::CT == W5_CHUNK, "activation tile matches the chunk");
-constexpr size_t w5_smem_bytes() { return (size_t)2 * W5_ABUF + 2 * W5X::PART + 64; }
+constexpr int W5_ROWS = 8 * KT;                  // real rows of an accumulator
+constexpr int W5_SUM = 4 * CH * W5_ROWS * 4;     // bytes of the drained sums, [channel group][co][row]
+constexpr size_t w5_smem_bytes() { return (size_t)2 * W5_ABUF + 2 * W5X::PART + 64 + W5_SUM; }
 // dynamic shared memory requested at launch: more than half an SM's, so that one CTA has the SM to
 // itself (its 544 threads need the register file)
-constexpr size_t W5_SMEM_LAUNCH = 120 * 1024;
-constexpr int W5_TMEM_COLS = 4 * 2 * CH;         // D_g of the four channel groups
+constexpr size_t W5_SMEM_LAUNCH = 144 * 1024;
+constexpr int W5_DCOLS = 4 * 2 * CH;             // D_g of the four channel groups
+constexpr int W5_TMEM_COLS = 2 * W5_DCOLS;       // two sets of them
 static_assert(w5_smem_bytes() <= W5_SMEM_LAUNCH, "launch request covers the layout");
 // the padding M-groups (taps 9-15) of the last plane of the second buffer read up to 4336 bytes
 // from that plane's start: still inside the launch allocation
@@ -765,10 +791,16 @@ static_assert((size_t)2 * W5_ABUF + W5X::PART + 3 * W5X::PLANE + (W5_CHUNK - 16)
 // ... and the 9 real taps stay inside their plane (rows < XW)
 static_assert((W5_CHUNK - 16) + 15 + (KT - 1) < W5X::XW, "real taps read staged rows only");
 
-__global__ void __launch_bounds__(W5_BLOCK, 1) wgrad_tc05_kernel(const __nv_bfloat16* __restrict__ h,
-                                                                   const float* __restrict__ da, int L, int n_rows,
-                                                                   float* __restrict__ dW, float* __restrict__ db)
+__global__ void __launch_bounds__(W5_BLOCK, 1) wgrad_tc05_kernel(const __grid_constant__ W5Args args)
 {
+    // CTAs are dealt to the layers in turn
+    const int layer = blockIdx.x % W5_LAYERS, part = blockIdx.x / W5_LAYERS;
+    const int parts = (gridDim.x - layer + W5_LAYERS - 1) / W5_LAYERS;
+    const __nv_bfloat16* __restrict__ h = args.h[layer];
+    const float* __restrict__ da = args.da[layer];
+    float* __restrict__ dW = args.dW[layer];
+    float* __restrict__ db = args.db[layer];
+    const int L = args.L, n_rows = args.n_rows;
     extern __shared__ __align__(128) unsigned char w5_smem[];
     unsigned char* abuf = w5_smem;                                  // [2][8 row groups][W5_ASBO]
     unsigned char* xbuf = w5_smem + 2 * W5_ABUF;                    // [2][W5X::PART]
@@ -777,12 +809,13 @@ __global__ void __launch_bounds__(W5_BLOCK, 1) wgrad_tc05_kernel(const __nv_bflo
     uint64_t* mbar = reinterpret_cast<uint64_t*>(w5_smem + 2 * W5_ABUF + 2 * W5X::PART);   // [2]
     uint64_t* full = mbar + 2;                                                              // [2]
     uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 4);
+    float* sum = reinterpret_cast<float*>(mbar + 8);
     __shared__ float db_s[CH];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int cpr = (L + W5_CHUNK - 1) / W5_CHUNK;                 // chunks per row
     const int64_t total = (int64_t)n_rows * cpr;
-    const int q_begin = (int)((int64_t)blockIdx.x * total / gridDim.x);
-    const int nch = (int)((int64_t)(blockIdx.x + 1) * total / gridDim.x) - q_begin;
+    const int q_begin = (int)(part * total / parts);
+    const int nch = (int)((part + 1) * total / parts) - q_begin;
     if (tid < CH) db_s[tid] = 0.f;
     if (tid == 0) {
         isr::mbar_init(isr::smem_u32(&mbar[0]), 1);
@@ -794,53 +827,52 @@ __global__ void __launch_bounds__(W5_BLOCK, 1) wgrad_tc05_kernel(const __nv_bflo
 
     // stage chunk c into buffer c & 1: da as hi / lo 8 x 8 blocks, the activations as planes; in
     // two phases, all global loads of the chunk (gradient and activations) into registers first,
-    // then the shared stores, so that one round trip to memory per chunk overlaps the MMAs
-    // items (8-position block kb, channel co) with the channel fastest: the eight lanes of a
-    // 16-byte store phase write one 128-byte core matrix (no bank conflicts)
-    constexpr int NITEM = CH * (W5_CHUNK / 8), PER = NITEM / W5_THREADS;
-    float4 q0[PER], q1[PER];
-    uint4 qa[C5Act<2, W5_THREADS>::PER];
-    float dbacc = 0.f;   // bias gradient of channel `lane` (every item of this thread has co = lane)
-    static_assert(W5_THREADS % CH == 0, "item e = tid + u W5_THREADS keeps channel e % 32 = lane");
-    auto load = [&](int c) {
+    // then the shared stores.  A warp's gradient items are four 8-position blocks (lane >> 3) of eight
+    // channels (lane & 7): 128 bytes of a row at a time, and the eight lanes of a 16-byte store phase
+    // write one 128-byte core matrix.
+    constexpr int PER = CH * (W5_CHUNK / 8) / W5_THREADS, KSTEP = W5_THREADS / CH;
+    static_assert(CH == 32 && W5_CHUNK / 8 == KSTEP * PER, "warp = channel group and four blocks");
+    const int co = 8 * (warp & 3) + (lane & 7), kb0 = 4 * ((warp >> 2) & 3) + (lane >> 3);
+    struct Regs {
+        float4 q0[PER], q1[PER];
+        uint4 qa[C5Act<2, W5_THREADS>::PER];
+    };
+    float dbacc = 0.f;   // bias gradient of channel co
+    auto load = [&](int c, Regs& v) {
         const int q = q_begin + c, b = q / cpr, p0 = (q - b * cpr) * W5_CHUNK;
         const int span_end = min(L, p0 + W5_CHUNK);
 #pragma unroll
         for (int u = 0; u < PER; ++u) {
-            const int e = tid + u * W5_THREADS;
-            const int co = e & (CH - 1), kb = e / CH;
-            const int pos = p0 + 8 * kb;
+            const int pos = p0 + 8 * (kb0 + KSTEP * u);
             const float* src = da + ((size_t)b * CH + co) * L + pos;
             if ((L & 3) == 0 && pos + 8 <= span_end) {
-                q0[u] = *reinterpret_cast<const float4*>(src);
-                q1[u] = *reinterpret_cast<const float4*>(src + 4);
+                v.q0[u] = *reinterpret_cast<const float4*>(src);
+                v.q1[u] = *reinterpret_cast<const float4*>(src + 4);
             } else {
                 float t[8];
 #pragma unroll
                 for (int k = 0; k < 8; ++k) t[k] = pos + k < span_end ? src[k] : 0.f;
-                q0[u] = make_float4(t[0], t[1], t[2], t[3]);
-                q1[u] = make_float4(t[4], t[5], t[6], t[7]);
+                v.q0[u] = make_float4(t[0], t[1], t[2], t[3]);
+                v.q1[u] = make_float4(t[4], t[5], t[6], t[7]);
             }
         }
-        c5_act_load<2, W5_THREADS>(reinterpret_cast<const unsigned short*>(h) + (size_t)b * CH * L, L, p0, qa);
+        c5_act_load<2, W5_THREADS>(reinterpret_cast<const unsigned short*>(h) + (size_t)b * CH * L, L, p0, v.qa);
     };
-    auto store = [&](int c) {
+    auto store = [&](int c, const Regs& v) {
         const int q = q_begin + c, b = q / cpr, p0 = (q - b * cpr) * W5_CHUNK;
         unsigned char* a = abuf + (c & 1) * W5_ABUF;
 #pragma unroll
         for (int u = 0; u < PER; ++u) {
-            const int e = tid + u * W5_THREADS;
-            const int co = e & (CH - 1), kb = e / CH;
-            const float t[8] = {q0[u].x, q0[u].y, q0[u].z, q0[u].w, q1[u].x, q1[u].y, q1[u].z, q1[u].w};
+            const float t[8] = {v.q0[u].x, v.q0[u].y, v.q0[u].z, v.q0[u].w, v.q1[u].x, v.q1[u].y, v.q1[u].z, v.q1[u].w};
             uint32_t hi[4], lo[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) isr::split2<true>(t[2 * k], t[2 * k + 1], hi[k], lo[k]);
-            const uint32_t o = (uint32_t)((co >> 3) * W5_ASBO + kb * 128 + (co & 7) * 16);
+            const uint32_t o = (uint32_t)((co >> 3) * W5_ASBO + (kb0 + KSTEP * u) * 128 + (co & 7) * 16);
             *reinterpret_cast<uint4*>(a + o) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
             *reinterpret_cast<uint4*>(a + o + 4 * W5_ASBO) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
             dbacc += ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
         }
-        c5_act_store<2, W5_THREADS>(reinterpret_cast<const unsigned short*>(h) + (size_t)b * CH * L, L, p0, qa,
+        c5_act_store<2, W5_THREADS>(reinterpret_cast<const unsigned short*>(h) + (size_t)b * CH * L, L, p0, v.qa,
                                     reinterpret_cast<unsigned short*>(xbuf + (c & 1) * W5X::PART));
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     };
@@ -851,18 +883,56 @@ __global__ void __launch_bounds__(W5_BLOCK, 1) wgrad_tc05_kernel(const __nv_bflo
     isr::tmem_fence_after_sync();
     const uint32_t tbase = *tslot;
     bool ok = true;
+    // D_g (columns 64 g ..) row 8 t + i (TMEM lane) = tap t, input channel 8 g + i; columns 0-31 the hi and
+    // 32-63 the lo part of output channel o.  Warp w reads lane quarter w % 4 (taps 4 (w % 4) ..) of channel
+    // group g = w / 4; taps 9-15 are padding.  out(o, value) with the sums drained before if there are any.
+    static_assert(W5_THREADS == 512, "sixteen epilogue warps: four lane quarters x four channel groups");
+    const int quarter = warp & 3, g4 = warp >> 2, row = 32 * quarter + lane;
+    float* sum_row = sum + (size_t)g4 * CH * W5_ROWS + row;
+    int seg = 0;   // segments drained
+    auto take = [&](auto out) {
+        if (quarter == 3) return;
+        const bool more = seg > 0;
+        const uint32_t d = isr::tmem_warp_lane_base(tbase) + (uint32_t)(W5_DCOLS * (seg & 1) + 2 * CH * g4);
+        uint32_t rh[32], rl[32];
+        isr::tmem_ld32(d, rh);
+        isr::tmem_ld32(d + CH, rl);
+        isr::tmem_wait_ld32(rh);
+        isr::tmem_wait_ld32(rl);
+        if (row < W5_ROWS) {
+#pragma unroll
+            for (int o = 0; o < CH; ++o) {
+                const float x = __uint_as_float(rh[o]) + __uint_as_float(rl[o]);
+                out(o, more ? sum_row[o * W5_ROWS] + x : x);
+            }
+        }
+    };
+    auto drain = [&]() {
+        isr::tmem_fence_after_sync();
+        take([&](int o, float d) { sum_row[o * W5_ROWS] = d; });
+        isr::tmem_fence_before_sync();
+        ++seg;
+    };
     if (warp < W5_THREADS / 32) {
-        // staging warps: chunk c + 1 goes into buffer (c + 1) & 1 once chunk c - 1's MMAs, which
-        // read that buffer, have completed; each warp then arrives on full[(c + 1) & 1]
-        for (int c = -1; c + 1 < nch; ++c) {
-            load(c + 1);
-            if (c >= 1 && !isr::mbar_wait(isr::smem_u32(&mbar[(c + 1) & 1]), (uint32_t)((c - 1) >> 1) & 1u, 1u << 26)) {
+        // staging warps: chunk c goes into buffer c & 1 once chunk c - 2's MMAs, which read that buffer,
+        // have completed; each warp then arrives on full[c & 1]
+        Regs v;
+        int left = args.drain + 1;
+        for (int c = 0; c < nch; ++c) {
+            if (left-- == 0) {   // chunk c - 2 ended a segment: drain it under the next one's MMAs
+                ok = isr::mbar_wait(isr::smem_u32(&mbar[c & 1]), (uint32_t)((c - 2) >> 1) & 1u, 1u << 26);
+                if (!ok) break;
+                drain();
+                left = args.drain - 1;
+            }
+            load(c, v);
+            if (c >= 2 && !isr::mbar_wait(isr::smem_u32(&mbar[c & 1]), (uint32_t)((c - 2) >> 1) & 1u, 1u << 26)) {
                 ok = false;
                 break;
             }
-            store(c + 1);
+            store(c, v);
             __syncwarp();
-            if (lane == 0) mbar_arrive(isr::smem_u32(&full[(c + 1) & 1]));
+            if (lane == 0) mbar_arrive(isr::smem_u32(&full[c & 1]));
         }
     } else if (lane == 0) {
         // the issuing warp: a tcgen05.mma issue holds its thread until the tensor pipe takes it,
@@ -872,14 +942,21 @@ __global__ void __launch_bounds__(W5_BLOCK, 1) wgrad_tc05_kernel(const __nv_bflo
         // 128 B along K, SBO = W5_ASBO along N (8 rows).  N = 64, M = 128 (M-groups 9-15 unused).
         constexpr uint32_t idesc =
             (isr::tc05_idesc<true>() & ~(0x3Fu << 17)) | ((uint32_t)(2 * CH >> 3) << 17) | (1u << 15);
-        for (int c = 0; c < nch; ++c) {
+        int left = 0;
+        uint32_t set = tbase + W5_DCOLS;
+        for (int c = 0; c < nch; ++c, --left) {
+            const bool anew = left == 0;
+            if (anew) {
+                left = args.drain;
+                set = tbase + (set == tbase ? W5_DCOLS : 0);
+            }
             if (!isr::mbar_wait(isr::smem_u32(&full[c & 1]), (uint32_t)(c >> 1) & 1u, 1u << 26)) {
                 ok = false;
                 break;
             }
             isr::tmem_fence_after_sync();
-            // descriptors built once per chunk; K-step s adds 16 (256 B) to the 16-byte-unit start
-            // field of both (addresses stay below 0x40000 B: the field never carries)
+            // descriptors built once per chunk; K-step s adds two blocks of eight positions to the
+            // 16-byte-unit start fields (addresses stay below 0x40000 B: the field never carries)
             const uint64_t bd0 = isr::tc05_desc(isr::smem_u32(abuf + (c & 1) * W5_ABUF), 128, W5_ASBO);
             const uint32_t xa = isr::smem_u32(xbuf + (c & 1) * W5X::PART);
             uint64_t ad0[4];
@@ -887,38 +964,29 @@ __global__ void __launch_bounds__(W5_BLOCK, 1) wgrad_tc05_kernel(const __nv_bflo
             for (int g = 0; g < 4; ++g) ad0[g] = isr::tc05_desc(xa + g * W5X::PLANE, 128, 16);
 #pragma unroll 1
             for (int s = 0; s < W5_CHUNK / 16; ++s) {
-                const uint32_t acc = (c > 0 || s > 0) ? 1u : 0u;
+                const uint32_t acc = !anew || s > 0 ? 1u : 0u;
 #pragma unroll
                 for (int g = 0; g < 4; ++g)
-                    isr::tc05_mma(tbase + (uint32_t)(2 * CH * g), ad0[g] + 16u * (uint32_t)s, bd0 + 16u * (uint32_t)s,
+                    isr::tc05_mma(set + (uint32_t)(2 * CH * g), ad0[g] + 16u * (uint32_t)s, bd0 + 16u * (uint32_t)s,
                                   idesc, acc);
             }
             isr::tc05_commit(isr::smem_u32(&mbar[c & 1]));
         }
     }
-    if (warp < W5_THREADS / 32) atomicAdd(&db_s[lane], dbacc);
+    if (warp < W5_THREADS / 32) {   // the four lanes of a channel
+        for (int o = 8; o < 32; o <<= 1) dbacc += __shfl_xor_sync(0xffffffffu, dbacc, o);
+        if (lane < 8) atomicAdd(&db_s[co], dbacc);
+    }
     // the last commit covers every MMA of this CTA; a thread whose wait ran out skips it
     if (nch > 0 && ok) ok = isr::mbar_wait(isr::smem_u32(&mbar[(nch - 1) & 1]), (uint32_t)((nch - 1) >> 1) & 1u, 1u << 26);
     isr::tmem_fence_before_sync();
     ok = __syncthreads_and(ok) != 0;
     isr::tmem_fence_after_sync();
-    // epilogue: D_g (columns 64 g ..) row 8 t + i (TMEM lane) = tap t, input channel 8 g + i;
-    // columns 0-31 the hi and 32-63 the lo part of output channel co.  Warp w reads lane quarter
-    // w % 4 (taps 4 (w % 4) ..) of channel group g = w / 4; taps 9-15 are padding.
-    static_assert(W5_THREADS == 512, "sixteen epilogue warps: four lane quarters x four channel groups");
-    const int quarter = warp & 3, g = warp >> 2;
-    if (ok && warp < W5_THREADS / 32 && quarter < 3) {
-        const int t = 4 * quarter + (lane >> 3), ci = 8 * g + (lane & 7);
-        uint32_t rh[32], rl[32];
-        isr::tmem_ld32(isr::tmem_warp_lane_base(tbase) + (uint32_t)(2 * CH * g), rh);
-        isr::tmem_ld32(isr::tmem_warp_lane_base(tbase) + (uint32_t)(2 * CH * g + CH), rl);
-        isr::tmem_wait_ld32(rh);
-        isr::tmem_wait_ld32(rl);
-        if (t < KT) {
-#pragma unroll
-            for (int co = 0; co < CH; ++co)
-                atomicAdd(&dW[((size_t)co * CH + ci) * KT + t], __uint_as_float(rh[co]) + __uint_as_float(rl[co]));
-        }
+    if (ok && warp < W5_THREADS / 32) {
+        while ((seg + 1) * args.drain < nch) drain();   // the segment before the last may end one chunk earlier
+        take([&](int o, float d) {
+            atomicAdd(&dW[((size_t)o * CH + 8 * g4 + (lane & 7)) * KT + (row >> 3)], d);
+        });
     }
     isr::tmem_fence_before_sync();
     __syncthreads();
@@ -2687,9 +2755,17 @@ isr_status backward_t(isr_est* e, int n, const float* fpos, const float* pres)
             a.nx = nxi;
             backward_kernel<<<std::min(e->sms, n * nxi), FB_SLOTS * FI_ST, FB_SMEM, s>>>(a);
             const int chunks = n * ((L + W5_CHUNK - 1) / W5_CHUNK), spans = n * ((L + W1_SPAN - 1) / W1_SPAN);
-            for (int l = 4; l >= 2; --l)
-                wgrad_tc05_kernel<<<std::min(chunks, e->sms), W5_BLOCK, W5_SMEM_LAUNCH, s>>>(
-                    act[l - 1], e->da[4 - l], L, n, e->grad + w_off(l), e->grad + b_off(l));
+            W5Args wa{};
+            for (int i = 0; i < W5_LAYERS; ++i) {
+                wa.h[i] = act[3 - i];
+                wa.da[i] = e->da[i];
+                wa.dW[i] = e->grad + w_off(4 - i);
+                wa.db[i] = e->grad + b_off(4 - i);
+            }
+            wa.L = L;
+            wa.n_rows = n;
+            wa.drain = (chunks + std::max(1, e->sms) - 1) / std::max(1, e->sms);
+            wgrad_tc05_kernel<<<std::min(W5_LAYERS * chunks, std::max(W5_LAYERS, e->sms)), W5_BLOCK, W5_SMEM_LAUNCH, s>>>(wa);
             wgrad1_kernel<T><<<std::min(spans, 2 * std::max(1, e->sms)), 256, 0, s>>>(act[0], e->da[3], L, n,
                                                                                      e->grad + OFF_W1, e->grad + OFF_B1);
             EST_TRY(cudaGetLastError());
