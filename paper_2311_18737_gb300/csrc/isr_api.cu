@@ -393,18 +393,19 @@ isr_status launch_block(isr_plan* p, const uint32_t* echo, const char* tx, int64
     while (done < n) {
         int64_t n_l = std::min<int64_t>(n - done, (int64_t)p->max_chunks * p->ipp_chunk);
         if (pack) n_l = std::min(n_l, p->sign_rows);
-        // at least enough chunks for the FP32 sum length cap, behind those that are pending (never all)
-        int64_t c_min = (n_l + p->ipp_chunk - 1) / p->ipp_chunk;
-        if (p->pending + c_min > p->max_chunks) {
-            if (cap == cudaStreamCaptureStatusNone) {
-                const isr_status st = flush_partials(p);
-                if (st != ISR_OK) return st;
-            } else {   // a replay must not reduce what is pending now once more
-                c_min = p->max_chunks - p->pending;
-                n_l = std::min(n_l, c_min * p->ipp_chunk);
-            }
+        // at least enough chunks for the FP32 sum length cap, behind those that are pending (never all); when
+        // the best split does not fit behind them they are reduced first, rather than leave SMs idle
+        int64_t c_min = (n_l + p->ipp_chunk - 1) / p->ipp_chunk, c_max = p->max_chunks;
+        if (cap != cudaStreamCaptureStatusNone) {   // a replay must not reduce what is pending now once more
+            c_max -= p->pending;
+            c_min = std::min(c_min, c_max);
+            n_l = std::min(n_l, c_min * p->ipp_chunk);
         }
-        int64_t C = isr::pick_chunks(n_l, rg, p->sm_count, c_min, p->max_chunks - p->pending, RN);
+        int64_t C = isr::pick_chunks(n_l, rg, p->sm_count, c_min, c_max, RN);
+        if (cap == cudaStreamCaptureStatusNone && p->pending + C > p->max_chunks) {
+            const isr_status st = flush_partials(p);
+            if (st != ISR_OK) return st;
+        }
         int64_t chunk = (n_l + C - 1) / C;
         C = (n_l + chunk - 1) / chunk;
 
