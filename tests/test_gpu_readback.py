@@ -78,3 +78,32 @@ def test_captured_integration_replayed_between_calls():
             graph.replay()
         out, _ = plan.spectra()
         assert_parity(out.numpy().astype(np.float64), _ref(echo[4:9], tx), what="a replay after the reset")
+
+
+@pytest.mark.parametrize("gates,row", [(5001, 7168), (5001, 1 << 20), (2431, 1 << 20)])
+def test_host_rows_in_blocks_and_gate_slices(gates, row):
+    """Host rows to host spectra: blocks of rows (36 MB of them, or one block of the short rows) and,
+    from 32 MB of spectra, a last launch in gate slices read back one by one (5001 gates: two, the last
+    one ragged; 2431: none).  Against the device-resident call: every bin is a sum of nine powers, in
+    FP32 in any order within 9 x 2^-24 of each other, twice over for two calls."""
+    n, nfft = 9, 2048
+    g = torch.Generator(device="cuda").manual_seed(3)
+    echo = torch.randint(-300, 300, (n, row, 2), generator=g, device="cuda", dtype=torch.int16)
+    code = torch.randint(0, 2, (nfft,), generator=g, device="cuda", dtype=torch.int8) * 2 - 1
+    hosts = [t.cpu().pin_memory() for t in (echo, code)]
+    with isr.Plan(nfft=nfft, n_ranges=gates, echo_stride=row, code_len=nfft, range_start=0, range_step=1,
+                  tx_type=isr.ISR_TX_PM1, stream=torch.cuda.current_stream()) as plan:
+        want = torch.empty((gates, nfft), device="cuda")
+        plan.integrate(echo, code, n)
+        plan.spectra(want, isr.ISR_RESET_AFTER)
+        want = want.cpu()
+        got = torch.empty((gates, nfft)).pin_memory()
+        plan.integrate(*hosts, n)
+        plan.spectra(got)
+        assert torch.allclose(got, want, rtol=2e-6, atol=0)
+        plan.integrate(echo, code, n)      # device rows on top: the slices are no longer the whole
+        plan.spectra(got)
+        assert torch.allclose(got, 2 * want, rtol=4e-6, atol=0)
+        plan.integrate(*hosts, n)          # host rows on top of sums already there
+        plan.spectra(got, isr.ISR_RESET_AFTER)
+        assert torch.allclose(got, 3 * want, rtol=6e-6, atol=0)
