@@ -38,7 +38,7 @@ UNIT = "spectra/s"
 FP32_LANES_PER_SM = 128  # FP32 FMA lanes per Blackwell SM
 # sources that define the fused kernel and its launch (the recorded DRAM traffic is tied to them)
 TRAFFIC_SOURCES = ("isr_fft.cuh", "isr_kernel.cuh", "isr_tc.cuh", "isr_tc05.cuh", "isr_tmem.cuh", "isr_paired.cuh",
-                   "isr_kernels.cuh", "isr_k_16384.cu", "isr_api.cu")
+                   "isr_xt.cuh", "isr_kernels.cuh", "isr_k_16384.cu", "isr_api.cu")
 
 
 def _peaks():
@@ -419,14 +419,15 @@ def run_ours(args):
                                         enumerate(("window_wait_and_barrier", "pass0", "middle_pass", "last_pass"))}
     if world == 1 and rank == 0 and not args.no_cpu_baseline:
         threads = os.cpu_count() or 1
-        v, ng, dt, ref, sel = _cpu_sample(w, args.ref_gates, args.ref_ipps, threads)
+        ref_ipps = min(args.ref_ipps, P)   # the echo on the device has P rows
+        v, ng, dt, ref, sel = _cpu_sample(w, args.ref_gates, ref_ipps, threads)
         line["cpu_baseline"] = {"value": v, "unit": UNIT, "cores": threads, "kind": "oracle",
-                                "sample": f"{ng} gates spread over the workload x the first {args.ref_ipps} IPPs "
+                                "sample": f"{ng} gates spread over the workload x the first {ref_ipps} IPPs "
                                           f"({dt:.1f} s wall)"}
         # the library on the same sample (same echo rows, all gates, then the sampled rows):
         # the largest per-bin relative difference from the FP64 oracle
         import numpy as np
-        plan.integrate(echo[:args.ref_ipps], code_d, args.ref_ipps)
+        plan.integrate(echo[:ref_ipps], code_d, ref_ipps)
         plan.spectra(out, isr.ISR_RESET_AFTER)
         got = out[torch.as_tensor(sel, dtype=torch.long, device=out.device)].double().cpu().numpy()
         line["cpu_baseline"]["max_rel_err_vs_oracle"] = float(np.max(np.abs(got - ref) / ref))
