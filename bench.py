@@ -343,8 +343,8 @@ def run_ours(args):
     timed = info1["kernel_timed"] - info0["kernel_timed"]
     kernel_ms = (info1["kernel_ms"] - info0["kernel_ms"]) / max(1, timed)
     launches_per_step = launches / args.steps
-    # our kernels per step: fused kernel + reduction per launch block, one conversion
-    gpu_launches = int(launches * 2 + args.steps)
+    # our kernels per step: the fused kernel per launch block, one read-back
+    gpu_launches = int(launches + args.steps)
 
     # end to end through the C ABI with host buffers (pinned), copies inside the timing
     e2e = None
