@@ -467,7 +467,7 @@ isr_status launch_block(isr_plan* p, const uint32_t* echo, const char* tx, int64
             void* args[] = {&a};
             CUDA_TRY(cudaLaunchKernel(p->ke.fn_tc[p->precision], dim3((unsigned)rg, (unsigned)C),
                                       dim3((unsigned)p->ke.threads), args, (size_t)p->ke.smem_tc, p->stream));
-        } else if (const int S = gate_slices(p, rg); slice && C == 1 && done + n_l == n && S > 1 && !p->captured && !p->prof &&
+        } else if (const int S = gate_slices(p, rg); slice && C == 1 && done + n_l == n && S > 1 && !p->captured &&
                                                      isr::takes_xt(p->ke, full, p->order)) {
             const int64_t rounds = (rg + p->sm_count - 1) / p->sm_count;
             for (int i = 0, u = 0; i < S; ++i) {
