@@ -666,15 +666,13 @@ isr_status isr_plan_create(isr_plan** out, const isr_plan_desc* desc)
     int64_t mc = d.max_chunks > 0 ? d.max_chunks : std::min<int64_t>(64, std::max<int64_t>(1, kScratchBudget / (RN * 4)));
     p->max_chunks = (int)mc;
     e = cudaMalloc(&p->acc, (size_t)(RN * 8));
-    // chunk partials, packed signs and the status word in one allocation
-    const int64_t part_bytes = mc * RN * 4, sign_row = (int64_t)d.nfft / 32 * 4;
+    const int64_t sign_row = (int64_t)d.nfft / 32 * 4;
     p->sign_rows = p->ke.fn_pack && d.tx_stride > 0 ? std::min<int64_t>(mc * p->ipp_chunk, kSignBytes / sign_row) : 0;
-    const int64_t sign_bytes = (p->sign_rows * sign_row + 15) / 16 * 16;
-    if (e == cudaSuccess) e = cudaMalloc(&p->partial, (size_t)(part_bytes + sign_bytes + 16));
-    if (e == cudaSuccess) {
-        p->signs = p->sign_rows ? reinterpret_cast<uint32_t*>(p->partial + part_bytes / 4) : nullptr;
-        p->status = reinterpret_cast<int*>(p->partial + (part_bytes + sign_bytes) / 4);
-    }
+    // the status word and the packed signs share one allocation; the partials, a multiple of 2 MiB for the
+    // large plans, keep one of their own: 16 bytes more made 4 GB of them take 1.1 instead of 0.2 ms
+    if (e == cudaSuccess) e = cudaMalloc(&p->partial, (size_t)(mc * RN * 4));
+    if (e == cudaSuccess) e = cudaMalloc(&p->status, (size_t)(16 + p->sign_rows * sign_row));
+    if (e == cudaSuccess) p->signs = p->sign_rows ? reinterpret_cast<uint32_t*>(p->status + 4) : nullptr;
     if (e == cudaSuccess) e = status_pool().take(&p->host_status);
 #ifdef ISR_DEBUG
     if (e == cudaSuccess) e = cudaMalloc(&p->phase, 5 * sizeof(unsigned long long));
@@ -1052,6 +1050,7 @@ void isr_destroy(isr_plan* p)
         if (e) cudaEventDestroy(e);
     cudaFree(p->acc);
     cudaFree(p->partial);
+    cudaFree(p->status);
     status_pool().give(p->host_status);
     cudaFree(p->phase);
     cudaFree(p->out_stage);
