@@ -260,7 +260,7 @@ isr_status isr_fp32_peak(int32_t device, int32_t paired, double* tflops, double*
  * or 256).  One thread per CTA issues 4096 MMAs back to back, one CTA per SM; 3 runs on an
  * internal stream, the best of runs 2-3 reported.  Writes *tflops (2 FLOP per multiply-add over
  * all SMs) and *cycles_per_mma (SM clock cycles per MMA, mean over the CTAs).  The learned
- * estimator's convolutions issue N = 32 and N = 64 MMAs, so this is their tensor roofline.
+ * estimator's convolutions issue N = 128 and N = 64 MMAs, so this is their tensor roofline.
  * Blocking; allocates a few bytes of device memory for the duration of the call.  The paper has
  * no counterpart.  Errors: ISR_ERR_INVALID_ARG (NULL output, n not one of the four; checked
  * before any CUDA call), ISR_ERR_CUDA, ISR_ERR_TIMEOUT (an MMA commit did not complete within the
@@ -310,6 +310,8 @@ isr_status isr_est_train_step(isr_est* est, const float* x, int32_t n, const flo
 /* line_bin[n]: position in bins of the full spectrum (band_lo + soft-argmax over the 7 bins
  * around the largest location logit); presence[n]: sigmoid of the presence logit. */
 isr_status isr_est_predict(isr_est* est, const float* x, int32_t n, float* line_bin, float* presence);
+/* The same for any number of rows, more than max_batch in as few launches as the estimator's buffers allow. */
+isr_status isr_est_predict_all(isr_est* est, const float* x, int64_t n, float* line_bin, float* presence);
 void isr_est_destroy(isr_est* est);
 
 /*

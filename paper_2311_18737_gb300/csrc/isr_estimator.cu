@@ -2657,6 +2657,38 @@ HeadArgs head_args(const isr_est* e, int nx, float* pos, float* pres)
     return HeadArgs{e->theta, e->L, nx, e->lo, e->pmax, e->psum, e->z, e->zmax, e->pidx, e->zidx, e->amax, e->pooled, e->u, e->q, pos, pres};
 }
 
+// Inference on the tcgen05 engine keeps no activations, so the buffers of h1 (logits) and h2 (the rest of
+// the head's scratch) hold the head of many more rows than max_batch, and a long prediction takes few
+// launches: 1000 rows x 4608 positions in eight launches of 128 rows left a fifth of the last of three
+// rounds of tiles idle in each and ran the head's small kernel eight times (506 us with the features;
+// 368 us in one launch).  Rows that fit; `a` points into the buffers for n of them.
+int predict_rows(const isr_est* e)
+{
+    const int64_t nx = (e->L + FI_P - 1) / FI_P, bytes = (int64_t)e->max_batch * CH * e->L * 2;
+    const int64_t row = 4 * (3 * nx * CH + 2 * nx + CH + 2 * CH + CH + 1);
+    return (int)std::max<int64_t>(e->max_batch, std::min<int64_t>({bytes / (4 * (int64_t)e->L), (bytes - 16 * 9) / row, 1 << 16}));
+}
+
+void place_head(const isr_est* e, int n, int nx, HeadArgs& a, FiFwdArgs& f)
+{
+    unsigned char* at = static_cast<unsigned char*>(e->act[2]);
+    auto take = [&](int per_row) {
+        void* p = at;
+        at += ((size_t)4 * n * per_row + 15) / 16 * 16;
+        return p;
+    };
+    a.z = f.z = static_cast<float*>(e->act[1]);
+    a.pmax = f.pmax = static_cast<float*>(take(nx * CH));
+    a.psum = f.psum = static_cast<float*>(take(nx * CH));
+    a.pidx = f.pidx = static_cast<int*>(take(nx * CH));
+    a.zmax = f.zmax = static_cast<float*>(take(nx));
+    a.zidx = f.zidx = static_cast<int*>(take(nx));
+    a.amax = static_cast<int*>(take(CH));
+    a.pooled = static_cast<float*>(take(2 * CH));
+    a.u = static_cast<float*>(take(CH));
+    a.q = static_cast<float*>(take(1));
+}
+
 // pos / pres: the prediction outputs (inference), or NULL
 template <class T>
 isr_status forward_t(isr_est* e, const float* x, int n, float* pos = nullptr, float* pres = nullptr)
@@ -2689,8 +2721,10 @@ isr_status forward_t(isr_est* e, const float* x, int n, float* pos = nullptr, fl
             a.pidx = e->pidx;
             a.zidx = e->zidx;
             if (pos) {
+                HeadArgs ha = head_args(e, nxi, pos, pres);
+                if (n > e->max_batch) place_head(e, n, nxi, ha, a);
                 forward_kernel<false><<<std::min(e->sms, tiles), fi_slots<false>() * FI_ST, fi_smem<false>(), s>>>(a);
-                head_mlp_kernel<true><<<n, HM_THREADS, 0, s>>>(head_args(e, nxi, pos, pres));
+                head_mlp_kernel<true><<<n, HM_THREADS, 0, s>>>(ha);
             } else {
                 // the weight gradient of the first layer reads x as stored
                 cast_kernel<T><<<(unsigned)std::min<size_t>((nx + 255) / 256, 4096), 256, 0, s>>>(x, nx, act[0]);
@@ -2997,6 +3031,23 @@ isr_status isr_est_predict(isr_est* e, const float* x, int32_t n, float* line_bi
     Dev guard(e->dev);
     return e->precision != ISR_EST_FP32 ? forward_t<__nv_bfloat16>(e, x, n, line_bin, presence)
                                         : forward_t<float>(e, x, n, line_bin, presence);
+}
+
+isr_status isr_est_predict_all(isr_est* e, const float* x, int64_t n, float* line_bin, float* presence)
+{
+    isr_status st = check_batch(e, x, 1);
+    if (st != ISR_OK) return st;
+    if (n < 1) return fail(ISR_ERR_INVALID_ARG, "n must be >= 1");
+    if (!line_bin || !presence) return fail(ISR_ERR_INVALID_ARG, "outputs must not be NULL");
+    Dev guard(e->dev);
+    const int most = e->conv05 ? predict_rows(e) : e->max_batch;
+    for (int64_t done = 0; done < n && st == ISR_OK; done += most) {
+        const int rows = (int)std::min<int64_t>(most, n - done);
+        const float* xr = x + done * e->L;
+        st = e->precision != ISR_EST_FP32 ? forward_t<__nv_bfloat16>(e, xr, rows, line_bin + done, presence + done)
+                                          : forward_t<float>(e, xr, rows, line_bin + done, presence + done);
+    }
+    return st;
 }
 
 void isr_est_destroy(isr_est* e)

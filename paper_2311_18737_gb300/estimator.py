@@ -96,6 +96,9 @@ class Estimator:
         n = x.shape[0]
         pos = torch.empty(n, dtype=torch.float32, device=self.dev)
         pres = torch.empty(n, dtype=torch.float32, device=self.dev)
+        if n > self.max_batch and x.is_contiguous():
+            isr.isr_est_predict_all(self.h, x, n, pos, pres)
+            return pos, pres
         for b0 in range(0, n, self.max_batch):
             b1 = min(n, b0 + self.max_batch)
             isr.isr_est_predict(self.h, x[b0:b1], b1 - b0, pos[b0:b1], pres[b0:b1])

@@ -63,3 +63,23 @@ def test_infinite_activation_stays_within_its_taps():
     assert np.isfinite(want[0]).all() and np.isfinite(want[1]).all()
     assert np.abs(got[0] - want[0]).max() <= 1e-3 and np.abs(got[1] - want[1]).max() <= 1e-5
     assert np.abs(plain[1] - want[1]).max() > 1e-5      # the infinities do reach the head
+
+
+@pytest.mark.parametrize("precision", [isr.ISR_EST_BF16, isr.ISR_EST_BF16_MMASYNC, isr.ISR_EST_FP32])
+@pytest.mark.parametrize("L,max_batch,n", [(16, 2, 37), (488, 3, 100), (1101, 8, 37), (4608, 5, 77), (1000, 4, 4)])
+def test_many_rows_as_their_batches(precision, L, max_batch, n):
+    """A prediction of more rows than a batch, in one launch or several (77 and 100 rows pass what the
+    buffers of 5 and 3 hold), against the rows batch by batch: bit for bit, since no row reads another's."""
+    dev = torch.device("cuda:0")
+    x = torch.randn((n, L), generator=torch.Generator(device="cuda").manual_seed(L), device=dev)
+    e = est_mod.Estimator(max_batch=max_batch, precision=precision, nfft=8192, band_lo=7, band_len=L)
+    e.set_params(ref.init_params(4).astype(np.float32))
+    want = [torch.empty(n, device=dev) for _ in range(2)]
+    for b in range(0, n, max_batch):
+        m = min(max_batch, n - b)
+        isr.isr_est_predict(e.h, x[b:b + m], m, want[0][b:b + m], want[1][b:b + m])
+    got = [torch.full((n,), -1.0, device=dev) for _ in range(2)]
+    isr.isr_est_predict_all(e.h, x, n, *got)
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    assert all(torch.equal(a, b) for a, b in zip(e.predict(x), want))
+    e.close()
