@@ -218,80 +218,104 @@ __global__ void relayout_kernel(const float* __restrict__ theta, T* __restrict__
 
 // ---------------------------------------------------------------- convolution
 // out[b][co][i] = sum_{ci,k} w[ci][k][co] in[b][ci][i + k - 4]  (+ bias, ReLU) or, for the
-// backward-data use, times the ReLU mask of `mask` (the layer below's activations).
-// CTA: 128 positions of one row; warp = 16 positions, lane = output channel.
-constexpr int CT = 128;
-constexpr size_t conv_smem_bytes(int cin) { return sizeof(float) * (size_t)cin * ((CT + KT - 1) + KT * CH); }
+// backward-data use, times the ReLU mask of `mask` (the layer below's activations).  FP32 storage.
+// CTA: 8 P positions of one row; warp = P positions, lane = output channel.  Bound by FMAs while enough
+// CTAs share an SM: the launch takes the P for which the fullest SM has least to do (conv_positions; 37
+// rows of 1101 positions at P = 16 gave some SMs three CTAs and most two).  The outputs go through
+// shared memory, since a store of one position of 32 channels touches 32 lines.  That launch, P = 16 and
+// direct stores: 29 us forward, 31 backward-data; now 21 and 25.
+constexpr size_t conv_smem_bytes(int p) { return sizeof(float) * (size_t)CH * ((8 * p + KT - 1) + KT * CH); }
 
-template <class TIN, class TW, class TOUT, class TM, int CIN, bool FWD>
-__global__ void __launch_bounds__(256) conv_kernel(const TIN* __restrict__ in, const TW* __restrict__ w,
-                                                   const float* __restrict__ bias, const TM* __restrict__ mask,
-                                                   int L, TOUT* __restrict__ out)
+template <bool FWD, int P>
+__global__ void __launch_bounds__(256) conv_kernel(const float* __restrict__ in, const float* __restrict__ w,
+                                                   const float* __restrict__ bias, const float* __restrict__ mask,
+                                                   int L, float* __restrict__ out)
 {
-    constexpr int XW = CT + KT - 1;
+    constexpr int CT = 8 * P, XW = CT + KT - 1;
+    static_assert(P % 4 == 0 && CH * (CT + 1) <= CH * XW + CH * KT * CH, "16-byte rows; the outputs fit");
     extern __shared__ __align__(16) float conv_smem[];
-    float* xs = conv_smem;                 // [CIN][XW]
-    float* ws = conv_smem + CIN * XW;      // [CIN][KT][CH]
+    float* xs = conv_smem;                // [CH][XW]
+    float* ws = conv_smem + CH * XW;      // [CH][KT][CH]
     const int b = blockIdx.y;
     const int i0 = blockIdx.x * CT;
-    const TIN* inb = in + (size_t)b * CIN * L;
+    const float* inb = in + (size_t)b * CH * L;
     // staging, every load of the thread in flight before its first store (with a few at a time the
     // 54 KB took half of the kernel)
-    constexpr int XPER = (CIN * XW + 255) / 256, WPER = CIN * KT * CH / 4 / 256;
-    static_assert(CIN * KT * CH == WPER * 4 * 256, "whole 16-byte pieces per thread");
+    constexpr int XPER = (CH * XW + 255) / 256, WPER = CH * KT * CH / 4 / 256;
+    static_assert(CH * KT * CH == WPER * 4 * 256, "whole 16-byte pieces per thread");
     float xq[XPER];
 #pragma unroll
     for (int u = 0; u < XPER; ++u) {
         const int e = threadIdx.x + u * 256, ci = e / XW, pos = i0 + e % XW - HALF;
-        xq[u] = (e < CIN * XW && pos >= 0 && pos < L) ? ld<TIN>(inb, (size_t)ci * L + pos) : 0.f;
+        xq[u] = (e < CH * XW && pos >= 0 && pos < L) ? inb[(size_t)ci * L + pos] : 0.f;
     }
-    if constexpr (std::is_same<TW, float>::value) {
-        float4 wq[WPER];
+    float4 wq[WPER];
 #pragma unroll
-        for (int u = 0; u < WPER; ++u) wq[u] = reinterpret_cast<const float4*>(w)[threadIdx.x + u * 256];
+    for (int u = 0; u < WPER; ++u) wq[u] = reinterpret_cast<const float4*>(w)[threadIdx.x + u * 256];
 #pragma unroll
-        for (int u = 0; u < WPER; ++u) reinterpret_cast<float4*>(ws)[threadIdx.x + u * 256] = wq[u];
-    } else {
-        for (int e = threadIdx.x; e < CIN * KT * CH; e += 256) ws[e] = ld<TW>(w, e);
-    }
+    for (int u = 0; u < WPER; ++u) reinterpret_cast<float4*>(ws)[threadIdx.x + u * 256] = wq[u];
 #pragma unroll
     for (int u = 0; u < XPER; ++u) {
         const int e = threadIdx.x + u * 256;
-        if (e < CIN * XW) xs[e] = xq[u];
+        if (e < CH * XW) xs[e] = xq[u];
     }
     __syncthreads();
     const int co = threadIdx.x & 31;
-    const int p0 = (threadIdx.x >> 5) * 16;
-    float acc[16];
+    const int p0 = (threadIdx.x >> 5) * P;
+    float acc[P];
     const float bv = FWD ? bias[co] : 0.f;
 #pragma unroll
-    for (int p = 0; p < 16; ++p) acc[p] = bv;
-    for (int ci = 0; ci < CIN; ++ci) {
-        float xv[16 + KT - 1];   // the same for all lanes: six 16-byte loads (XW and p0 are multiples of 4)
+    for (int p = 0; p < P; ++p) acc[p] = bv;
+    for (int ci = 0; ci < CH; ++ci) {
+        float xv[P + KT - 1];   // the same for all lanes: 16-byte loads (XW and p0 are multiples of 4)
 #pragma unroll
-        for (int j = 0; j < 16 + KT - 1; j += 4)
+        for (int j = 0; j < P + KT - 1; j += 4)
             *reinterpret_cast<float4*>(xv + j) = *reinterpret_cast<const float4*>(xs + ci * XW + p0 + j);
 #pragma unroll
         for (int k = 0; k < KT; ++k) {
             const float wv = ws[(ci * KT + k) * CH + co];
 #pragma unroll
-            for (int p = 0; p < 16; ++p) acc[p] = fmaf(wv, xv[p + k], acc[p]);
+            for (int p = 0; p < P; ++p) acc[p] = fmaf(wv, xv[p + k], acc[p]);
         }
     }
-    TOUT* ob = out + ((size_t)b * CH + co) * L;
+    __syncthreads();
+    float* os = conv_smem;   // [CH][CT + 1]
 #pragma unroll
-    for (int p = 0; p < 16; ++p) {
-        const int i = i0 + p0 + p;
+    for (int p = 0; p < P; ++p) os[co * (CT + 1) + p0 + p] = acc[p];
+    __syncthreads();
+#pragma unroll 8
+    for (int e = threadIdx.x; e < CH * CT; e += 256) {
+        const int c = e / CT, j = e % CT, i = i0 + j;
         if (i < L) {
-            float v = acc[p];
-            if (FWD) {
-                v = fmaxf(v, 0.f);
-            } else if (mask) {
-                v = ld<TM>(mask, ((size_t)b * CH + co) * L + i) > 0.f ? v : 0.f;
-            }
-            ob[i] = cvt<TOUT>(v);
+            const size_t o = ((size_t)b * CH + c) * L + i;
+            float v = os[c * (CT + 1) + j];
+            if (FWD) v = fmaxf(v, 0.f);
+            else v = mask[o] > 0.f ? v : 0.f;
+            out[o] = v;
         }
     }
+}
+
+// Positions per warp: the choice whose fullest SM has least to do, a CTA's staging and stores counted as
+// two positions (P = 16 for many rows).
+inline int conv_positions(int L, int n, int sms)
+{
+    int best = 16;
+    int64_t best_cost = INT64_MAX;
+    for (int p : {16, 12, 8}) {
+        const int64_t ctas = (int64_t)n * ((L + 8 * p - 1) / (8 * p)), cost = (ctas + sms - 1) / sms * (p + 2);
+        if (cost < best_cost) best = p, best_cost = cost;
+    }
+    return best;
+}
+
+template <bool FWD>
+void launch_conv(const float* in, const float* w, const float* bias, const float* mask, int L, int n, int sms, float* out,
+                 cudaStream_t s)
+{
+    const int p = conv_positions(L, n, sms);
+    auto* k = p == 16 ? conv_kernel<FWD, 16> : p == 12 ? conv_kernel<FWD, 12> : conv_kernel<FWD, 8>;
+    k<<<dim3((L + 8 * p - 1) / (8 * p), n), 256, conv_smem_bytes(p), s>>>(in, w, bias, mask, L, out);
 }
 
 // ---------------------------------------------------------------- tensor-core convolution
@@ -1003,6 +1027,8 @@ __global__ void __launch_bounds__(W5_BLOCK, 1) wgrad_tc05_kernel(const __grid_co
 // go out through shared memory so that the atomics of a warp fall on runs of 18 addresses instead of 32
 // sectors.
 constexpr int WG_MAX_SPAN = 1152;
+
+constexpr int CT = 128;   // positions of a tile
 
 inline int wgrad_span(int L, int n, int sms)
 {
@@ -2631,11 +2657,11 @@ struct Dev {
 template <class T>
 isr_status set_smem_attrs()
 {
-    [[maybe_unused]] const int big = (int)conv_smem_bytes(CH);
     if constexpr (!kTensorConv<T>) {
-        EST_TRY(cudaFuncSetAttribute(conv_kernel<T, T, T, T, CH, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-        EST_TRY(cudaFuncSetAttribute(conv_kernel<float, T, float, T, CH, false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+        EST_TRY(cudaFuncSetAttribute(conv_kernel<true, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_smem_bytes(16)));
+        EST_TRY(cudaFuncSetAttribute(conv_kernel<true, 12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_smem_bytes(12)));
+        EST_TRY(cudaFuncSetAttribute(conv_kernel<false, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_smem_bytes(16)));
+        EST_TRY(cudaFuncSetAttribute(conv_kernel<false, 12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_smem_bytes(12)));
     } else {
         EST_TRY(cudaFuncSetAttribute(backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FB_SMEM));
         EST_TRY(cudaFuncSetAttribute(forward_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fi_smem<false>()));
@@ -2739,7 +2765,6 @@ isr_status forward_t(isr_est* e, const float* x, int n, float* pos = nullptr, fl
     }
     cast_kernel<T><<<(unsigned)std::min<size_t>((nx + 255) / 256, 4096), 256, 0, s>>>(x, nx, act[0]);
     const T* wf = static_cast<const T*>(e->wf);
-    dim3 grid((L + CT - 1) / CT, n);
     conv1_kernel<T><<<dim3((L + L1_CT - 1) / L1_CT, n), 256, 0, s>>>(act[0], wf, e->theta + OFF_B1, L, act[1]);
     for (int l = 2; l <= 4; ++l) {
         if constexpr (kTensorConv<T>)
@@ -2747,8 +2772,8 @@ isr_status forward_t(isr_est* e, const float* x, int n, float* pos = nullptr, fl
                 act[l - 1], static_cast<const T*>(e->tf) + (size_t)(l - 2) * CH * CH * KT, e->theta + b_off(l), nullptr, L,
                 act[l]);
         else
-            conv_kernel<T, T, T, T, CH, true><<<grid, 256, conv_smem_bytes(CH), s>>>(
-                act[l - 1], wf + CH * KT + (size_t)(l - 2) * CH * CH * KT, e->theta + b_off(l), nullptr, L, act[l]);
+            launch_conv<true>(act[l - 1], wf + CH * KT + (size_t)(l - 2) * CH * CH * KT, e->theta + b_off(l), nullptr, L, n,
+                              std::max(1, e->sms), act[l], s);
     }
     const int nxh = (L + HD_CT - 1) / HD_CT;
     head_chunk_kernel<T><<<dim3(nxh, n), 256, 0, s>>>(act[4], e->theta, L, nxh, e->z, e->pmax, e->pidx, e->psum,
@@ -2811,7 +2836,6 @@ isr_status backward_t(isr_est* e, int n, const float* fpos, const float* pres)
     const T* wbk = static_cast<const T*>(e->wb);
     float* da = e->da[0];
     float* dn = e->da[1];
-    dim3 gc((L + CT - 1) / CT, n);
     const int fspan = wgrad_span(L, n, std::max(1, e->sms));
     const int span = TC_CT * wgrad_span_chunks(L, n, std::max(1, e->wgrad_slots));
     for (int l = 4; l >= 1; --l) {
@@ -2831,8 +2855,7 @@ isr_status backward_t(isr_est* e, int n, const float* fpos, const float* pres)
                 conv_tc_kernel<false><<<dim3((L + CF_CT - 1) / CF_CT, n), CF_THREADS, tc_smem_bytes(false), s>>>(
                     da, static_cast<const T*>(e->tb) + (size_t)(l - 2) * CH * CH * KT, nullptr, act[l - 1], L, dn);
             else
-                conv_kernel<float, T, float, T, CH, false><<<gc, 256, conv_smem_bytes(CH), s>>>(
-                    da, wbk + (size_t)(l - 2) * CH * CH * KT, nullptr, act[l - 1], L, dn);
+                launch_conv<false>(da, wbk + (size_t)(l - 2) * CH * CH * KT, nullptr, act[l - 1], L, n, std::max(1, e->sms), dn, s);
             std::swap(da, dn);
         }
     }

@@ -274,3 +274,31 @@ def test_bf16_fused_gradients_at_tile_edges(B, L):
         err = np.abs(gd[name] - rd[name]).max() / scale
         assert err <= 1e-3, f"{name}: max error {err:.2e} of the block's largest gradient"
     e.close()
+
+
+@pytest.mark.parametrize("B,L", [(37, 1101), (152, 128), (19, 1000)])
+def test_fp32_batches_as_their_rows(B, L):
+    """FP32 convolutions take 8, 12 or 16 positions per warp, by the batch (here 12, 16 and 16 on 152 SMs, 8
+    for a single row), with ragged last tiles: predictions bit for bit as row by row (the sums' order
+    is the same), the batch gradient the mean of the rows' up to FP32 summation (1e-4 of each block's
+    largest)."""
+    rng = np.random.default_rng(B + L)
+    theta = (ref.init_params(3) + 0.05 * rng.standard_normal(ref.N_PARAMS)).astype(np.float32)
+    arrays = [torch.from_numpy(a).cuda() for a in (rng.standard_normal((B, L)).astype(np.float32),
+                                                   rng.uniform(3, L - 3, B).astype(np.float32),
+                                                   np.resize(np.array([1, 0, 1, 1], dtype=np.float32), B))]
+    e = est_mod.Estimator(max_batch=B, precision=isr.ISR_EST_FP32, nfft=L, band_lo=0, band_len=L)
+    e.set_params(theta)
+    whole = e.predict(arrays[0])
+    _, g = e.grad(*arrays)
+    rows = np.zeros(ref.N_PARAMS)
+    for r in range(B):
+        row = [a[r:r + 1].contiguous() for a in arrays]
+        assert all(torch.equal(a[r:r + 1], b) for a, b in zip(whole, e.predict(row[0])))
+        rows += e.grad(*row)[1].astype(np.float64)
+    e.close()
+    gd, rd = ref.unpack(g.astype(np.float64)), ref.unpack(rows / B)
+    gmax = np.abs(rows / B).max()
+    for name, _ in ref.SHAPES:
+        scale = max(np.abs(rd[name]).max(), 1e-3 * gmax)
+        assert np.abs(gd[name] - rd[name]).max() <= 1e-4 * scale, name
