@@ -24,13 +24,14 @@
 // 256 exchange columns + 64 + 4 x 48 fill the 512 columns).
 //
 // Measured (binary-phase code, M spectra/s; before: the best Stockham order of that size): nfft 16384
-// 31.6 -> 34.0, 8192 66.4 -> 80.0, 4096 147 -> 173, 2048 322 -> 372, 1024 750 -> 842; with a code per IPP
-// 16384 18.2 -> 33.8, 2048 190 -> 366, 1024 383 -> 830; complex int16 codes at 4096 105-120 -> 150.  At
-// 16384 it issues on 77 % of cycles with the FMA pipe at 60 % and shared-memory wavefronts at 28 %
-// (before: 76, 57 and 47 %): one transform fills the register file, so its load phases still run beside
-// little else, while the gates of the smaller sizes fill each other's.  The paired FP32 instructions on
-// (re, im), an mbarrier in place of the barrier at the top of an IPP, and wider TMEM stores (which need
-// copies into consecutive registers) each measured slower.
+// 31.6 -> 34.2, 8192 66.4 -> 78.9, 4096 147 -> 170, 2048 322 -> 370, 1024 750 -> 842; with a code per IPP
+// 16384 18.2 -> 33.9, 2048 190 -> 365, 1024 383 -> 830; complex int16 codes at 4096 105-120 -> 149.  At
+// 16384 it issues on 74 % of cycles with the FMA pipe at 55 % and shared-memory wavefronts at 31 %
+// (before: 76, 57 and 47 %, with 1,853 instead of 1,668 instructions per warp and transform): one
+// transform fills the register file, so its load phases still run beside little else, while the gates of
+// the smaller sizes fill each other's.  The paired FP32 instructions on (re, im), an mbarrier in place of
+// the barrier at the top of an IPP, and wider TMEM stores (which need copies into consecutive registers)
+// each measured slower.
 #pragma once
 
 #include "isr_kernel.cuh"
