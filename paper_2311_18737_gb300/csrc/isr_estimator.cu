@@ -1023,21 +1023,31 @@ __global__ void __launch_bounds__(W5_BLOCK, 1) wgrad_tc05_kernel(const __grid_co
 // CTA: one row b, positions [i0, i0 + span); lane = co, warp = four input channels.  Bound by shared
 // loads and FMAs: the activations are the same for all lanes, so they come 16 bytes at a time (16 loads
 // per 144 FMAs instead of 52).  The span shrinks until the launch has about four CTAs per SM: with one of
-// 1152 positions per row, 37 rows of 1101 left three quarters of the SMs idle (121 -> 32 us).  The sums
+// 1152 positions per row, 37 rows of 1101 left three quarters of the SMs idle (121 -> 32 us, 26-29 with tiles of 96).  The sums
 // go out through shared memory so that the atomics of a warp fall on runs of 18 addresses instead of 32
 // sectors.
 constexpr int WG_MAX_SPAN = 1152;
 
-constexpr int CT = 128;   // positions of a tile
-
-inline int wgrad_span(int L, int n, int sms)
+inline int wgrad_span(int L, int n, int sms, int ct)
 {
     int span = WG_MAX_SPAN;
-    while (span > CT && (int64_t)n * ((L + span - 1) / span) < 4 * (int64_t)sms) span -= CT;
+    while (span > ct && (int64_t)n * ((L + span - 1) / span) < 4 * (int64_t)sms) span -= ct;
     return span;
 }
 
-template <class TH>
+// Positions of a tile, 128 or 96: the one whose fullest SM has least to do, a CTA's staging and atomics
+// counted as 32 positions (37 rows of 1101 positions: 444 CTAs of 96 make three on every SM, 333 of 128
+// three on some and two on most: 26-29 us, 32).
+inline int wgrad_tile(int L, int n, int sms)
+{
+    auto cost = [&](int ct) {
+        const int span = wgrad_span(L, n, sms, ct);
+        return ((int64_t)n * ((L + span - 1) / span) + sms - 1) / sms * (span + 32);
+    };
+    return cost(96) < cost(128) ? 96 : 128;
+}
+
+template <class TH, int CT>
 __global__ void __launch_bounds__(256) wgrad_kernel(const TH* __restrict__ h, const float* __restrict__ da, int L, int span,
                                                     float* __restrict__ dW, float* __restrict__ db)
 {
@@ -2836,7 +2846,7 @@ isr_status backward_t(isr_est* e, int n, const float* fpos, const float* pres)
     const T* wbk = static_cast<const T*>(e->wb);
     float* da = e->da[0];
     float* dn = e->da[1];
-    const int fspan = wgrad_span(L, n, std::max(1, e->sms));
+    const int ftile = wgrad_tile(L, n, std::max(1, e->sms)), fspan = wgrad_span(L, n, std::max(1, e->sms), ftile);
     const int span = TC_CT * wgrad_span_chunks(L, n, std::max(1, e->wgrad_slots));
     for (int l = 4; l >= 1; --l) {
         if (l == 1) {
@@ -2848,8 +2858,8 @@ isr_status backward_t(isr_est* e, int n, const float* fpos, const float* pres)
                 wgrad_tc_kernel<<<dim3((L + span - 1) / span, n), 256, wgrad_tc_smem_bytes(), s>>>(
                     act[l - 1], da, L, span, e->grad + w_off(l), e->grad + b_off(l));
             else
-                wgrad_kernel<T><<<dim3((L + fspan - 1) / fspan, n), 256, 0, s>>>(act[l - 1], da, L, fspan, e->grad + w_off(l),
-                                                                                 e->grad + b_off(l));
+                (ftile == 96 ? wgrad_kernel<T, 96> : wgrad_kernel<T, 128>)<<<dim3((L + fspan - 1) / fspan, n), 256, 0, s>>>(
+                    act[l - 1], da, L, fspan, e->grad + w_off(l), e->grad + b_off(l));
             // gradient into the layer below, masked by its ReLU: da_{l-1} = (W_l^T * da_l) (h_{l-1} > 0)
             if constexpr (kTensorConv<T>)
                 conv_tc_kernel<false><<<dim3((L + CF_CT - 1) / CF_CT, n), CF_THREADS, tc_smem_bytes(false), s>>>(
