@@ -117,8 +117,9 @@ inline KernelEntry kernel_entry(int log2n, int txt)
 // memory and fill the twiddle tables if that has not happened on this device (synchronises `stream` then).
 cudaError_t prepare_entry(const KernelEntry& ke, int log2n, int dev, cudaStream_t stream);
 
-// whether launch_integrate takes the tensor-memory kernel
-inline bool takes_xt(const KernelEntry& ke, bool full, int order) { return ke.fn_xt && (!full || order == 0 || order == 6); }
+// whether launch_integrate takes the tensor-memory kernel: for every code and order that has no kernel of
+// its own, which only the orders 1-5 and 7-9 of full-length binary phase have
+inline bool takes_xt(const KernelEntry& ke, bool full, int order) { return ke.fn_xt && (!full || !ke.fn_order[order]); }
 
 // IPP chunks of a launch over n IPPs and rg gate groups on sm_count SMs, c_min .. c_max of them.  One CTA
 // per SM works through rg x C units of ceil(n / C) IPPs each; a unit costs its IPPs (about 4.3 us each

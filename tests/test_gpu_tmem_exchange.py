@@ -73,3 +73,26 @@ def test_orders_0_and_6_at_full_scale_samples(order):
     # a bin may be small beside the rms bin, whose rounding it shares
     tol = RTOL * np.maximum(ref, ref.mean(axis=1, keepdims=True))
     assert (np.abs(out.numpy().astype(np.float64) - ref) <= tol).all()
+
+
+@pytest.mark.parametrize("kind", ["ci16", "c32"])
+@pytest.mark.parametrize("log2n", [11, 14])
+def test_orders_of_full_length_complex_codes(log2n, kind):
+    """The radix orders tell kernels of binary-phase codes apart; with any other code a plan takes orders
+    1 to 3 as well, through the one kernel there is, and the autotuner times them on the caller's data."""
+    nfft, R, P = 1 << log2n, 5, 3
+    echo, tx = _case(5 * log2n, nfft, R, P, 1, 3, nfft, kind, False)
+    ref = oracle.integrate(echo, tx, nfft=nfft, n_ranges=R, range_start=1, range_step=3)
+    e, t = torch.from_numpy(echo).cuda(), torch.from_numpy(tx).cuda()
+    with isr.Plan(nfft=nfft, n_ranges=R, echo_stride=echo.shape[1], range_start=1, range_step=3,
+                  tx_type=isr.ISR_TX_CI16 if kind == "ci16" else isr.ISR_TX_C32, device=0,
+                  stream=torch.cuda.current_stream()) as plan:
+        for order in (1, 2, 3):
+            isr.isr_plan_set_order(plan.handle, order)
+            plan.integrate(e, t, P)
+            out, _ = plan.spectra(flags=isr.ISR_RESET_AFTER)
+            assert_parity(out.numpy().astype(np.float64), ref, what=f"nfft={nfft} {kind} order {order}")
+        tuned = plan.autotune(e, t, P)
+        assert tuned["order"] in range(4) and len(tuned["ms"]) == 4
+        plan.integrate(e, t, P)
+        assert_parity(plan.spectra()[0].numpy().astype(np.float64), ref, what=f"nfft={nfft} {kind} tuned")
