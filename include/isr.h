@@ -344,7 +344,8 @@ typedef struct {
 } isr_window;
 
 #define ISR_BATCH_GRAPH 1    /* capture launch + reduction in a CUDA graph; runs replay it */
-#define ISR_BATCH_AUTOTUNE 2 /* at creation, time the radix orders of each nfft on these windows */
+#define ISR_BATCH_AUTOTUNE 2 /* at creation, time the radix orders of each nfft on these windows (reads their
+                                echoes and codes then; `out` is written by runs only) */
 
 typedef struct {
     int32_t n_windows;

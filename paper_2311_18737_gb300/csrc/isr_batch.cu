@@ -455,10 +455,12 @@ isr_status isr_batch_create(isr_batch** out, const isr_window* windows, int32_t 
         return bail(fail(e == cudaErrorMemoryAllocation ? ISR_ERR_NO_MEMORY : ISR_ERR_CUDA, "allocation failed: %s",
                          cudaGetErrorString(e)));
     std::vector<RedSeg> segs;
+    int64_t probe_bins = 0;   // of the largest window without chunk partials
     for (int i = 0; i < n_windows; ++i) {
         const bool direct = b->hw[i].n_cy == 1;
-        b->hw[i].a.partial = direct ? windows[i].out : b->partial + part_off[i];
+        b->hw[i].a.partial = direct ? nullptr : b->partial + part_off[i];
         b->hw[i].a.status = b->status;
+        if (direct) probe_bins = std::max(probe_bins, (int64_t)windows[i].n_ranges * windows[i].nfft);
         if (!direct)
             segs.push_back(RedSeg{b->partial + part_off[i], windows[i].out, (int64_t)windows[i].n_ranges * windows[i].nfft,
                                   b->hw[i].n_cy});
@@ -469,8 +471,22 @@ isr_status isr_batch_create(isr_batch** out, const isr_window* windows, int32_t 
     if (e != cudaSuccess) return bail(fail(ISR_ERR_CUDA, "upload failed: %s", cudaGetErrorString(e)));
 
     isr_status st = ISR_OK;
-    if (flags & ISR_BATCH_AUTOTUNE) st = autotune(b);
-    if (st != ISR_OK) return bail(st);
+    if (flags & ISR_BATCH_AUTOTUNE) {
+        // the probes' sums go to scratch, never to the caller's outputs (one for all windows: no one reads it)
+        float* probe = nullptr;
+        if (probe_bins > 0) e = cudaMalloc(&probe, sizeof(float) * probe_bins);
+        if (e != cudaSuccess)
+            return bail(fail(e == cudaErrorMemoryAllocation ? ISR_ERR_NO_MEMORY : ISR_ERR_CUDA, "allocation failed: %s",
+                             cudaGetErrorString(e)));
+        for (auto& bw : b->hw)
+            if (bw.n_cy == 1) bw.a.partial = probe;
+        st = autotune(b);
+        cudaStreamSynchronize(b->cap_stream);   // a failed probe may have left launches behind
+        cudaFree(probe);
+        if (st != ISR_OK) return bail(st);
+    }
+    for (int i = 0; i < n_windows; ++i)
+        if (b->hw[i].n_cy == 1) b->hw[i].a.partial = windows[i].out;
     build_units(b, -1, 0);
     b->n_units = (int64_t)b->hu.size();
     st = upload(b, b->cap_stream);

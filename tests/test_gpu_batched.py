@@ -121,3 +121,34 @@ def test_mixed_code_lengths_and_gate_counts_in_one_launch():
         tol = RTOL * np.maximum(ref, 0.01 * ref.mean(axis=1, keepdims=True))
         assert (np.abs(got - ref) <= tol).all(), (nfft, L, R, P, per)
     isr.isr_batch_destroy(h)
+
+
+def test_creation_leaves_the_outputs_alone():
+    """Autotuning probes the windows at creation; only isr_batch_run writes `out`, of windows of one chunk
+    (10 IPPs) and of several (600)."""
+    rng = np.random.default_rng(23)
+    dev = torch.device("cuda:0")
+    keep, ws = [], []
+    for nfft, R, P in [(2048, 40, 10), (16384, 30, 10), (4096, 9, 600)]:
+        stride = (R + nfft + 3) // 4 * 4
+        e = torch.from_numpy(rng.integers(-500, 500, (P, stride, 2)).astype(np.int16)).to(dev)
+        c = torch.ones(nfft, dtype=torch.int8, device=dev)
+        o = torch.full((R, nfft), -7.0, device=dev)
+        keep.append((e, c, o))
+        x = isr.IsrWindow()
+        x.echo, x.tx_code, x.out = e.data_ptr(), c.data_ptr(), o.data_ptr()
+        x.echo_stride, x.tx_stride, x.nfft, x.code_len = stride, 0, nfft, nfft
+        x.n_ranges, x.range_start, x.range_step, x.n_ipp, x.order, x.reserved = R, 0, 1, P, -1, 0
+        ws.append(x)
+    torch.cuda.synchronize()
+    for flags in (0, isr.ISR_BATCH_GRAPH | isr.ISR_BATCH_AUTOTUNE):
+        h = isr.isr_batch_create(ws, flags, 0, torch.cuda.current_stream())
+        torch.cuda.synchronize()
+        assert all((o == -7.0).all() for _, _, o in keep), flags
+        isr.isr_batch_run(h)
+        isr.isr_batch_wait(h)
+        assert all((o >= 0.0).all() for _, _, o in keep), flags
+        isr.isr_batch_destroy(h)
+        for _, _, o in keep:
+            o.fill_(-7.0)
+        torch.cuda.synchronize()
