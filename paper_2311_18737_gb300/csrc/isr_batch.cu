@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <new>
 #include <queue>
+#include <utility>
 #include <vector>
 
 #include "isr.h"
@@ -139,7 +140,8 @@ struct RedSeg {
 };
 
 // out[i] = sum_c part[c][i], FP32 with Kahan compensation (error ~2 ulp for any chunk count);
-// one window per blockIdx.y.  A window of one chunk needs none: its units write into out.
+// one window per blockIdx.y.  A window of one chunk needs none, its units write into out, unless out
+// shares memory with an input of the run: then it is written here, after every unit has read its input.
 __global__ void batch_reduce_kernel(const RedSeg* __restrict__ segs)
 {
     const RedSeg s = segs[blockIdx.y];
@@ -163,6 +165,32 @@ bool dev_ptr(const void* p)
         return false;
     }
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+}
+
+// Bytes [lo, hi) that the units read, as disjoint ranges in ascending order.
+using Range = std::pair<uintptr_t, uintptr_t>;
+std::vector<Range> input_ranges(const isr_window* windows, int n)
+{
+    std::vector<Range> in, out;
+    for (int i = 0; i < n; ++i) {
+        const isr_window& w = windows[i];
+        const int64_t row = (int64_t)w.range_start + (int64_t)(w.n_ranges - 1) * w.range_step + w.code_len;
+        const uintptr_t e = reinterpret_cast<uintptr_t>(w.echo), c = reinterpret_cast<uintptr_t>(w.tx_code);
+        in.push_back({e, e + 4 * ((w.n_ipp - 1) * w.echo_stride + (row + 3) / 4 * 4)});
+        in.push_back({c, c + (w.n_ipp - 1) * w.tx_stride + w.code_len});
+    }
+    std::sort(in.begin(), in.end());
+    for (const Range& r : in) {
+        if (out.empty() || r.first > out.back().second) out.push_back(r);
+        else out.back().second = std::max(out.back().second, r.second);
+    }
+    return out;
+}
+bool overlaps(const std::vector<Range>& ranges, uintptr_t lo, uintptr_t hi)
+{
+    // the first range that ends behind lo
+    auto it = std::upper_bound(ranges.begin(), ranges.end(), lo, [](uintptr_t v, const Range& r) { return v < r.second; });
+    return it != ranges.end() && it->first < hi;
 }
 
 #define B_TRY(expr)                                                                                     \
@@ -412,6 +440,8 @@ isr_status isr_batch_create(isr_batch** out, const isr_window* windows, int32_t 
     // chunking and scratch layout
     int64_t part_floats = 0;
     std::vector<int64_t> part_off(n_windows);
+    std::vector<char> direct(n_windows);   // whether a window's units write into out
+    const std::vector<Range> inputs = input_ranges(windows, n_windows);
     for (int i = 0; i < n_windows; ++i) {
         const isr_window& w = windows[i];
         int lg = 0;
@@ -437,7 +467,9 @@ isr_status isr_batch_create(isr_batch** out, const isr_window* windows, int32_t 
         bw.a.drop_ipp = -1;
         bw.a.chip_bytes = 1;
         part_off[i] = part_floats;
-        if (bw.n_cy > 1) part_floats += (int64_t)bw.n_cy * w.n_ranges * w.nfft;
+        const uintptr_t out_at = reinterpret_cast<uintptr_t>(w.out);
+        direct[i] = bw.n_cy == 1 && !overlaps(inputs, out_at, out_at + sizeof(float) * w.n_ranges * w.nfft);
+        if (!direct[i]) part_floats += (int64_t)bw.n_cy * w.n_ranges * w.nfft;
         b->hw.push_back(bw);
         b->transforms += (int64_t)w.n_ranges * w.n_ipp;
         b->max_bins = std::max<int64_t>(b->max_bins, (int64_t)w.n_ranges * w.nfft);
@@ -457,11 +489,10 @@ isr_status isr_batch_create(isr_batch** out, const isr_window* windows, int32_t 
     std::vector<RedSeg> segs;
     int64_t probe_bins = 0;   // of the largest window without chunk partials
     for (int i = 0; i < n_windows; ++i) {
-        const bool direct = b->hw[i].n_cy == 1;
-        b->hw[i].a.partial = direct ? nullptr : b->partial + part_off[i];
+        b->hw[i].a.partial = direct[i] ? nullptr : b->partial + part_off[i];
         b->hw[i].a.status = b->status;
-        if (direct) probe_bins = std::max(probe_bins, (int64_t)windows[i].n_ranges * windows[i].nfft);
-        if (!direct)
+        if (direct[i]) probe_bins = std::max(probe_bins, (int64_t)windows[i].n_ranges * windows[i].nfft);
+        if (!direct[i])
             segs.push_back(RedSeg{b->partial + part_off[i], windows[i].out, (int64_t)windows[i].n_ranges * windows[i].nfft,
                                   b->hw[i].n_cy});
     }
@@ -478,15 +509,15 @@ isr_status isr_batch_create(isr_batch** out, const isr_window* windows, int32_t 
         if (e != cudaSuccess)
             return bail(fail(e == cudaErrorMemoryAllocation ? ISR_ERR_NO_MEMORY : ISR_ERR_CUDA, "allocation failed: %s",
                              cudaGetErrorString(e)));
-        for (auto& bw : b->hw)
-            if (bw.n_cy == 1) bw.a.partial = probe;
+        for (int i = 0; i < n_windows; ++i)
+            if (direct[i]) b->hw[i].a.partial = probe;
         st = autotune(b);
         cudaStreamSynchronize(b->cap_stream);   // a failed probe may have left launches behind
         cudaFree(probe);
         if (st != ISR_OK) return bail(st);
     }
     for (int i = 0; i < n_windows; ++i)
-        if (b->hw[i].n_cy == 1) b->hw[i].a.partial = windows[i].out;
+        if (direct[i]) b->hw[i].a.partial = windows[i].out;
     build_units(b, -1, 0);
     b->n_units = (int64_t)b->hu.size();
     st = upload(b, b->cap_stream);

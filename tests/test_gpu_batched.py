@@ -152,3 +152,40 @@ def test_creation_leaves_the_outputs_alone():
         for _, _, o in keep:
             o.fill_(-7.0)
         torch.cuda.synchronize()
+
+
+def test_outputs_that_share_memory_with_an_input():
+    """A run reads every echo and code before it writes an output: a window integrated in place (its output
+    over its own echo), one whose output lies over another's echo, one over its own code, and one that ends
+    where an echo begins, all of one chunk, give the same sums as with outputs of their own."""
+    dev = torch.device("cuda:0")
+    stride, P, base = 70000, 6, 1 << 20
+    shapes = [(2048, 100), (4096, 60), (2048, 77), (8192, 20)]
+
+    def run(shared):
+        rng = np.random.default_rng(31)
+        pool = torch.from_numpy(rng.integers(-2**31, 2**31, base + 4 * stride * P).astype(np.int32)).to(dev)
+        echoes = [pool[base + i * stride * P:][:stride * P] for i in range(4)]
+        ws, outs = [], []
+        for i, (nfft, R) in enumerate(shapes):
+            n = R * nfft
+            code = torch.from_numpy(np.where(rng.random(4 * n) < 0.5, -1, 1).astype(np.int8)).to(dev)
+            o = torch.empty(n, device=dev)
+            if shared:
+                o = (echoes[0][:n], echoes[2][5:5 + n], code.view(torch.int32), pool[base - n:base])[i].view(torch.float32)
+            x = isr.IsrWindow()
+            x.echo, x.tx_code, x.out = echoes[i].data_ptr(), code.data_ptr(), o.data_ptr()
+            x.echo_stride, x.tx_stride, x.nfft, x.code_len = stride, 0, nfft, nfft
+            x.n_ranges, x.range_start, x.range_step, x.n_ipp, x.order, x.reserved = R, 1, 3, P, -1, 0
+            ws.append(x)
+            outs.append((o, code))
+        torch.cuda.synchronize()
+        h = isr.isr_batch_create(ws, 0, 0, torch.cuda.current_stream())
+        isr.isr_batch_run(h)
+        isr.isr_batch_wait(h)
+        got = [o.cpu().numpy() for o, _ in outs]
+        isr.isr_batch_destroy(h)
+        return got
+
+    for i, (a, b) in enumerate(zip(run(True), run(False))):
+        assert np.isfinite(a).all() and np.array_equal(a, b), f"window {i}"
