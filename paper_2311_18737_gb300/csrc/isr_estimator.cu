@@ -1025,8 +1025,14 @@ __global__ void __launch_bounds__(W5_BLOCK, 1) wgrad_tc05_kernel(const __grid_co
 // per 144 FMAs instead of 52).  The span shrinks until the launch has about four CTAs per SM: with one of
 // 1152 positions per row, 37 rows of 1101 left three quarters of the SMs idle (121 -> 32 us, 26-29 with tiles of 96).  The sums
 // go out through shared memory so that the atomics of a warp fall on runs of 18 addresses instead of 32
-// sectors.
+// sectors.  The CTAs add to WG_COPIES copies of the gradient in turn, which wgrad_sum_kernel adds up: in
+// one copy each of the 444 additions rounds at the size of the whole sum, which leaves a layer's gradient a
+// relative RMS error of 3e-7 to 4e-7 (one span per row 1e-7 to 2e-7, the copies 3e-8 to 4e-8; the sums of
+// such a batch formed in these orders).  The whole gradient is within 1.5e-7 of FP64 (one copy 3.3e-7), and
+// the pass no slower (37 rows of 1101: 309 -> 304 us).
 constexpr int WG_MAX_SPAN = 1152;
+constexpr int WG_COPIES = 16;
+constexpr int WG_SIZE = OFF_W5 - OFF_W2;   // floats of a copy: weights and biases of layers 2 to 4
 
 inline int wgrad_span(int L, int n, int sms, int ct)
 {
@@ -1047,10 +1053,14 @@ inline int wgrad_tile(int L, int n, int sms)
     return cost(96) < cost(128) ? 96 : 128;
 }
 
+// dW, db: the layer's gradients in the first copy
 template <class TH, int CT>
 __global__ void __launch_bounds__(256) wgrad_kernel(const TH* __restrict__ h, const float* __restrict__ da, int L, int span,
                                                     float* __restrict__ dW, float* __restrict__ db)
 {
+    const size_t copy = (blockIdx.y * gridDim.x + blockIdx.x) % WG_COPIES;
+    dW += copy * WG_SIZE;
+    db += copy * WG_SIZE;
     constexpr int CPW = CH / 8, HW = CT + KT - 1, RUN = CPW / 2 * KT;
     static_assert(HW % 4 == 0 && WG_MAX_SPAN % CT == 0, "aligned window rows, whole tiles");
     __shared__ __align__(16) float sm[CT * (CH + 1) + CH * HW];
@@ -1109,6 +1119,20 @@ __global__ void __launch_bounds__(256) wgrad_kernel(const TH* __restrict__ h, co
         for (int e = lane; e < CH * RUN; e += 32)
             atomicAdd(&dW[(size_t)(e / RUN) * CH * KT + (warp * CPW + half * (CPW / 2)) * KT + e % RUN], st[e]);
     }
+}
+
+// grad[i] = sum over the copies, in FP64 (under half a million additions)
+__global__ void __launch_bounds__(256) wgrad_sum_kernel(const float* __restrict__ copies, float* __restrict__ grad)
+{
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= WG_SIZE) return;
+    float v[WG_COPIES];
+#pragma unroll
+    for (int c = 0; c < WG_COPIES; ++c) v[c] = copies[(size_t)c * WG_SIZE + i];
+    double s = 0.0;
+#pragma unroll
+    for (int c = 0; c < WG_COPIES; ++c) s += (double)v[c];
+    grad[i] = (float)s;
 }
 
 // Weight gradient of the one-channel first layer:
@@ -2616,6 +2640,7 @@ struct isr_est {
     int nfft = 0, lo = 0, L = 0, max_batch = 0, precision = 0, dev = 0;
     cudaStream_t stream = nullptr;
     float *theta = nullptr, *m = nullptr, *v = nullptr, *grad = nullptr;
+    float* wcopies = nullptr;   // FP32 storage: [WG_COPIES][WG_SIZE] sums of the weight gradients
     int64_t step = 0;
     void* wf = nullptr;       // forward working weights (storage type)
     void* wb = nullptr;       // backward-data working weights
@@ -2803,6 +2828,7 @@ isr_status backward_t(isr_est* e, int n, const float* fpos, const float* pres)
     for (int i = 0; i < 5; ++i) act[i] = static_cast<T*>(e->act[i]);
     EST_TRY(cudaMemsetAsync(e->grad, 0, sizeof(float) * NPARAM, s));
     EST_TRY(cudaMemsetAsync(e->loss, 0, sizeof(float), s));
+    if constexpr (!kTensorConv<T>) EST_TRY(cudaMemsetAsync(e->wcopies, 0, sizeof(float) * WG_COPIES * WG_SIZE, s));
     head_bwd_row_kernel<<<n, 256, 0, s>>>(e->theta, L, n, e->z, e->pooled, e->u, e->q, fpos, pres, e->hscal,
                                           e->dpool, e->grad, e->loss);
     if constexpr (kTensorConv<T>) {
@@ -2859,7 +2885,7 @@ isr_status backward_t(isr_est* e, int n, const float* fpos, const float* pres)
                     act[l - 1], da, L, span, e->grad + w_off(l), e->grad + b_off(l));
             else
                 (ftile == 96 ? wgrad_kernel<T, 96> : wgrad_kernel<T, 128>)<<<dim3((L + fspan - 1) / fspan, n), 256, 0, s>>>(
-                    act[l - 1], da, L, fspan, e->grad + w_off(l), e->grad + b_off(l));
+                    act[l - 1], da, L, fspan, e->wcopies + (w_off(l) - OFF_W2), e->wcopies + (b_off(l) - OFF_W2));
             // gradient into the layer below, masked by its ReLU: da_{l-1} = (W_l^T * da_l) (h_{l-1} > 0)
             if constexpr (kTensorConv<T>)
                 conv_tc_kernel<false><<<dim3((L + CF_CT - 1) / CF_CT, n), CF_THREADS, tc_smem_bytes(false), s>>>(
@@ -2869,6 +2895,7 @@ isr_status backward_t(isr_est* e, int n, const float* fpos, const float* pres)
             std::swap(da, dn);
         }
     }
+    if constexpr (!kTensorConv<T>) wgrad_sum_kernel<<<(WG_SIZE + 255) / 256, 256, 0, s>>>(e->wcopies, e->grad + OFF_W2);
     EST_TRY(cudaGetLastError());
     return ISR_OK;
 }
@@ -2935,6 +2962,7 @@ isr_status isr_est_create(isr_est** out, int32_t nfft, int32_t band_lo, int32_t 
         A(&e->tf, es * 3 * CH * CH * KT);
         A(&e->tb, es * 3 * CH * CH * KT);
     }
+    if (!bf16) A((void**)&e->wcopies, sizeof(float) * WG_COPIES * WG_SIZE);
     A(&e->act[0], es * B * L);
     for (int i = 1; i < 5; ++i) A(&e->act[i], es * B * CH * L);
     A((void**)&e->z, 4 * B * L);
@@ -3088,7 +3116,7 @@ void isr_est_destroy(isr_est* e)
     if (!e) return;
     Dev guard(e->dev);
     cudaStreamSynchronize(e->stream);
-    void* ptrs[] = {e->theta, e->m, e->v, e->grad, e->wf, e->wb, e->tf, e->tb, e->act[0], e->act[1], e->act[2], e->act[3],
+    void* ptrs[] = {e->theta, e->m, e->v, e->grad, e->wcopies, e->wf, e->wb, e->tf, e->tb, e->act[0], e->act[1], e->act[2], e->act[3],
                     e->act[4], e->z, e->pooled, e->u, e->q, e->loss, e->amax, e->da[0], e->da[1], e->da[2], e->da[3],
                     e->pmax, e->pidx, e->psum, e->hscal, e->dpool, e->zmax, e->zidx, e->hbits};
     for (void* p : ptrs) cudaFree(p);
