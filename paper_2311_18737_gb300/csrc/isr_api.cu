@@ -92,8 +92,6 @@ constexpr int64_t kSignBytes = int64_t(16) << 20;      // packed chip signs of o
 constexpr int64_t kHostStageBytes = int64_t(1) << 30;   // per host-input staging buffer
 constexpr int64_t kHostFirstBytes = int64_t(64) << 20;   // first block of a host-input call, at most
 constexpr int64_t kHostSplitBytes = int64_t(32) << 20;   // host-input calls from here on take several blocks
-constexpr int kMaxSlices = 6;                            // gate slices of a host-input call's last launch ...
-constexpr int64_t kSliceBytes = int64_t(16) << 20;       // ... each of at least this many bytes of spectra
 
 int chip_bytes(int tx_type) { return tx_type == ISR_TX_CI16 ? 4 : tx_type == ISR_TX_C32 ? 8 : 1; }
 
@@ -224,11 +222,11 @@ __global__ void reduce_partials_kernel(const float* __restrict__ part, int n_chu
 }
 
 // out[i] = (float)((acc[i] + sum_c part[c][i]) * scale), and the status word to host memory: the whole
-// read-back in one pass over the partials (`chunk` bins apart) that no reduction has taken yet.  Without accumulated sums
-// (ACC false) it stays on the FP32 pipe: the product with scale = sc.h + sc.l as a float pair, one
-// rounding.  V4: out is 16-byte aligned.
+// read-back in one pass over the partials that no reduction has taken yet.  Without accumulated sums (ACC
+// false) it stays on the FP32 pipe: the product with scale = sc.h + sc.l as a float pair, one rounding.
+// V4: out is 16-byte aligned.
 template <bool ACC, bool V4>
-__global__ void spectra_kernel(const float* __restrict__ part, int n_chunks, int64_t chunk, int64_t n, const double* __restrict__ acc,
+__global__ void spectra_kernel(const float* __restrict__ part, int n_chunks, int64_t n, const double* __restrict__ acc,
                                double scale, isr::ff sc, float* __restrict__ out, const int* __restrict__ status,
                                int* __restrict__ host_status)
 {
@@ -236,7 +234,7 @@ __global__ void spectra_kernel(const float* __restrict__ part, int n_chunks, int
     const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4;
     for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i < n; i += stride) {
         float s[4], cp[4], o[4];
-        sum_partials(part + i, n_chunks, chunk, s, cp);
+        sum_partials(part + i, n_chunks, n, s, cp);
         if constexpr (ACC) {
             const double2 a0 = *reinterpret_cast<const double2*>(acc + i), a1 = *reinterpret_cast<const double2*>(acc + i + 2);
             const double d[4] = {a0.x, a0.y, a1.x, a1.y};
@@ -307,12 +305,6 @@ struct isr_plan {
     cudaEvent_t hs_copied[2] = {nullptr, nullptr};
     cudaEvent_t hs_free[2] = {nullptr, nullptr};
     cudaEvent_t hs_t[4] = {nullptr, nullptr, nullptr, nullptr};   // block 0: copy start / end, kernels start / end
-    // Gate slices of the last launch of a host-input call: gates up to slice_end[i] are integrated once
-    // slice_done[i] has passed.  None (n_slices 0) as soon as anything else touches the partials.
-    int n_slices = 0;
-    int slice_end[kMaxSlices] = {};
-    cudaEvent_t slice_done[kMaxSlices] = {};
-    cudaStream_t read_stream = nullptr;
     int64_t hs_growth = 0;    // block growth the last multi-block host-input call measured (0: none yet)
     uint32_t* signs = nullptr;   // packed chip signs of per-IPP binary-phase codes, sign_rows x nfft / 32 words
     int64_t sign_rows = 0;
@@ -372,7 +364,6 @@ int bin_threads(const isr_plan* p, int64_t bins) { return bins / 4 < (int64_t)p-
 isr_status flush_partials(isr_plan* p)
 {
     if (p->pending == 0) return ISR_OK;
-    p->n_slices = 0;
     const int64_t RN = (int64_t)p->d.n_ranges * p->d.nfft;
     const int threads = bin_threads(p, RN);
     const unsigned blocks = bin_blocks(p, RN, threads);
@@ -386,21 +377,9 @@ isr_status flush_partials(isr_plan* p)
     return ISR_OK;
 }
 
-// Gate slices for the last launch of a host-input call, which a read-back to host memory can then copy
-// one by one while the rest still computes (4096 gates x nfft 16384, 100 IPPs: 268 MB, 1.5 of the call's
-// 14.0 ms; 1191 x 8192, 6 IPPs: 370 -> 319 us).  Whole rounds of one gate group per SM, so that no slice ends with idle SMs.
-int gate_slices(const isr_plan* p, int rg)
-{
-    const int64_t rounds = (rg + p->sm_count - 1) / p->sm_count, bytes = (int64_t)p->d.n_ranges * p->d.nfft * 4;
-    return (int)std::min<int64_t>({rounds, bytes / kSliceBytes, kMaxSlices});
-}
-
 // Launch the fused kernel for n rows of device-resident input; its chunk partials are left pending.
-// slice: the last launch in gate slices, if that pays.
-isr_status launch_block(isr_plan* p, const uint32_t* echo, const char* tx, int64_t n, int64_t start, int64_t step,
-                        bool slice = false)
+isr_status launch_block(isr_plan* p, const uint32_t* echo, const char* tx, int64_t n, int64_t start, int64_t step)
 {
-    p->n_slices = 0;
     const int R = p->d.n_ranges;
     const int64_t N = p->d.nfft;
     const int64_t RN = (int64_t)R * N;
@@ -467,18 +446,6 @@ isr_status launch_block(isr_plan* p, const uint32_t* echo, const char* tx, int64
             void* args[] = {&a};
             CUDA_TRY(cudaLaunchKernel(p->ke.fn_tc[p->precision], dim3((unsigned)rg, (unsigned)C),
                                       dim3((unsigned)p->ke.threads), args, (size_t)p->ke.smem_tc, p->stream));
-        } else if (const int S = gate_slices(p, rg); slice && C == 1 && done + n_l == n && S > 1 && !p->captured &&
-                                                     isr::takes_xt(p->ke, full, p->order)) {
-            const int64_t rounds = (rg + p->sm_count - 1) / p->sm_count;
-            for (int i = 0, u = 0; i < S; ++i) {
-                const int end = (int)std::min<int64_t>(rg, rounds * (i + 1) / S * p->sm_count);
-                CUDA_TRY(isr::launch_xt(p->ke, a, rg, u, end, p->sm_count, p->stream));
-                CUDA_TRY(cudaEventRecord(p->slice_done[i], p->stream));
-                p->slice_end[i] = std::min(R, end * p->ke.gates);
-                u = end;
-            }
-            p->n_slices = S;
-            p->launches += S - 1;
         } else {
             CUDA_TRY(isr::launch_integrate(p->ke, a, full, p->order, rg, (int)C, p->sm_count, p->stream));
         }
@@ -524,13 +491,6 @@ isr_status ensure_host_staging(isr_plan* p, int64_t rows)
     }
     for (auto& e : p->hs_t)
         if (!e) CUDA_TRY(cudaEventCreate(&e));
-    for (auto& e : p->slice_done)
-        if (!e) CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    if (!p->read_stream) {   // its read-back kernels go before the next slice's
-        int least = 0, greatest = 0;
-        CUDA_TRY(cudaDeviceGetStreamPriorityRange(&least, &greatest));
-        CUDA_TRY(cudaStreamCreateWithPriority(&p->read_stream, cudaStreamNonBlocking, greatest));
-    }
     if (!p->copy_stream) CUDA_TRY(cudaStreamCreateWithFlags(&p->copy_stream, cudaStreamNonBlocking));
     p->hs_rows = rows;
     return ISR_OK;
@@ -554,9 +514,8 @@ isr_status integrate_host(isr_plan* p, const int16_t* echo, const void* tx, int6
     // while growth <= (kernel time) / (copy time) of equal blocks; the host link differs from box
     // to box, so block 0's copy and kernels are timed, block 1 doubles meanwhile, and once block 1
     // is queued the host waits for block 0's kernels and takes growth = that ratio, within 1..4.
-    // A call under kHostSplitBytes (0.17 ms to copy) that fits one buffer is one block.  (100 IPPs of
-    // 4096 gates, 100 MB: 14.0 -> 12.9 ms together with the slices above; 512 MB of short transforms,
-    // 872 x 3041 of 512 points: 4.87 -> 3.21 ms; 46 MB for 9 gates: 436 -> 361 us.)
+    // A call under kHostSplitBytes (0.17 ms to copy) that fits one buffer is one block.  (512 MB of short
+    // transforms, 872 x 3041 of 512 points: 4.87 -> 3.21 ms; 46 MB for 9 gates: 436 -> 361 us.)
     const bool several = n > rows || (n > 1 && n * row_bytes >= kHostSplitBytes);
     const int64_t first_bytes = std::min<int64_t>(kHostFirstBytes, n * row_bytes / 8);
     int64_t cur = several ? std::max<int64_t>(1, std::min<int64_t>(rows, first_bytes / row_bytes)) : rows;
@@ -584,7 +543,7 @@ isr_status integrate_host(isr_plan* p, const int16_t* echo, const void* tx, int6
         if (time0) CUDA_TRY(cudaEventRecord(p->hs_t[1], p->copy_stream));
         CUDA_TRY(cudaStreamWaitEvent(p->stream, p->hs_copied[b], 0));
         if (time0) CUDA_TRY(cudaEventRecord(p->hs_t[2], p->stream));
-        st = launch_block(p, p->hs_echo[b], txblk, nb, start, step, done + nb == n);
+        st = launch_block(p, p->hs_echo[b], txblk, nb, start, step);
         if (st != ISR_OK) return st;
         if (time0) CUDA_TRY(cudaEventRecord(p->hs_t[3], p->stream));
         CUDA_TRY(cudaEventRecord(p->hs_free[b], p->stream));
@@ -749,23 +708,9 @@ isr_status isr_spectra(isr_plan* p, float* out, int32_t flags, int64_t* n_ipp_ou
         const bool v4 = reinterpret_cast<uintptr_t>(dst) % 16 == 0, from_acc = !p->acc_zero || p->captured;
         auto* k = from_acc ? (v4 ? spectra_kernel<true, true> : spectra_kernel<true, false>)
                            : (v4 ? spectra_kernel<false, true> : spectra_kernel<false, false>);
-        if (!dev_out && p->n_slices > 0) {
-            int64_t at = 0;
-            for (int i = 0; i < p->n_slices; ++i) {
-                const int64_t bins = (int64_t)p->slice_end[i] * p->d.nfft - at;
-                CUDA_TRY(cudaStreamWaitEvent(p->read_stream, p->slice_done[i], 0));
-                k<<<bin_blocks(p, bins, threads), threads, 0, p->read_stream>>>(p->partial + at, p->pending, RN, bins, p->acc + at,
-                                                                               scale, sc, dst + at, p->status, p->host_status);
-                CUDA_TRY(cudaGetLastError());
-                CUDA_TRY(cudaMemcpyAsync(out + at, dst + at, (size_t)(bins * 4), cudaMemcpyDeviceToHost, p->read_stream));
-                at += bins;
-            }
-            CUDA_TRY(cudaStreamSynchronize(p->read_stream));
-        } else {
-            k<<<blocks, threads, 0, p->stream>>>(p->partial, p->pending, RN, RN, p->acc, scale, sc, dst, p->status, p->host_status);
-            CUDA_TRY(cudaGetLastError());
-            if (!dev_out) CUDA_TRY(cudaMemcpyAsync(out, dst, (size_t)(RN * 4), cudaMemcpyDeviceToHost, p->stream));
-        }
+        k<<<blocks, threads, 0, p->stream>>>(p->partial, p->pending, RN, p->acc, scale, sc, dst, p->status, p->host_status);
+        CUDA_TRY(cudaGetLastError());
+        if (!dev_out) CUDA_TRY(cudaMemcpyAsync(out, dst, (size_t)(RN * 4), cudaMemcpyDeviceToHost, p->stream));
     } else {
         CUDA_TRY(cudaMemcpyAsync(p->host_status, p->status, sizeof(int), cudaMemcpyDeviceToHost, p->stream));
     }
@@ -775,7 +720,6 @@ isr_status isr_spectra(isr_plan* p, float* out, int32_t flags, int64_t* n_ipp_ou
     if (n_ipp_out) *n_ipp_out = p->n_ipp_total;
     if (flags & ISR_RESET_AFTER) {
         p->pending = 0;
-        p->n_slices = 0;
         if (!p->acc_zero || p->captured) CUDA_TRY(cudaMemsetAsync(p->acc, 0, (size_t)(RN * 8), p->stream));
         p->acc_zero = true;
         p->n_ipp_total = 0;
@@ -1025,10 +969,6 @@ void isr_destroy(isr_plan* p)
     if (!p) return;
     DeviceGuard guard(p->dev);
     if (p->stream || p->acc) cudaStreamSynchronize(p->stream);
-    if (p->read_stream) {
-        cudaStreamSynchronize(p->read_stream);
-        cudaStreamDestroy(p->read_stream);
-    }
     if (p->copy_stream) {
         cudaStreamSynchronize(p->copy_stream);
         cudaStreamDestroy(p->copy_stream);
@@ -1045,8 +985,6 @@ void isr_destroy(isr_plan* p)
         if (p->hs_free[b]) cudaEventDestroy(p->hs_free[b]);
     }
     for (auto e : p->hs_t)
-        if (e) cudaEventDestroy(e);
-    for (auto e : p->slice_done)
         if (e) cudaEventDestroy(e);
     cudaFree(p->acc);
     cudaFree(p->partial);

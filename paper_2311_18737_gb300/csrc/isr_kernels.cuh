@@ -153,20 +153,16 @@ inline int64_t pick_chunks(int64_t n, int64_t rg, int64_t sm_count, int64_t c_mi
     return best;
 }
 
-// The tensor-memory kernel over units [unit0, unit1) of rg gate groups x IPP chunks of `a`.
-inline cudaError_t launch_xt(const KernelEntry& ke, const KArgs& a, int rg, int unit0, int unit1, int sm_count, cudaStream_t stream)
-{
-    XtPlanSrc src{a, rg, unit0, unit1};
-    void* args[] = {&src};
-    const int grid = std::min(unit1 - unit0, sm_count);   // persistent: one CTA per SM
-    return cudaLaunchKernel(ke.fn_xt, dim3((unsigned)grid), dim3(kThreads), args, (size_t)ke.smem_xt, stream);
-}
-
 // One launch over rg gate groups x n_chunks IPP chunks of `a` with radix order `order`.
 inline cudaError_t launch_integrate(const KernelEntry& ke, KArgs a, bool full, int order, int rg, int n_chunks,
                                     int sm_count, cudaStream_t stream)
 {
-    if (takes_xt(ke, full, order)) return launch_xt(ke, a, rg, 0, rg * n_chunks, sm_count, stream);
+    if (takes_xt(ke, full, order)) {
+        XtPlanSrc src{a, rg, rg * n_chunks};
+        void* args[] = {&src};
+        const int grid = std::min(src.n_units, sm_count);   // persistent: one CTA per SM
+        return cudaLaunchKernel(ke.fn_xt, dim3((unsigned)grid), dim3(kThreads), args, (size_t)ke.smem_xt, stream);
+    }
     void* args[] = {&a};
     return cudaLaunchKernel(full ? ke.fn_order[order] : ke.fn, dim3((unsigned)rg, (unsigned)n_chunks),
                             dim3((unsigned)ke.threads), args, (size_t)(full ? ke.smem_order[order] : ke.smem), stream);

@@ -281,8 +281,8 @@ __device__ __forceinline__ void xt_fill(XtUnit& x, const KArgs& a, int gx, int c
 // chunk) grid, gate groups first.
 struct XtPlanSrc {
     KArgs a;
-    int rg, unit0, n_units;   // units unit0 .. n_units - 1 of rg gate groups x IPP chunks
-    __device__ __forceinline__ int first() const { return unit0 + blockIdx.x; }
+    int rg, n_units;   // n_units = rg gate groups x IPP chunks
+    __device__ __forceinline__ int first() const { return blockIdx.x; }
     __device__ __forceinline__ int next(int un) const { return un + gridDim.x; }
     __device__ __forceinline__ bool valid(int un) const { return un < n_units; }
     template <int LOG2N>

@@ -107,3 +107,27 @@ def test_host_rows_in_blocks_and_gate_slices(gates, row):
         plan.integrate(*hosts, n)          # host rows on top of sums already there
         plan.spectra(got, isr.ISR_RESET_AFTER)
         assert torch.allclose(got, 3 * want, rtol=6e-6, atol=0)
+
+
+@pytest.mark.parametrize("gates", [5001, 700])
+def test_read_back_to_the_host_keeps_the_stream_order(gates):
+    """Work that the caller queues on the plan's stream between isr_integrate (host rows) and isr_spectra
+    comes before the copy into the host buffer, here an upload from that very buffer behind a long delay."""
+    n, nfft = 9, 2048
+    g = torch.Generator(device="cuda").manual_seed(4)
+    echo = torch.randint(-300, 300, (n, 7168, 2), generator=g, device="cuda", dtype=torch.int16)
+    code = torch.randint(0, 2, (nfft,), generator=g, device="cuda", dtype=torch.int8) * 2 - 1
+    hosts = [t.cpu().pin_memory() for t in (echo, code)]
+    buf = torch.full((gates, nfft), -5.0).pin_memory()
+    before = torch.zeros((gates, nfft), device="cuda")
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with isr.Plan(nfft=nfft, n_ranges=gates, echo_stride=7168, code_len=nfft, range_start=0, range_step=1,
+                  tx_type=isr.ISR_TX_PM1, stream=side) as plan:
+        plan.integrate(*hosts, n)
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(40_000_000)      # about 20 ms
+            before.copy_(buf, non_blocking=True)
+        plan.spectra(buf)
+        assert (before == -5.0).all()
+        assert (buf > 0.0).all()
