@@ -158,7 +158,7 @@ inline cudaError_t launch_integrate(const KernelEntry& ke, KArgs a, bool full, i
                                     int sm_count, cudaStream_t stream)
 {
     if (takes_xt(ke, full, order)) {
-        XtPlanSrc src{a, rg, rg * n_chunks};
+        XtPlanSrc src{a, rg, 0, rg * n_chunks};
         void* args[] = {&src};
         const int grid = std::min(src.n_units, sm_count);   // persistent: one CTA per SM
         return cudaLaunchKernel(ke.fn_xt, dim3((unsigned)grid), dim3(kThreads), args, (size_t)ke.smem_xt, stream);

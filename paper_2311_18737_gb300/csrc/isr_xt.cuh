@@ -281,8 +281,10 @@ __device__ __forceinline__ void xt_fill(XtUnit& x, const KArgs& a, int gx, int c
 // chunk) grid, gate groups first.
 struct XtPlanSrc {
     KArgs a;
-    int rg, n_units;   // n_units = rg gate groups x IPP chunks
-    __device__ __forceinline__ int first() const { return blockIdx.x; }
+    // units unit0 .. n_units - 1 of rg gate groups x IPP chunks; unit0 is 0, but without it the kernel is
+    // compiled to one that takes 0.3 % longer (nfft 16384: 291.5 -> 292.5 ms for 1000 gates x 10,000 IPPs)
+    int rg, unit0, n_units;
+    __device__ __forceinline__ int first() const { return unit0 + blockIdx.x; }
     __device__ __forceinline__ int next(int un) const { return un + gridDim.x; }
     __device__ __forceinline__ bool valid(int un) const { return un < n_units; }
     template <int LOG2N>
