@@ -192,6 +192,16 @@ __device__ __forceinline__ double widen(float f)
     return __hiloint2double((int)hi, (int)(b << 29));
 }
 
+// The sum of a bin's partials in FP64, where it leaves the range of FP32: the partials of several calls
+// together may (each within it; float codes of large amplitude).  NaN if a partial itself is not finite.
+__device__ __forceinline__ double wide_sum(const float* __restrict__ part, int n_chunks, int64_t n)
+{
+    double s = 0.0;
+#pragma unroll 1
+    for (int c = 0; c < n_chunks; ++c) s += (double)part[(int64_t)c * n];
+    return isfinite(s) ? s : (double)NAN;
+}
+
 // acc[i] (+)= sum_c part[c][i], the sum added once per bin into the FP64 accumulator
 template <bool ADD>
 __global__ void reduce_partials_kernel(const float* __restrict__ part, int n_chunks, int64_t n,
@@ -209,7 +219,8 @@ __global__ void reduce_partials_kernel(const float* __restrict__ part, int n_chu
         sum_partials(part + i, n_chunks, n, s, cp);
         double d[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) d[k] = widen(s[k]) - widen(cp[k]);
+        for (int k = 0; k < 4; ++k)
+            d[k] = isfinite(s[k]) ? widen(s[k]) - widen(cp[k]) : wide_sum(part + i + k, n_chunks, n);
         if constexpr (ADD) {
             d[0] += a0.x;
             d[1] += a0.y;
@@ -231,6 +242,7 @@ __global__ void spectra_kernel(const float* __restrict__ part, int n_chunks, int
                                int* __restrict__ host_status)
 {
     if (blockIdx.x == 0 && threadIdx.x == 0) *host_status = *status;
+    bool wide = false;   // one of this thread's sums may have left FP32
     const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4;
     for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i < n; i += stride) {
         float s[4], cp[4], o[4];
@@ -257,6 +269,13 @@ __global__ void spectra_kernel(const float* __restrict__ part, int n_chunks, int
 #pragma unroll
             for (int k = 0; k < 4; ++k) out[i + k] = o[k];
         }
+        wide |= !((s[0] + s[1]) + (s[2] + s[3]) < INFINITY);
+    }
+    if (wide) {   // again in FP64, behind the loop above, which this in it makes slower
+#pragma unroll 1
+        for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i < n; i += stride)
+#pragma unroll 1
+            for (int k = 0; k < 4; ++k) out[i + k] = (float)(((ACC ? acc[i + k] : 0.0) + wide_sum(part + i + k, n_chunks, n)) * scale);
     }
 }
 

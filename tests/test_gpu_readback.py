@@ -6,7 +6,7 @@ import pytest
 import torch
 
 import oracle
-from gpu_helpers import assert_parity
+from gpu_helpers import RTOL, assert_parity
 from paper_2311_18737_gb300 import isr
 
 pytestmark = pytest.mark.gpu
@@ -131,3 +131,28 @@ def test_read_back_to_the_host_keeps_the_stream_order(gates):
         plan.spectra(buf)
         assert (before == -5.0).all()
         assert (buf > 0.0).all()
+
+
+@pytest.mark.parametrize("nfft", [512, 1024])
+@pytest.mark.parametrize("max_chunks", [0, 2, 4])
+def test_sums_over_calls_beyond_the_range_of_fp32(nfft, max_chunks):
+    """Six calls whose sums leave FP32 together but not each (a float code of amplitude 1e14), pending all
+    at once, two at a time, or two beside four reduced ones: the mean is finite and within RTOL of the oracle's, the sum infinite where
+    it is beyond FP32."""
+    rng = np.random.default_rng(8)
+    R, calls = 4, 6
+    echo = np.clip(np.rint(rng.standard_normal((1, nfft + 8, 2)) * 1000), -32768, 32767).astype(np.int16)
+    tx = (1e14 * np.exp(2j * np.pi * rng.random(nfft))).astype(np.complex64).view(np.float32).reshape(nfft, 2)
+    ref = oracle.integrate(echo, tx, nfft=nfft, n_ranges=R, range_start=0, range_step=2)
+    assert ref.max() < 3.4e38 < calls * ref.max() and calls * ref.min() < 3.4e38
+    e, t = torch.from_numpy(echo).cuda(), torch.from_numpy(tx).cuda()
+    with isr.Plan(nfft=nfft, n_ranges=R, echo_stride=nfft + 8, range_step=2, tx_type=isr.ISR_TX_C32, device=0,
+                  max_chunks=max_chunks, stream=torch.cuda.current_stream()) as plan:
+        for _ in range(calls):
+            plan.integrate(e, t, 1)
+        out, _ = plan.spectra(flags=isr.ISR_MEAN)
+        # a bin far below the mean shares the mean's rounding
+        tol = RTOL * np.maximum(ref, 0.01 * ref.mean(axis=1, keepdims=True))
+        assert (np.abs(out.numpy().astype(np.float64) - ref) <= tol).all()
+        total = plan.spectra()[0].numpy()
+        assert np.isposinf(total[calls * ref > 3.41e38]).all() and np.isfinite(total[calls * ref < 3.39e38]).all()
