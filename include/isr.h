@@ -213,13 +213,13 @@ isr_status isr_plan_test_drop_window(isr_plan* plan, int32_t ipp);
  * reduction each).  The first block's reduction writes `out`; each later block adds its
  * sum (formed in double) to `out` with one FP32 rounding, so a call of B blocks carries at
  * most B extra roundings of 2^-24 relative per bin (B = 1 whenever n_ipp <= C * 256).
- * The first call on a device looks up the array's device address (once per device, with
- * that device current), so make that first call before any stream capture.  Every call
- * shares the array and its contents stay from the last call: calls that overlap on the
- * GPU (other host threads or other streams) race and corrupt each other's results.  The
- * call is synchronous: it enqueues its work on desc->stream and then waits for that
- * stream (so it can report ISR_ERR_TIMEOUT from a bounded wait that ran out); a stream
- * that is being captured does not allow that wait, so no call belongs inside a capture.
+ * The first call on a device loads the array there, so make that first call before any
+ * stream capture.  Every call shares the array and its contents stay from the last call:
+ * calls that overlap on the GPU (other host threads or other streams) race and corrupt each
+ * other's results.  The call is synchronous: it enqueues its work on desc->stream and then
+ * waits for that stream (so it can report ISR_ERR_TIMEOUT from a bounded wait that ran out);
+ * a stream that is being captured does not allow that wait, so no call belongs inside a
+ * capture.
  */
 #define ISR_STATIC_SCRATCH_FLOATS (4 * 1024 * 1024)
 isr_status isr_integrate_static(const isr_plan_desc* desc, const int16_t* echo, const void* tx_code,

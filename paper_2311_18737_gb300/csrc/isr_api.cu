@@ -10,11 +10,15 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdarg>
-#include <mutex>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "isr.h"
@@ -36,7 +40,26 @@ isr_status fail(isr_status st, const char* fmt, ...)
 }
 void clear_error() { g_err[0] = 0; }
 
-cudaError_t prepare_entry(const KernelEntry& ke, int log2n, int dev, cudaStream_t stream)
+// What this library keeps in a CUDA context beside its handles, recorded in the context itself: one that was
+// made anew (cudaDeviceReset, by this or any other copy of the CUDA runtime) has the zeros of a freshly
+// loaded module here, whatever the process remembers of the one before.
+struct ContextRecord {
+    unsigned long long pool;   // id of the pinned page of status words, 0 = none
+    uint32_t tables;           // bit log2n: the twiddle tables of that transform length are filled
+    int static_status;         // status word of isr_integrate_static
+};
+static __device__ ContextRecord g_context;
+
+static std::mutex g_context_mu;   // held from the look at a record until what it lacks is there
+
+static cudaError_t read_record(ContextRecord& r, cudaStream_t stream)
+{
+    cudaError_t e = cudaMemcpyFromSymbolAsync(&r, g_context, sizeof(r), 0, cudaMemcpyDeviceToHost, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    return e;
+}
+
+static cudaError_t set_attributes(const KernelEntry& ke)
 {
     cudaError_t e = cudaSuccess;
     auto set = [&](const void* fn, int smem) {
@@ -46,16 +69,31 @@ cudaError_t prepare_entry(const KernelEntry& ke, int log2n, int dev, cudaStream_
     for (int o = 0; o < kNumOrders; ++o) set(ke.fn_order[o], ke.smem_order[o]);
     set(ke.fn_xt, ke.smem_xt);
     set(ke.fn_xt_batch, ke.smem_xt);
-    if (e != cudaSuccess || !ke.fn_tables) return e;
-    // the tables are the same for every user: filled under the lock, complete before it is released
-    static std::mutex mu;
-    static uint32_t filled[64] = {};   // bit log2n per device
-    std::lock_guard<std::mutex> lock(mu);
-    if (dev >= 0 && dev < 64 && (filled[dev] >> log2n & 1u)) return cudaSuccess;
-    e = cudaLaunchKernel(ke.fn_tables, dim3(32), dim3(128), nullptr, 0, stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-    if (e == cudaSuccess && dev >= 0 && dev < 64) filled[dev] |= 1u << log2n;
     return e;
+}
+
+// Fill the tables if record r (of the current context, read under the lock) says they are not.
+static cudaError_t fill_tables(const KernelEntry& ke, int log2n, ContextRecord& r, cudaStream_t stream)
+{
+    if (!ke.fn_tables || (r.tables >> log2n & 1u)) return cudaSuccess;
+    cudaError_t e = cudaLaunchKernel(ke.fn_tables, dim3(32), dim3(128), nullptr, 0, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    r.tables |= 1u << log2n;
+    if (e == cudaSuccess)
+        e = cudaMemcpyToSymbolAsync(g_context, &r.tables, sizeof(r.tables), offsetof(ContextRecord, tables),
+                                    cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    return e;
+}
+
+cudaError_t prepare_entry(const KernelEntry& ke, int log2n, cudaStream_t stream)
+{
+    cudaError_t e = set_attributes(ke);
+    if (e != cudaSuccess || !ke.fn_tables) return e;
+    std::lock_guard<std::mutex> lock(g_context_mu);
+    ContextRecord r;
+    e = read_record(r, stream);
+    return e == cudaSuccess ? fill_tables(ke, log2n, r, stream) : e;
 }
 }  // namespace isr
 
@@ -105,42 +143,76 @@ bool is_device_ptr(const void* p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// Host copies of the plans' status words: slots of one pinned page, taken and given back by plans of any
-// thread and device.  A pinned allocation per plan would cost 0.2 ms at each creation; the page is made
-// by the first plan and stays, and a plan that finds no slot free allocates its own word.
-struct StatusPool {
+// Host copies of the plans' status words: slots of one pinned page per context, taken and given back by
+// plans of any thread.  A pinned allocation per plan would cost 0.2 ms at each creation; the page (4 KB) is
+// made by the context's first plan and goes with the context, and a plan that finds no slot free allocates
+// its own word.  The context's record names its page by an id that no other page of the process has, so
+// a page that went with its context is never written again.
+struct StatusPage {
     static constexpr int kSlots = 1024;
-    std::mutex mu;
-    int* page = nullptr;
+    int* words = nullptr;
     std::vector<int> free_slots;
-    cudaError_t take(int** out)
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        if (!page) {
-            const cudaError_t e = cudaHostAlloc(&page, kSlots * sizeof(int), cudaHostAllocPortable);
-            if (e != cudaSuccess) {
-                page = nullptr;
-                return e;
-            }
-            for (int i = kSlots; i-- > 0;) free_slots.push_back(i);
-        }
-        if (free_slots.empty()) return cudaHostAlloc(out, sizeof(int), cudaHostAllocPortable);
-        *out = page + free_slots.back();
-        free_slots.pop_back();
-        return cudaSuccess;
-    }
-    void give(int* w)
-    {
-        if (!w) return;
-        std::lock_guard<std::mutex> lock(mu);
-        if (page && w >= page && w < page + kSlots) free_slots.push_back((int)(w - page));
-        else cudaFreeHost(w);
-    }
 };
-StatusPool& status_pool()
+struct StatusSlot {
+    unsigned long long pool = 0;   // 0: the word is an allocation of its own
+    int* word = nullptr;
+};
+std::map<unsigned long long, StatusPage>& status_pages()   // under g_context_mu
 {
-    static StatusPool* pool = new StatusPool();   // never destroyed: plans may outlive static destructors
-    return *pool;
+    static auto* pages = new std::map<unsigned long long, StatusPage>();   // plans may outlive static destructors
+    return *pages;
+}
+
+// A slot of the current context, whose record is r (under g_context_mu).
+cudaError_t take_status(StatusSlot& out, isr::ContextRecord& r, cudaStream_t stream)
+{
+    if (r.pool == 0) {
+        static unsigned long long last_id = 0;
+        StatusPage page;
+        cudaError_t e = cudaHostAlloc(&page.words, StatusPage::kSlots * sizeof(int), cudaHostAllocPortable);
+        if (e != cudaSuccess) return e;
+        for (int i = StatusPage::kSlots; i-- > 0;) page.free_slots.push_back(i);
+        r.pool = ++last_id;
+        e = cudaMemcpyToSymbolAsync(isr::g_context, &r.pool, sizeof(r.pool), offsetof(isr::ContextRecord, pool),
+                                    cudaMemcpyHostToDevice, stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+        if (e != cudaSuccess) {
+            cudaFreeHost(page.words);
+            return e;
+        }
+        status_pages()[r.pool] = std::move(page);
+    }
+    StatusPage& page = status_pages()[r.pool];
+    if (page.free_slots.empty()) return cudaHostAlloc(&out.word, sizeof(int), cudaHostAllocPortable);
+    out.pool = r.pool;
+    out.word = page.words + page.free_slots.back();
+    page.free_slots.pop_back();
+    return cudaSuccess;
+}
+
+void give_status(const StatusSlot& s)
+{
+    if (!s.word) return;
+    if (s.pool == 0) {
+        cudaFreeHost(s.word);
+        return;
+    }
+    std::lock_guard<std::mutex> lock(isr::g_context_mu);
+    StatusPage& page = status_pages()[s.pool];
+    page.free_slots.push_back((int)(s.word - page.words));
+}
+
+// What a plan needs of its context: the kernels' attributes and tables, and a status slot.
+cudaError_t enter_context(const isr::KernelEntry& ke, int log2n, cudaStream_t stream, StatusSlot& slot)
+{
+    cudaError_t e = isr::set_attributes(ke);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(isr::g_context_mu);
+    isr::ContextRecord r;
+    e = isr::read_record(r, stream);
+    if (e == cudaSuccess) e = isr::fill_tables(ke, log2n, r, stream);
+    if (e == cudaSuccess) e = take_status(slot, r, stream);
+    return e;
 }
 
 // s + x with the rounding error carried in c (Kahan compensated summation, FP32)
@@ -302,7 +374,7 @@ struct isr_plan {
     bool captured = false;
     int ipp_chunk = 0;
     int* status = nullptr;       // device word, bit 0 = timed-out wait
-    int* host_status = nullptr;  // its copy in pinned host memory
+    StatusSlot host_status;      // its copy in pinned host memory
     float* out_stage = nullptr;  // [R][N] for host readback
     int64_t n_ipp_total = 0;
     int64_t launches = 0;
@@ -637,8 +709,6 @@ isr_status isr_plan_create(isr_plan** out, const isr_plan_desc* desc)
     const int smem = std::max(p->ke.smem, p->ke.smem_xt);
     if (smem > smem_optin)
         return bail(fail(ISR_ERR_UNSUPPORTED, "kernel needs %d B shared memory, device allows %d", smem, smem_optin));
-    e = isr::prepare_entry(p->ke, lg, dev, p->stream);
-    if (e != cudaSuccess) return bail(fail(ISR_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e)));
 
     const int64_t RN = (int64_t)d.n_ranges * d.nfft;
     int64_t mc = d.max_chunks > 0 ? d.max_chunks : std::min<int64_t>(64, std::max<int64_t>(1, kScratchBudget / (RN * 4)));
@@ -651,7 +721,6 @@ isr_status isr_plan_create(isr_plan** out, const isr_plan_desc* desc)
     if (e == cudaSuccess) e = cudaMalloc(&p->partial, (size_t)(mc * RN * 4));
     if (e == cudaSuccess) e = cudaMalloc(&p->status, (size_t)(16 + p->sign_rows * sign_row));
     if (e == cudaSuccess) p->signs = p->sign_rows ? reinterpret_cast<uint32_t*>(p->status + 4) : nullptr;
-    if (e == cudaSuccess) e = status_pool().take(&p->host_status);
 #ifdef ISR_DEBUG
     if (e == cudaSuccess) e = cudaMalloc(&p->phase, 5 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemsetAsync(p->phase, 0, 5 * sizeof(unsigned long long), p->stream);
@@ -663,8 +732,10 @@ isr_status isr_plan_create(isr_plan** out, const isr_plan_desc* desc)
     }
     e = cudaMemsetAsync(p->acc, 0, (size_t)(RN * 8), p->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(p->status, 0, sizeof(int), p->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);
-    if (e != cudaSuccess) return bail(fail(ISR_ERR_CUDA, "initialisation failed: %s", cudaGetErrorString(e)));
+    if (e == cudaSuccess) e = enter_context(p->ke, lg, p->stream, p->host_status);   // waits for the stream
+    if (e != cudaSuccess)
+        return bail(fail(e == cudaErrorMemoryAllocation ? ISR_ERR_NO_MEMORY : ISR_ERR_CUDA, "initialisation failed: %s",
+                         cudaGetErrorString(e)));
     *out = p;
     return ISR_OK;
 }
@@ -727,14 +798,14 @@ isr_status isr_spectra(isr_plan* p, float* out, int32_t flags, int64_t* n_ipp_ou
         const bool v4 = reinterpret_cast<uintptr_t>(dst) % 16 == 0, from_acc = !p->acc_zero || p->captured;
         auto* k = from_acc ? (v4 ? spectra_kernel<true, true> : spectra_kernel<true, false>)
                            : (v4 ? spectra_kernel<false, true> : spectra_kernel<false, false>);
-        k<<<blocks, threads, 0, p->stream>>>(p->partial, p->pending, RN, p->acc, scale, sc, dst, p->status, p->host_status);
+        k<<<blocks, threads, 0, p->stream>>>(p->partial, p->pending, RN, p->acc, scale, sc, dst, p->status, p->host_status.word);
         CUDA_TRY(cudaGetLastError());
         if (!dev_out) CUDA_TRY(cudaMemcpyAsync(out, dst, (size_t)(RN * 4), cudaMemcpyDeviceToHost, p->stream));
     } else {
-        CUDA_TRY(cudaMemcpyAsync(p->host_status, p->status, sizeof(int), cudaMemcpyDeviceToHost, p->stream));
+        CUDA_TRY(cudaMemcpyAsync(p->host_status.word, p->status, sizeof(int), cudaMemcpyDeviceToHost, p->stream));
     }
     CUDA_TRY(cudaStreamSynchronize(p->stream));
-    const int status = *p->host_status;
+    const int status = *p->host_status.word;
     harvest_events(p);
     if (n_ipp_out) *n_ipp_out = p->n_ipp_total;
     if (flags & ISR_RESET_AFTER) {
@@ -837,16 +908,10 @@ isr_status isr_plan_test_drop_window(isr_plan* p, int32_t ipp)
 // ---------------------------------------------------------------- allocation-free variant
 namespace {
 
-// IPP-chunk partials of isr_integrate_static: [chunks][n_ranges][nfft] floats, plus the
-// variant's own status word.  Host code must not use these names as addresses (they are
-// host-side shadows); it looks up each device's copy with cudaGetSymbolAddress.
+// IPP-chunk partials of isr_integrate_static: [chunks][n_ranges][nfft] floats.  Host code must not use
+// this name as an address (it is a host-side shadow); each call looks up its context's copy with
+// cudaGetSymbolAddress.
 __device__ __align__(256) float g_static_scratch[ISR_STATIC_SCRATCH_FLOATS];
-__device__ __align__(16) int g_static_status[4];
-
-constexpr int kMaxDevices = 64;
-std::mutex g_static_mu;
-float* g_static_scratch_ptr[kMaxDevices] = {};
-int* g_static_status_ptr[kMaxDevices] = {};
 
 // out[i] = (float) sum_c part[c][i] (first block of IPPs) or (float)(out[i] + sum_c part[c][i])
 // (later blocks), summed in double: one FP32 rounding of the running sum per block
@@ -860,25 +925,19 @@ __global__ void reduce_to_spectra_kernel(const float* __restrict__ part, int n_c
     }
 }
 
-// device addresses of the file-scope arrays on `dev` (looked up once per device)
-isr_status static_buffers(int dev, float** scratch, int** status)
+// device addresses of the scratch and the status word on the current device
+isr_status static_buffers(float** scratch, int** status)
 {
-    if (dev < 0 || dev >= kMaxDevices) return fail(ISR_ERR_UNSUPPORTED, "device ordinal %d out of range", dev);
-    std::lock_guard<std::mutex> lock(g_static_mu);
-    if (!g_static_scratch_ptr[dev]) {
-        void* a = nullptr;
-        void* b = nullptr;
-        cudaError_t e = cudaGetSymbolAddress(&a, g_static_scratch);
-        if (e == cudaSuccess) e = cudaGetSymbolAddress(&b, g_static_status);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return fail(ISR_ERR_CUDA, "cudaGetSymbolAddress: %s", cudaGetErrorString(e));
-        }
-        g_static_scratch_ptr[dev] = static_cast<float*>(a);
-        g_static_status_ptr[dev] = static_cast<int*>(b);
+    void* a = nullptr;
+    void* b = nullptr;
+    cudaError_t e = cudaGetSymbolAddress(&a, g_static_scratch);
+    if (e == cudaSuccess) e = cudaGetSymbolAddress(&b, isr::g_context);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return fail(ISR_ERR_CUDA, "cudaGetSymbolAddress: %s", cudaGetErrorString(e));
     }
-    *scratch = g_static_scratch_ptr[dev];
-    *status = g_static_status_ptr[dev];
+    *scratch = static_cast<float*>(a);
+    *status = &static_cast<isr::ContextRecord*>(b)->static_status;
     return ISR_OK;
 }
 
@@ -923,7 +982,7 @@ isr_status isr_integrate_static(const isr_plan_desc* desc, const int16_t* echo, 
     if (!guard.ok) return fail(ISR_ERR_CUDA, "cannot select CUDA device %d", dev);
     float* scratch = nullptr;
     int* status = nullptr;
-    st = static_buffers(dev, &scratch, &status);
+    st = static_buffers(&scratch, &status);
     if (st != ISR_OK) return st;
 
     int lg = 0;
@@ -932,7 +991,14 @@ isr_status isr_integrate_static(const isr_plan_desc* desc, const int16_t* echo, 
     int sm_count = 0;
     CUDA_TRY(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev));
     cudaStream_t stream = static_cast<cudaStream_t>(d.stream);
-    CUDA_TRY(isr::prepare_entry(ke, lg, dev, stream));
+    // Whether this context has the tables of this length comes back with the status.  Where this process
+    // has seen them on the device, a call does without the look before (about 10 us): in a context made
+    // anew since, it finds out at the end, fills them and runs once more.
+    static std::atomic<uint32_t> seen[64];   // bit log2n per device
+    std::atomic<uint32_t>* hint = dev < 64 ? &seen[dev] : nullptr;
+    if (!hint || !(hint->load() >> lg & 1u)) CUDA_TRY(isr::prepare_entry(ke, lg, stream));
+    else CUDA_TRY(isr::set_attributes(ke));
+    if (hint) hint->fetch_or(1u << lg);
 
     // Chunks: FP32 sums of at most kDefaultChunk IPPs (the bound the per-bin tolerance rests
     // on), at most c_cap of them in the scratch at once.  The IPPs run in blocks of at most
@@ -942,11 +1008,12 @@ isr_status isr_integrate_static(const isr_plan_desc* desc, const int16_t* echo, 
     const int64_t c_cap = std::min<int64_t>(65535, ISR_STATIC_SCRATCH_FLOATS / RN);
     const int64_t block_cap = c_cap * kDefaultChunk;
 
-    CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int), stream));
     const int cb = chip_bytes(d.tx_type);
     const int threads = 256;
     const int64_t blocks = std::min<int64_t>((RN + threads - 1) / threads, (int64_t)sm_count * 8);
+    isr::ContextRecord rec;
     for (int64_t done = 0; done < n_ipp;) {
+        if (done == 0) CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int), stream));
         const int64_t n_l = std::min<int64_t>(n_ipp - done, block_cap);
         const int64_t c_min = (n_l + kDefaultChunk - 1) / kDefaultChunk;
         int64_t C = isr::pick_chunks(n_l, rg, sm_count, c_min, c_cap, RN);
@@ -973,10 +1040,14 @@ isr_status isr_integrate_static(const isr_plan_desc* desc, const int16_t* echo, 
         reduce_to_spectra_kernel<<<(unsigned)blocks, threads, 0, stream>>>(scratch, (int)C, RN, out, done > 0);
         CUDA_TRY(cudaGetLastError());
         done += n_l;
+        if (done < n_ipp) continue;
+        CUDA_TRY(isr::read_record(rec, stream));
+        if (ke.fn_tables && !(rec.tables >> lg & 1u)) {
+            CUDA_TRY(isr::prepare_entry(ke, lg, stream));
+            done = 0;
+        }
     }
-    int flag = 0;
-    CUDA_TRY(cudaMemcpyAsync(&flag, status, sizeof(int), cudaMemcpyDeviceToHost, stream));
-    CUDA_TRY(cudaStreamSynchronize(stream));
+    const int flag = rec.static_status;
     if (flag & 2)
         return fail(ISR_ERR_OUT_OF_RANGE, "a kernel found a gate window outside its echo row (debug build check)");
     if (flag) return fail(ISR_ERR_TIMEOUT, "a kernel timed out waiting for its staged echo window");
@@ -1008,7 +1079,7 @@ void isr_destroy(isr_plan* p)
     cudaFree(p->acc);
     cudaFree(p->partial);
     cudaFree(p->status);
-    status_pool().give(p->host_status);
+    give_status(p->host_status);
     cudaFree(p->phase);
     cudaFree(p->out_stage);
     cudaGetLastError();

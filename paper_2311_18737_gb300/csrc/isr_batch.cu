@@ -433,7 +433,7 @@ isr_status isr_batch_create(isr_batch** out, const isr_window* windows, int32_t 
         if (cudaStreamCreateWithFlags(&b->side[l], cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&b->join[l], cudaEventDisableTiming) != cudaSuccess)
             return bail(fail(ISR_ERR_CUDA, "stream creation failed"));
-        e = isr::prepare_entry(b->ke[l], kMinLog2 + l, dev, b->cap_stream);
+        e = isr::prepare_entry(b->ke[l], kMinLog2 + l, b->cap_stream);
         if (e != cudaSuccess) return bail(fail(ISR_ERR_CUDA, "kernel preparation: %s", cudaGetErrorString(e)));
     }
 

@@ -113,9 +113,9 @@ inline KernelEntry kernel_entry(int log2n, int txt)
     return entry_16384(txt);
 }
 
-// Ready the entry's kernels on the current device `dev` (once per plan): opt them into their shared
-// memory and fill the twiddle tables if that has not happened on this device (synchronises `stream` then).
-cudaError_t prepare_entry(const KernelEntry& ke, int log2n, int dev, cudaStream_t stream);
+// Ready the entry's kernels on the current device (once per plan): opt them into their shared memory and
+// fill the twiddle tables if its context does not have them (synchronises `stream`).
+cudaError_t prepare_entry(const KernelEntry& ke, int log2n, cudaStream_t stream);
 
 // whether launch_integrate takes the tensor-memory kernel: for every code and order that has no kernel of
 // its own, which only the orders 1-5 and 7-9 of full-length binary phase have

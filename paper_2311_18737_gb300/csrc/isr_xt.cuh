@@ -191,7 +191,7 @@ struct SchedX {
 };
 
 // The twiddle groups as the threads of a CTA keep them, [group][half][128 blk + 32 s + lane]: the same for
-// every launch, filled once per device (xt_tables_kernel), so that a CTA starts with a few loads
+// every launch, filled once per context (xt_tables_kernel), so that a CTA starts with a few loads
 // instead of some forty sines and thirty quotients per thread (a launch of 8 gates x 1 IPP at nfft 16384:
 // 17.9 us formed in the kernel, 14.0 us loaded).
 template <int LOG2N>
