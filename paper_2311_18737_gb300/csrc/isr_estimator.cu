@@ -2658,7 +2658,8 @@ struct isr_est {
     bool conv05 = false;                      // BF16 convolutions on tcgen05 (else mma.sync)
     int sms = 0;                              // multiprocessors of the device
     int* pidx = nullptr;
-    float* da[4] = {};                    // masked gradients [B][32][L]: of h4 .. h1 (tcgen05 engine), else two in turn
+    float* da[4] = {};                    // masked gradients [da_rows][32][L]: of h4 .. h1 (tcgen05 engine), else two in turn
+    int da_rows = 0;                      // rows they hold: max_batch, or fewer on the tcgen05 engine
     // tcgen05 engine: ReLU masks of h1..h3 as written by a training forward pass, [3][B][L] words,
     // bit co of word (b, i) set when h_l[b][co][i] > 0 as stored
     uint32_t* hbits = nullptr;
@@ -2834,35 +2835,39 @@ isr_status backward_t(isr_est* e, int n, const float* fpos, const float* pres)
     if constexpr (kTensorConv<T>) {
         if (e->conv05) {
             const int nxi = (L + FI_P - 1) / FI_P;
-            FiBwdArgs a{};
-            a.h4 = act[4];
-            a.wt = static_cast<const T*>(e->tb);
-            a.theta = e->theta;
-            a.z = e->z;
-            a.scal = e->hscal;
-            a.dpool = e->dpool;
-            a.amax = e->amax;
-            for (int i = 0; i < 3; ++i) a.bits[i] = e->hbits + (size_t)(2 - i) * e->max_batch * L;
-            for (int i = 0; i < 4; ++i) a.da[i] = e->da[i];
-            a.grad = e->grad;
-            a.L = L;
-            a.n_rows = n;
-            a.nx = nxi;
-            backward_kernel<<<std::min(e->sms, n * nxi), FB_SLOTS * FI_ST, FB_SMEM, s>>>(a);
-            const int chunks = n * ((L + W5_CHUNK - 1) / W5_CHUNK), spans = n * ((L + W1_SPAN - 1) / W1_SPAN);
-            W5Args wa{};
-            for (int i = 0; i < W5_LAYERS; ++i) {
-                wa.h[i] = act[3 - i];
-                wa.da[i] = e->da[i];
-                wa.dW[i] = e->grad + w_off(4 - i);
-                wa.db[i] = e->grad + b_off(4 - i);
+            for (int r0 = 0; r0 < n; r0 += e->da_rows) {   // rows r0 .. r0 + rows - 1
+                const int rows = std::min(e->da_rows, n - r0);
+                const size_t at = (size_t)r0 * L;
+                FiBwdArgs a{};
+                a.h4 = act[4] + at * CH;
+                a.wt = static_cast<const T*>(e->tb);
+                a.theta = e->theta;
+                a.z = e->z + at;
+                a.scal = e->hscal + (size_t)r0 * HB_SCAL;
+                a.dpool = e->dpool + (size_t)r0 * 2 * CH;
+                a.amax = e->amax + (size_t)r0 * CH;
+                for (int i = 0; i < 3; ++i) a.bits[i] = e->hbits + (size_t)(2 - i) * e->max_batch * L + at;
+                for (int i = 0; i < 4; ++i) a.da[i] = e->da[i];
+                a.grad = e->grad;
+                a.L = L;
+                a.n_rows = rows;
+                a.nx = nxi;
+                backward_kernel<<<std::min(e->sms, rows * nxi), FB_SLOTS * FI_ST, FB_SMEM, s>>>(a);
+                const int chunks = rows * ((L + W5_CHUNK - 1) / W5_CHUNK), spans = rows * ((L + W1_SPAN - 1) / W1_SPAN);
+                W5Args wa{};
+                for (int i = 0; i < W5_LAYERS; ++i) {
+                    wa.h[i] = act[3 - i] + at * CH;
+                    wa.da[i] = e->da[i];
+                    wa.dW[i] = e->grad + w_off(4 - i);
+                    wa.db[i] = e->grad + b_off(4 - i);
+                }
+                wa.L = L;
+                wa.n_rows = rows;
+                wa.drain = (chunks + std::max(1, e->sms) - 1) / std::max(1, e->sms);
+                wgrad_tc05_kernel<<<std::min(W5_LAYERS * chunks, std::max(W5_LAYERS, e->sms)), W5_BLOCK, W5_SMEM_LAUNCH, s>>>(wa);
+                wgrad1_kernel<T><<<std::min(spans, 2 * std::max(1, e->sms)), 256, 0, s>>>(act[0] + at, e->da[3], L, rows,
+                                                                                         e->grad + OFF_W1, e->grad + OFF_B1);
             }
-            wa.L = L;
-            wa.n_rows = n;
-            wa.drain = (chunks + std::max(1, e->sms) - 1) / std::max(1, e->sms);
-            wgrad_tc05_kernel<<<std::min(W5_LAYERS * chunks, std::max(W5_LAYERS, e->sms)), W5_BLOCK, W5_SMEM_LAUNCH, s>>>(wa);
-            wgrad1_kernel<T><<<std::min(spans, 2 * std::max(1, e->sms)), 256, 0, s>>>(act[0], e->da[3], L, n,
-                                                                                     e->grad + OFF_W1, e->grad + OFF_B1);
             EST_TRY(cudaGetLastError());
             return ISR_OK;
         }
@@ -2980,8 +2985,22 @@ isr_status isr_est_create(isr_est** out, int32_t nfft, int32_t band_lo, int32_t 
     A((void**)&e->dpool, 4 * B * 2 * CH);
     A((void**)&e->zmax, 4 * B * nxh);
     A((void**)&e->zidx, 4 * B * nxh);
-    for (int i = 0; i < (e->conv05 ? 4 : 2); ++i) A((void**)&e->da[i], 4 * B * CH * L);
     if (e->conv05) A((void**)&e->hbits, 4 * 3 * B * L);
+    // the tcgen05 engine's backward pass takes as many rows at a time as four gradient buffers fit for: all
+    // of them, or where memory is short a half (the two full buffers that the other engines need), and so on
+    const int n_da = e->conv05 ? 4 : 2;
+    e->da_rows = max_batch;
+    while (r == cudaSuccess) {
+        for (int i = 0; i < n_da; ++i) A((void**)&e->da[i], (size_t)4 * e->da_rows * CH * L);
+        if (r != cudaErrorMemoryAllocation || !e->conv05 || e->da_rows == 1) break;
+        cudaGetLastError();
+        for (int i = 0; i < n_da; ++i) {
+            cudaFree(e->da[i]);
+            e->da[i] = nullptr;
+        }
+        e->da_rows = (e->da_rows + 1) / 2;
+        r = cudaSuccess;
+    }
     if (r == cudaSuccess) r = cudaMemset(e->theta, 0, 4 * NPARAM);
     if (r == cudaSuccess) r = cudaMemset(e->m, 0, 4 * NPARAM);
     if (r == cudaSuccess) r = cudaMemset(e->v, 0, 4 * NPARAM);

@@ -330,3 +330,42 @@ def test_fp32_weight_gradients_round_no_worse_than_their_rows(B, L):
     for name in ("W2", "W3", "W4"):
         err = np.linalg.norm(gd[name] - rd[name]) / np.linalg.norm(rd[name])
         assert err <= 1.5e-7, f"{name}: relative error {err:.2e}"
+
+
+@pytest.mark.parametrize("L", [4608, 4601])
+def test_bf16_gradients_where_memory_holds_two_gradient_buffers(L):
+    """With device memory for the activations and two full gradient buffers, but not four, a tcgen05
+    estimator is still created, and its gradient, taken in two halves of the rows (the second ragged), is
+    that of one with memory for all, at the bound of the gradient tests against the reference (1e-3 of
+    each block's largest)."""
+    B, n = 256, 251
+    rng = np.random.default_rng(13)
+    arrays = [torch.from_numpy(a).cuda() for a in (rng.standard_normal((n, L)).astype(np.float32),
+                                                   rng.uniform(3, L - 3, n).astype(np.float32),
+                                                   (rng.random(n) < 0.8).astype(np.float32))]
+    theta = ref.init_params(3).astype(np.float32)
+
+    def grad():
+        e = est_mod.Estimator(max_batch=B, precision=isr.ISR_EST_BF16, nfft=L, band_lo=0, band_len=L)
+        e.set_params(theta)
+        out = e.grad(*arrays)
+        e.close()
+        return out
+
+    loss, g = grad()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    row = 2 * L * (1 + 4 * 32) + 4 * L * 4 + 12 * 32 * (L // 488 + 1)      # activations, masks, logits, statistics
+    one = 4 * 32 * L * B                                                    # a full gradient buffer
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - (row * B + 2 * one + one), dtype=torch.uint8, device="cuda")
+    try:
+        loss2, g2 = grad()
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+    assert abs(loss2 - loss) <= 1e-6 * abs(loss)
+    gd, rd = ref.unpack(g2.astype(np.float64)), ref.unpack(g.astype(np.float64))
+    gmax = np.abs(g).max()
+    for name, _ in ref.SHAPES:
+        scale = max(np.abs(rd[name]).max(), 1e-3 * gmax)
+        assert np.abs(gd[name] - rd[name]).max() <= 1e-3 * scale, name
