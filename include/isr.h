@@ -312,6 +312,13 @@ isr_status isr_est_train_step(isr_est* est, const float* x, int32_t n, const flo
 isr_status isr_est_predict(isr_est* est, const float* x, int32_t n, float* line_bin, float* presence);
 /* The same for any number of rows, more than max_batch in as few launches as the estimator's buffers allow. */
 isr_status isr_est_predict_all(isr_est* est, const float* x, int64_t n, float* line_bin, float* presence);
+/* The tcgen05 kernels (ISR_EST_BF16) wait for their tensor-core products with a bound.  Where one runs out,
+ * the results of that call are incomplete (a train step leaves the parameters as they were), and a call
+ * that synchronises (isr_est_grad, isr_est_train_step with a loss, isr_est_get_params) returns
+ * ISR_ERR_TIMEOUT, or the next prediction or train step does, which then does nothing else.
+ * Test hook: the following calls leave out the products of `pass` (0 forward, 1 backward, 2 weight
+ * gradient; -1 turns the hook off), and every wait ends after `polls` polls. */
+isr_status isr_est_test_drop_products(isr_est* est, int32_t pass, uint32_t polls);
 void isr_est_destroy(isr_est* est);
 
 /*

@@ -780,6 +780,21 @@ __global__ void __launch_bounds__(256, 4) wgrad_tc_kernel(const __nv_bfloat16* _
 // registers) and M = 64 with tap 8 as a fifth product, for no padding rows (+19 us: as many cycles per
 // MMA), gave nothing.
 // one arrival (release semantics at CTA scope) on the barrier's current phase
+// Bounded waits of the tcgen05 kernels on their products.  One that runs out ends the work of its threads:
+// they note it, wait once more for what is in flight (with the same bound) and give the tensor memory back;
+// the host reports it.
+struct EstWait {
+    unsigned limit;   // polls
+    int* status;      // device word
+    int* host;        // pinned host word
+};
+__device__ __forceinline__ void est_timed_out(const EstWait& w)
+{
+    atomicOr(w.status, 1);
+    *static_cast<volatile int*>(w.host) = 1;
+    __threadfence_system();
+}
+
 __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
@@ -796,6 +811,7 @@ struct W5Args {
     const float* da[W5_LAYERS];
     float *dW[W5_LAYERS], *db[W5_LAYERS];
     int L, n_rows, drain;   // chunks between drains of the accumulators
+    EstWait wait;
 };
 using W5X = C5<2>;                               // activation tile: 256 + 8 rows, 4 planes
 static_assert(W5X::CT == W5_CHUNK, "activation tile matches the chunk");
@@ -815,6 +831,7 @@ static_assert((size_t)2 * W5_ABUF + W5X::PART + 3 * W5X::PLANE + (W5_CHUNK - 16)
 // ... and the 9 real taps stay inside their plane (rows < XW)
 static_assert((W5_CHUNK - 16) + 15 + (KT - 1) < W5X::XW, "real taps read staged rows only");
 
+template <bool DROP>
 __global__ void __launch_bounds__(W5_BLOCK, 1) wgrad_tc05_kernel(const __grid_constant__ W5Args args)
 {
     // CTAs are dealt to the layers in turn
@@ -833,6 +850,7 @@ __global__ void __launch_bounds__(W5_BLOCK, 1) wgrad_tc05_kernel(const __grid_co
     uint64_t* mbar = reinterpret_cast<uint64_t*>(w5_smem + 2 * W5_ABUF + 2 * W5X::PART);   // [2]
     uint64_t* full = mbar + 2;                                                              // [2]
     uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 4);
+    uint64_t* drained = mbar + 5;   // everything issued completed, where a wait ran out
     float* sum = reinterpret_cast<float*>(mbar + 8);
     __shared__ float db_s[CH];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -844,6 +862,7 @@ __global__ void __launch_bounds__(W5_BLOCK, 1) wgrad_tc05_kernel(const __grid_co
     if (tid == 0) {
         isr::mbar_init(isr::smem_u32(&mbar[0]), 1);
         isr::mbar_init(isr::smem_u32(&mbar[1]), 1);
+        isr::mbar_init(isr::smem_u32(drained), 1);
         isr::mbar_init(isr::smem_u32(&full[0]), W5_THREADS / 32);
         isr::mbar_init(isr::smem_u32(&full[1]), W5_THREADS / 32);
     }
@@ -944,13 +963,13 @@ __global__ void __launch_bounds__(W5_BLOCK, 1) wgrad_tc05_kernel(const __grid_co
         int left = args.drain + 1;
         for (int c = 0; c < nch; ++c) {
             if (left-- == 0) {   // chunk c - 2 ended a segment: drain it under the next one's MMAs
-                ok = isr::mbar_wait(isr::smem_u32(&mbar[c & 1]), (uint32_t)((c - 2) >> 1) & 1u, 1u << 26);
+                ok = isr::mbar_wait(isr::smem_u32(&mbar[c & 1]), (uint32_t)((c - 2) >> 1) & 1u, args.wait.limit);
                 if (!ok) break;
                 drain();
                 left = args.drain - 1;
             }
             load(c, v);
-            if (c >= 2 && !isr::mbar_wait(isr::smem_u32(&mbar[c & 1]), (uint32_t)((c - 2) >> 1) & 1u, 1u << 26)) {
+            if (c >= 2 && !isr::mbar_wait(isr::smem_u32(&mbar[c & 1]), (uint32_t)((c - 2) >> 1) & 1u, args.wait.limit)) {
                 ok = false;
                 break;
             }
@@ -974,10 +993,11 @@ __global__ void __launch_bounds__(W5_BLOCK, 1) wgrad_tc05_kernel(const __grid_co
                 left = args.drain;
                 set = tbase + (set == tbase ? W5_DCOLS : 0);
             }
-            if (!isr::mbar_wait(isr::smem_u32(&full[c & 1]), (uint32_t)(c >> 1) & 1u, 1u << 26)) {
+            if (!isr::mbar_wait(isr::smem_u32(&full[c & 1]), (uint32_t)(c >> 1) & 1u, args.wait.limit)) {
                 ok = false;
                 break;
             }
+            if constexpr (DROP) continue;
             isr::tmem_fence_after_sync();
             // descriptors built once per chunk; K-step s adds two blocks of eight positions to the
             // 16-byte-unit start fields (addresses stay below 0x40000 B: the field never carries)
@@ -996,16 +1016,21 @@ __global__ void __launch_bounds__(W5_BLOCK, 1) wgrad_tc05_kernel(const __grid_co
             }
             isr::tc05_commit(isr::smem_u32(&mbar[c & 1]));
         }
+        if (!ok) {
+            isr::tc05_commit(isr::smem_u32(drained));
+            isr::mbar_wait(isr::smem_u32(drained), 0u, args.wait.limit);
+        }
     }
     if (warp < W5_THREADS / 32) {   // the four lanes of a channel
         for (int o = 8; o < 32; o <<= 1) dbacc += __shfl_xor_sync(0xffffffffu, dbacc, o);
         if (lane < 8) atomicAdd(&db_s[co], dbacc);
     }
     // the last commit covers every MMA of this CTA; a thread whose wait ran out skips it
-    if (nch > 0 && ok) ok = isr::mbar_wait(isr::smem_u32(&mbar[(nch - 1) & 1]), (uint32_t)((nch - 1) >> 1) & 1u, 1u << 26);
+    if (nch > 0 && ok) ok = isr::mbar_wait(isr::smem_u32(&mbar[(nch - 1) & 1]), (uint32_t)((nch - 1) >> 1) & 1u, args.wait.limit);
     isr::tmem_fence_before_sync();
     ok = __syncthreads_and(ok) != 0;
     isr::tmem_fence_after_sync();
+    if (!ok && tid == 0) est_timed_out(args.wait);
     if (ok && warp < W5_THREADS / 32) {
         while ((seg + 1) * args.drain < nch) drain();   // the segment before the last may end one chunk earlier
         take([&](int o, float d) {
@@ -1799,7 +1824,8 @@ __device__ __forceinline__ void fi_mask_to_rows(uint32_t* __restrict__ bits, int
 }
 
 struct FiFwdSlot {
-    uint64_t mbar;
+    uint64_t mbar, drained;
+    int last;            // tiles end here; 0 once a wait ran out
     float zm[4];
     int zi[4];
     float mx[4][CH], sum[4][CH];
@@ -1831,9 +1857,11 @@ struct FiFwdArgs {
     int *pidx, *zidx;
     __nv_bfloat16* h[4];       // training: h1 .. h4
     uint32_t* bits[3];         // training: ReLU masks of h1 .. h3
+    EstWait wait;
 };
 
-template <bool TRAIN>
+// DROP (test hook, here and below): no products are issued, so that the waits for them run out
+template <bool TRAIN, bool DROP>
 __global__ void __launch_bounds__(fi_slots<TRAIN>() * FI_ST, 1) forward_kernel(const __grid_constant__ FiFwdArgs a)
 {
     constexpr int SLOTS = fi_slots<TRAIN>(), NT = SLOTS * FI_ST;
@@ -1848,7 +1876,11 @@ __global__ void __launch_bounds__(fi_slots<TRAIN>() * FI_ST, 1) forward_kernel(c
     const uint32_t mbar = isr::smem_u32(&sl.mbar);
     const int L = a.L, nx = a.nx;
 
-    if (st == 0) isr::mbar_init(mbar, 1);
+    if (st == 0) {
+        isr::mbar_init(mbar, 1);
+        isr::mbar_init(isr::smem_u32(&sl.drained), 1);
+        sl.last = a.n_rows * a.nx;
+    }
     isr::fence_barrier_init();
     if (tid < 32) isr::tmem_alloc(isr::smem_u32(&sh.tslot), fi_cols(SLOTS));
     fi_stage_weights<NT>(smem, a.wt, tid);
@@ -1880,9 +1912,13 @@ __global__ void __launch_bounds__(fi_slots<TRAIN>() * FI_ST, 1) forward_kernel(c
         }
     };
     uint32_t phase = 0;
+    auto stop = [&]() {   // a wait ran out: this is the slot's last tile
+        sl.last = 0;
+        est_timed_out(a.wait);
+    };
     int tile = slot * gridDim.x + blockIdx.x;   // what is left after full rounds goes to different SMs
     if (tile < n_tiles) load_x(tile);
-    for (; tile < n_tiles; tile += step) {
+    for (; tile < sl.last; tile += step) {
         const int b = tile / nx, xc = tile - b * nx, i0 = xc * FI_P, end = min(i0 + FI_P, L);
 #pragma unroll
         for (int k = 0; k < XPER; ++k) {
@@ -1943,7 +1979,7 @@ __global__ void __launch_bounds__(fi_slots<TRAIN>() * FI_ST, 1) forward_kernel(c
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         inf = fi_slot_or(slot, inf);
-        if (st == 0) fi_issue<1>(tacc, mbar, buf, smem, inf);
+        if (!DROP && st == 0) fi_issue<1>(tacc, mbar, buf, smem, inf);
         // relu(accumulator + bias) of layer l + 2, as stored
         auto outputs = [&](int l, int g, FiQuad& q) {
             float v[4][GC];
@@ -1961,7 +1997,7 @@ __global__ void __launch_bounds__(fi_slots<TRAIN>() * FI_ST, 1) forward_kernel(c
         // ---- layers 2 and 3
 #pragma unroll 1
         for (int l = 0; l < 2; ++l) {
-            const bool done = isr::mbar_wait(mbar, phase, 1u << 26);
+            if (!isr::mbar_wait(mbar, phase, a.wait.limit)) stop();
             phase ^= 1u;
             isr::tmem_fence_after_sync();
             const int pos = i0 - 8 + 4 * l + 4 * r;
@@ -1972,7 +2008,7 @@ __global__ void __launch_bounds__(fi_slots<TRAIN>() * FI_ST, 1) forward_kernel(c
                 outputs(l, g, q[g]);
 #pragma unroll
                 for (int p = 0; p < 4; ++p) {
-                    const uint32_t in = done ? inside(pos + p) : 0u;
+                    const uint32_t in = inside(pos + p);
 #pragma unroll
                     for (int k = 0; k < GC / 2; ++k) {
                         q[g][p][k] &= in;
@@ -1985,7 +2021,7 @@ __global__ void __launch_bounds__(fi_slots<TRAIN>() * FI_ST, 1) forward_kernel(c
             isr::tmem_fence_before_sync();
             inf = fi_slot_or(slot, fi_inf2(top));
             isr::tmem_fence_after_sync();
-            if (st == 0) fi_issue<1>(tacc, mbar, buf, smem + (l + 1) * FI_WLAYER, inf);
+            if (!DROP && st == 0) fi_issue<1>(tacc, mbar, buf, smem + (l + 1) * FI_WLAYER, inf);
             if constexpr (TRAIN) {   // beside the next layer's MMAs
                 if (const int n = owned(pos)) {
                     uint32_t mask[4] = {0u, 0u, 0u, 0u};
@@ -2000,10 +2036,10 @@ __global__ void __launch_bounds__(fi_slots<TRAIN>() * FI_ST, 1) forward_kernel(c
         }
         // ---- layer 4 stays in registers: the logits (lower channels first, the order of head_chunk_kernel)
         // and the head's statistics
-        const bool done = isr::mbar_wait(mbar, phase, 1u << 26);
+        if (!isr::mbar_wait(mbar, phase, a.wait.limit)) stop();
         phase ^= 1u;
         isr::tmem_fence_after_sync();
-        const int pos = i0 + 4 * r, n_own = done ? owned(pos) : 0;
+        const int pos = i0 + 4 * r, n_own = owned(pos);
         auto logits = [&](int g, const FiQuad& q, float (&s)[4]) {
 #pragma unroll
             for (int c4 = 0; c4 < GC / 4; ++c4) {
@@ -2151,6 +2187,10 @@ __global__ void __launch_bounds__(fi_slots<TRAIN>() * FI_ST, 1) forward_kernel(c
                 a.zidx[(size_t)b * nx + xc] = at;
             }
         }
+    }
+    if (sl.last == 0 && st == 0) {   // what was issued meanwhile completes before the tensor memory goes
+        isr::tc05_commit(isr::smem_u32(&sl.drained));
+        isr::mbar_wait(isr::smem_u32(&sl.drained), 0u, a.wait.limit);
     }
     isr::tmem_fence_before_sync();
     __syncthreads();
@@ -2440,8 +2480,10 @@ struct FiBwdArgs {
     float* da[4];              // masked gradients of h4 .. h1
     float* grad;
     int L, n_rows, nx;
+    EstWait wait;
 };
 
+template <bool DROP>
 __global__ void __launch_bounds__(FB_SLOTS * FI_ST, 1) backward_kernel(const __grid_constant__ FiBwdArgs a)
 {
     constexpr int NT = FB_SLOTS * FI_ST;
@@ -2505,7 +2547,8 @@ __global__ void __launch_bounds__(FB_SLOTS * FI_ST, 1) backward_kernel(const __g
 #pragma unroll
     for (int c = 0; c < HC; ++c) dw5[c] = 0.f;
     uint32_t phase = 0;
-    for (int tile = slot * gridDim.x + blockIdx.x; tile < n_tiles; tile += step) {
+    bool failed = false;   // a wait of this slot's threads ran out
+    for (int tile = slot * gridDim.x + blockIdx.x; tile < n_tiles && !failed; tile += step) {
         const int b = tile / nx, xc = tile - b * nx, i0 = xc * FI_P, end = min(i0 + FI_P, L);
         auto owned = [&](int pos) { return pos >= i0 && pos < end ? min(4, end - pos) : 0; };
         auto inside = [&](int pos) { return pos >= 0 && pos < L; };
@@ -2569,7 +2612,7 @@ __global__ void __launch_bounds__(FB_SLOTS * FI_ST, 1) backward_kernel(const __g
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         bool inf = fi_slot_or(slot, fi_inf2(top));
-        if (st == 0) fi_issue<2>(tacc, mbar, buf, fb_smem + 2 * FI_WLAYER, inf);
+        if (!DROP && st == 0) fi_issue<2>(tacc, mbar, buf, fb_smem + 2 * FI_WLAYER, inf);
         // ---- layers 4, 3, 2: gradients of h3, h2, h1
 #pragma unroll 1
         for (int l = 0; l < 3; ++l) {
@@ -2586,7 +2629,7 @@ __global__ void __launch_bounds__(FB_SLOTS * FI_ST, 1) backward_kernel(const __g
                 for (int p = 0; p < 4; ++p)
                     if (inside(pos + p)) m[p] = mb[p];
             }
-            const bool done = isr::mbar_wait(mbar, phase, 1u << 26);
+            const bool done = isr::mbar_wait(mbar, phase, a.wait.limit);
             phase ^= 1u;
             isr::tmem_fence_after_sync();
             top = 0u;
@@ -2598,16 +2641,24 @@ __global__ void __launch_bounds__(FB_SLOTS * FI_ST, 1) backward_kernel(const __g
                 for (int p = 0; p < 4; ++p)
 #pragma unroll
                     for (int c = 0; c < GC; ++c)
-                        v[p][c] = done && (m[p] >> (HC * half + GC * g + c) & 1u) ? v[p][c] : 0.f;
+                        v[p][c] = m[p] >> (HC * half + GC * g + c) & 1u ? v[p][c] : 0.f;
                 to_rows(a.da[l + 1], b, pos, n_own, g, v);
                 if (l < 2) to_planes(g, v, top);
             }
             isr::tmem_fence_before_sync();
             if (l < 2) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            inf = fi_slot_or(slot, fi_inf2(top));
+            inf = fi_slot_or(slot, fi_inf2(top) || !done);
+            if (inf) {   // one of the two, both of them rare
+                if ((failed = fi_slot_or(slot, !done))) break;
+                inf = fi_slot_or(slot, fi_inf2(top));
+            }
             isr::tmem_fence_after_sync();
-            if (l < 2 && st == 0) fi_issue<2>(tacc, mbar, buf, fb_smem + (1 - l) * FI_WLAYER, inf);
+            if (!DROP && l < 2 && st == 0) fi_issue<2>(tacc, mbar, buf, fb_smem + (1 - l) * FI_WLAYER, inf);
         }
+    }
+    if (failed) {
+        if (st == 0) est_timed_out(a.wait);
+        isr::mbar_wait(mbar, phase ^ 1u, a.wait.limit);
     }
     const float d5 = fi_scatter(dw5, lane, [](float u, float v) { return u + v; });
     if ((lane & 1) == 0) atomicAdd(&a.grad[OFF_W5 + HC * half + (lane >> 1)], d5);
@@ -2621,9 +2672,12 @@ __global__ void __launch_bounds__(FB_SLOTS * FI_ST, 1) backward_kernel(const __g
     if (tid < 32) isr::tmem_dealloc(sh.tslot, fi_cols(FB_SLOTS));
 }
 
+// status: set where the gradient is incomplete (tcgen05 engine; else NULL), which then leaves everything as it was
 __global__ void adam_kernel(float* __restrict__ theta, const float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, int n, float lr, float b1, float b2, float eps, float c1, float c2)
+                            float* __restrict__ v, int n, float lr, float b1, float b2, float eps, float c1, float c2,
+                            const int* __restrict__ status)
 {
+    if (status && *status) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const float gi = g[i];
         const float mi = b1 * m[i] + (1.f - b1) * gi;
@@ -2663,6 +2717,11 @@ struct isr_est {
     // tcgen05 engine: ReLU masks of h1..h3 as written by a training forward pass, [3][B][L] words,
     // bit co of word (b, i) set when h_l[b][co][i] > 0 as stored
     uint32_t* hbits = nullptr;
+    // tcgen05 engine: whether a bounded wait ran out, in device memory and in pinned host memory
+    int *status = nullptr, *host_status = nullptr;
+    unsigned wait_limit = 1u << 26;       // polls
+    int drop_pass = -1;                   // test hook: the pass that leaves out its products
+    EstWait wait() const { return EstWait{wait_limit, status, host_status}; }
 };
 
 namespace {
@@ -2699,17 +2758,20 @@ isr_status set_smem_attrs()
         EST_TRY(cudaFuncSetAttribute(conv_kernel<false, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_smem_bytes(16)));
         EST_TRY(cudaFuncSetAttribute(conv_kernel<false, 12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_smem_bytes(12)));
     } else {
-        EST_TRY(cudaFuncSetAttribute(backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FB_SMEM));
-        EST_TRY(cudaFuncSetAttribute(forward_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fi_smem<false>()));
-        EST_TRY(cudaFuncSetAttribute(forward_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, fi_smem<true>()));
+        for (auto* k : {backward_kernel<false>, backward_kernel<true>})
+            EST_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, FB_SMEM));
+        for (auto* k : {forward_kernel<false, false>, forward_kernel<false, true>})
+            EST_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, fi_smem<false>()));
+        for (auto* k : {forward_kernel<true, false>, forward_kernel<true, true>})
+            EST_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, fi_smem<true>()));
         EST_TRY(cudaFuncSetAttribute(conv_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)tc_smem_bytes(true)));
         EST_TRY(cudaFuncSetAttribute(conv_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)tc_smem_bytes(false)));
         EST_TRY(cudaFuncSetAttribute(wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)wgrad_tc_smem_bytes()));
-        EST_TRY(cudaFuncSetAttribute(wgrad_tc05_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)W5_SMEM_LAUNCH));
+        for (auto* k : {wgrad_tc05_kernel<false>, wgrad_tc05_kernel<true>})
+            EST_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W5_SMEM_LAUNCH));
     }
     return ISR_OK;
 }
@@ -2782,17 +2844,20 @@ isr_status forward_t(isr_est* e, const float* x, int n, float* pos = nullptr, fl
             a.zmax = e->zmax;
             a.pidx = e->pidx;
             a.zidx = e->zidx;
+            a.wait = e->wait();
             if (pos) {
                 HeadArgs ha = head_args(e, nxi, pos, pres);
                 if (n > e->max_batch) place_head(e, n, nxi, ha, a);
-                forward_kernel<false><<<std::min(e->sms, tiles), fi_slots<false>() * FI_ST, fi_smem<false>(), s>>>(a);
+                auto* k = e->drop_pass == 0 ? forward_kernel<false, true> : forward_kernel<false, false>;
+                k<<<std::min(e->sms, tiles), fi_slots<false>() * FI_ST, fi_smem<false>(), s>>>(a);
                 head_mlp_kernel<true><<<n, HM_THREADS, 0, s>>>(ha);
             } else {
                 // the weight gradient of the first layer reads x as stored
                 cast_kernel<T><<<(unsigned)std::min<size_t>((nx + 255) / 256, 4096), 256, 0, s>>>(x, nx, act[0]);
                 for (int l = 0; l < 4; ++l) a.h[l] = act[l + 1];
                 for (int l = 0; l < 3; ++l) a.bits[l] = e->hbits + (size_t)l * e->max_batch * L;
-                forward_kernel<true><<<std::min(e->sms, tiles), fi_slots<true>() * FI_ST, fi_smem<true>(), s>>>(a);
+                auto* k = e->drop_pass == 0 ? forward_kernel<true, true> : forward_kernel<true, false>;
+                k<<<std::min(e->sms, tiles), fi_slots<true>() * FI_ST, fi_smem<true>(), s>>>(a);
                 head_mlp_kernel<false><<<n, HM_THREADS, 0, s>>>(head_args(e, nxi, nullptr, nullptr));
             }
             EST_TRY(cudaGetLastError());
@@ -2852,7 +2917,8 @@ isr_status backward_t(isr_est* e, int n, const float* fpos, const float* pres)
                 a.L = L;
                 a.n_rows = rows;
                 a.nx = nxi;
-                backward_kernel<<<std::min(e->sms, rows * nxi), FB_SLOTS * FI_ST, FB_SMEM, s>>>(a);
+                a.wait = e->wait();
+                (e->drop_pass == 1 ? backward_kernel<true> : backward_kernel<false>)<<<std::min(e->sms, rows * nxi), FB_SLOTS * FI_ST, FB_SMEM, s>>>(a);
                 const int chunks = rows * ((L + W5_CHUNK - 1) / W5_CHUNK), spans = rows * ((L + W1_SPAN - 1) / W1_SPAN);
                 W5Args wa{};
                 for (int i = 0; i < W5_LAYERS; ++i) {
@@ -2863,8 +2929,9 @@ isr_status backward_t(isr_est* e, int n, const float* fpos, const float* pres)
                 }
                 wa.L = L;
                 wa.n_rows = rows;
+                wa.wait = e->wait();
                 wa.drain = (chunks + std::max(1, e->sms) - 1) / std::max(1, e->sms);
-                wgrad_tc05_kernel<<<std::min(W5_LAYERS * chunks, std::max(W5_LAYERS, e->sms)), W5_BLOCK, W5_SMEM_LAUNCH, s>>>(wa);
+                (e->drop_pass == 2 ? wgrad_tc05_kernel<true> : wgrad_tc05_kernel<false>)<<<std::min(W5_LAYERS * chunks, std::max(W5_LAYERS, e->sms)), W5_BLOCK, W5_SMEM_LAUNCH, s>>>(wa);
                 wgrad1_kernel<T><<<std::min(spans, 2 * std::max(1, e->sms)), 256, 0, s>>>(act[0] + at, e->da[3], L, rows,
                                                                                          e->grad + OFF_W1, e->grad + OFF_B1);
             }
@@ -2913,6 +2980,17 @@ bool dev_ptr(const void* p)
         return false;
     }
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+}
+
+// ISR_ERR_TIMEOUT, once, if a kernel since the last report gave up waiting.  Between calls it may come late
+// (the kernel may still run), after a synchronisation it does not.
+isr_status check_waits(isr_est* e)
+{
+    if (!e->host_status || *static_cast<volatile int*>(e->host_status) == 0) return ISR_OK;
+    EST_TRY(cudaMemsetAsync(e->status, 0, sizeof(int), e->stream));
+    EST_TRY(cudaStreamSynchronize(e->stream));
+    *static_cast<volatile int*>(e->host_status) = 0;
+    return fail(ISR_ERR_TIMEOUT, "an estimator kernel timed out waiting for its tensor-core products");
 }
 
 isr_status check_batch(isr_est* e, const float* x, int n)
@@ -2985,7 +3063,13 @@ isr_status isr_est_create(isr_est** out, int32_t nfft, int32_t band_lo, int32_t 
     A((void**)&e->dpool, 4 * B * 2 * CH);
     A((void**)&e->zmax, 4 * B * nxh);
     A((void**)&e->zidx, 4 * B * nxh);
-    if (e->conv05) A((void**)&e->hbits, 4 * 3 * B * L);
+    if (e->conv05) {
+        A((void**)&e->hbits, 4 * 3 * B * L);
+        A((void**)&e->status, sizeof(int));
+        if (r == cudaSuccess) r = cudaMemset(e->status, 0, sizeof(int));
+        if (r == cudaSuccess) r = cudaHostAlloc((void**)&e->host_status, sizeof(int), cudaHostAllocPortable);
+        if (r == cudaSuccess) *e->host_status = 0;
+    }
     // the tcgen05 engine's backward pass takes as many rows at a time as four gradient buffers fit for: all
     // of them, or where memory is short a half (the two full buffers that the other engines need), and so on
     const int n_da = e->conv05 ? 4 : 2;
@@ -3047,7 +3131,7 @@ isr_status isr_est_get_params(isr_est* e, float* params)
     Dev guard(e->dev);
     EST_TRY(cudaMemcpyAsync(params, e->theta, 4 * NPARAM, cudaMemcpyDefault, e->stream));
     EST_TRY(cudaStreamSynchronize(e->stream));
-    return ISR_OK;
+    return check_waits(e);
 }
 
 isr_status isr_est_features(isr_est* e, const float* spectra, int32_t n, float* x)
@@ -3074,7 +3158,7 @@ isr_status isr_est_grad(isr_est* e, const float* x, int32_t n, const float* line
     if (grad) EST_TRY(cudaMemcpyAsync(grad, e->grad, 4 * NPARAM, cudaMemcpyDefault, e->stream));
     if (loss) EST_TRY(cudaMemcpyAsync(loss, e->loss, 4, cudaMemcpyDefault, e->stream));
     EST_TRY(cudaStreamSynchronize(e->stream));
-    return ISR_OK;
+    return check_waits(e);
 }
 
 isr_status isr_est_train_step(isr_est* e, const float* x, int32_t n, const float* line_bin, const float* present,
@@ -3084,6 +3168,8 @@ isr_status isr_est_train_step(isr_est* e, const float* x, int32_t n, const float
     if (st != ISR_OK) return st;
     if (!line_bin || !present || !(lr > 0.f)) return fail(ISR_ERR_INVALID_ARG, "labels NULL or lr <= 0");
     Dev guard(e->dev);
+    st = check_waits(e);
+    if (st != ISR_OK) return st;
     st = e->precision != ISR_EST_FP32 ? forward_t<__nv_bfloat16>(e, x, n) : forward_t<float>(e, x, n);
     if (st == ISR_OK)
         st = e->precision != ISR_EST_FP32 ? backward_t<__nv_bfloat16>(e, n, line_bin, present)
@@ -3093,12 +3179,13 @@ isr_status isr_est_train_step(isr_est* e, const float* x, int32_t n, const float
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f / (1.f - powf(b1, (float)e->step)), c2 = 1.f / (1.f - powf(b2, (float)e->step));
     adam_kernel<<<(NPARAM + 255) / 256, 256, 0, e->stream>>>(e->theta, e->grad, e->m, e->v, NPARAM, lr, b1, b2, 1e-8f,
-                                                              c1, c2);
+                                                              c1, c2, e->status);
     e->weights_stale = true;
     EST_TRY(cudaGetLastError());
     if (loss) {
         EST_TRY(cudaMemcpyAsync(loss, e->loss, 4, cudaMemcpyDefault, e->stream));
         EST_TRY(cudaStreamSynchronize(e->stream));
+        return check_waits(e);
     }
     return ISR_OK;
 }
@@ -3109,6 +3196,8 @@ isr_status isr_est_predict(isr_est* e, const float* x, int32_t n, float* line_bi
     if (st != ISR_OK) return st;
     if (!line_bin || !presence) return fail(ISR_ERR_INVALID_ARG, "outputs must not be NULL");
     Dev guard(e->dev);
+    st = check_waits(e);
+    if (st != ISR_OK) return st;
     return e->precision != ISR_EST_FP32 ? forward_t<__nv_bfloat16>(e, x, n, line_bin, presence)
                                         : forward_t<float>(e, x, n, line_bin, presence);
 }
@@ -3120,6 +3209,7 @@ isr_status isr_est_predict_all(isr_est* e, const float* x, int64_t n, float* lin
     if (n < 1) return fail(ISR_ERR_INVALID_ARG, "n must be >= 1");
     if (!line_bin || !presence) return fail(ISR_ERR_INVALID_ARG, "outputs must not be NULL");
     Dev guard(e->dev);
+    st = check_waits(e);
     const int most = e->conv05 ? predict_rows(e) : e->max_batch;
     for (int64_t done = 0; done < n && st == ISR_OK; done += most) {
         const int rows = (int)std::min<int64_t>(most, n - done);
@@ -3130,6 +3220,15 @@ isr_status isr_est_predict_all(isr_est* e, const float* x, int64_t n, float* lin
     return st;
 }
 
+isr_status isr_est_test_drop_products(isr_est* e, int32_t pass, uint32_t polls)
+{
+    if (!e || pass < -1 || pass > 2 || (pass >= 0 && polls == 0))
+        return fail(ISR_ERR_INVALID_ARG, "estimator is NULL, pass not in -1..2 or polls is 0");
+    e->drop_pass = pass;
+    e->wait_limit = pass >= 0 ? polls : 1u << 26;
+    return ISR_OK;
+}
+
 void isr_est_destroy(isr_est* e)
 {
     if (!e) return;
@@ -3137,8 +3236,9 @@ void isr_est_destroy(isr_est* e)
     cudaStreamSynchronize(e->stream);
     void* ptrs[] = {e->theta, e->m, e->v, e->grad, e->wcopies, e->wf, e->wb, e->tf, e->tb, e->act[0], e->act[1], e->act[2], e->act[3],
                     e->act[4], e->z, e->pooled, e->u, e->q, e->loss, e->amax, e->da[0], e->da[1], e->da[2], e->da[3],
-                    e->pmax, e->pidx, e->psum, e->hscal, e->dpool, e->zmax, e->zidx, e->hbits};
+                    e->pmax, e->pidx, e->psum, e->hscal, e->dpool, e->zmax, e->zidx, e->hbits, e->status};
     for (void* p : ptrs) cudaFree(p);
+    cudaFreeHost(e->host_status);
     cudaGetLastError();
     delete e;
 }

@@ -37,7 +37,7 @@ STATUS_NAMES = {0: "ISR_OK", 1: "ISR_ERR_INVALID_ARG", 2: "ISR_ERR_UNSUPPORTED",
 EXPORTS = ("isr_plan_create", "isr_integrate", "isr_spectra", "isr_plan_query", "isr_plan_set_profiling",
            "isr_plan_set_wait_limit", "isr_plan_set_order", "isr_plan_set_precision", "isr_plan_test_drop_window", "isr_destroy", "isr_last_error",
            "isr_integrate_static", "isr_peak_fit", "isr_fp32_peak", "isr_tc05_rate", "isr_plan_phase_cycles", "isr_est_create", "isr_est_set_params", "isr_est_get_params",
-           "isr_est_features", "isr_est_grad", "isr_est_train_step", "isr_est_predict", "isr_est_predict_all", "isr_est_destroy",
+           "isr_est_features", "isr_est_grad", "isr_est_train_step", "isr_est_predict", "isr_est_predict_all", "isr_est_test_drop_products", "isr_est_destroy",
            "isr_batch_create", "isr_batch_run", "isr_batch_wait", "isr_batch_query", "isr_batch_destroy")
 
 # radix orders of isr_plan_set_order (4..8 at nfft 16384 with binary-phase codes only)
@@ -187,6 +187,7 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.isr_est_train_step.argtypes = [P, P, ctypes.c_int32, P, P, ctypes.c_float, P]
     lib.isr_est_predict.argtypes = [P, P, ctypes.c_int32, P, P]
     lib.isr_est_predict_all.argtypes = [P, P, ctypes.c_int64, P, P]
+    lib.isr_est_test_drop_products.argtypes = [P, ctypes.c_int32, ctypes.c_uint32]
     lib.isr_est_destroy.argtypes = [P]
     lib.isr_est_destroy.restype = None
     lib.isr_batch_create.argtypes = [ctypes.POINTER(P), ctypes.POINTER(IsrWindow), ctypes.c_int32, ctypes.c_int32,
@@ -358,6 +359,11 @@ def isr_est_predict(est, x, n: int, line_bin, presence) -> None:
 def isr_est_predict_all(est, x, n: int, line_bin, presence) -> None:
     _check(load_library().isr_est_predict_all(est, _addr(x), int(n), _addr(line_bin), _addr(presence)),
            "isr_est_predict_all")
+
+
+def isr_est_test_drop_products(est, which: int, polls: int) -> None:
+    """Test hook: products of pass ``which`` are left out, so that a bounded wait runs out (-1: off)."""
+    _check(load_library().isr_est_test_drop_products(est, int(which), int(polls)), "isr_est_test_drop_products")
 
 
 def isr_est_destroy(est) -> None:

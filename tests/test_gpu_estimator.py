@@ -369,3 +369,39 @@ def test_bf16_gradients_where_memory_holds_two_gradient_buffers(L):
     for name, _ in ref.SHAPES:
         scale = max(np.abs(rd[name]).max(), 1e-3 * gmax)
         assert np.abs(gd[name] - rd[name]).max() <= 1e-3 * scale, name
+
+
+@pytest.mark.parametrize("which", [0, 1, 2])
+def test_bounded_waits_for_products_are_reported(which):
+    """Products left out in the forward pass, the backward pass or the weight gradient: the wait
+    for them runs out and the call, or the next one, reports it instead of returning incomplete numbers; a
+    train step leaves the parameters alone; afterwards everything works as before."""
+    e, theta, x, f, y, (xd, fd, yd) = _dyadic_case(L=600, seed=12)
+    want_pos, want_pres = (t.clone() for t in e.predict(xd))
+    want_loss, want = e.grad(xd, fd, yd)
+
+    def times_out(call):
+        with pytest.raises(isr.IsrError) as ei:
+            call()
+        assert ei.value.status == isr.ISR_ERR_TIMEOUT
+
+    isr.isr_est_test_drop_products(e.h, which, 20000)
+    times_out(lambda: e.grad(xd, fd, yd))
+    times_out(lambda: e.train_step(xd, fd, yd, 1e-2, want_loss=True))
+    e.train_step(xd, fd, yd, 1e-2)
+    times_out(e.get_params)
+    if which == 0:
+        e.predict(xd)
+        torch.cuda.synchronize()
+        times_out(lambda: e.predict(xd))
+    isr.isr_est_test_drop_products(e.h, -1, 0)
+    assert np.array_equal(e.get_params(), theta)
+    pos, pres = e.predict(xd)
+    assert torch.equal(pos, want_pos) and torch.equal(pres, want_pres)
+    loss, g = e.grad(xd, fd, yd)
+    assert abs(loss - want_loss) <= 1e-6 * abs(want_loss)
+    assert np.linalg.norm(g - want) <= 1e-5 * np.linalg.norm(want)
+    with pytest.raises(isr.IsrError) as ei:
+        isr.isr_est_test_drop_products(e.h, 3, 1)
+    assert ei.value.status == isr.ISR_ERR_INVALID_ARG
+    e.close()
