@@ -96,3 +96,14 @@ def test_orders_of_full_length_complex_codes(log2n, kind):
         assert tuned["order"] in range(4) and len(tuned["ms"]) == 4
         plan.integrate(e, t, P)
         assert_parity(plan.spectra()[0].numpy().astype(np.float64), ref, what=f"nfft={nfft} {kind} tuned")
+
+
+def test_autotuner_times_each_kernel_once():
+    """Orders 0 and 6 are one kernel: it is timed once, and reported as order 0."""
+    nfft, R, P = 16384, 4, 2
+    echo, tx = _case(7, nfft, R, P, 0, 1, nfft, "pm1", False)
+    e, t = torch.from_numpy(echo).cuda(), torch.from_numpy(tx).cuda()
+    with isr.Plan(nfft=nfft, n_ranges=R, echo_stride=echo.shape[1], range_step=1, device=0,
+                  stream=torch.cuda.current_stream()) as plan:
+        tuned = plan.autotune(e, t, P)
+    assert len(tuned["ms"]) == isr.N_ORDERS and tuned["ms"][6] == tuned["ms"][0] and tuned["order"] != 6
