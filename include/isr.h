@@ -52,7 +52,7 @@ typedef struct {
     int32_t tx_type;     /* isr_tx_type                                                       */
     int64_t echo_stride; /* complex samples per echo row (IPP); multiple of 4                 */
     int64_t tx_stride;   /* chips between per-IPP code rows; 0 = one code for every IPP       */
-    int32_t ipp_chunk;   /* max IPPs summed in FP32 before the FP64 reduction; 0 = 256        */
+    int32_t ipp_chunk;   /* max IPPs in one FP32 partial sum; 0 = 256                         */
     int32_t max_chunks;  /* IPP chunks in flight per launch (scratch = max_chunks * R * nfft
                             floats); 0 = automatic (<= 64, <= 4 GiB)                          */
     int32_t device;      /* CUDA device ordinal; -1 = the calling thread's current device     */
@@ -94,6 +94,9 @@ typedef struct isr_plan isr_plan;
 /*
  * Create a plan: validates the description and allocates, on the plan's device, the
  * persistent [n_ranges][nfft] accumulators (FP64, zeroed) and the IPP-chunk scratch.
+ * Partial sums, of one call or several, wait in the scratch until it is full or read back;
+ * they are added up in FP32 with compensation (about 2 ulp for any number of them), or in
+ * FP64 where a sum leaves the range of FP32, and from a full scratch into the accumulators.
  * The plan owns that memory until isr_destroy.  On failure *out is set to NULL.
  * Errors: ISR_ERR_INVALID_ARG, ISR_ERR_UNSUPPORTED, ISR_ERR_OUT_OF_RANGE (the last gate's
  * window, range_start + (n_ranges-1)*range_step + code_len, exceeds echo_stride),
@@ -137,7 +140,7 @@ isr_status isr_plan_query(const isr_plan* plan, isr_plan_info* info);
 /* Turn per-launch CUDA-event timing of the fused kernel on (1) or off (0). */
 isr_status isr_plan_set_profiling(isr_plan* plan, int32_t enable);
 
-/* Tracing, debug build only (-DISR_DEBUG): the Stockham fused kernels (every nfft; at nfft 16384
+/* Tracing, debug build only (-DISR_DEBUG): the three-pass fused kernels (every nfft; at nfft 16384
  * radix orders 0-2 and 6-8) time the phases of their IPP loop with the SM clock, as seen by
  * thread 0 of each CTA, and add them up over all CTAs and launches of the plan:
  *   out[0] waiting for the staged window + the first barrier, out[1] pass 0 (decode, first DFT,

@@ -7,7 +7,7 @@
 // length, longest first to the CTA with the least work (their cost is known: it goes by IPPs), and
 // run in the fused kernel with its exchange in tensor memory, one launch per transform
 // length on streams of their own, so that an SM that is done with one length starts the next
-// (32 windows with 10-100 IPPs: 22.7 ms from one queue of every shape in one kernel, 18.5 ms so).
+// (32 windows with 10-100 IPPs: 22.7 ms from one queue of every shape in one kernel, 18.1 ms so).
 // Units of the other radix orders form one queue, longest first, from which one CTA per SM
 // pulls with an atomic counter.  The launches and the chunk reduction can be captured once in
 // a CUDA graph and replayed.  The radix order of each transform length can be picked by

@@ -57,7 +57,7 @@ template <> __device__ __forceinline__ __nv_bfloat16 cvt<__nv_bfloat16>(float v)
 // x[i] = (ln max(P[lo+i], 1e-30) - mean) / (std + 1e-6) over the band; one CTA per gate.
 // Bytes bound it (4 in, 4 out per bin), so the logarithm and both moments run in float-float on the
 // FP32 pipe instead of FP64, of which the part has about two operations per SM and clock: 1000 gates
-// x 4608 bins took 618 us with two FP64 logarithms per bin, 38 us now.  The moments are taken about the first
+// x 4608 bins took 618 us with two FP64 logarithms per bin, 32 us now.  The moments are taken about the first
 // bin's logarithm, so the variance loses nothing to cancellation.  A thread keeps the logarithms of
 // up to FT_KEEP bins in registers; bands beyond FT_THREADS x FT_KEEP bins form the rest again in the
 // second pass.  A band with an infinite bin goes through the FP64 form, whose infinities and NaN are

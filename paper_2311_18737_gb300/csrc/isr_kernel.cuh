@@ -1,4 +1,6 @@
-// isr_kernel.cuh -- fused decode -> FFT -> |X|^2 integration kernel for sm_103a.
+// isr_kernel.cuh -- fused decode -> FFT -> |X|^2 integration kernels for sm_103a: all codes below nfft
+// 1024, and from 2048 up the radix orders 1 to 3 and 7 to 9 of binary-phase codes (everything else is in
+// isr_xt.cuh, orders 4 and 5 in isr_paired.cuh).
 //
 // One CTA (512 threads) owns G = 16384 / nfft range gates for one chunk of IPPs (for
 // nfft = 16384: one gate).  Per IPP and gate it
@@ -13,8 +15,8 @@
 //      transform of Sec. 3.2.2);
 //   4. adds |X[f]|^2 into 32 FP32 accumulators per thread that stay in registers for the
 //      whole IPP chunk (Eq. 8, the "spectrum accumulation" kernel of Sec. 3.2.3).
-// At the end of the chunk each thread writes its 32 partial sums once; a separate
-// reduction adds the chunk partials into FP64 accumulators.
+// At the end of the chunk each thread writes its 32 partial sums once; the read-back, or a
+// reduction into FP64 accumulators, sums the chunk partials.
 #pragma once
 
 #include <cstdint>
@@ -31,8 +33,9 @@ enum TxKind { TX_CI16 = 0, TX_C32 = 1, TX_PM1 = 2 };
 constexpr int kThreads = 512;
 
 // ---------------------------------------------------------------- per-size schedule
-// Radix orders of the three-pass sizes (nfft 2048 .. 16384).  ORDER 0 is the default;
-// Plan.autotune and the batched launch time them on the caller's data and pick per size.
+// Radix orders of the three-pass sizes (nfft 2048 .. 16384).  Plan.autotune and the batched launch time
+// them on the caller's data and pick per size; the default, ORDER 0, is isr_xt.cuh's kernel there, and
+// its row gives only the shape (gates per CTA, stage) that all orders share.
 __host__ __device__ constexpr int radix_of(int log2n, int order, int p)
 {
     if (log2n <= 5) return p == 0 ? (1 << log2n) : 1;
@@ -227,7 +230,7 @@ __device__ __forceinline__ float2 iq_of(uint32_t w)
 // Binary-phase codes: CVT picks how a sample's int16 pair becomes floats.  The first passes decode
 // even samples with the conversion instruction and odd ones with the magic-number form below, so
 // that both pipes share the work: at nfft 16384 either form alone took 320-323 ms per
-// integration of the realistic workload (order 6), the split 312.5 ms.
+// integration of 1000 gates x 10,000 IPPs (passes [32, 32, 16]), the split 312.5 ms.
 template <int TXT, bool CVT = false>
 __device__ __forceinline__ float2 decode(uint32_t w, const void* txrow, int pos, uint32_t sbit)
 {
@@ -469,6 +472,7 @@ __device__ __forceinline__ bool integrate_unit(A a, const int gx, const int c, u
     // gates per CTA each gate's threads sync on a named barrier of their own (1 + g), so the
     // gates of a CTA run their passes independently and their FFT and exchange phases overlap
     constexpr bool CTA_SYNC = T > 32;
+    static_assert(LOG2N < 10 || (ORDER > 0 && TXT == TX_PM1), "isr_xt.cuh has order 0 and the other codes");
     static_assert(P0 == P0_SIMT || (LOG2N == 14 && ORDER == 1 && TXT == TX_PM1 && FULL),
                   "the tensor-core first pass exists for nfft 16384, radix order 1, full binary-phase codes");
     uint4* afrag = reinterpret_cast<uint4*>(smem + S::SMEM);   // tensor-core A fragments (mma.sync)

@@ -405,3 +405,17 @@ def test_bounded_waits_for_products_are_reported(which):
         isr.isr_est_test_drop_products(e.h, 3, 1)
     assert ei.value.status == isr.ISR_ERR_INVALID_ARG
     e.close()
+
+
+@pytest.mark.parametrize("L,at", [(16, 0), (700, 699), (5121, 5120), (6000, 17)])
+def test_features_of_a_band_with_an_infinite_bin(L, at):
+    """The mean is infinite and the variance, infinity less infinity, counts as 0: every finite bin gives
+    minus infinity and the infinite one NaN, and other gates of the launch are not touched by it."""
+    rng = np.random.default_rng(L)
+    P = rng.gamma(30.0, 2.0, size=(3, L)).astype(np.float32)
+    P[1, at] = np.inf
+    e = est_mod.Estimator(max_batch=4, precision=isr.ISR_EST_FP32, nfft=L, band_lo=0, band_len=L)
+    x = e.features(torch.from_numpy(P).cuda()).cpu().numpy()
+    e.close()
+    assert np.isnan(x[1, at]) and np.isneginf(np.delete(x[1], at)).all()
+    assert np.abs(x[[0, 2]] - ref.features(P[[0, 2]], 0, L)).max() <= 1e-5
