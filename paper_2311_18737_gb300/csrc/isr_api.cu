@@ -90,6 +90,8 @@ cudaError_t prepare_entry(const KernelEntry& ke, int log2n, cudaStream_t stream)
 {
     cudaError_t e = set_attributes(ke);
     if (e != cudaSuccess || !ke.fn_tables) return e;
+    e = cudaStreamSynchronize(stream);   // not under the lock: what is queued there may take long
+    if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lock(g_context_mu);
     ContextRecord r;
     e = read_record(r, stream);
@@ -206,12 +208,17 @@ void give_status(const StatusSlot& s)
 cudaError_t enter_context(const isr::KernelEntry& ke, int log2n, cudaStream_t stream, StatusSlot& slot)
 {
     cudaError_t e = isr::set_attributes(ke);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);   // not under the lock: what is queued there may take long
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lock(isr::g_context_mu);
     isr::ContextRecord r;
     e = isr::read_record(r, stream);
     if (e == cudaSuccess) e = isr::fill_tables(ke, log2n, r, stream);
-    if (e == cudaSuccess) e = take_status(slot, r, stream);
+    try {
+        if (e == cudaSuccess) e = take_status(slot, r, stream);
+    } catch (const std::bad_alloc&) {
+        e = cudaErrorMemoryAllocation;
+    }
     return e;
 }
 
