@@ -6,7 +6,8 @@ import pytest
 import torch
 
 import oracle
-from gpu_helpers import RTOL, assert_parity
+from gpu_helpers import assert_parity
+from gpu_helpers import RTOL
 from paper_2311_18737_gb300 import isr
 
 pytestmark = pytest.mark.gpu
