@@ -145,20 +145,17 @@ bool is_device_ptr(const void* p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// Host copies of the plans' status words: slots of one pinned page per context, taken and given back by
-// plans of any thread.  A pinned allocation per plan would cost 0.2 ms at each creation; the page (4 KB) is
-// made by the context's first plan and goes with the context, and a plan that finds no slot free allocates
-// its own word.  The context's record names its page by an id that no other page of the process has, so
+// Host words for the status of plans and estimators: slots of one pinned page per context, taken and given
+// back by handles of any thread.  A pinned allocation per handle would cost 0.2 ms at each creation; the
+// page (4 KB) is made by the context's first handle and goes with the context, and a handle that finds no
+// slot free allocates its own word.  The context's record names its page by an id that no other page of the process has, so
 // a page that went with its context is never written again.
 struct StatusPage {
     static constexpr int kSlots = 1024;
     int* words = nullptr;
     std::vector<int> free_slots;
 };
-struct StatusSlot {
-    unsigned long long pool = 0;   // 0: the word is an allocation of its own
-    int* word = nullptr;
-};
+using isr::StatusSlot;
 std::map<unsigned long long, StatusPage>& status_pages()   // under g_context_mu
 {
     static auto* pages = new std::map<unsigned long long, StatusPage>();   // plans may outlive static destructors
@@ -192,28 +189,15 @@ cudaError_t take_status(StatusSlot& out, isr::ContextRecord& r, cudaStream_t str
     return cudaSuccess;
 }
 
-void give_status(const StatusSlot& s)
+// What a handle needs of its context: a status slot and, for a plan, the tables of its kernels (ke).
+cudaError_t enter_context(const isr::KernelEntry* ke, int log2n, cudaStream_t stream, StatusSlot& slot)
 {
-    if (!s.word) return;
-    if (s.pool == 0) {
-        cudaFreeHost(s.word);
-        return;
-    }
-    std::lock_guard<std::mutex> lock(isr::g_context_mu);
-    StatusPage& page = status_pages()[s.pool];
-    page.free_slots.push_back((int)(s.word - page.words));
-}
-
-// What a plan needs of its context: the kernels' attributes and tables, and a status slot.
-cudaError_t enter_context(const isr::KernelEntry& ke, int log2n, cudaStream_t stream, StatusSlot& slot)
-{
-    cudaError_t e = isr::set_attributes(ke);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);   // not under the lock: what is queued there may take long
+    cudaError_t e = cudaStreamSynchronize(stream);   // not under the lock: what is queued there may take long
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lock(isr::g_context_mu);
     isr::ContextRecord r;
     e = isr::read_record(r, stream);
-    if (e == cudaSuccess) e = isr::fill_tables(ke, log2n, r, stream);
+    if (e == cudaSuccess && ke) e = isr::fill_tables(*ke, log2n, r, stream);
     try {
         if (e == cudaSuccess) e = take_status(slot, r, stream);
     } catch (const std::bad_alloc&) {
@@ -221,6 +205,34 @@ cudaError_t enter_context(const isr::KernelEntry& ke, int log2n, cudaStream_t st
     }
     return e;
 }
+}  // namespace
+
+namespace isr {
+// on a stream of its own: the caller's may be busy or in capture
+cudaError_t take_status(StatusSlot& slot)
+{
+    cudaStream_t s = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return e;
+    e = enter_context(nullptr, 0, s, slot);
+    cudaStreamDestroy(s);
+    return e;
+}
+
+void give_status(const StatusSlot& s)
+{
+    if (!s.word) return;
+    if (s.pool == 0) {
+        cudaFreeHost(s.word);
+        return;
+    }
+    std::lock_guard<std::mutex> lock(g_context_mu);
+    StatusPage& page = status_pages()[s.pool];
+    page.free_slots.push_back((int)(s.word - page.words));
+}
+}  // namespace isr
+
+namespace {
 
 // s + x with the rounding error carried in c (Kahan compensated summation, FP32)
 __device__ __forceinline__ void kahan_add(float& s, float& c, float x)
@@ -739,7 +751,8 @@ isr_status isr_plan_create(isr_plan** out, const isr_plan_desc* desc)
     }
     e = cudaMemsetAsync(p->acc, 0, (size_t)(RN * 8), p->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(p->status, 0, sizeof(int), p->stream);
-    if (e == cudaSuccess) e = enter_context(p->ke, lg, p->stream, p->host_status);   // waits for the stream
+    if (e == cudaSuccess) e = isr::set_attributes(p->ke);
+    if (e == cudaSuccess) e = enter_context(&p->ke, lg, p->stream, p->host_status);   // waits for the stream
     if (e != cudaSuccess)
         return bail(fail(e == cudaErrorMemoryAllocation ? ISR_ERR_NO_MEMORY : ISR_ERR_CUDA, "initialisation failed: %s",
                          cudaGetErrorString(e)));
@@ -1086,7 +1099,7 @@ void isr_destroy(isr_plan* p)
     cudaFree(p->acc);
     cudaFree(p->partial);
     cudaFree(p->status);
-    give_status(p->host_status);
+    isr::give_status(p->host_status);
     cudaFree(p->phase);
     cudaFree(p->out_stage);
     cudaGetLastError();

@@ -2718,10 +2718,11 @@ struct isr_est {
     // bit co of word (b, i) set when h_l[b][co][i] > 0 as stored
     uint32_t* hbits = nullptr;
     // tcgen05 engine: whether a bounded wait ran out, in device memory and in pinned host memory
-    int *status = nullptr, *host_status = nullptr;
+    int* status = nullptr;
+    isr::StatusSlot host_status;
     unsigned wait_limit = 1u << 26;       // polls
     int drop_pass = -1;                   // test hook: the pass that leaves out its products
-    EstWait wait() const { return EstWait{wait_limit, status, host_status}; }
+    EstWait wait() const { return EstWait{wait_limit, status, host_status.word}; }
 };
 
 namespace {
@@ -2749,6 +2750,16 @@ struct Dev {
     }
 };
 
+template <bool DROP>
+isr_status set_tc05_attrs()
+{
+    EST_TRY(cudaFuncSetAttribute(forward_kernel<false, DROP>, cudaFuncAttributeMaxDynamicSharedMemorySize, fi_smem<false>()));
+    EST_TRY(cudaFuncSetAttribute(forward_kernel<true, DROP>, cudaFuncAttributeMaxDynamicSharedMemorySize, fi_smem<true>()));
+    EST_TRY(cudaFuncSetAttribute(backward_kernel<DROP>, cudaFuncAttributeMaxDynamicSharedMemorySize, FB_SMEM));
+    EST_TRY(cudaFuncSetAttribute(wgrad_tc05_kernel<DROP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W5_SMEM_LAUNCH));
+    return ISR_OK;
+}
+
 template <class T>
 isr_status set_smem_attrs()
 {
@@ -2758,20 +2769,14 @@ isr_status set_smem_attrs()
         EST_TRY(cudaFuncSetAttribute(conv_kernel<false, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_smem_bytes(16)));
         EST_TRY(cudaFuncSetAttribute(conv_kernel<false, 12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_smem_bytes(12)));
     } else {
-        for (auto* k : {backward_kernel<false>, backward_kernel<true>})
-            EST_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, FB_SMEM));
-        for (auto* k : {forward_kernel<false, false>, forward_kernel<false, true>})
-            EST_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, fi_smem<false>()));
-        for (auto* k : {forward_kernel<true, false>, forward_kernel<true, true>})
-            EST_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, fi_smem<true>()));
+        const isr_status st = set_tc05_attrs<false>();
+        if (st != ISR_OK) return st;
         EST_TRY(cudaFuncSetAttribute(conv_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)tc_smem_bytes(true)));
         EST_TRY(cudaFuncSetAttribute(conv_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)tc_smem_bytes(false)));
         EST_TRY(cudaFuncSetAttribute(wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)wgrad_tc_smem_bytes()));
-        for (auto* k : {wgrad_tc05_kernel<false>, wgrad_tc05_kernel<true>})
-            EST_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W5_SMEM_LAUNCH));
     }
     return ISR_OK;
 }
@@ -2986,10 +2991,10 @@ bool dev_ptr(const void* p)
 // (the kernel may still run), after a synchronisation it does not.
 isr_status check_waits(isr_est* e)
 {
-    if (!e->host_status || *static_cast<volatile int*>(e->host_status) == 0) return ISR_OK;
+    if (!e->host_status.word || *static_cast<volatile int*>(e->host_status.word) == 0) return ISR_OK;
     EST_TRY(cudaMemsetAsync(e->status, 0, sizeof(int), e->stream));
     EST_TRY(cudaStreamSynchronize(e->stream));
-    *static_cast<volatile int*>(e->host_status) = 0;
+    *static_cast<volatile int*>(e->host_status.word) = 0;
     return fail(ISR_ERR_TIMEOUT, "an estimator kernel timed out waiting for its tensor-core products");
 }
 
@@ -3067,8 +3072,8 @@ isr_status isr_est_create(isr_est** out, int32_t nfft, int32_t band_lo, int32_t 
         A((void**)&e->hbits, 4 * 3 * B * L);
         A((void**)&e->status, sizeof(int));
         if (r == cudaSuccess) r = cudaMemset(e->status, 0, sizeof(int));
-        if (r == cudaSuccess) r = cudaHostAlloc((void**)&e->host_status, sizeof(int), cudaHostAllocPortable);
-        if (r == cudaSuccess) *e->host_status = 0;
+        if (r == cudaSuccess) r = isr::take_status(e->host_status);
+        if (r == cudaSuccess) *e->host_status.word = 0;
     }
     // the tcgen05 engine's backward pass takes as many rows at a time as four gradient buffers fit for: all
     // of them, or where memory is short a half (the two full buffers that the other engines need), and so on
@@ -3224,6 +3229,11 @@ isr_status isr_est_test_drop_products(isr_est* e, int32_t pass, uint32_t polls)
 {
     if (!e || pass < -1 || pass > 2 || (pass >= 0 && polls == 0))
         return fail(ISR_ERR_INVALID_ARG, "estimator is NULL, pass not in -1..2 or polls is 0");
+    Dev guard(e->dev);
+    if (pass >= 0) {
+        const isr_status st = set_tc05_attrs<true>();
+        if (st != ISR_OK) return st;
+    }
     e->drop_pass = pass;
     e->wait_limit = pass >= 0 ? polls : 1u << 26;
     return ISR_OK;
@@ -3238,7 +3248,7 @@ void isr_est_destroy(isr_est* e)
                     e->act[4], e->z, e->pooled, e->u, e->q, e->loss, e->amax, e->da[0], e->da[1], e->da[2], e->da[3],
                     e->pmax, e->pidx, e->psum, e->hscal, e->dpool, e->zmax, e->zidx, e->hbits, e->status};
     for (void* p : ptrs) cudaFree(p);
-    cudaFreeHost(e->host_status);
+    isr::give_status(e->host_status);
     cudaGetLastError();
     delete e;
 }

@@ -117,6 +117,14 @@ inline KernelEntry kernel_entry(int log2n, int txt)
 // fill the twiddle tables if its context does not have them (synchronises `stream`).
 cudaError_t prepare_entry(const KernelEntry& ke, int log2n, cudaStream_t stream);
 
+// A word of pinned host memory for a handle's status, from a page that the current context's handles share.
+struct StatusSlot {
+    unsigned long long pool = 0;   // 0: the word is an allocation of its own
+    int* word = nullptr;
+};
+cudaError_t take_status(StatusSlot& slot);
+void give_status(const StatusSlot& slot);
+
 // whether launch_integrate takes the tensor-memory kernel: for every code and order that has no kernel of
 // its own, which only the orders 1-5 and 7-9 of full-length binary phase have
 inline bool takes_xt(const KernelEntry& ke, bool full, int order) { return ke.fn_xt && (!full || !ke.fn_order[order]); }
